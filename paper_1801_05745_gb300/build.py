@@ -25,7 +25,7 @@ NVCC = os.path.join(CUDA_HOME, "bin", "nvcc")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 CU = ["bin.cu", "stats.cu", "sht.cu", "capi.cu"]
 CPP = ["cosmo.cpp", "welford.cpp"]
-HEADERS = ["common.cuh", "pixel.cuh", "ctx.h"]
+HEADERS = ["common.cuh", "packed.cuh", "pixel.cuh", "ctx.h"]
 
 
 def _stale(target: str, deps: list[str]) -> bool:

@@ -29,6 +29,7 @@
 
 #include "common.cuh"
 #include "ctx.h"
+#include "packed.cuh"
 
 namespace ufc {
 
@@ -135,52 +136,7 @@ __device__ __forceinline__ float4 cdf_sub(float4 a, float4 b) {
 }
 __device__ __forceinline__ float4 cdf_conj(float4 a) { return make_float4(a.x, a.y, -a.z, -a.w); }
 
-// Two double-floats side by side in the packed FP32 instructions of sm_100
-// and later (add/sub/mul/fma.rn.f32x2: one issue slot for two correctly
-// rounded FP32 operations).  The Legendre kernels are bound by the FP32 pipe
-// and, with scalar instructions, by the issue slots as well; packing two ring
-// pairs leaves slots for the loads, shuffles and votes around the arithmetic.
-typedef unsigned long long u64;
-__device__ __forceinline__ u64 x2_pack(float a, float b) {
-  u64 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-  return r;
-}
-__device__ __forceinline__ float2 x2_get(u64 v) {
-  float2 r;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-  return r;
-}
-__device__ __forceinline__ u64 x2_add(u64 a, u64 b) {
-  u64 r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ u64 x2_sub(u64 a, u64 b) {
-  u64 r;
-  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ u64 x2_mul(u64 a, u64 b) {
-  u64 r;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ u64 x2_fma(u64 a, u64 b, u64 c) {
-  u64 r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-__device__ __forceinline__ u64 x2_neg(u64 a) { return a ^ 0x8000000080000000ull; }
-struct dfx { u64 h, l; };
 __device__ __forceinline__ dfx dfx_set(dfl a, dfl b) { return {x2_pack(a.h, b.h), x2_pack(a.l, b.l)}; }
-// a + b, the low part not renormalised (the tree sums of k_legendre)
-__device__ __forceinline__ dfx dfx_add_raw(dfx a, dfx b) {
-  const u64 s = x2_add(a.h, b.h);
-  const u64 bb = x2_sub(s, a.h);
-  const u64 er = x2_add(x2_sub(a.h, x2_sub(s, bb)), x2_sub(b.h, bb));
-  return {s, x2_add(er, x2_add(a.l, b.l))};
-}
 // v * f, the exact product of the high parts plus the cross terms (not
 // renormalised); nv = -v.h
 __device__ __forceinline__ dfx dfx_mul_raw(dfx v, dfx f) {

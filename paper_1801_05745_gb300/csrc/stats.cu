@@ -12,6 +12,7 @@
 
 #include "common.cuh"
 #include "ctx.h"
+#include "packed.cuh"
 #include "pixel.cuh"
 
 namespace ufc {
@@ -68,6 +69,13 @@ __device__ __forceinline__ double block_sum_d(double v, double* sh) {
   if (threadIdx.x == 0)
     for (int i = 0; i < NT / 32; ++i) t += sh[i];
   return t;   // valid in thread 0
+}
+
+// Clears the PDF that the moment pass after this kernel adds to (block 0; pdf
+// may be NULL).  One launch less than a memset between the two passes.
+__device__ __forceinline__ void clear_pdf(unsigned long long* pdf, int n) {
+  if (pdf && blockIdx.x == 0)
+    for (int i = threadIdx.x; i < n; i += blockDim.x) pdf[i] = 0ull;
 }
 
 struct Coef {
@@ -152,7 +160,8 @@ struct AdjRow { I128 s[3]; long long n; long long pad_; };
 // aligned.
 __global__ void __launch_bounds__(kKT)
 k_kappa_plain(const int32_t* __restrict__ counts, Coef cf, float* __restrict__ kappa,
-              double* __restrict__ ksum_part) {
+              double* __restrict__ ksum_part, unsigned long long* __restrict__ pdf, int npdf) {
+  clear_pdf(pdf, npdf);
   __shared__ float ah_s[kMaxShells], al_s[kMaxShells];
   __shared__ double red[kKT / 32];
   const int S = cf.nshell;
@@ -213,7 +222,8 @@ __device__ __forceinline__ double kappa_vec_block(const int32_t* __restrict__ co
 
 __global__ void __launch_bounds__(kKV)
 k_kappa_vec(const int32_t* __restrict__ counts, Coef cf, float* __restrict__ kappa,
-            double* __restrict__ ksum_part) {
+            double* __restrict__ ksum_part, unsigned long long* __restrict__ pdf, int npdf) {
+  clear_pdf(pdf, npdf);
   __shared__ float ah_s[kMaxShells], al_s[kMaxShells];
   __shared__ double red[kKV / 32];
   const int S = cf.nshell;
@@ -267,7 +277,9 @@ k_kappa_partial(const int32_t* __restrict__ counts, Coef cf, double* __restrict_
 // the moment pass treats it exactly as a map from the counts.
 __global__ void __launch_bounds__(kKV)
 k_kappa_finish(const double* __restrict__ part, float ch, float cl, int npix,
-               float* __restrict__ kappa, double* __restrict__ ksum_part) {
+               float* __restrict__ kappa, double* __restrict__ ksum_part,
+               unsigned long long* __restrict__ pdf, int npdf) {
+  clear_pdf(pdf, npdf);
   __shared__ double red[kKV / 32];
   const int ng = npix >> 2;
   const f2 mc{-ch, -cl};
@@ -323,7 +335,9 @@ __global__ void __launch_bounds__(NT, 1)
 k_adj_main(const int32_t* __restrict__ counts, Coef cf, const float* __restrict__ g,
            double* __restrict__ rows_out, double* __restrict__ sumpart,
            unsigned long long* range_flag, int s0, float* __restrict__ kappa_out,
-           double* __restrict__ ksum_out, const double* __restrict__ ext) {
+           double* __restrict__ ksum_out, const double* __restrict__ ext,
+           unsigned long long* __restrict__ pdf, int npdf) {
+  if (kappa_out) clear_pdf(pdf, npdf);
   extern __shared__ __align__(16) uint8_t adj_sm[];
   constexpr int T = NT, NW = T / 32, TP = 4 * T;
   int* q_s = reinterpret_cast<int*>(adj_sm);                 // [6][TP] quantised e, e^2, g
@@ -554,7 +568,9 @@ k_adj_main(const int32_t* __restrict__ counts, Coef cf, const float* __restrict_
 // the moments of an arbitrary map (ufc_map_stats).  Needs a 16-byte aligned
 // map of a multiple of 4 values.
 __global__ void __launch_bounds__(kKV)
-k_map_sum(const float* __restrict__ map, int npix, double* __restrict__ ksum_part) {
+k_map_sum(const float* __restrict__ map, int npix, double* __restrict__ ksum_part,
+          unsigned long long* __restrict__ pdf, int npdf) {
+  clear_pdf(pdf, npdf);
   __shared__ double red[kKV / 32];
   const int ng = npix >> 2;
   f2 ks{0.f, 0.f};
@@ -576,7 +592,7 @@ constexpr int kMaxBins = 4096;
 
 struct PdfParam {
   double lo, hi, scale;     // scale = nbins / (hi - lo)
-  float lo_f, scale_f, band_rel;
+  float lo_f, scale_f, band;
   float lo_dn, lo_up, hi_dn, hi_up;   // FP32 brackets of lo and hi
   int32_t nbins;
 };
@@ -586,94 +602,111 @@ struct PdfParam {
 // lane ends with the same value (each pairwise sum is formed by both lanes).
 __device__ __forceinline__ double warp_sum_fixed(const double* v, int n, int stride) {
   double s = 0.0;
-  for (int i = threadIdx.x & 31; i < n; i += 32) s += v[(size_t)i * stride];
+  for (int i = threadIdx.x & 31; i < n; i += 32) s += __ldcg(v + (size_t)i * stride);
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
   return s;
 }
 
-// PDF slot of one FP32 value: floor((k - lo) * scale) in FP64, decided in FP32
-// unless k lies within a proven band of a bin edge; under/overflow and NaN.
+// PDF slot of one FP32 value by the FP64 definition: floor((k - lo) * scale),
+// under/overflow and NaN.  A call of its own: inlined, the compiler evaluates
+// the FP64 expressions for every value (they have no side effects) and selects
+// afterwards, and at GB300's FP64 rate that alone is 200 us for the 12.6 M
+// pixels of Nside 1024.
+__device__ __noinline__ int pdf_slot_exact(float k, double lo, double hi, double scale, int nbins) {
+  if (isnan(k)) return nbins + 2;
+  const double x = (double)k;
+  if (x < lo) return nbins;
+  if (x >= hi) return nbins + 1;
+  const int b = (int)floor(__dmul_rn(__dsub_rn(x, lo), scale));
+  return b >= nbins ? nbins - 1 : (b < 0 ? 0 : b);
+}
+
+// PDF slot of one FP32 value, decided in FP32 where the value lies outside
+// the FP32 neighbours of lo and hi and farther than a proven band from every
+// bin edge, else by the FP64 definition.
 __device__ __forceinline__ int pdf_slot(float k, const PdfParam& pp) {
-  // k < lo and k >= hi decided in FP32 unless k lies between the FP32
-  // neighbours of lo (resp. hi)
-  const bool under = k < pp.lo_dn || (k < pp.lo_up && (double)k < pp.lo);
-  const bool over = k >= pp.hi_up || (k >= pp.hi_dn && (double)k >= pp.hi);
-  if (isnan(k)) return pp.nbins + 2;
-  if (under) return pp.nbins;
-  if (over) return pp.nbins + 1;
-  const float x = (k - pp.lo_f) * pp.scale_f;   // in [-1, nbins + 1] up to rounding
+  const float x = (k - pp.lo_f) * pp.scale_f;
   float xr;
   int b = round_fast(x, xr);
-  if (xr > x) { b -= 1; xr -= 1.0f; }          // floor
-  const float rem = x - xr;
-  const float band = pp.band_rel * (fabsf(x) + 1.0f);
-  if (!(rem >= band && rem < 1.0f - band))
-    b = (int)floor(__dmul_rn(__dsub_rn((double)k, pp.lo), pp.scale));
-  return b >= pp.nbins ? pp.nbins - 1 : (b < 0 ? 0 : b);
+  const float d = x - xr;                       // distance to the nearest edge, signed
+  b = d < 0.f ? b - 1 : b;                      // floor
+  const bool inside = k >= pp.lo_up && k < pp.hi_dn && fabsf(d) >= pp.band;
+  if (inside) return min(max(b, 0), pp.nbins - 1);
+  if (k < pp.lo_dn) return pp.nbins;
+  if (k >= pp.hi_up) return pp.nbins + 1;
+  return pdf_slot_exact(k, pp.lo, pp.hi, pp.scale, pp.nbins);
 }
 
 // One block's share of the moment pass: block vb of a grid of nb blocks of
 // kMT threads (every thread calls it).  Central power sums about `mean` into
-// out[0..2] (valid in thread 0); PDF counts into the shared histogram.
+// out[0..2] (valid in thread 0); PDF counts into the shared histogram.  Two
+// of a thread's pixels at a time, side by side in packed double-float.
 __device__ __forceinline__ void moments_block(const float* __restrict__ kappa, int npix,
                                               double mean, const PdfParam& pp, int vb, int nb,
                                               unsigned int* hist, double* red, double* out) {
   const float mh = (float)mean;
   const float ml = (float)(mean - (double)mh);
-  f2 a2{0.f, 0.f}, a3{0.f, 0.f}, a4{0.f, 0.f};
-  for (int p = vb * kMT + threadIdx.x; p < npix; p += nb * kMT) {
-    const float k = kappa[p];
-    f2 d = f2_add(f2_two_sum(k, -mh), f2{-ml, 0.f});
-    f2 d2 = f2_mul(d, d);
-    a2 = f2_add(a2, d2);
-    a3 = f2_add(a3, f2_mul(d2, d));
-    a4 = f2_add(a4, f2_mul(d2, d2));
-    atomicAdd(hist + pdf_slot(k, pp), 1u);
+  const u64 nmh = x2_pack(-mh, -mh), nml = x2_pack(-ml, -ml);
+  dfx a2{0ull, 0ull}, a3{0ull, 0ull}, a4{0ull, 0ull};
+  auto acc = [](dfx& a, dfx x) { a = dfx_add_raw(a, x); };
+  auto add_pair = [&](float k0, float k1, bool both) {
+    // d = (k - mh) - ml: two exact sums, renormalised
+    const u64 k = x2_pack(k0, k1);
+    const u64 s = x2_add(k, nmh), bb = x2_sub(s, k);
+    const u64 e = x2_add(x2_sub(k, x2_sub(s, bb)), x2_sub(nmh, bb));
+    dfx d = dfx_add_raw(dfx{s, e}, dfx{nml, 0ull});
+    d = dfx_norm(d.h, d.l);
+    if (!both) {                                       // (the second half counts as d = 0)
+      d.h = x2_pack(x2_get(d.h).x, 0.f);
+      d.l = x2_pack(x2_get(d.l).x, 0.f);
+    }
+    const dfx d2 = dfx_mul(d, d);
+    acc(a2, d2);
+    acc(a3, dfx_mul(d2, d));
+    acc(a4, dfx_mul(d2, d2));
+    atomicAdd(hist + pdf_slot(k0, pp), 1u);
+    if (both) atomicAdd(hist + pdf_slot(k1, pp), 1u);
+  };
+  const int step = nb * kMT;
+  int p = vb * kMT + threadIdx.x;
+  for (; p < npix - 3 * step; p += 4 * step) {         // four loads in flight
+    const float k0 = kappa[p], k1 = kappa[p + step], k2 = kappa[p + 2 * step],
+                k3 = kappa[p + 3 * step];
+    add_pair(k0, k1, true);
+    add_pair(k2, k3, true);
   }
-  out[0] = block_sum_d<kMT>(f2_to_d(a2), red);
-  out[1] = block_sum_d<kMT>(f2_to_d(a3), red);
-  out[2] = block_sum_d<kMT>(f2_to_d(a4), red);
+  for (; p < npix; p += 2 * step) {
+    const bool both = p < npix - step;
+    const float k0 = kappa[p], k1 = both ? kappa[p + step] : k0;
+    add_pair(k0, k1, both);
+  }
+  auto total = [](dfx a) {                             // the halves, in FP64
+    const float2 h = x2_get(a.h), l = x2_get(a.l);
+    return ((double)h.x + (double)l.x) + ((double)h.y + (double)l.y);
+  };
+  out[0] = block_sum_d<kMT>(total(a2), red);
+  out[1] = block_sum_d<kMT>(total(a3), red);
+  out[2] = block_sum_d<kMT>(total(a4), red);
 }
 
-__global__ void __launch_bounds__(kMT)
-k_moments(const float* __restrict__ kappa, int npix, const double* __restrict__ ksum_part,
-          int nksum, PdfParam pp, double* __restrict__ part /*[grid][3]*/,
-          unsigned long long* __restrict__ pdf /*[nbins+3]*/) {
-  extern __shared__ unsigned int hist[];   // [nbins + 3]
-  __shared__ double red[kMT / 32];
-  __shared__ double mean_s;
-  for (int i = threadIdx.x; i < pp.nbins + 3; i += blockDim.x) hist[i] = 0;
-  if (threadIdx.x < 32) {
-    const double s = warp_sum_fixed(ksum_part, nksum, 1);   // fixed order
-    if (threadIdx.x == 0) mean_s = s / double(npix);
+// moments[10] from the partial sums, by a block of kMT threads (fixed orders:
+// warp q sums quantity q; thread 0 writes).
+__device__ __forceinline__ void moments_final_block(const double* ksum_part, int nksum,
+                                                    const double* part, int npart, int npix,
+                                                    double* red, double* m) {
+  const int w = threadIdx.x >> 5;
+  __syncthreads();
+  if (w < 4) {
+    // the mean as k_moments forms it, then the power sums
+    const double s = w == 0 ? warp_sum_fixed(ksum_part, nksum, 1)
+                            : warp_sum_fixed(part + (w - 1), npart, 3);
+    if ((threadIdx.x & 31) == 0) red[w] = s;
   }
   __syncthreads();
-  double o[3];
-  moments_block(kappa, npix, mean_s, pp, blockIdx.x, gridDim.x, hist, red, o);
-  if (threadIdx.x == 0) {
-    part[3 * blockIdx.x + 0] = o[0];
-    part[3 * blockIdx.x + 1] = o[1];
-    part[3 * blockIdx.x + 2] = o[2];
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < pp.nbins + 3; i += blockDim.x)
-    if (hist[i]) atomicAdd(pdf + i, (unsigned long long)hist[i]);
-}
-
-// moments[10] from the partial sums (one warp, fixed orders; every lane of
-// warp 0 calls it, lane 0 writes).
-__device__ __forceinline__ void moments_final_warp(const double* ksum_part, int nksum,
-                                                   const double* part, int npart, int npix,
-                                                   double* m) {
-  // the mean as k_moments forms it
-  const double s = warp_sum_fixed(ksum_part, nksum, 1);
-  const double s2 = warp_sum_fixed(part, npart, 3);
-  const double s3 = warp_sum_fixed(part + 1, npart, 3);
-  const double s4 = warp_sum_fixed(part + 2, npart, 3);
   if (threadIdx.x != 0) return;
   const double N = double(npix);
-  const double mu2 = s2 / N, mu3 = s3 / N, mu4 = s4 / N;
-  m[0] = s / N;
+  const double mu2 = red[1] / N, mu3 = red[2] / N, mu4 = red[3] / N;
+  m[0] = red[0] / N;
   m[1] = mu2;
   m[2] = mu3;
   m[3] = mu4;
@@ -690,11 +723,48 @@ __device__ __forceinline__ void moments_final_warp(const double* ksum_part, int 
   m[9] = N;
 }
 
-__global__ void k_moments_final(const double* __restrict__ ksum_part, int nksum,
-                                const double* __restrict__ part, int npart, int npix,
-                                double* __restrict__ m) {
-  if (threadIdx.x >= 32 || blockIdx.x != 0) return;
-  moments_final_warp(ksum_part, nksum, part, npart, npix, m);
+// Blocks of the moment pass: 4 per SM (32 warps; four loads in flight per
+// thread), no more than there are pixels for.  What bounds the pass is the
+// latency of a pixel's chain (load, shared-memory histogram, double-float
+// sums): with 2 blocks per SM and one pixel at a time it took 200 us for the
+// 12.6 M pixels of Nside 1024.
+static int moments_grid(int num_sms, int npix) {
+  return std::min(4 * num_sms, (npix + kMT - 1) / kMT);
+}
+
+// The last block to finish (ticket) turns the partial sums into the moments:
+// one launch less, and nothing waits.  The ticket is left at 0.
+__global__ void __launch_bounds__(kMT)
+k_moments(const float* __restrict__ kappa, int npix, const double* __restrict__ ksum_part,
+          int nksum, PdfParam pp, double* __restrict__ part /*[grid][3]*/,
+          unsigned long long* __restrict__ pdf /*[nbins+3]*/, double* __restrict__ m,
+          unsigned int* __restrict__ ticket) {
+  extern __shared__ unsigned int hist[];   // [nbins + 3]
+  __shared__ double red[kMT / 32];
+  __shared__ double mean_s;
+  __shared__ bool last_s;
+  for (int i = threadIdx.x; i < pp.nbins + 3; i += blockDim.x) hist[i] = 0;
+  if (threadIdx.x < 32) {
+    const double s = warp_sum_fixed(ksum_part, nksum, 1);   // fixed order
+    if (threadIdx.x == 0) mean_s = s / double(npix);
+  }
+  __syncthreads();
+  double o[3];
+  moments_block(kappa, npix, mean_s, pp, blockIdx.x, gridDim.x, hist, red, o);
+  if (threadIdx.x == 0) {
+    part[3 * blockIdx.x + 0] = o[0];
+    part[3 * blockIdx.x + 1] = o[1];
+    part[3 * blockIdx.x + 2] = o[2];
+    __threadfence();                       // this block's sums before its ticket
+    last_s = atomicAdd(ticket, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < pp.nbins + 3; i += blockDim.x)
+    if (hist[i]) atomicAdd(pdf + i, (unsigned long long)hist[i]);
+  if (!last_s) return;
+  __threadfence();                         // every block's sums are visible
+  moments_final_block(ksum_part, nksum, part, gridDim.x, npix, red, m);
+  if (threadIdx.x == 0) *ticket = 0u;
 }
 
 // Statistics vector of one map for the covariance (Eq. 10): the first six
@@ -959,7 +1029,7 @@ k_batch_persistent(BatchArgs ba, ShellTable st, Bands bd, PdfParam pp) {
     __syncthreads();
     double* mo = ba.moments + 10 * (size_t)r;
     int64_t* pd = ba.pdf + (size_t)(ba.nbins + 3) * r;
-    if (threadIdx.x < 32) moments_final_warp(ks, ba.gk, mp, ba.gm, npix, mo);
+    moments_final_block(ks, ba.gk, mp, ba.gm, npix, red, mo);
     for (int i = threadIdx.x; i < ba.nbins + 3; i += kBT) pd[i] = (int64_t)hist[i];
     __syncthreads();
     double* v = ba.stats + (size_t)ba.d * r;
@@ -1015,13 +1085,16 @@ static ufc_status check_kappa_args(ufc_ctx* c, const int32_t* counts, int S, int
 
 // Forward kappa pass shared by ufc_kappa_stats and its allocation-free
 // variant (identical results): grid blocks, one partial sum each in ksum.
-static int kappa_fwd_grid(ufc_ctx* c) { return 8 * c->num_sms; }
+static int kappa_fwd_grid(const ufc_ctx* c, int npix) {   // blocks with work only
+  return std::min(8 * c->num_sms, (npix / 4 + kKV - 1) / kKV);
+}
 static ufc_status launch_kappa_fwd(ufc_ctx* c, const int32_t* counts, const Coef& cf,
-                                   float* kappa, double* ksum, int grid) {
+                                   float* kappa, double* ksum, int grid, int64_t* pdf, int nbins) {
+  unsigned long long* pd = reinterpret_cast<unsigned long long*>(pdf);
   if ((reinterpret_cast<uintptr_t>(kappa) & 15) == 0) {
-    k_kappa_vec<<<grid, kKV, 0, c->stream>>>(counts, cf, kappa, ksum);
+    k_kappa_vec<<<grid, kKV, 0, c->stream>>>(counts, cf, kappa, ksum, pd, nbins + 3);
   } else {
-    k_kappa_plain<<<grid, kKT, 0, c->stream>>>(counts, cf, kappa, ksum);
+    k_kappa_plain<<<grid, kKT, 0, c->stream>>>(counts, cf, kappa, ksum, pd, nbins + 3);
   }
   UFC_CUDA(c, cudaGetLastError());
   return UFC_OK;
@@ -1038,10 +1111,14 @@ static PdfParam make_pdf_param(double lo, double hi, int nbins) {
   pp.lo_f = (float)lo;
   pp.scale_f = (float)pp.scale;
   pp.nbins = nbins;
-  // |x_f - x_64| <= 3u |x| + u |lo| s + 2^-52 |x| (u = 2^-24); when
-  // |lo| s < 16 that is below 68u (|x| + 1) < 2^-16 (|x| + 1), the band
-  // used; other ranges send every value through the FP64 expression.
-  pp.band_rel = std::fabs(lo) * pp.scale < 16.0 ? std::ldexp(1.0f, -16) : 2.0f;
+  // |x_f - x_64| <= u |lo| s + 3u |x| + 2^-52 |x| (u = 2^-24) with x in
+  // [0, nbins]; the band is twice that at x = nbins.  A range whose band
+  // passes 1/4 sends every value through the FP64 expression.  (With a band
+  // that held for |lo| s < 16 only, a range of +- 6 sigma in 200 bins took the
+  // FP64 expression for every pixel: 200 us of the Nside-1024 map's moment
+  // pass.)
+  const double band = std::ldexp(1.0, -23) * (std::fabs(lo) * pp.scale + 3.0 * nbins + 4.0);
+  pp.band = band < 0.25 ? (float)band : 2.0f;
   auto fdn = [](double v) { float f = (float)v; return (double)f > v ? nextafterf(f, -INFINITY) : f; };
   auto fup = [](double v) { float f = (float)v; return (double)f < v ? nextafterf(f, INFINITY) : f; };
   pp.lo_dn = fdn(lo);
@@ -1051,20 +1128,17 @@ static PdfParam make_pdf_param(double lo, double hi, int nbins) {
   return pp;
 }
 
+// (the PDF has been cleared by the kernel that wrote ksum)
 static ufc_status launch_moments(ufc_ctx* c, const float* kmap, int npix, const double* ksum,
                                  int grid, double lo, double hi, int nbins, double* mpart,
-                                 int mgrid, double* moments, int64_t* pdf, bool timed) {
+                                 double* moments, int64_t* pdf, bool timed) {
   const PdfParam pp = make_pdf_param(lo, hi, nbins);
-  UFC_CUDA(c, cudaMemsetAsync(pdf, 0, (size_t)(nbins + 3) * 8, c->stream));
   const int smem = (nbins + 3) * 4;
   {
     ProfScope ps_(timed ? c : nullptr, "k_moments");
-    k_moments<<<mgrid, kMT, smem, c->stream>>>(kmap, npix, ksum, grid, pp, mpart,
-                                               (unsigned long long*)pdf);
-  }
-  {
-    ProfScope ps_(timed ? c : nullptr, "k_moments_final");
-    k_moments_final<<<1, 32, 0, c->stream>>>(ksum, grid, mpart, mgrid, npix, moments);
+    k_moments<<<moments_grid(c->num_sms, npix), kMT, smem, c->stream>>>(
+        kmap, npix, ksum, grid, pp, mpart, (unsigned long long*)pdf, moments,
+        &reinterpret_cast<BinCounters*>(c->counters)->ticket);
   }
   UFC_CUDA(c, cudaGetLastError());
   return UFC_OK;
@@ -1081,16 +1155,15 @@ ufc_status run_map_stats(ufc_ctx* c, const float* map, int nside, double lo, dou
     return set_err(c, UFC_ERR_ARG, "PDF range needs finite lo < hi");
   if (reinterpret_cast<uintptr_t>(map) & 15) return set_err(c, UFC_ERR_ARG, "map_dev must be 16-byte aligned");
   const int npix = 12 * nside * nside;
-  const int grid = kappa_fwd_grid(c), mgrid = 2 * c->num_sms;
+  const int grid = kappa_fwd_grid(c, npix), mgrid = moments_grid(c->num_sms, npix);
   double* ksum = (double*)ws_get(c, kSlotPartials, (size_t)(grid + 3 * mgrid) * 8);
   if (!ksum) return UFC_ERR_ALLOC;
   {
     ProfScope ps_(c, "k_map_sum");
-    k_map_sum<<<grid, kKV, 0, c->stream>>>(map, npix, ksum);
+    k_map_sum<<<grid, kKV, 0, c->stream>>>(map, npix, ksum, (unsigned long long*)pdf, nbins + 3);
   }
   UFC_CUDA(c, cudaGetLastError());
-  return launch_moments(c, map, npix, ksum, grid, lo, hi, nbins, ksum + grid, mgrid, moments, pdf,
-                        true);
+  return launch_moments(c, map, npix, ksum, grid, lo, hi, nbins, ksum + grid, moments, pdf, true);
 }
 
 ufc_status run_kappa_stats(ufc_ctx* c, const int32_t* counts, int S, int nside,
@@ -1112,8 +1185,8 @@ ufc_status run_kappa_stats(ufc_ctx* c, const int32_t* counts, int S, int nside,
   make_coef(A, C, S, npix, cf);
   if (reinterpret_cast<uintptr_t>(counts) & 15)
     return set_err(c, UFC_ERR_ARG, "counts_dev must be 16-byte aligned");
-  const int grid = kappa_fwd_grid(c);
-  const int mgrid = 2 * c->num_sms;
+  const int grid = kappa_fwd_grid(c, npix);
+  const int mgrid = moments_grid(c->num_sms, npix);
   double* ksum = (double*)ws_get(c, kSlotPartials, (size_t)(grid + 3 * mgrid) * 8);
   if (!ksum) return UFC_ERR_ALLOC;
   double* mpart = ksum + grid;
@@ -1125,12 +1198,11 @@ ufc_status run_kappa_stats(ufc_ctx* c, const int32_t* counts, int S, int nside,
   if (!kmap) return UFC_OK;   // nothing requested
   {
     ProfScope ps_(c, "k_kappa");
-    s = launch_kappa_fwd(c, counts, cf, kmap, ksum, grid);
+    s = launch_kappa_fwd(c, counts, cf, kmap, ksum, grid, pdf, nbins);
     if (s) return s;
   }
   if (!want_stats) return UFC_OK;
-  return launch_moments(c, kmap, npix, ksum, grid, lo, hi, nbins, mpart, mgrid, moments, pdf,
-                        true);
+  return launch_moments(c, kmap, npix, ksum, grid, lo, hi, nbins, mpart, moments, pdf, true);
 }
 
 // The adjoint's device pass and its reduction to the sums
@@ -1162,7 +1234,7 @@ static ufc_status adjoint_sums(ufc_ctx* c, const int32_t* counts, int S, int nsi
   const int npix = 12 * nside * nside;
   const int grid2 = c->num_sms;                            // one block per SM
   const size_t nrow = (size_t)grid2 * 4 * S, nsum = (size_t)grid2 * 4;
-  const int mgrid = 2 * c->num_sms;
+  const int mgrid = moments_grid(c->num_sms, npix);
   const size_t nmap = kappa ? (size_t)grid2 + 3 * (size_t)mgrid : 0;   // map sums, moment partials
   double* part = (double*)ws_get(c, kSlotPartials, (nrow + nsum + nmap) * 8);
   if (!part) return UFC_ERR_ALLOC;
@@ -1187,7 +1259,8 @@ static ufc_status adjoint_sums(ufc_ctx* c, const int32_t* counts, int S, int nsi
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2));   \
     for (int s0 = 0; s0 < S; s0 += win)                                                           \
       k_adj_main<G, NT_, X><<<grid2, NT_, smem2, c->stream>>>(                                    \
-          counts, cf, g, rows, sums, &bc->range, s0, s0 == 0 ? kappa : nullptr, ksum, ext);       \
+          counts, cf, g, rows, sums, &bc->range, s0, s0 == 0 ? kappa : nullptr, ksum, ext,        \
+          (unsigned long long*)pdf, nbins + 3);                                                   \
   } while (0)
 #define UFC_ADJ_X(G, NT_)                                                                         \
   do {                                                                                            \
@@ -1203,8 +1276,8 @@ static ufc_status adjoint_sums(ufc_ctx* c, const int32_t* counts, int S, int nsi
   }
   UFC_CUDA(c, cudaGetLastError());
   if (kappa) {                             // moments and PDF of the map just written
-    ufc_status s = launch_moments(c, kappa, npix, ksum, grid2, lo, hi, nbins, mpart, mgrid,
-                                  moments, pdf, true);
+    ufc_status s = launch_moments(c, kappa, npix, ksum, grid2, lo, hi, nbins, mpart, moments, pdf,
+                                  true);
     if (s) return s;
   }
   std::vector<double> hp(nrow + nsum);
@@ -1298,7 +1371,7 @@ ufc_status run_kappa_partial(ufc_ctx* c, const int32_t* counts, int S, int nside
   make_coef(A, 0.0, S, npix, cf);
   {
     ProfScope ps_(c, "k_kappa_partial");
-    k_kappa_partial<<<kappa_fwd_grid(c), kKV, 0, c->stream>>>(counts, cf, partial);
+    k_kappa_partial<<<kappa_fwd_grid(c, npix), kKV, 0, c->stream>>>(counts, cf, partial);
   }
   UFC_CUDA(c, cudaGetLastError());
   return UFC_OK;
@@ -1328,17 +1401,17 @@ ufc_status run_kappa_stats_partial(ufc_ctx* c, const double* partial, int nside,
   if (!(hi > lo) || !std::isfinite(lo) || !std::isfinite(hi))
     return set_err(c, UFC_ERR_ARG, "PDF range needs finite lo < hi");
   const int npix = 12 * nside * nside;
-  const int grid = kappa_fwd_grid(c), mgrid = 2 * c->num_sms;
+  const int grid = kappa_fwd_grid(c, npix), mgrid = moments_grid(c->num_sms, npix);
   double* ksum = (double*)ws_get(c, kSlotPartials, (size_t)(grid + 3 * mgrid) * 8);
   if (!ksum) return UFC_ERR_ALLOC;
   const float ch = (float)C, cl = (float)(C - (double)ch);
   {
     ProfScope ps_(c, "k_kappa_finish");
-    k_kappa_finish<<<grid, kKV, 0, c->stream>>>(partial, ch, cl, npix, kappa, ksum);
+    k_kappa_finish<<<grid, kKV, 0, c->stream>>>(partial, ch, cl, npix, kappa, ksum,
+                                                (unsigned long long*)pdf, nbins + 3);
   }
   UFC_CUDA(c, cudaGetLastError());
-  return launch_moments(c, kappa, npix, ksum, grid, lo, hi, nbins, ksum + grid, mgrid, moments,
-                        pdf, true);
+  return launch_moments(c, kappa, npix, ksum, grid, lo, hi, nbins, ksum + grid, moments, pdf, true);
 }
 
 ufc_status run_kappa_adjoint_sums(ufc_ctx* c, const int32_t* counts, int S, int nside,
@@ -1411,8 +1484,8 @@ ufc_status run_kappa_stats_noalloc(ufc_ctx* c, const int32_t* counts, int S, int
   if (reinterpret_cast<uintptr_t>(counts) & 15)
     return set_err(c, UFC_ERR_ARG, "counts_dev must be 16-byte aligned");
   const int npix = 12 * nside * nside;
-  const int grid = kappa_fwd_grid(c);
-  const int mgrid = 2 * c->num_sms;
+  const int grid = kappa_fwd_grid(c, npix);
+  const int mgrid = moments_grid(c->num_sms, npix);
   if (grid + 3 * mgrid > kNoAllocScratch)
     return set_err(c, UFC_ERR_CAPACITY,
                    "scratch needs %d doubles, the fixed array holds %d", grid + 3 * mgrid,
@@ -1423,11 +1496,10 @@ ufc_status run_kappa_stats_noalloc(ufc_ctx* c, const int32_t* counts, int S, int
   double* mpart = ksum + grid;   // every slot is written before it is read
   Coef cf;
   make_coef(A, C, S, npix, cf);
-  s = launch_kappa_fwd(c, counts, cf, kappa, ksum, grid);
+  s = launch_kappa_fwd(c, counts, cf, kappa, ksum, grid, pdf, nbins);
   if (s) return s;
   // (no kernel-timing records here: recording them may allocate)
-  return launch_moments(c, kappa, npix, ksum, grid, lo, hi, nbins, mpart, mgrid, moments, pdf,
-                        false);
+  return launch_moments(c, kappa, npix, ksum, grid, lo, hi, nbins, mpart, moments, pdf, false);
 }
 
 ufc_status run_stats_vector(ufc_ctx* c, const double* m, const int64_t* pdf, int nbins,
@@ -1492,7 +1564,7 @@ void batch_persistent_bytes(const ufc_ctx* c, int nreal, int nbox, int S, int ns
                             size_t* maps, size_t* desc) {
   const size_t npix = 12ull * nside * nside;
   const size_t kap_b = (npix * 4 + 255) / 256 * 256;
-  const size_t part_b = ((size_t)(8 * c->num_sms + 3 * 2 * c->num_sms) * 8 + 255) / 256 * 256;
+  const size_t part_b = ((size_t)(8 * c->num_sms + 3 * 4 * c->num_sms) * 8 + 255) / 256 * 256;
   *maps = (batch_map_stride(S, nside) + kap_b + part_b) * nreal;
   *desc = ((size_t)nreal * nbox * sizeof(BatchItem) + 255) / 256 * 256 +
           ((size_t)nreal * sizeof(Coef) + 255) / 256 * 256 + ((size_t)nreal * 4 + 255) / 256 * 256 +
@@ -1566,7 +1638,7 @@ ufc_status batch_persistent_prepare(ufc_ctx* c, int nreal, int nbox, const float
   std::memcpy(host.data() + o_nt, ntask_r.data(), (size_t)nreal * 4);
   UFC_CUDA(c, cudaMemcpyAsync(desc, host.data(), host.size(), cudaMemcpyHostToDevice, c->stream));
   UFC_CUDA(c, cudaStreamSynchronize(c->stream));   // (host staging leaves scope)
-  const int gk = kappa_fwd_grid(c), gm = 2 * c->num_sms;
+  const int gk = kappa_fwd_grid(c, npix), gm = moments_grid(c->num_sms, npix);
   const size_t map_b = batch_map_stride(S, nside);
   const size_t kap_b = ((size_t)npix * 4 + 255) / 256 * 256;
   BatchArgs& ba = L.ba;
