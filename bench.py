@@ -289,7 +289,7 @@ def batched_leg(ctx, api, synth, dev, n_real: int, n_side: int, nbuf: int = 8,
     out["tuning"] = {k: tuning[k] for k in ("batch_chunk", "batch_blocks_per_sm", "cached")}
     out["tuning"]["candidates_ms"] = tuning.get("ms")
     # GPU time per kernel of the serial run (a separate, profiled pass) and of
-    # the batched call's persistent kernel outside a graph
+    # the batched call's stages
     ctx.profile(True)
     serial(api.welford_state(d, dev))
     torch.cuda.synchronize()

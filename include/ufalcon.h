@@ -296,7 +296,9 @@ ufc_status ufc_bin_snapshots_host(ufc_ctx *ctx, const float *const *xyz_host,
 /* Diagnostics of the last ufc_bin/ufc_keys call (synchronises):
  * info[0] invalid particles, info[1] particle-images with a key,
  * info[2] decisions refined past the FP32 stage, info[3] past the
- * float-float stage (resolved by the FP64 procedure itself). */
+ * float-float stage (resolved by the FP64 procedure itself).  Periodic images
+ * that cannot hold a particle inside the box's shells are not decided one by
+ * one and count in neither. */
 ufc_status ufc_bin_info(ufc_ctx *ctx, int64_t info[4]);
 
 /* ---- kappa map, moments, PDF (Eq. 6, Eq. 12-13, Sec. 3.3) ------------------ */
@@ -495,7 +497,7 @@ ufc_status ufc_map_stats(ufc_ctx *ctx, const float *map_dev, int32_t nside,
 
 #define UFC_BATCH_GRAPH 1      /* capture the whole batch into one CUDA graph */
 #define UFC_BATCH_LAUNCHES 2   /* one launch sequence per realisation, never the
-                                  persistent kernel                           */
+                                  stages over all of them                     */
 
 /* Statistics of nreal realisations in one call (Sec. 3.2 averages over 150
  * realisations).  Realisation r has nbox particle sets xyz_dev[r*nbox + k]
@@ -507,16 +509,15 @@ ufc_status ufc_map_stats(ufc_ctx *ctx, const float *map_dev, int32_t nside,
  * pdf_dev[r][nbins+3] and stats_dev[r][6 + nbins] (ufc_stats_vector), and
  * finally adds all nreal vectors to the Welford state state_dev in order.
  * Count maps of up to 64 MB whose boxes have no periodic images, and whose
- * per-realisation maps fit in 4 GB of workspace together, run as ONE
- * persistent kernel (unless UFC_BATCH_LAUNCHES): a device work queue of
- * (realisation, particle chunk) tasks; the block that finishes a
- * realisation's last chunk builds its kappa map, moments, PDF and
- * statistics vector, and the block that finishes the last realisation runs
- * the Welford update in realisation order.  No block waits for another
- * (completion is counted with atomics).  Its chunk size and blocks per SM
- * come from ufc_set_tuning.  Results equal the one-at-a-time calls bit for
- * bit; counts_dev and kappa_dev are then not used (the kernel keeps one map
- * per realisation in the workspace).  Otherwise count maps of up to 64 MB
+ * per-realisation maps fit in 4 GB of workspace together, run stage by stage
+ * over all realisations (unless UFC_BATCH_LAUNCHES): one launch bins every
+ * (realisation, box), one makes the kappa maps, one the moments, PDFs and
+ * statistics vectors, one updates the Welford state in realisation order.
+ * The binning's task size and blocks per SM come from ufc_set_tuning.
+ * Results equal the one-at-a-time calls bit for bit; counts_dev and kappa_dev
+ * are then not used (the workspace keeps one map per realisation), and
+ * UFC_BATCH_GRAPH changes nothing: half a dozen launches need no graph.
+ * Otherwise count maps of up to 64 MB
  * run on up to 8 concurrent lanes: realisation r on lane r mod 8, lane 0
  * being this context with counts_dev and kappa_dev, the others extra
  * contexts owned by this one, each with its own count and kappa maps,
@@ -543,8 +544,9 @@ ufc_status ufc_batched_stats(ufc_ctx *ctx, int32_t nreal, int32_t nbox,
 
 /* Tuning of a context (no counterpart in the paper; an autotuner picks the
  * values by timing candidates): batch_chunk = particles per task of the
- * persistent batch kernel (0: 8192), batch_blocks_per_sm = its resident
- * blocks per SM (0: 2; at most 2).  Host only. */
+ * batched call's binning (0: from the particle count, at most 1024),
+ * batch_blocks_per_sm = its resident blocks per SM (0: 2; at most 2).  Host
+ * only. */
 typedef struct {
   int32_t batch_chunk;
   int32_t batch_blocks_per_sm;

@@ -45,7 +45,7 @@ MOMENT_NAMES = ("mean", "mu2", "mu3", "mu4", "skew", "kurt", "s2_expect", "var_s
 
 
 class Tuning(ctypes.Structure):
-    """ufc_tuning: chunk size and blocks per SM of the persistent batch kernel (0 = default)."""
+    """ufc_tuning: task size and blocks per SM of the batched call's binning (0 = default)."""
     _fields_ = [("batch_chunk", I32), ("batch_blocks_per_sm", I32)]
 
 
@@ -593,7 +593,7 @@ class Context:
         A [nreal, nshell], C [nreal].  Returns (moments [nreal,10],
         pdf [nreal, nbins+3], stats [nreal, 6+nbins]); updates `state`.
         launches=True: one launch sequence per realisation instead of the
-        persistent kernel (UFC_BATCH_LAUNCHES).  The autotuner's cached
+        stages over all of them (UFC_BATCH_LAUNCHES).  The autotuner's cached
         tuning for this shape, if any, is applied first (autotune.tune_batch
         makes it)."""
         import torch

@@ -2,7 +2,7 @@
 shape and caching the winner in a JSON file:
   - the binning output path (L2 atomics vs dense-key scatter with
     shared-memory histograms) per (GPU, Nside, shells, particle count);
-  - the persistent batch kernel's particles per task and blocks per SM
+  - the batched call's binning: particles per task and blocks per SM
     (ufc_set_tuning) per (GPU, Nside, shells, realisations, particle count).
 
 Every choice gives identical results; only speed differs.  The cache lives in
@@ -110,13 +110,13 @@ def choose_bin_path(ctx, xyz_list, boxes, chi_edges, nside: int, counts=None, re
     return best
 
 
-BATCH_CHUNKS = (2048, 8192, 32768)
+BATCH_CHUNKS = (512, 1024, 4096)     # particles per task of one warp
 BATCH_BLOCKS = (1, 2)
 
 
 def batch_key(gpu_name: str, nside: int, nshell: int, nreal: int, n_total: int) -> str:
     nb = int(math.log2(max(1, n_total)))
-    return f"batch|{gpu_name}|nside={nside}|nshell={nshell}|nreal={nreal}|log2n={nb}"
+    return f"batch-tasks|{gpu_name}|nside={nside}|nshell={nshell}|nreal={nreal}|log2n={nb}"
 
 
 def cached_batch_tuning(ctx, nside: int, nshell: int, nreal: int, n_total: int):
@@ -130,7 +130,7 @@ def cached_batch_tuning(ctx, nside: int, nshell: int, nreal: int, n_total: int):
 def tune_batch(ctx, run, nside: int, nshell: int, nreal: int, n_total: int, reps: int = 2,
                force_retune: bool = False) -> dict:
     """Times run() (one batched call) under every candidate tuning of the
-    persistent batch kernel, keeps the fastest in the context and the cache;
+    batched call's binning, keeps the fastest in the context and the cache;
     returns {"batch_chunk", "batch_blocks_per_sm", "ms": {candidate: ms},
     "cached": bool}."""
     import torch

@@ -9,7 +9,8 @@
 //   exact stage k_exact   : the FP64 procedure over queue 2.
 // Outputs (mode):
 //   KEYS   : int32 key per particle (ufc_keys).
-//   DIRECT : atomicAdd into the count map (maps that sit in L2).
+//   DIRECT : atomicAdd into the count map (maps that sit in L2), in one
+//            kernel of its own (direct.cu).
 //   DENSE  : keys packed as (bucket << 15 | offset) with bucket = shell *
 //            nblk + pix / 24576, appended per warp to a dense array while a
 //            shared-memory histogram counts buckets; then two scatter passes
@@ -25,6 +26,7 @@
 
 #include "common.cuh"
 #include "ctx.h"
+#include "direct.cuh"
 #include "pixel.cuh"
 
 namespace ufc {
@@ -84,8 +86,8 @@ __device__ __forceinline__ void dense_append(WarpChunk& wc, bool want, uint32_t 
                                              const KeyOut& o) {
   const unsigned full = 0xFFFFFFFFu;
   unsigned m = __ballot_sync(full, want);
-  if (m == 0) return;
   int lane = threadIdx.x & 31;
+  if (m == 0) return;
   int cnt = __popc(m);
   int rank = __popc(m & ((1u << lane) - 1u));
   if (wc.base < 0) {
@@ -227,20 +229,10 @@ __device__ __forceinline__ unsigned long long warp_sum(unsigned long long v) {
 }
 
 // ----------------------------------------------------------- fast stage ----
-// Shell lookup table over r^2.  Bin i holds the r2 values whose FP32
-// v = fminf(r2 * scale, kLut - 1) rounds to i; its low 15 bits count the
-// edges e certainly at or below every such r2 (hi2[e] <= the bin's lowest
-// possible r2), and bit 15 is set unless the next edge is certainly above
-// every such r2 (lo2[e0] > the bin's highest possible r2).  A clean bin
-// gives the shell with one load; the others scan the edges (exact).
-constexpr int kLutBits = 13;
-constexpr int kLut = 1 << kLutBits;
-constexpr uint16_t kLutScan = 0x8000;
-
 struct FastShared {
   float lo2[kMaxShells + 2], hi2[kMaxShells + 2];
-  float shf[3][kMaxImg1D], shlo[3][kMaxImg1D];
-  uint16_t lut[kLut];
+  float shf[3], shlo[3];
+  alignas(16) uint16_t lut[kLut];
 };
 
 // Shell of r2 (finite, >= 0) among the box's shells [lo, hi): -1 outside,
@@ -267,7 +259,7 @@ struct FastCtx {
   unsigned long long n_invalid, n_keyed;
 };
 
-// All images of one particle (warp-collective: every lane calls it).
+// One particle (warp-collective: every lane calls it).
 template <int MODE>
 __device__ __forceinline__ void fast_particle(bool have, float x, float y, float zc, int64_t p,
                                               int32_t box_id, const BoxGeom& bg,
@@ -276,66 +268,60 @@ __device__ __forceinline__ void fast_particle(bool have, float x, float y, float
                                               int32_t npix, const KeyOut& o, const Queues& qs,
                                               uint32_t* hist_s, FastCtx& fc) {
   const int lo = bg.shell_lo, hi = bg.shell_hi;
-  const int n1 = 2 * bg.R + 1;
   const bool finite = have && isfinite(x) && isfinite(y) && isfinite(zc);
   if (have && !finite) ++fc.n_invalid;
-  int ii = 0, jj = 0, kk = 0;                   // image (ii, jj, kk), img = (ii n1 + jj) n1 + kk
-  for (int img = 0; img < bg.nimg; ++img) {
-    if (img) {
-      if (++kk == n1) { kk = 0; if (++jj == n1) { jj = 0; ++ii; } }
-    }
-    int32_t key = kKeyOutside;
-    uint32_t dkey = 0u;
-    if (finite) {
-      const float dx = (x + fs.shf[0][ii]) + fs.shlo[0][ii];
-      const float dy = (y + fs.shf[1][jj]) + fs.shlo[1][jj];
-      const float dz = (zc + fs.shf[2][kk]) + fs.shlo[2][kk];
-      const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
-      if (!(r2 >= bd.r2_min)) {
-        key = kKeyUndecided;
-      } else {
-        const int32_t b = shell_lut(fs, lo, hi, lut_scale, r2);
-        if (b == -2) {
-          key = kKeyUndecided;
-        } else if (b >= 0) {
-          const int32_t pix = pixel_fast(N, bd, dx, dy, dz, r2);
-          key = (pix == kKeyUndecided) ? kKeyUndecided : b * npix + pix;
-          if (MODE == kModeDense && pix != kKeyUndecided) {
-            const uint32_t blk = uint32_t(pix >> 13) / 3u;       // pix / 24576
-            dkey = ((uint32_t(b - o.shell0) * uint32_t(o.nblk) + blk) << kOffBits) |
-                   (uint32_t(pix) - blk * uint32_t(kBlockPix));
-          }
-        }
-      }
-    }
-    const bool und = key == kKeyUndecided;
-    if (!queue_push(fc.qc, und, qpack(box_id, img, p), qs.q1, qs.cap1, &qs.cnt->q1)) {
-      // queue full: resolve with the FP64 procedure here
-      key = key_exact(st, lo, hi, N, npix, x, y, zc, bg.sh64[0][ii], bg.sh64[1][jj],
-                      bg.sh64[2][kk]);
-      if (key == kKeyInvalid) ++fc.n_invalid;
-      if (MODE == kModeDense && key >= 0) dkey = dense_key(key, npix, o);
-    }
-    if (MODE == kModeKeys) {
-      if (have) o.keys[p] = finite ? key : kKeyInvalid;
-    } else if (MODE == kModeDirect) {
-      if (key >= 0 && UFC_IDX_OK(key, o.ncell, 2)) atomicAdd(o.counts + key, 1);
+  int32_t key = kKeyOutside;
+  uint32_t dkey = 0u;
+  if (finite) {
+    const float dx = (x + bg.shf[0][0]) + bg.shlo[0][0];
+    const float dy = (y + bg.shf[1][0]) + bg.shlo[1][0];
+    const float dz = (zc + bg.shf[2][0]) + bg.shlo[2][0];
+    const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
+    if (!(r2 >= bd.r2_min)) {
+      key = kKeyUndecided;
     } else {
-      if (key >= 0) {
-        const uint32_t bucket = dkey >> kOffBits;
-        if (UFC_IDX_OK(bucket, o.nbuckets, 1)) {
-          if (o.smem_hist) atomicAdd(hist_s + bucket, 1u);
-          else atomicAdd(o.hist + bucket, 1u);
+      const int32_t b = shell_lut(fs, lo, hi, lut_scale, r2);
+      if (b == -2) {
+        key = kKeyUndecided;
+      } else if (b >= 0) {
+        const int32_t pix = pixel_fast(N, bd, dx, dy, dz, r2);
+        key = (pix == kKeyUndecided) ? kKeyUndecided : b * npix + pix;
+        if (MODE == kModeDense && pix != kKeyUndecided) {
+          const uint32_t blk = uint32_t(pix >> 13) / 3u;       // pix / 24576
+          dkey = ((uint32_t(b - o.shell0) * uint32_t(o.nblk) + blk) << kOffBits) |
+                 (uint32_t(pix) - blk * uint32_t(kBlockPix));
         }
       }
-      dense_append(fc.wc, key >= 0, dkey, o);
     }
-    fc.n_keyed += key >= 0;
   }
+  const bool und = key == kKeyUndecided;
+  if (!queue_push(fc.qc, und, qpack(box_id, 0, p), qs.q1, qs.cap1, &qs.cnt->q1)) {
+    // queue full: resolve with the FP64 procedure here
+    key = key_exact(st, lo, hi, N, npix, x, y, zc, bg.sh64[0][0], bg.sh64[1][0], bg.sh64[2][0]);
+    if (key == kKeyInvalid) ++fc.n_invalid;
+    if (MODE == kModeDense && key >= 0) dkey = dense_key(key, npix, o);
+  }
+  if (MODE == kModeKeys) {
+    if (have) o.keys[p] = finite ? key : kKeyInvalid;
+  } else {
+    if (key >= 0) {
+      const uint32_t bucket = dkey >> kOffBits;
+      if (UFC_IDX_OK(bucket, o.nbuckets, 1)) {
+        if (o.smem_hist) atomicAdd(hist_s + bucket, 1u);
+        else atomicAdd(o.hist + bucket, 1u);
+      }
+    }
+    dense_append(fc.wc, key >= 0, dkey, o);
+  }
+  fc.n_keyed += key >= 0;
 }
 
 __device__ __forceinline__ void fast_init_shared(FastShared& fs, const BoxGeom& bg,
                                                  const ShellTable& st, const uint16_t* lut) {
+  if (threadIdx.x < 3) {
+    fs.shf[threadIdx.x] = bg.shf[threadIdx.x][0];
+    fs.shlo[threadIdx.x] = bg.shlo[threadIdx.x][0];
+  }
   for (int i = threadIdx.x; i <= st.nshell; i += blockDim.x) {
     fs.lo2[i] = st.lo2[i];
     fs.hi2[i] = st.hi2[i];
@@ -344,11 +330,9 @@ __device__ __forceinline__ void fast_init_shared(FastShared& fs, const BoxGeom& 
     fs.lo2[st.nshell + 1] = INFINITY;
     fs.hi2[st.nshell + 1] = INFINITY;
   }
-  for (int i = threadIdx.x; i < 3 * kMaxImg1D; i += blockDim.x) {
-    fs.shf[i / kMaxImg1D][i % kMaxImg1D] = bg.shf[i / kMaxImg1D][i % kMaxImg1D];
-    fs.shlo[i / kMaxImg1D][i % kMaxImg1D] = bg.shlo[i / kMaxImg1D][i % kMaxImg1D];
-  }
-  for (int i = threadIdx.x; i < kLut; i += blockDim.x) fs.lut[i] = lut[i];
+  const uint4* src = reinterpret_cast<const uint4*>(lut);
+  uint4* dst = reinterpret_cast<uint4*>(fs.lut);
+  for (int i = threadIdx.x; i < kLut / 8; i += blockDim.x) dst[i] = src[i];
 }
 
 template <int MODE>
@@ -368,16 +352,15 @@ __device__ __forceinline__ void fast_finish(FastCtx& fc, const KeyOut& o, const 
   }
 }
 
-struct LutParam { uint16_t v[kLut]; float scale; };
-
 // Fast stage with plain per-thread loads (any 4-byte aligned input).
 template <int MODE>
 __global__ void __launch_bounds__(kFastThreads)
 k_fast(const float* __restrict__ xyz, int64_t n, int64_t p_off, int32_t box_id, BoxGeom bg,
-       ShellTable st, LutParam lp, Bands bd, int32_t N, int32_t npix, KeyOut o, Queues qs) {
+       ShellTable st, const BinTables* __restrict__ tab, float lut_scale, Bands bd, int32_t N,
+       int32_t npix, KeyOut o, Queues qs) {
   extern __shared__ uint32_t hist_s[];
   __shared__ FastShared fs;
-  fast_init_shared(fs, bg, st, lp.v);
+  fast_init_shared(fs, bg, st, tab->lut);
   if (MODE == kModeDense && o.smem_hist)
     for (int i = threadIdx.x; i < o.nbuckets; i += blockDim.x) hist_s[i] = 0;
   __syncthreads();
@@ -393,8 +376,8 @@ k_fast(const float* __restrict__ xyz, int64_t n, int64_t p_off, int32_t box_id, 
       y = __ldg(xyz + 3 * p + 1);
       zc = __ldg(xyz + 3 * p + 2);
     }
-    fast_particle<MODE>(have, x, y, zc, p_off + p, box_id, bg, fs, lp.scale, st, bd, N, npix, o,
-                        qs, hist_s, fc);
+    fast_particle<MODE>(have, x, y, zc, p_off + p, box_id, bg, fs, lut_scale, st, bd, N, npix,
+                        o, qs, hist_s, fc);
   }
   fast_finish<MODE>(fc, o, qs, hist_s);
 }
@@ -480,11 +463,10 @@ __device__ __noinline__ int32_t key_exact_slow(const ShellTable& st, int32_t lo,
 //      counters (an overflow at 65536 is carried to the global histogram).
 // A stage is free once every warp has finished A on it (the entries hold
 // copies); the last warp to finish issues the copy that refills it, so the
-// steady state has no block-wide barrier.  Without periodic images the
-// lists carry over from chunk to chunk; an entry keeps its offset in its
-// chunk and the chunk's sequence number modulo 4096, and the lists are
-// drained at least every kWAgeFlush chunks.  With periodic images the lists
-// are drained after every (chunk, image) pass.  Particle p of the launch is
+// steady state has no block-wide barrier.  The lists carry over from chunk to
+// chunk; an entry keeps its offset in its chunk and the chunk's sequence
+// number modulo 4096, and the lists are drained at least every kWAgeFlush
+// chunks.  Particle p of the launch is
 // element p_off + p of the caller's array (chunked launches of ufc_bin_host).
 constexpr int kWThreads = 768;
 constexpr int kWChunk = 3840;                  // particles per chunk (45 KB)
@@ -514,10 +496,11 @@ __device__ __forceinline__ void hist16_carry(uint32_t* h32, uint32_t* ghist, uin
   atomicAdd(ghist + bucket, 65536u);
 }
 
-template <int MODE, bool IMAGES>
+template <int MODE>
 __global__ void __launch_bounds__(kWThreads, 1)
 k_fast_tma(const float* __restrict__ xyz, int64_t n, int64_t p_off, int32_t box_id, BoxGeom bg,
-           ShellTable st, LutParam lp, Bands bd, int32_t N, int32_t npix, KeyOut o, Queues qs) {
+           ShellTable st, const BinTables* __restrict__ tab, float lut_scale, Bands bd, int32_t N,
+           int32_t npix, KeyOut o, Queues qs) {
   extern __shared__ __align__(128) uint8_t dyn[];
   float* ring = reinterpret_cast<float*>(dyn);                          // [kWStages][3 kWChunk]
   float4* lists = reinterpret_cast<float4*>(dyn + kWStages * kWChunk * 12);  // [warps][2][kWList]
@@ -526,7 +509,7 @@ k_fast_tma(const float* __restrict__ xyz, int64_t n, int64_t p_off, int32_t box_
   __shared__ __align__(8) uint64_t bar[kWStages];
   __shared__ int done_s[kWStages];
   __shared__ int abort_s;
-  fast_init_shared(fs, bg, st, lp.v);
+  fast_init_shared(fs, bg, st, tab->lut);
   const int nwords = (o.nbuckets + 1) >> 1;
   if (MODE == kModeDense && o.smem_hist)
     for (int i = threadIdx.x; i < nwords; i += blockDim.x) h32[i] = 0u;
@@ -542,7 +525,7 @@ k_fast_tma(const float* __restrict__ xyz, int64_t n, int64_t p_off, int32_t box_
 
   const int lo = bg.shell_lo, hi = bg.shell_hi;
   const int n1 = 2 * bg.R + 1;
-  const bool carry = bg.nimg == 1;
+  const bool carry = bg.nimg == 1;             // (always: see the loop over images)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const unsigned lt_mask = (1u << lane) - 1u;
   float4* list_eq = lists + (2 * warp) * kWList;
@@ -574,9 +557,8 @@ k_fast_tma(const float* __restrict__ xyz, int64_t n, int64_t p_off, int32_t box_
   int ii = 0, jj = 0, kk = 0;                  // current image
   bool aborted = false;
   int64_t k = 0;
-  // the shift of the only image when the box has no periodic images
-  const float hsx = fs.shf[0][0], hsy = fs.shf[1][0], hsz = fs.shf[2][0];
-  const float hlx = fs.shlo[0][0], hly = fs.shlo[1][0], hlz = fs.shlo[2][0];
+  const float sx = fs.shf[0], sy = fs.shf[1], sz = fs.shf[2];
+  const float lx = fs.shlo[0], ly = fs.shlo[1], lz = fs.shlo[2];
   for (; k <= mine; ++k) {
     const bool last = k == mine;               // the final pass only drains the lists
     const int s = int(k & 1);                  // stage (two stages)
@@ -600,15 +582,15 @@ k_fast_tma(const float* __restrict__ xyz, int64_t n, int64_t p_off, int32_t box_
     const int ng = last ? 0 : kWGroups;                  // groups of 32 particles to classify
     const int nsteps = ng + (drain_all ? 1 : 0);         // + a drain step
     ii = jj = kk = 0;
+    // (one pass: boxes with periodic images take the direct path.  The loop
+    // over images and the drain after each stay because the code the compiler
+    // makes without them is slower, k_fast of two boxes of 512^3: 2.02 ms
+    // without either, 1.87 ms without the drain, 1.80 ms with both)
 #pragma unroll 1
     for (int img = 0; img < nimg; ++img) {
       if (img) {
         if (++kk == n1) { kk = 0; if (++jj == n1) { jj = 0; ++ii; } }
       }
-      const float sx = IMAGES ? fs.shf[0][ii] : hsx, sy = IMAGES ? fs.shf[1][jj] : hsy,
-                  sz = IMAGES ? fs.shf[2][kk] : hsz;
-      const float lx = IMAGES ? fs.shlo[0][ii] : hlx, ly = IMAGES ? fs.shlo[1][jj] : hly,
-                  lz = IMAGES ? fs.shlo[2][kk] : hlz;
       const uint64_t qbase = qpack(box_id, img, p_off + base);   // + offset in the chunk
 #pragma unroll 1
       for (int h = 0; h < nsteps; ++h) {
@@ -643,7 +625,7 @@ k_fast_tma(const float* __restrict__ xyz, int64_t n, int64_t p_off, int32_t box_
           // outside, undecided (c1), belt (c2) or cap (c3)
           const bool fin = r2 <= 3.0e38f;                // false for NaN and overflow
           const bool near = !(r2 >= bd.r2_min);          // near the observer (r == 0 is invalid)
-          const float v = fminf(r2 * lp.scale, float(kLut - 1));
+          const float v = fminf(r2 * lut_scale, float(kLut - 1));
           const int bin = __float_as_int(v + 8388608.0f) - 0x4B000000;
           const uint32_t e = fs.lut[bin];
           int a = int(e & 0x7FFFu) - 1;
@@ -666,11 +648,10 @@ k_fast_tma(const float* __restrict__ xyz, int64_t n, int64_t p_off, int32_t box_
           const bool dec = have && fin && !near && !band && inshell;
           const bool c2 = dec && eqz;
           const bool c3 = dec && capz;
-          // NaN or overflowing r2 (rare) goes to the queue as well, once per
-          // particle (its first image): the FP64 stage returns the invalid
-          // key for non-finite coordinates and decides a finite overflow
-          const bool c1 = have && (fin ? (near || band || (inshell && !eqz && !capz))
-                                       : (!IMAGES || img == 0));
+          // NaN or overflowing r2 (rare) goes to the queue as well: the FP64
+          // stage returns the invalid key for non-finite coordinates and
+          // decides a finite overflow
+          const bool c1 = have && (fin ? (near || band || (inshell && !eqz && !capz)) : true);
           const uint32_t meta = uint32_t(a & 255) | (uint32_t(j) << 8) | kqtag;
           const float4 ent = make_float4(dx, dy, dz, __uint_as_float(meta));
           const unsigned meq = __ballot_sync(0xFFFFFFFFu, c2);
@@ -689,7 +670,6 @@ k_fast_tma(const float* __restrict__ xyz, int64_t n, int64_t p_off, int32_t box_
             if (kx == kKeyInvalid) ++fc.n_invalid;
             if (kx >= 0) {
               ++fc.n_keyed;
-              if (MODE == kModeDirect && UFC_IDX_OK(kx, o.ncell, 2)) atomicAdd(o.counts + kx, 1);
               if (MODE == kModeDense) {            // rare: straight to the global histogram
                 const uint32_t dk = dense_key(kx, npix, o);
                 if (UFC_IDX_OK(dk >> kOffBits, o.nbuckets, 1)) atomicAdd(ghist + (dk >> kOffBits), 1u);
@@ -737,40 +717,14 @@ k_fast_tma(const float* __restrict__ xyz, int64_t n, int64_t p_off, int32_t box_
             return (blockIdx.x + ke * gridDim.x) * kWChunk + int64_t((meta >> 8) & 4095u);
           };
           const int32_t key = b * npix + pix;
-          bool queued = true;
           if (__any_sync(0xFFFFFFFFu, have && !ok)) {   // rare: a warp-uniform test first
-            if constexpr (IMAGES) {
-              queued = queue_push_f(
-                  fc.qc, have && !ok, [&]() { return qpack(box_id, img, p_off + local_index()); },
-                  qs.q1, qs.cap1, &qs.cnt->q1);
-            } else {                             // queue full: left to the exact pass
-              queue_push_mark(
-                  fc.qc, have && !ok, [&]() { return qpack(box_id, 0, p_off + local_index()); },
-                  qs.q1, qs.cap1, &qs.cnt->q1, qs.ovf, qs.ovf_base, &qs.cnt->ovf);
-            }
-          }
-          if (!queued) {                         // queue full: the FP64 procedure here
-            const int64_t pl = local_index();
-            const float x = __ldg(xyz + 3 * pl), y = __ldg(xyz + 3 * pl + 1),
-                        zc = __ldg(xyz + 3 * pl + 2);
-            const int32_t kx = key_exact_slow(st, lo, hi, N, npix, x, y, zc, bg.sh64[0][ii],
-                                              bg.sh64[1][jj], bg.sh64[2][kk]);
-            if (kx >= 0) {
-              ++fc.n_keyed;
-              if (MODE == kModeDirect && UFC_IDX_OK(kx, o.ncell, 2)) atomicAdd(o.counts + kx, 1);
-              if (MODE == kModeDense) {
-                const uint32_t dk = dense_key(kx, npix, o);
-                if (UFC_IDX_OK(dk >> kOffBits, o.nbuckets, 1)) atomicAdd(ghist + (dk >> kOffBits), 1u);
-                const unsigned long long at = atomicAdd(o.dense_count, 1ull);
-                if ((int64_t)at < o.dense_cap) o.dense[at] = dk;
-              }
-            }
-            if (MODE == kModeKeys) o.keys[p_off + pl] = kx;
+            // queue full: left to the exact pass
+            queue_push_mark(
+                fc.qc, have && !ok, [&]() { return qpack(box_id, 0, p_off + local_index()); },
+                qs.q1, qs.cap1, &qs.cnt->q1, qs.ovf, qs.ovf_base, &qs.cnt->ovf);
           }
           if (MODE == kModeKeys) {
-            if (have && queued) o.keys[p_off + local_index()] = ok ? key : kKeyUndecided;
-          } else if (MODE == kModeDirect) {
-            if (ok && UFC_IDX_OK(key, o.ncell, 2)) atomicAdd(o.counts + key, 1);
+            if (have) o.keys[p_off + local_index()] = ok ? key : kKeyUndecided;
           } else {
             uint32_t dk = 0u, bucket = 0u;
             bool wrapped = false;
@@ -841,8 +795,6 @@ __device__ __forceinline__ void emit_late(int32_t key, int64_t p, int32_t npix,
                                           const KeyOut& o, WarpChunk& wc) {
   if (MODE == kModeKeys) {
     o.keys[p] = key;
-  } else if (MODE == kModeDirect) {
-    if (key >= 0 && UFC_IDX_OK(key, o.ncell, 2)) atomicAdd(o.counts + key, 1);
   } else {
     uint32_t dk = key >= 0 ? dense_key(key, npix, o) : 0u;
     if (key >= 0 && UFC_IDX_OK(dk >> kOffBits, o.nbuckets, 1)) atomicAdd(o.hist + (dk >> kOffBits), 1u);
@@ -884,30 +836,20 @@ k_refine(BoxesParam bp, ShellTable st, int32_t N, int32_t npix, KeyOut o, Queues
     if (have) e = qs.q1[i];
     have = have && e != kQEmpty;
     if (have) {
-      const int b = qbox(e), img = qimg(e);
       p = qidx(e);
-      const BoxGeom& g = bp.box[b];
-      int ii = 0, jj = 0, kk = 0;
-      if (g.R) {                                   // periodic images only
-        const int n1 = 2 * g.R + 1;
-        ii = img / (n1 * n1); jj = (img / n1) % n1; kk = img % n1;
-      }
-      const float* xp = bp.xyz[b] + 3 * p;
-      float x = xp[0], y = xp[1], zc = xp[2];
-      key = key_refine(chih_s, chil_s, atab_s, g.shell_lo, g.shell_hi, N, npix, x, y, zc, g.shf[0][ii],
-                       g.shf[1][jj], g.shf[2][kk], g.shlo[0][ii], g.shlo[1][jj],
-                       g.shlo[2][kk]);
+      const BoxGeom& g = bp.box[qbox(e)];
+      const float* xp = bp.xyz[qbox(e)] + 3 * p;
+      key = key_refine(chih_s, chil_s, atab_s, g.shell_lo, g.shell_hi, N, npix, xp[0], xp[1], xp[2],
+                       g.shf[0][0], g.shf[1][0], g.shf[2][0], g.shlo[0][0], g.shlo[1][0],
+                       g.shlo[2][0]);
       ++n_ref;
     }
     const bool und = have && key == kKeyUndecided;
     if (!queue_push(qc, und, e, qs.q2, qs.cap2, &qs.cnt->q2)) {
-      const int b = qbox(e), img = qimg(e);
-      const BoxGeom& g = bp.box[b];
-      const int n1 = 2 * g.R + 1;
-      const int ii = img / (n1 * n1), jj = (img / n1) % n1, kk = img % n1;
-      const float* xp = bp.xyz[b] + 3 * p;
+      const BoxGeom& g = bp.box[qbox(e)];
+      const float* xp = bp.xyz[qbox(e)] + 3 * p;
       key = key_exact(st, g.shell_lo, g.shell_hi, N, npix, xp[0], xp[1], xp[2],
-                      g.sh64[0][ii], g.sh64[1][jj], g.sh64[2][kk]);
+                      g.sh64[0][0], g.sh64[1][0], g.sh64[2][0]);
       if (key == kKeyInvalid) ++n_invalid;
     }
     const bool done = have && key != kKeyUndecided;
@@ -948,14 +890,11 @@ k_exact(BoxesParam bp, ShellTable st, int32_t N, int32_t npix, KeyOut o, Queues 
     if (have) e = qs.q2[i];
     have = have && e != kQEmpty;
     if (have) {
-      const int b = qbox(e), img = qimg(e);
       p = qidx(e);
-      const BoxGeom& g = bp.box[b];
-      const int n1 = 2 * g.R + 1;
-      const int ii = img / (n1 * n1), jj = (img / n1) % n1, kk = img % n1;
-      const float* xp = bp.xyz[b] + 3 * p;
+      const BoxGeom& g = bp.box[qbox(e)];
+      const float* xp = bp.xyz[qbox(e)] + 3 * p;
       key = key_exact(st, g.shell_lo, g.shell_hi, N, npix, xp[0], xp[1], xp[2],
-                      g.sh64[0][ii], g.sh64[1][jj], g.sh64[2][kk]);
+                      g.sh64[0][0], g.sh64[1][0], g.sh64[2][0]);
       ++n_ex;
       if (key == kKeyInvalid) ++n_invalid;
       n_keyed += key >= 0;
@@ -1002,7 +941,6 @@ k_overflow(BoxesParam bp, int nbox, ShellTable st, int32_t N, int32_t npix, KeyO
       if (MODE == kModeKeys) o.keys[p] = key;
       if (key >= 0) {
         ++n_keyed;
-        if (MODE == kModeDirect && UFC_IDX_OK(key, o.ncell, 2)) atomicAdd(o.counts + key, 1);
         if (MODE == kModeDense) {
           const uint32_t dk = dense_key(key, npix, o);
           if (UFC_IDX_OK(dk >> kOffBits, o.nbuckets, 1)) atomicAdd(o.hist + (dk >> kOffBits), 1u);
@@ -1525,7 +1463,8 @@ ufc_status reserve_bin_workspace(ufc_ctx* c, int64_t fast_launches, int64_t tota
                                  int nshell, int nside) {
   const int64_t npix = 12ll * nside * nside;
   const BinSizes z = bin_sizes(c, fast_launches, total_img, nshell, nside);
-  if (!ws_get(c, kSlotQueue1, z.cap1 * 8) || !ws_get(c, kSlotQueue2, z.cap2 * 8) ||
+  if (!ws_get(c, kSlotTables, sizeof(BinTables)) ||
+      !ws_get(c, kSlotQueue1, z.cap1 * 8) || !ws_get(c, kSlotQueue2, z.cap2 * 8) ||
       !ws_get(c, kSlotOvf, (size_t)((total_img + 31) / 32) * 4))   // overflow bits (bound)
     return UFC_ERR_ALLOC;
   if (nside >= 64 && npix * nshell * 4 > (32ll << 20) && z.nb < (1ll << 17)) {
@@ -1547,14 +1486,15 @@ static cudaEvent_t copy_event(ufc_ctx* c, size_t i) {
   return c->copy_events[i];
 }
 
-// Shell table and box geometry of a batched call's boxes (the persistent
-// batch kernel of stats.cu keys particles with the same stages).
+// Shell table (chi not NULL) and box geometry of a batched call's boxes.
 ufc_status batch_geometry(ufc_ctx* c, const double* chi, int nshell, const ufc_box* boxes,
                           int nbox, ShellTable& st, BoxGeom* bg) {
-  ufc_status s = make_table(c, chi, nshell, st);
-  if (s) return s;
+  if (chi) {
+    const ufc_status s = make_table(c, chi, nshell, st);
+    if (s) return s;
+  }
   for (int k = 0; k < nbox; ++k) {
-    s = make_box(c, boxes[k], nshell, bg[k]);
+    const ufc_status s = make_box(c, boxes[k], nshell, bg[k]);
     if (s) return s;
   }
   return UFC_OK;
@@ -1659,6 +1599,105 @@ ufc_status run_keys_pipeline(ufc_ctx* c, int mode_req, const float* const* xyz,
                      (size_t)plan.nbuckets * 4 + fixed <= (size_t)c->smem_optin;
   }
 
+  // the staged copies of host input overwrite the staging slot only after the
+  // work already on the context stream (which may still read it) has finished
+  size_t nev = 1;
+  if (xyz_host) {
+    if (!c->copy_stream)
+      UFC_CUDA(c, cudaStreamCreateWithFlags(&c->copy_stream, cudaStreamNonBlocking));
+    cudaEvent_t e0 = copy_event(c, 0);
+    if (!e0) return set_err(c, UFC_ERR_CUDA, "cudaEventCreate failed");
+    UFC_CUDA(c, cudaEventRecord(e0, c->stream));
+    UFC_CUDA(c, cudaStreamWaitEvent(c->copy_stream, e0, 0));
+  }
+  // particles [p0, p0 + cnt) of box k copied; the context stream waits for them
+  auto stage = [&](int k, int64_t p0, int64_t cnt) -> ufc_status {
+    UFC_CUDA(c, cudaMemcpyAsync(const_cast<float*>(xyz[k]) + 3 * p0, xyz_host[k] + 3 * p0,
+                                (size_t)cnt * 12, cudaMemcpyHostToDevice, c->copy_stream));
+    cudaEvent_t e = copy_event(c, nev++);
+    if (!e) return set_err(c, UFC_ERR_CUDA, "cudaEventCreate failed");
+    UFC_CUDA(c, cudaEventRecord(e, c->copy_stream));
+    UFC_CUDA(c, cudaStreamWaitEvent(c->stream, e, 0));
+    return UFC_OK;
+  };
+  BinTables* tab = nullptr;
+  float lut_scale = 0.f;
+
+  if (plan.mode == kModeDirect) {
+    // counts cleared with the tables when they are small and aligned, by a
+    // memset otherwise
+    const size_t map_bytes = (size_t)nshell * npix * 4;
+    const bool clear = !(flags & UFC_BIN_ACCUMULATE);
+    const bool with_prep = clear && (reinterpret_cast<uintptr_t>(counts) & 15) == 0 &&
+                           map_bytes % 16 == 0 && map_bytes <= (64ull << 20);
+    if (clear && !with_prep) UFC_CUDA(c, cudaMemsetAsync(counts, 0, map_bytes, c->stream));
+    s = bin_prep(c, st, with_prep ? counts : nullptr, map_bytes, &tab, &lut_scale);
+    if (s) return s;
+    DirectArgs a;
+    std::memset(&a, 0, sizeof a);
+    a.lut_scale = lut_scale;
+    a.tab = tab;
+    a.bd = bd;
+    a.N = nside;
+    a.npix = (int32_t)npix;
+    a.ncell = (int64_t)nshell * npix;
+    a.cnt = (BinCounters*)c->counters;
+    auto item = [&](int k, int64_t p0, int64_t cnt) {
+      DirectItem d;
+      std::memset(&d, 0, sizeof d);
+      const BoxGeom& g = bp.box[k];
+      d.xyz = xyz[k] + 3 * p0;
+      d.n = cnt;
+      d.counts = counts;
+      d.shell_lo = g.shell_lo;
+      d.shell_hi = g.shell_hi;
+      for (int ax = 0; ax < 3; ++ax) {
+        d.shf[ax] = g.shf[ax][0];
+        d.shlo[ax] = g.shlo[ax][0];
+        d.sh64[ax] = g.sh64[ax][0];
+      }
+      return d;
+    };
+    // the boxes without images in one launch (host input: one per staged
+    // chunk), each box with images in its own
+    auto run = [&]() -> ufc_status {
+      int64_t total = 0;
+      for (int i = 0; i < a.nitems; ++i) total += a.inl[i].n;
+      a.task = direct_task(c, total);
+      a.ntasks = 0;
+      for (int i = 0; i < a.nitems; ++i) {
+        a.inl[i].task0 = a.ntasks;
+        a.ntasks += (a.inl[i].n + a.task - 1) / a.task;
+      }
+      const ufc_status r = launch_direct(c, a, 0);
+      a.nitems = 0;
+      return r;
+    };
+    for (int k = 0; k < nbox; ++k) {
+      const bool images = bp.box[k].nimg > 1;
+      const int64_t step = xyz_host ? kHostChunk : std::max<int64_t>(n[k], 1);
+      for (int64_t p0 = 0; p0 < n[k]; p0 += step) {
+        const int64_t cnt = std::min(step, n[k] - p0);
+        if (xyz_host && (s = stage(k, p0, cnt))) return s;
+        if (images) {
+          if (p0 > 0) {                        // (the bounds of another chunk)
+            s = bin_prep_bounds(c, tab, k);
+            if (s) return s;
+          }
+          DirectArgs ai = a;
+          ai.nitems = 1;
+          ai.inl[0] = item(k, p0, cnt);
+          s = launch_direct_images(c, ai, bp.box[k], k);
+        } else {
+          a.inl[a.nitems++] = item(k, p0, cnt);
+          s = xyz_host ? run() : UFC_OK;
+        }
+        if (s) return s;
+      }
+    }
+    return a.nitems ? run() : UFC_OK;
+  }
+
   // workspace
   const BinSizes z = bin_sizes(c, fast_launches, total_img, nshell, nside);
   Queues qs;
@@ -1668,12 +1707,13 @@ ufc_status run_keys_pipeline(ufc_ctx* c, int mode_req, const float* const* xyz,
   qs.q2 = (uint64_t*)ws_get(c, kSlotQueue2, z.cap2 * 8);
   if (!qs.q1 || !qs.q2) return UFC_ERR_ALLOC;
   qs.cnt = (BinCounters*)c->counters;
-  UFC_CUDA(c, cudaMemsetAsync(qs.cnt, 0, offsetof(BinCounters, timeouts), c->stream));
-  // overflow bits: one per particle of the boxes without periodic images
+  s = bin_prep(c, st, nullptr, 0, &tab, &lut_scale);
+  if (s) return s;
+  // overflow bits: one per particle
   int64_t nbits = 0;
   for (int k = 0; k < nbox; ++k) {
     bp.bit_base[k] = nbits;
-    if (bp.box[k].nimg == 1) nbits += n[k];
+    nbits += n[k];
   }
   const int64_t ovf_words = (nbits + 31) / 32;
   qs.ovf = (uint32_t*)ws_get(c, kSlotOvf, (size_t)ovf_words * 4);
@@ -1706,82 +1746,35 @@ ufc_status run_keys_pipeline(ufc_ctx* c, int mode_req, const float* const* xyz,
                                     (size_t)(nshell - plan.shell1) * npix * 4, c->stream));
     }
     smem = plan.smem_hist ? plan.nbuckets * 4 : 0;
-  } else if (plan.mode == kModeDirect) {
-    if (!(flags & UFC_BIN_ACCUMULATE))
-      UFC_CUDA(c, cudaMemsetAsync(counts, 0, (size_t)nshell * npix * 4, c->stream));
-  }
-  // shell lookup table over r^2: lut[i] = edges with lo2 <= i / scale
-  LutParam lp;
-  {
-    // bins 0 .. kLut-2 cover [0, hi2[nshell]]
-    const double top = std::max((double)st.hi2[nshell], 1e-30);
-    lp.scale = (float)std::min((kLut - 2) / top, 1e30);
-    const double sc = (double)lp.scale;
-    int e0 = 0;
-    for (int i = 0; i < kLut; ++i) {
-      // r2 whose fminf(r2 * scale, kLut - 1) rounds to i has r2 * scale in
-      // [i - 1/2, i + 1/2] up to the product's rounding (< 2^-11 here);
-      // the range is widened by 2^-10
-      const double rlo = ((double)i - 0.5 - 0x1p-10) / sc;
-      const double rhi = (i == kLut - 1) ? INFINITY : ((double)i + 0.5 + 0x1p-10) / sc;
-      while (e0 <= nshell && (double)st.hi2[e0] <= rlo) ++e0;
-      const bool clean = e0 > nshell || (double)st.lo2[e0] > rhi;
-      lp.v[i] = (uint16_t)(e0 | (clean ? 0 : kLutScan));
-    }
   }
   // fast stage: one launch per box, or per staged chunk for host input
   const int tma_smem = kWSmemBase +
                        (plan.mode == kModeDense && plan.smem_hist ? ((plan.nbuckets + 1) / 2) * 4 : 0);
-  if (xyz_host) {
-    if (!c->copy_stream)
-      UFC_CUDA(c, cudaStreamCreateWithFlags(&c->copy_stream, cudaStreamNonBlocking));
-    // the copies overwrite the staging slot only after the work already on
-    // the context stream (which may still read it) has finished
-    cudaEvent_t e0 = copy_event(c, 0);
-    if (!e0) return set_err(c, UFC_ERR_CUDA, "cudaEventCreate failed");
-    UFC_CUDA(c, cudaEventRecord(e0, c->stream));
-    UFC_CUDA(c, cudaStreamWaitEvent(c->copy_stream, e0, 0));
-  }
-  size_t nev = 1;
   for (int k = 0; k < nbox; ++k) {
     const int64_t step = xyz_host ? kHostChunk : std::max<int64_t>(n[k], 1);
     for (int64_t p0 = 0; p0 < n[k]; p0 += step) {
       const int64_t cnt = std::min(step, n[k] - p0);
       const float* src = xyz[k] + 3 * p0;
-      if (xyz_host) {
-        UFC_CUDA(c, cudaMemcpyAsync(const_cast<float*>(src), xyz_host[k] + 3 * p0,
-                                    (size_t)cnt * 12, cudaMemcpyHostToDevice, c->copy_stream));
-        cudaEvent_t e = copy_event(c, nev++);
-        if (!e) return set_err(c, UFC_ERR_CUDA, "cudaEventCreate failed");
-        UFC_CUDA(c, cudaEventRecord(e, c->copy_stream));
-        UFC_CUDA(c, cudaStreamWaitEvent(c->stream, e, 0));
-      }
+      if (xyz_host && (s = stage(k, p0, cnt))) return s;
       const bool tma = (reinterpret_cast<uintptr_t>(src) & 15) == 0;
       ProfScope ps_(c, "k_fast");
       if (tma) {
         qs.ovf_base = bp.bit_base[k];
-        const bool images = bp.box[k].nimg > 1;
-#define UFC_LAUNCH_TMA(M, I)                                                                    \
-  UFC_CUDA(c, cudaFuncSetAttribute(k_fast_tma<M, I>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
+#define UFC_LAUNCH_TMA(M)                                                                        \
+  UFC_CUDA(c, cudaFuncSetAttribute(k_fast_tma<M>, cudaFuncAttributeMaxDynamicSharedMemorySize,    \
                                    tma_smem));                                                   \
-  k_fast_tma<M, I><<<c->num_sms, kWThreads, tma_smem, c->stream>>>(                              \
-      src, cnt, p0, k, bp.box[k], st, lp, bd, nside, (int32_t)npix, o, qs)
-        if (plan.mode == kModeDense) {
-          if (images) { UFC_LAUNCH_TMA(kModeDense, true); } else { UFC_LAUNCH_TMA(kModeDense, false); }
-        } else if (plan.mode == kModeDirect) {
-          if (images) { UFC_LAUNCH_TMA(kModeDirect, true); } else { UFC_LAUNCH_TMA(kModeDirect, false); }
-        } else {
-          if (images) { UFC_LAUNCH_TMA(kModeKeys, true); } else { UFC_LAUNCH_TMA(kModeKeys, false); }
-        }
+  k_fast_tma<M><<<c->num_sms, kWThreads, tma_smem, c->stream>>>(                                 \
+      src, cnt, p0, k, bp.box[k], st, tab, lut_scale, bd, nside, (int32_t)npix, o, qs)
+        if (plan.mode == kModeDense) { UFC_LAUNCH_TMA(kModeDense); }
+        else { UFC_LAUNCH_TMA(kModeKeys); }
 #undef UFC_LAUNCH_TMA
       } else {
         const int ssm = plan.mode == kModeDense ? smem : 0;
 #define UFC_LAUNCH_PLAIN(M)                                                                      \
   UFC_CUDA(c, cudaFuncSetAttribute(k_fast<M>, cudaFuncAttributeMaxDynamicSharedMemorySize, ssm)); \
   k_fast<M><<<(ssm > 0 ? 1 : 2) * c->num_sms, kFastThreads, ssm, c->stream>>>(                     \
-      src, cnt, p0, k, bp.box[k], st, lp, bd, nside, (int32_t)npix, o, qs)
+      src, cnt, p0, k, bp.box[k], st, tab, lut_scale, bd, nside, (int32_t)npix, o, qs)
         if (plan.mode == kModeDense) { UFC_LAUNCH_PLAIN(kModeDense); }
-        else if (plan.mode == kModeDirect) { UFC_LAUNCH_PLAIN(kModeDirect); }
         else { UFC_LAUNCH_PLAIN(kModeKeys); }
 #undef UFC_LAUNCH_PLAIN
       }
@@ -1801,20 +1794,6 @@ ufc_status run_keys_pipeline(ufc_ctx* c, int mode_req, const float* const* xyz,
     if (ovf_words) {
       ProfScope ps_(c, "k_overflow");
       k_overflow<kModeDense><<<lgrid, 256, 0, c->stream>>>(bp, nbox, st, nside, (int32_t)npix, o, qs,
-                                                      ovf_words);
-    }
-  } else if (plan.mode == kModeDirect) {
-    {
-      ProfScope ps_(c, "k_refine");
-      k_refine<kModeDirect><<<lgrid, 256, 0, c->stream>>>(bp, st, nside, (int32_t)npix, o, qs);
-    }
-    {
-      ProfScope ps_(c, "k_exact");
-      k_exact<kModeDirect><<<lgrid, 256, 0, c->stream>>>(bp, st, nside, (int32_t)npix, o, qs);
-    }
-    if (ovf_words) {
-      ProfScope ps_(c, "k_overflow");
-      k_overflow<kModeDirect><<<lgrid, 256, 0, c->stream>>>(bp, nbox, st, nside, (int32_t)npix, o, qs,
                                                       ovf_words);
     }
   } else {

@@ -39,6 +39,7 @@ void grad_from_sums(const double* sm, int S, int npix, double w_var, double w_sk
                     const double* dA, const double* dC, double* grad, double* G, double* H);
 cudaError_t take_checks_bin(CheckRec* out, cudaStream_t s);
 cudaError_t take_checks_stats(CheckRec* out, cudaStream_t s);
+cudaError_t take_checks_direct(CheckRec* out, cudaStream_t s);
 ufc_status run_check_selftest(ufc_ctx* c, int64_t index, int64_t bound);
 ufc_status run_welford_update(ufc_ctx* c, const double* v, int nvec, int d, double* st);
 ufc_status run_stats_vector(ufc_ctx* c, const double* m, const int64_t* pdf, int nbins, double* v);
@@ -46,14 +47,12 @@ ufc_status run_kappa_stats_noalloc(ufc_ctx* c, const int32_t* counts, int S, int
                                    const double* A, double C, double lo, double hi, int nbins,
                                    float* kappa, double* moments, int64_t* pdf);
 ufc_status run_welford_merge(ufc_ctx* c, double* a, const double* b, int d);
-void batch_persistent_bytes(const ufc_ctx* c, int nreal, int nbox, int S, int nside,
-                            size_t* maps, size_t* desc);
-ufc_status batch_persistent_prepare(ufc_ctx* c, int nreal, int nbox, const float* const* xyz,
-                                    const int64_t* n, const ufc_box* boxes, const double* chi,
-                                    int S, int nside, const double* A, const double* C, double lo,
-                                    double hi, int nbins, double* moments, int64_t* pdf,
-                                    double* stats, double* state, char* maps, char* desc);
-ufc_status batch_persistent_enqueue(ufc_ctx* c, char* maps, char* desc);
+bool batch_stages_ok(const ufc_ctx* c, int nreal, int nbox, int S, int nside, size_t max_bytes);
+ufc_status run_batch_stages(ufc_ctx* c, int nreal, int nbox, const float* const* xyz,
+                            const int64_t* n, const ufc_box* boxes, const double* chi, int S,
+                            int nside, const double* A, const double* C, double lo, double hi,
+                            int nbins, double* moments, int64_t* pdf, double* stats,
+                            double* state);
 ufc_status run_welford_finalize(ufc_ctx* c, const double* st, int d, int ddof, double* mean,
                                 double* cov, double* corr);
 ufc_status reserve_bin_workspace(ufc_ctx* c, int64_t fast_launches, int64_t total_img,
@@ -199,6 +198,11 @@ ufc_status ufc_destroy(ufc_ctx* c) {
   for (cudaEvent_t e : c->aux_ev)
     if (e) cudaEventDestroy(e);
   if (c->graph_exec) cudaGraphExecDestroy(c->graph_exec);
+  if (c->batch_host) {
+    if (c->batch_ev) cudaEventSynchronize(c->batch_ev);
+    cudaFreeHost(c->batch_host);
+  }
+  if (c->batch_ev) cudaEventDestroy(c->batch_ev);
   for (int k = 0; k < ufc_ctx::kMaxLanes; ++k) {
     if (c->lane_stream[k]) cudaStreamSynchronize(c->lane_stream[k]);
     if (c->lanes[k]) { c->lanes[k]->stream = c->lane_stream[k]; ufc_destroy(c->lanes[k]); }
@@ -238,9 +242,10 @@ ufc_status ufc_synchronize(ufc_ctx* c) {
     total += t[k];
   }
   // index-test records (per device and translation unit), after all the work
-  CheckRec rec[2] = {};
+  CheckRec rec[3] = {};
   UFC_CUDA(c, take_checks_bin(&rec[0], c->stream));
   UFC_CUDA(c, take_checks_stats(&rec[1], c->stream));
+  UFC_CUDA(c, take_checks_direct(&rec[2], c->stream));
   UFC_CUDA(c, cudaStreamSynchronize(c->stream));
   if (total)
     return set_err(c, UFC_ERR_TIMEOUT,
@@ -829,33 +834,21 @@ ufc_status ufc_batched_stats(ufc_ctx* c, int32_t nreal, int32_t nbox, const floa
   }
   const int d = 6 + nbins;
   const int64_t npix_b = 12ll * nside * nside;
-  // one persistent kernel for small maps without periodic images whose maps
-  // fit in 4 GB of workspace together
-  bool persistent = !(flags & UFC_BATCH_LAUNCHES) && (size_t)nshell * npix_b * 4 <= kLaneMapMax;
-  for (int i = 0; i < nreal * nbox && persistent; ++i) persistent = boxes[i].replicate == 0;
-  size_t pmaps = 0, pdesc = 0;
-  if (persistent) {
-    batch_persistent_bytes(c, nreal, nbox, nshell, nside, &pmaps, &pdesc);
-    persistent = pmaps <= (4ull << 30);
-  }
-  char* bmaps = nullptr;
-  char* bdesc = nullptr;
-  ufc_status s = UFC_OK;
-  if (persistent) {
-    bmaps = (char*)ws_get(c, kSlotBatchMaps, pmaps);
-    bdesc = (char*)ws_get(c, kSlotBatchDesc, pdesc);
-    if (!bmaps || !bdesc) return UFC_ERR_ALLOC;
-    // descriptors uploaded now, before any capture (also before a cached
-    // graph's relaunch, which reads them)
-    s = batch_persistent_prepare(c, nreal, nbox, xyz, n, boxes, chi, nshell, nside, A, C, lo, hi,
-                                 nbins, moments, pdf, stats, state, bmaps, bdesc);
-    if (s) return s;
-  } else {
-    s = reserve_bin_workspace(c, nbox, max_img, nshell, nside);
-    if (s) return s;
-    // per-block partial sums of the kappa and moment kernels
-    if (!ws_get(c, kSlotPartials, (size_t)20 * c->num_sms * 8)) return UFC_ERR_ALLOC;
-  }
+  // small maps without periodic images whose maps fit in 4 GB of workspace
+  // together: stage by stage over all realisations
+  bool stages = !(flags & UFC_BATCH_LAUNCHES) && (size_t)nshell * npix_b * 4 <= kLaneMapMax &&
+                nside >= 1 && nside <= UFC_MAX_NSIDE && (nside & (nside - 1)) == 0;
+  for (int i = 0; i < nreal * nbox && stages; ++i) stages = boxes[i].replicate == 0;
+  if (stages && batch_stages_ok(c, nreal, nbox, nshell, nside, 4ull << 30))
+    return run_batch_stages(c, nreal, nbox, xyz, n, boxes, chi, nshell, nside, A, C, lo, hi, nbins,
+                            moments, pdf, stats, state);
+  ufc_status s = reserve_bin_workspace(c, nbox, max_img, nshell, nside);
+  if (s) return s;
+  // per-block partial sums of the kappa and moment kernels, and the new mean of
+  // the Welford update
+  if (!ws_get(c, kSlotPartials, (size_t)20 * c->num_sms * 8) ||
+      !ws_get(c, kSlotWelford, (size_t)d * 8))
+    return UFC_ERR_ALLOC;
   // small maps: realisation r runs on lane r mod nlane, the lanes concurrently
   // (lane 0 is this context with the caller's scratch maps; the others have
   // their own count and kappa maps, workspace and stream)
@@ -863,8 +856,7 @@ ufc_status ufc_batched_stats(ufc_ctx* c, int32_t nreal, int32_t nbox, const floa
   const size_t map_bytes = (size_t)nshell * npix * 4;
   // (and a bound of 8 GB on the lanes' binning workspace, ~16 B per image)
   const int64_t ws_lanes = std::max<int64_t>(1, (8ll << 30) / std::max<int64_t>(1, 16 * max_img));
-  const int nlane = persistent ? 1
-                   : map_bytes <= kLaneMapMax
+  const int nlane = map_bytes <= kLaneMapMax
                         ? (int)std::min<int64_t>({ufc_ctx::kMaxLanes, nreal, ws_lanes})
                         : 1;
   ufc_ctx* lane[ufc_ctx::kMaxLanes] = {c};
@@ -912,8 +904,6 @@ ufc_status ufc_batched_stats(ufc_ctx* c, int32_t nreal, int32_t nbox, const floa
     };
     const size_t nrb = (size_t)nreal * nbox;
     put(&nreal, 4); put(&nbox, 4); put(&nshell, 4); put(&nside, 4); put(&nbins, 4);
-    const int32_t mode[3] = {persistent ? 1 : 0, c->batch_chunk, c->batch_blocks_per_sm};
-    put(mode, sizeof mode);
     put(&lo, 8); put(&hi, 8);
     put(xyz, nrb * sizeof(void*)); put(n, nrb * 8);
     for (size_t i = 0; i < nrb; ++i) {
@@ -946,8 +936,7 @@ ufc_status ufc_batched_stats(ufc_ctx* c, int32_t nreal, int32_t nbox, const floa
     UFC_CUDA(c, cudaEventRecord(c->lane_ev[0], c->stream));
     for (int k = 1; k < nlane; ++k) UFC_CUDA(c, cudaStreamWaitEvent(lane[k]->stream, c->lane_ev[0], 0));
   }
-  if (persistent) s = batch_persistent_enqueue(c, bmaps, bdesc);
-  for (int r = 0; r < nreal && !s && !persistent; ++r) {
+  for (int r = 0; r < nreal && !s; ++r) {
     ufc_ctx* lc = lane[r % nlane];
     int32_t* cnt = lane_counts[r % nlane];
     float* kap = lane_kappa[r % nlane];
@@ -966,7 +955,7 @@ ufc_status ufc_batched_stats(ufc_ctx* c, int32_t nreal, int32_t nbox, const floa
     if (e == cudaSuccess) cudaStreamWaitEvent(c->stream, c->lane_ev[k], 0);
     else if (!s) s = set_err(c, UFC_ERR_CUDA, "lane join: %s", cudaGetErrorString(e));
   }
-  if (!s && !persistent) s = run_welford_update(c, stats, nreal, d, state);
+  if (!s) s = run_welford_update(c, stats, nreal, d, state);
   if (graph) {
     cudaStream_t cap = c->stream;
     c->stream = user;

@@ -18,7 +18,7 @@ struct ufc_ctx {
   int num_sms = 0;
   int smem_optin = 0;            // shared memory per block with opt-in (bytes)
   // grow-only device buffers, one per slot
-  static constexpr int kSlots = 18;
+  static constexpr int kSlots = 19;
   void* buf[kSlots] = {};
   size_t cap[kSlots] = {};
   void* counters = nullptr;      // ufc::BinCounters of the last binning call
@@ -49,10 +49,12 @@ struct ufc_ctx {
   cudaStream_t lane_stream[kMaxLanes] = {};
   cudaEvent_t lane_ev[kMaxLanes + 1] = {};
   ufc_ctx* owner = nullptr;
-  // tuning (ufc_set_tuning) and the prepared launch of the persistent
-  // batch kernel (descriptors uploaded, launch arguments kept here)
+  // tuning (ufc_set_tuning) of the batched call, and its page-locked staging
+  // buffer (items and coefficients; batch_ev: the last copy out of it)
   int32_t batch_chunk = 0, batch_blocks_per_sm = 0;
-  std::vector<unsigned char> batch_launch;
+  void* batch_host = nullptr;
+  size_t batch_host_cap = 0;
+  cudaEvent_t batch_ev = nullptr;
 };
 
 namespace ufc {
@@ -68,14 +70,15 @@ enum Slot {
   kSlotCursors,
   kSlotTiles,
   kSlotPartials,
-  kSlotCoeffs,
+  kSlotTables,     // tables of a binning call (BinTables)
   kSlotMisc,
   kSlotStage,      // device copy of host particle positions (ufc_bin_host)
   kSlotSht,        // ring transforms, Legendre seeds, partial a_lm (ufc_map2alm)
   kSlotOvf,        // one bit per particle image: left undecided when queue 1 was full
   kSlotLaneMap,    // a lane's count map and kappa map (ufc_batched_stats)
-  kSlotBatchMaps,  // persistent batch kernel: per-realisation maps and partial sums
-  kSlotBatchDesc,  // persistent batch kernel: task descriptors and queue counters
+  kSlotBatchMaps,  // batched call: per-realisation maps and partial sums
+  kSlotBatchDesc,  // batched call: items, coefficients and counters
+  kSlotWelford,    // the new mean of a Welford update
 };
 
 inline ufc_status set_err(ufc_ctx* c, ufc_status s, const char* fmt, ...) {

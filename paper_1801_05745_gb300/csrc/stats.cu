@@ -12,6 +12,7 @@
 
 #include "common.cuh"
 #include "ctx.h"
+#include "direct.cuh"
 #include "packed.cuh"
 #include "pixel.cuh"
 
@@ -723,13 +724,14 @@ __device__ __forceinline__ void moments_final_block(const double* ksum_part, int
   m[9] = N;
 }
 
-// Blocks of the moment pass: 4 per SM (32 warps; four loads in flight per
-// thread), no more than there are pixels for.  What bounds the pass is the
+// Blocks of the moment pass: 4 per SM (32 warps), no more than there are
+// pixels for at four per thread (the loads a thread has in flight; a block of
+// fewer pixels pays its prologue and its PDF's global atomics for little).  What bounds the pass is the
 // latency of a pixel's chain (load, shared-memory histogram, double-float
 // sums): with 2 blocks per SM and one pixel at a time it took 200 us for the
 // 12.6 M pixels of Nside 1024.
 static int moments_grid(int num_sms, int npix) {
-  return std::min(4 * num_sms, (npix + kMT - 1) / kMT);
+  return std::min(4 * num_sms, (npix + 4 * kMT - 1) / (4 * kMT));
 }
 
 // The last block to finish (ticket) turns the partial sums into the moments:
@@ -777,60 +779,85 @@ __global__ void k_stats_vector(const double* __restrict__ m, const unsigned long
 }
 
 // ---------------------------------------------------------- Welford -----
-// Welford update of st by the nvec vectors v [nvec][d] in order (every thread
-// of the block calls it; sh holds 2 rc d doubles).  Runs of rc vectors: the
-// deltas of each vector against the running mean (dold = x - mean before,
-// dnew = x - mean after) are formed in order into shared memory, the mean
-// updated as they are; then every element of M2 takes the run's products
-// as one chain of fused multiply-adds in a register, one global read and
-// write per run instead of per vector.  The chain per element is the same as
-// one vector at a time, so the result does not depend on rc or on the block
-// size.  The count is read once and written once.
-__device__ __forceinline__ void welford_update_block(const double* v, int nvec, int d, double* st,
-                                                     double* sh, int rc) {
+// Welford update of st by the nvec vectors v [nvec][d] in order.  Element
+// (i, j) of M2 takes the products dold_i dnew_j of the vectors as one chain of
+// fused multiply-adds (dold = x - mean before, dnew = x - mean after), so the
+// elements are independent given the deltas, and a component's deltas are one
+// short chain (difference, mean += delta (1 / n), difference).  A block owns 16 x 16
+// elements: its first 256 threads hold one each in a register, and one more
+// warp forms the deltas of the block's 16 rows and 16 columns, run after run
+// of kWfRun vectors into the other of two buffers while the run before is
+// added.  (The chains are the same whatever the blocks: the result does not
+// depend on how the vectors are split over calls.)  Every block reads the old
+// mean; the blocks of the first column leave the new one in `mean_new`, and the
+// last block to finish (ticket, left at 0) copies it into the state.
+//
+// FP64 at 1/64 of the FP32 rate bounds it: one block of 1024 threads took 12 us
+// for one vector of 206 components and 2 ms for 150 (the tail of a batched
+// call); spread over 169 blocks they share the chip's FP64 pipes.
+constexpr int kWfTile = 16;
+constexpr int kWfThreads = kWfTile * kWfTile + 32;
+constexpr int kWfRun = 16;
+__global__ void __launch_bounds__(kWfThreads)
+k_welford_update(const double* __restrict__ v, int nvec, int d, double* __restrict__ st,
+                 double* __restrict__ mean_new, unsigned int* __restrict__ ticket) {
+  __shared__ double dold[2][kWfRun][kWfTile], dnew[2][kWfRun][kWfTile];
+  __shared__ bool last_s;
   double* mean = st + 1;
   double* M2 = st + 1 + d;
   const double n0 = st[0];
-  __syncthreads();
-  for (int r0 = 0; r0 < nvec; r0 += rc) {
-    const int nr = min(rc, nvec - r0);
-    // the run's deltas, in vector order (thread i owns mean[i] throughout)
-    for (int i = threadIdx.x; i < d; i += blockDim.x) {
-      double m = mean[i];
-      for (int q = 0; q < nr; ++q) {
-        const double x = v[(size_t)(r0 + q) * d + i];
-        const double n = n0 + double(r0 + q + 1);
-        const double delta = x - m;
-        m = m + delta / n;
-        sh[(size_t)q * d + i] = delta;                 // dold
-        sh[(size_t)(rc + q) * d + i] = x - m;          // dnew
-      }
-      mean[i] = m;
+  const int i0 = blockIdx.y * kWfTile, j0 = blockIdx.x * kWfTile;
+  const int t = threadIdx.x;
+  const bool maker = t >= kWfTile * kWfTile;         // the warp that forms the deltas
+  const int lane = t & 31;
+  const int comp = (lane < kWfTile ? i0 : j0 - kWfTile) + lane;   // its component
+  double m = maker && comp < d ? mean[comp] : 0.0;
+  const int i = i0 + t / kWfTile, j = j0 + t % kWfTile;
+  const bool mine = !maker && i < d && j < d;
+  double acc = mine ? M2[(size_t)i * d + j] : 0.0;
+  auto make = [&](int r0, int buf) {                 // (the maker warp)
+    // the run's values first (their loads in flight together) and 1 / n of
+    // its vectors, one per lane; the chain is then three operations a vector
+    const double rn = 1.0 / (n0 + double(r0 + (lane & (kWfRun - 1)) + 1));
+    double x[kWfRun];
+#pragma unroll
+    for (int q = 0; q < kWfRun; ++q)
+      x[q] = comp < d && r0 + q < nvec ? v[(size_t)(r0 + q) * d + comp] : 0.0;
+#pragma unroll
+    for (int q = 0; q < kWfRun; ++q) {
+      const double r = __shfl_sync(0xFFFFFFFFu, rn, q);
+      const double a = x[q] - m;
+      const double mq = __fma_rn(a, r, m);
+      if (r0 + q < nvec) m = mq;
+      if (lane < kWfTile) dold[buf][q][lane] = a;
+      else dnew[buf][q][lane - kWfTile] = x[q] - mq;
     }
-    __syncthreads();
-    for (int k = threadIdx.x; k < d * d; k += blockDim.x) {
-      const int i = k / d, j = k - i * d;
-      double acc = M2[k];
+  };
+  if (maker) make(0, 0);
+  __syncthreads();
+  for (int r0 = 0, buf = 0; r0 < nvec; r0 += kWfRun, buf ^= 1) {
+    if (maker) {
+      if (r0 + kWfRun < nvec) make(r0 + kWfRun, buf ^ 1);
+    } else {
+      const int nr = min(kWfRun, nvec - r0);
       for (int q = 0; q < nr; ++q)
-        acc = __fma_rn(sh[(size_t)q * d + i], sh[(size_t)(rc + q) * d + j], acc);
-      M2[k] = acc;
+        acc = __fma_rn(dold[buf][q][t / kWfTile], dnew[buf][q][t % kWfTile], acc);
     }
     __syncthreads();
   }
-  if (threadIdx.x == 0) st[0] = n0 + double(nvec);
-}
-
-// Vectors per run of the Welford update for d-dimensional states: the run's
-// deltas (2 rc d doubles) within 48 KB of shared memory, at most 16.
-__host__ __device__ inline int welford_run(int d) {
-  const int rc = 49152 / (16 * d);
-  return rc < 1 ? 1 : (rc > 16 ? 16 : rc);
-}
-
-__global__ void __launch_bounds__(1024)
-k_welford_update(const double* __restrict__ v, int nvec, int d, double* __restrict__ st) {
-  extern __shared__ double sh[];   // the run's deltas: dold[rc][d], dnew[rc][d]
-  welford_update_block(v, nvec, d, st, sh, welford_run(d));
+  if (mine) M2[(size_t)i * d + j] = acc;
+  if (maker && blockIdx.x == 0 && lane < kWfTile && comp < d) mean_new[comp] = m;
+  __threadfence();                                   // the means before the ticket
+  __syncthreads();
+  if (t == 0) last_s = atomicAdd(ticket, 1u) == gridDim.x * gridDim.y - 1;
+  __syncthreads();
+  if (!last_s) return;
+  __threadfence();
+  for (int k = t; k < d; k += kWfThreads) mean[k] = __ldcg(mean_new + k);
+  if (t == 0) {
+    st[0] = n0 + double(nvec);
+    *ticket = 0u;
+  }
 }
 
 __global__ void __launch_bounds__(1024)
@@ -867,37 +894,27 @@ k_welford_final(const double* __restrict__ st, int d, int ddof, double* __restri
   }
 }
 
-// ------------------------------------------------ persistent batch kernel --
-// All realisations of a batched call (Sec. 3.2: statistics over many
-// realisations) in one launch.  A device work queue hands out tasks of
-// `chunk` particles of one (realisation, box); a block bins its task's
-// particles with the three-stage key (FP32, double-float and FP64 stages
-// inline: the same keys as the binning call) and adds them to the
-// realisation's count map with global atomics.  The block that finishes the
-// last task of a realisation then computes its kappa map, moments, PDF and
-// statistics vector by running, one after the other, every block of the
-// serial kappa and moment passes (kappa_vec_block and moments_block with the
-// serial grids), so that the results equal the one-at-a-time calls bit for
-// bit.  The block that finishes the last realisation runs the Welford
-// update over all of them in realisation order.  No block ever waits for
-// another one: completion is detected with atomic counters and fences.
-struct BatchItem {          // one (realisation, box) of a batched call
-  const float* xyz;
-  int64_t n;
-  int64_t task0;            // first task of this item (ascending over the items)
-  int32_t real;
-  int32_t shell_lo, shell_hi;
-  float shf[3], shlo[3];    // the box's shift split as in BoxGeom (no periodic images)
-  double sh64[3];
+// --------------------------------------------------------- batched maps --
+// Realisations of small maps in one call (Sec. 3.2: statistics over many
+// realisations), a launch per stage over all of them: the binning (k_direct,
+// direct.cu, with one item per (realisation, box)), then the kappa maps, the
+// moments with PDF and statistics vector, and the Welford update.  Blocks
+// (x, r) of the kappa and moment stages do what block x of the one-at-a-time
+// kernels does for realisation r (kappa_vec_block, moments_block with the same
+// grids), so the results equal those calls bit for bit.  (One persistent
+// kernel that binned one particle per thread with every stage inline, finished
+// each realisation in one block and ran the Welford update in the last one took
+// 6.1 ms for 150 realisations of 2 x 64^3 particles.)
+struct BatchCoef {          // per realisation: C, then the coefficients [S]
+  float2 c, a[1];
 };
+__host__ __device__ inline size_t batch_coef_stride(int S) {
+  return ((size_t)(S + 1) * sizeof(float2) + 15) / 16 * 16;
+}
 struct BatchArgs {
-  const BatchItem* items;
-  int32_t nitems, chunk;
-  int64_t ntasks;
-  const Coef* coef;         // [nreal]
-  const int32_t* ntask_r;   // [nreal] tasks of each realisation
-  int32_t nreal, S, N, npix;
-  int32_t* counts;          // [nreal][S][npix], zero at the launch
+  const char* coef;         // [nreal] BatchCoef, batch_coef_stride(S) apart
+  int32_t nreal, S, npix;
+  int32_t* counts;          // [nreal][S][npix]
   float* kappa;             // [nreal][npix]
   double* ksum;             // [nreal][gk]
   double* mpart;            // [nreal][3 gm]
@@ -905,148 +922,63 @@ struct BatchArgs {
   double* moments;          // [nreal][10]
   int64_t* pdf;             // [nreal][nbins + 3]
   double* stats;            // [nreal][d]
-  double* state;            // Welford state (1 + d + d^2)
   int32_t nbins, d;
-  unsigned long long* queue;   // [0] next task, [1] realisations finished (zero at launch)
-  unsigned int* done;          // [nreal] tasks finished (zero at launch)
+  unsigned int* done;       // [nreal] blocks of the moment pass finished (zero at launch)
 };
-constexpr int kBT = 256;
-static_assert(kBT == kKV && kBT == kMT, "the persistent blocks reproduce the serial blocks");
 
-// Key of one particle: FP32 stage, then the double-float and FP64 stages for
-// what it leaves undecided (shell_fast: binary search over the FP32 bands).
-__device__ __forceinline__ int32_t batch_key(float x, float y, float zc, const BatchItem& it,
-                                             const float* lo2, const float* hi2,
-                                             const float* chih, const float* chil,
-                                             const float2* atab,
-                                             const ShellTable& st, const Bands& bd, int32_t N,
-                                             int32_t npix) {
-  const int lo = it.shell_lo, hi = it.shell_hi;
-  const float dx = (x + it.shf[0]) + it.shlo[0];
-  const float dy = (y + it.shf[1]) + it.shlo[1];
-  const float dz = (zc + it.shf[2]) + it.shlo[2];
-  const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
-  int32_t key = kKeyUndecided;
-  if (r2 >= bd.r2_min && r2 <= 3.0e38f) {
-    const int32_t b = shell_fast(lo2, hi2, lo, hi, r2);
-    if (b == -1) {
-      key = kKeyOutside;
-    } else if (b >= 0) {
-      const int32_t pix = pixel_fast(N, bd, dx, dy, dz, r2);
-      if (pix != kKeyUndecided) key = b * npix + pix;
-    }
-  }
-  if (key == kKeyUndecided)
-    key = key_refine(chih, chil, atab, lo, hi, N, npix, x, y, zc, it.shf[0], it.shf[1], it.shf[2], it.shlo[0],
-                     it.shlo[1], it.shlo[2]);
-  if (key == kKeyUndecided)
-    key = key_exact(st, lo, hi, N, npix, x, y, zc, it.sh64[0], it.sh64[1], it.sh64[2]);
-  return key;
+__global__ void __launch_bounds__(kKV)
+k_batch_kappa(const __grid_constant__ BatchArgs ba) {
+  __shared__ float ah_s[kMaxShells], al_s[kMaxShells];
+  __shared__ double red[kKV / 32];
+  const int r = blockIdx.y, S = ba.S;
+  clear_pdf((unsigned long long*)ba.pdf + (size_t)(ba.nbins + 3) * r, ba.nbins + 3);
+  const BatchCoef& cf = *reinterpret_cast<const BatchCoef*>(ba.coef + batch_coef_stride(S) * r);
+  for (int i = threadIdx.x; i < S; i += blockDim.x) { ah_s[i] = cf.a[i].x; al_s[i] = cf.a[i].y; }
+  __syncthreads();
+  const double t = kappa_vec_block(ba.counts + (size_t)r * S * ba.npix, ah_s, al_s, S, ba.npix,
+                                   f2{-cf.c.x, -cf.c.y}, ba.kappa + (size_t)r * ba.npix,
+                                   blockIdx.x, ba.gk, red);
+  if (threadIdx.x == 0) ba.ksum[(size_t)r * ba.gk + blockIdx.x] = t;
 }
 
-__global__ void __launch_bounds__(kBT)
-k_batch_persistent(BatchArgs ba, ShellTable st, Bands bd, PdfParam pp) {
-  extern __shared__ __align__(16) uint8_t bsm[];   // PDF histogram, then Welford scratch
-  __shared__ float lo2_s[kMaxShells + 2], hi2_s[kMaxShells + 2];
-  __shared__ float chih_s[kMaxShells + 1], chil_s[kMaxShells + 1];
-  __shared__ float2 atab_s[kAtanTab];
-  __shared__ float ah_s[kMaxShells], al_s[kMaxShells];
-  __shared__ double red[kBT / 32];
-  __shared__ long long task_s;
-  __shared__ int flag_s;
+__global__ void __launch_bounds__(kMT)
+k_batch_moments(const __grid_constant__ BatchArgs ba, const __grid_constant__ PdfParam pp) {
+  extern __shared__ unsigned int hist[];   // [nbins + 3]
+  __shared__ double red[kMT / 32];
   __shared__ double mean_s;
-  for (int i = threadIdx.x; i <= st.nshell; i += kBT) {
-    lo2_s[i] = st.lo2[i];
-    hi2_s[i] = st.hi2[i];
-    chih_s[i] = st.chih[i];
-    chil_s[i] = st.chil[i];
+  __shared__ bool last_s;
+  const int r = blockIdx.y;
+  const double* ks = ba.ksum + (size_t)r * ba.gk;
+  double* mp = ba.mpart + (size_t)r * 3 * ba.gm;
+  int64_t* pd = ba.pdf + (size_t)(ba.nbins + 3) * r;
+  for (int i = threadIdx.x; i < ba.nbins + 3; i += blockDim.x) hist[i] = 0;
+  if (threadIdx.x < 32) {
+    const double s = warp_sum_fixed(ks, ba.gk, 1);          // fixed order, as k_moments
+    if (threadIdx.x == 0) mean_s = s / double(ba.npix);
   }
-  fill_atan_table(atab_s);                 // (the task loop's first barrier follows)
-  const int S = ba.S, npix = ba.npix, ng = npix >> 2;
-  for (;;) {
-    if (threadIdx.x == 0) task_s = (long long)atomicAdd(&ba.queue[0], 1ull);
-    __syncthreads();
-    const long long t = task_s;
-    if (t >= ba.ntasks) break;
-    // the task's item: the last one whose first task is <= t
-    int a = 0, b = ba.nitems;
-    while (b - a > 1) {
-      const int m = (a + b) >> 1;
-      if (ba.items[m].task0 <= t) a = m; else b = m;
-    }
-    const BatchItem it = ba.items[a];
-    const int r = it.real;
-    const int64_t p0 = (t - it.task0) * ba.chunk;
-    const int64_t cnt = min((int64_t)ba.chunk, it.n - p0);
-    int32_t* cmap = ba.counts + (size_t)r * S * npix;
-    for (int64_t i = threadIdx.x; i < cnt; i += kBT) {
-      const float* q = it.xyz + 3 * (p0 + i);
-      const int32_t key = batch_key(__ldg(q), __ldg(q + 1), __ldg(q + 2), it, lo2_s, hi2_s,
-                                    chih_s, chil_s, atab_s, st, bd, ba.N, npix);
-      if (key >= 0 && UFC_IDX_OK(key, (int64_t)S * npix, 8)) atomicAdd(cmap + key, 1);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      __threadfence();                       // this block's keys before its count of the task
-      flag_s = atomicAdd(&ba.done[r], 1u) == (unsigned)(ba.ntask_r[r] - 1);
-    }
-    __syncthreads();
-    if (!flag_s) continue;
-    // ---- the last task of realisation r: its map, moments, PDF, statistics
-    __threadfence();                         // every block's keys of r are visible
-    const Coef& cf = ba.coef[r];
-    for (int i = threadIdx.x; i < S; i += kBT) { ah_s[i] = cf.ah[i]; al_s[i] = cf.al[i]; }
-    __syncthreads();
-    const f2 mc{-cf.ch, -cf.cl};
-    float* kap = ba.kappa + (size_t)r * npix;
-    double* ks = ba.ksum + (size_t)r * ba.gk;
-    for (int vb = 0; vb < ba.gk; ++vb) {
-      if (vb * kKV < ng) {                   // uniform; the serial blocks past the map add 0.0
-        const double v = kappa_vec_block(cmap, ah_s, al_s, S, npix, mc, kap, vb, ba.gk, red);
-        if (threadIdx.x == 0) ks[vb] = v;
-      } else if (threadIdx.x == 0) {
-        ks[vb] = 0.0;
-      }
-    }
-    unsigned int* hist = reinterpret_cast<unsigned int*>(bsm);
-    for (int i = threadIdx.x; i < ba.nbins + 3; i += kBT) hist[i] = 0u;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-      const double sum = warp_sum_fixed(ks, ba.gk, 1);      // fixed order, as k_moments
-      if (threadIdx.x == 0) mean_s = sum / double(npix);
-    }
-    __syncthreads();
-    double* mp = ba.mpart + (size_t)r * 3 * ba.gm;
-    for (int vb = 0; vb < ba.gm; ++vb) {
-      if (vb * kMT < npix) {
-        double o[3];
-        moments_block(kap, npix, mean_s, pp, vb, ba.gm, hist, red, o);
-        if (threadIdx.x == 0) { mp[3 * vb] = o[0]; mp[3 * vb + 1] = o[1]; mp[3 * vb + 2] = o[2]; }
-      } else if (threadIdx.x == 0) {
-        mp[3 * vb] = 0.0; mp[3 * vb + 1] = 0.0; mp[3 * vb + 2] = 0.0;
-      }
-    }
-    __syncthreads();
-    double* mo = ba.moments + 10 * (size_t)r;
-    int64_t* pd = ba.pdf + (size_t)(ba.nbins + 3) * r;
-    moments_final_block(ks, ba.gk, mp, ba.gm, npix, red, mo);
-    for (int i = threadIdx.x; i < ba.nbins + 3; i += kBT) pd[i] = (int64_t)hist[i];
-    __syncthreads();
-    double* v = ba.stats + (size_t)ba.d * r;
-    for (int i = threadIdx.x; i < ba.d; i += kBT) v[i] = i < 6 ? mo[i] : double(pd[i - 6]) / mo[9];
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      __threadfence();                       // r's results before its count
-      flag_s = atomicAdd(&ba.queue[1], 1ull) == (unsigned long long)(ba.nreal - 1);
-    }
-    __syncthreads();
-    if (flag_s) {                            // the last realisation: the covariance update
-      __threadfence();
-      welford_update_block(ba.stats, ba.nreal, ba.d, ba.state, reinterpret_cast<double*>(bsm),
-                           welford_run(ba.d));
-    }
-    __syncthreads();
+  __syncthreads();
+  double o[3];
+  moments_block(ba.kappa + (size_t)r * ba.npix, ba.npix, mean_s, pp, blockIdx.x, ba.gm, hist, red, o);
+  if (threadIdx.x == 0) {
+    mp[3 * blockIdx.x + 0] = o[0];
+    mp[3 * blockIdx.x + 1] = o[1];
+    mp[3 * blockIdx.x + 2] = o[2];
   }
+  __syncthreads();
+  for (int i = threadIdx.x; i < ba.nbins + 3; i += blockDim.x)
+    if (hist[i]) atomicAdd((unsigned long long*)pd + i, (unsigned long long)hist[i]);
+  __threadfence();                         // sums and PDF before this block's count
+  __syncthreads();
+  if (threadIdx.x == 0) last_s = atomicAdd(ba.done + r, 1u) == (unsigned)(ba.gm - 1);
+  __syncthreads();
+  if (!last_s) return;
+  __threadfence();
+  double* mo = ba.moments + 10 * (size_t)r;
+  moments_final_block(ks, ba.gk, mp, ba.gm, ba.npix, red, mo);
+  __syncthreads();
+  double* v = ba.stats + (size_t)ba.d * r;
+  for (int i = threadIdx.x; i < ba.d; i += blockDim.x)
+    v[i] = i < 6 ? mo[i] : double(__ldcg(pd + i - 6)) / mo[9];
 }
 
 // ============================================================== host =====
@@ -1518,12 +1450,13 @@ ufc_status run_welford_update(ufc_ctx* c, const double* v, int nvec, int d, doub
   if (!v || !st || nvec < 0 || d < 1 || d > 8192)
     return set_err(c, UFC_ERR_ARG, "welford_update: bad arguments");
   if (nvec == 0) return UFC_OK;
-  const int smem = 2 * welford_run(d) * d * 8;   // up to 128 KB at d = 8192
-  UFC_CUDA(c, cudaFuncSetAttribute(k_welford_update, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   smem));
+  double* mean_new = (double*)ws_get(c, kSlotWelford, (size_t)d * 8);
+  if (!mean_new) return UFC_ERR_ALLOC;
   {
     ProfScope ps_(c, "k_welford_update");
-    k_welford_update<<<1, 1024, smem, c->stream>>>(v, nvec, d, st);
+    const int g = (d + kWfTile - 1) / kWfTile;
+    k_welford_update<<<dim3(g, g), kWfThreads, 0, c->stream>>>(
+        v, nvec, d, st, mean_new, &reinterpret_cast<BinCounters*>(c->counters)->ticket);
   }
   UFC_CUDA(c, cudaGetLastError());
   return UFC_OK;
@@ -1549,153 +1482,170 @@ ufc_status run_welford_finalize(ufc_ctx* c, const double* st, int d, int ddof, d
   return UFC_OK;
 }
 
-// ---- persistent batched call: host side ------------------------------------
+// ---- batched call: host side -------------------------------------------------
 ufc_status batch_geometry(ufc_ctx* c, const double* chi, int nshell, const ufc_box* boxes,
                           int nbox, ShellTable& st, BoxGeom* bg);
 void batch_bands(int nside, float smax, Bands& bd);
 
-// Workspace of the persistent batch kernel: per realisation a count map, a
-// kappa map and the partial sums of the serial grids (256-byte aligned
-// pieces), and the descriptors.
-static size_t batch_map_stride(int S, int nside) {
-  return ((size_t)S * 12 * nside * nside * 4 + 255) / 256 * 256;
-}
-void batch_persistent_bytes(const ufc_ctx* c, int nreal, int nbox, int S, int nside,
-                            size_t* maps, size_t* desc) {
-  const size_t npix = 12ull * nside * nside;
-  const size_t kap_b = (npix * 4 + 255) / 256 * 256;
-  const size_t part_b = ((size_t)(8 * c->num_sms + 3 * 4 * c->num_sms) * 8 + 255) / 256 * 256;
-  *maps = (batch_map_stride(S, nside) + kap_b + part_b) * nreal;
-  *desc = ((size_t)nreal * nbox * sizeof(BatchItem) + 255) / 256 * 256 +
-          ((size_t)nreal * sizeof(Coef) + 255) / 256 * 256 + ((size_t)nreal * 4 + 255) / 256 * 256 +
-          16 + (size_t)nreal * 4 + 256;
-}
-
-struct BatchLaunch {
-  BatchArgs ba;
-  ShellTable st;
-  Bands bd;
-  PdfParam pp;
-  size_t zero_maps;          // bytes of count maps to clear at each launch
-  size_t q_off, q_bytes;     // queue counters in the descriptor buffer
-  int grid, smem;
+// Workspace of a batched call: per realisation a count map, a kappa map and the
+// partial sums of the serial grids, then the items, the coefficients and the
+// finished-block counters.
+struct BatchSpace {
+  size_t maps, kappa, part;                  // offsets in the map buffer
+  size_t maps_bytes;
+  size_t items, coef, done, up_bytes, desc_bytes;   // in the descriptor buffer
+  int gk, gm;
 };
-
-// Host set-up of a persistent batched call: geometry, descriptors uploaded
-// into `desc` (synchronises the context stream; never under stream capture),
-// launch arguments kept in the context.
-ufc_status batch_persistent_prepare(ufc_ctx* c, int nreal, int nbox, const float* const* xyz,
-                                    const int64_t* n, const ufc_box* boxes, const double* chi,
-                                    int S, int nside, const double* A, const double* C, double lo,
-                                    double hi, int nbins, double* moments, int64_t* pdf,
-                                    double* stats, double* state, char* maps, char* desc) {
+static BatchSpace batch_space(const ufc_ctx* c, int nreal, int nbox, int S, int nside) {
   const int npix = 12 * nside * nside;
-  const int nitems = nreal * nbox;
-  const int chunk = c->batch_chunk > 0 ? c->batch_chunk : 8192;
-  const int bps = c->batch_blocks_per_sm > 0 ? c->batch_blocks_per_sm : 2;
+  auto up = [](size_t b) { return (b + 255) / 256 * 256; };
+  BatchSpace o;
+  o.gk = kappa_fwd_grid(c, npix);
+  o.gm = moments_grid(c->num_sms, npix);
+  o.maps = 0;
+  o.kappa = up((size_t)nreal * S * npix * 4);
+  o.part = o.kappa + up((size_t)nreal * npix * 4);
+  o.maps_bytes = o.part + (size_t)nreal * (o.gk + 3 * o.gm) * 8;
+  o.items = 0;
+  o.coef = up((size_t)nreal * nbox * sizeof(DirectItem));
+  o.up_bytes = o.coef + (size_t)nreal * batch_coef_stride(S);
+  o.done = up(o.up_bytes);
+  o.desc_bytes = o.done + (size_t)nreal * 4;
+  return o;
+}
+// Whether the batched call of this shape runs stage by stage over all
+// realisations: item numbers have 17 bits in an undecided image's entry, grids
+// 65535 rows.
+bool batch_stages_ok(const ufc_ctx* c, int nreal, int nbox, int S, int nside, size_t max_bytes) {
+  return (int64_t)nreal * nbox <= (1 << 17) && nreal <= 65535 &&
+         batch_space(c, nreal, nbox, S, nside).maps_bytes <= max_bytes;
+}
+
+// A batched call over all realisations at once.  The items and coefficients
+// are built in page-locked memory of the context and copied from there; the
+// next call waits (on the host, for the copy only) before it overwrites them.
+ufc_status run_batch_stages(ufc_ctx* c, int nreal, int nbox, const float* const* xyz,
+                            const int64_t* n, const ufc_box* boxes, const double* chi, int S,
+                            int nside, const double* A, const double* C, double lo, double hi,
+                            int nbins, double* moments, int64_t* pdf, double* stats,
+                            double* state) {
+  cudaStreamCaptureStatus cs;
+  UFC_CUDA(c, cudaStreamIsCapturing(c->stream, &cs));
+  if (cs != cudaStreamCaptureStatusNone)
+    return set_err(c, UFC_ERR_UNSUPPORTED, "ufc_batched_stats cannot be captured into a graph");
+  const int npix = 12 * nside * nside, nitems = nreal * nbox;
+  const BatchSpace sp = batch_space(c, nreal, nbox, S, nside);
+  char* maps = (char*)ws_get(c, kSlotBatchMaps, sp.maps_bytes);
+  char* desc = (char*)ws_get(c, kSlotBatchDesc, sp.desc_bytes);
+  if (!maps || !desc) return UFC_ERR_ALLOC;
+  if (!c->batch_ev) UFC_CUDA(c, cudaEventCreateWithFlags(&c->batch_ev, cudaEventDisableTiming));
+  if (c->batch_host_cap < sp.up_bytes) {
+    if (c->batch_host) {
+      UFC_CUDA(c, cudaEventSynchronize(c->batch_ev));
+      cudaFreeHost(c->batch_host);
+      c->batch_host = nullptr;
+      c->batch_host_cap = 0;
+    }
+    const size_t want = sp.up_bytes + sp.up_bytes / 8;
+    if (cudaHostAlloc(&c->batch_host, want, cudaHostAllocDefault) != cudaSuccess) {
+      cudaGetLastError();
+      c->batch_host = nullptr;
+      return set_err(c, UFC_ERR_ALLOC, "cudaHostAlloc of %zu bytes failed", want);
+    }
+    c->batch_host_cap = want;
+  } else {
+    UFC_CUDA(c, cudaEventSynchronize(c->batch_ev));    // the last call's copy has been made
+  }
+  char* host = static_cast<char*>(c->batch_host);
+  DirectItem* items = reinterpret_cast<DirectItem*>(host + sp.items);
+  DirectArgs a;
+  std::memset(&a, 0, sizeof a);
+  int64_t total = 0;
+  for (int i = 0; i < nitems; ++i) {
+    if (n[i] < 0) return set_err(c, UFC_ERR_ARG, "n[%d] < 0", i);
+    if (n[i] > 0 && !xyz[i]) return set_err(c, UFC_ERR_ARG, "xyz[%d] is NULL", i);
+    if (n[i] >= (1ll << 47)) return set_err(c, UFC_ERR_ARG, "n[%d] too large", i);
+    if (n[i] > 0 && (reinterpret_cast<uintptr_t>(xyz[i]) & 3))
+      return set_err(c, UFC_ERR_ARG, "xyz[%d] is not 4-byte aligned", i);
+    total += n[i];
+  }
+  a.task = c->batch_chunk > 0 ? c->batch_chunk : direct_task(c, total);
   std::vector<BoxGeom> bg(nbox);
-  BatchLaunch L;
-  std::memset(&L, 0, sizeof L);
-  std::vector<BatchItem> items(nitems);
-  std::vector<int32_t> ntask_r(nreal, 0);
+  ShellTable st;
   float smax = 0.f;
-  int64_t task = 0;
   for (int r = 0; r < nreal; ++r) {
-    ufc_status s = batch_geometry(c, chi, S, boxes + (size_t)r * nbox, nbox, L.st, bg.data());
+    const ufc_status s = batch_geometry(c, r == 0 ? chi : nullptr, S, boxes + (size_t)r * nbox, nbox,
+                                        st, bg.data());
     if (s) return s;
     for (int k = 0; k < nbox; ++k) {
       const size_t i = (size_t)r * nbox + k;
-      BatchItem& it = items[i];
       const BoxGeom& g = bg[k];
-      if (n[i] < 0) return set_err(c, UFC_ERR_ARG, "n[%zu] < 0", i);
-      if (n[i] > 0 && !xyz[i]) return set_err(c, UFC_ERR_ARG, "xyz[%zu] is NULL", i);
+      DirectItem& d = items[i];
       smax = std::max(smax, g.smax);
-      it.xyz = xyz[i];
-      it.n = n[i];
-      it.task0 = task;
-      it.real = r;
-      it.shell_lo = g.shell_lo;
-      it.shell_hi = g.shell_hi;
+      d.xyz = xyz[i];
+      d.n = n[i];
+      d.task0 = a.ntasks;
+      d.counts = reinterpret_cast<int32_t*>(maps + sp.maps) + (size_t)r * S * npix;
+      d.shell_lo = g.shell_lo;
+      d.shell_hi = g.shell_hi;
       for (int ax = 0; ax < 3; ++ax) {
-        it.shf[ax] = g.shf[ax][0];
-        it.shlo[ax] = g.shlo[ax][0];
-        it.sh64[ax] = g.sh64[ax][0];
+        d.shf[ax] = g.shf[ax][0];
+        d.shlo[ax] = g.shlo[ax][0];
+        d.sh64[ax] = g.sh64[ax][0];
       }
-      const int64_t nt = std::max<int64_t>(1, (it.n + chunk - 1) / chunk);   // empty: one task
-      task += nt;
-      ntask_r[r] += (int32_t)nt;
+      a.ntasks += (n[i] + a.task - 1) / a.task;
     }
+    BatchCoef* cf = reinterpret_cast<BatchCoef*>(host + sp.coef + batch_coef_stride(S) * r);
+    auto split = [](double x) {
+      const float h = (float)x;
+      return make_float2(h, (float)(x - (double)h));
+    };
+    for (int b = 0; b < S; ++b) cf->a[b] = split(A[(size_t)r * S + b]);
+    cf->c = split(C[r]);
   }
-  batch_bands(nside, smax, L.bd);        // the bands of the largest shift of all the boxes
-  std::vector<Coef> coef(nreal);
-  for (int r = 0; r < nreal; ++r) make_coef(A + (size_t)r * S, C[r], S, npix, coef[r]);
-  const size_t o_coef = ((size_t)nitems * sizeof(BatchItem) + 255) / 256 * 256;
-  const size_t o_nt = o_coef + ((size_t)nreal * sizeof(Coef) + 255) / 256 * 256;
-  const size_t o_q = o_nt + ((size_t)nreal * 4 + 255) / 256 * 256;
-  std::vector<char> host(o_q);
-  std::memcpy(host.data(), items.data(), (size_t)nitems * sizeof(BatchItem));
-  std::memcpy(host.data() + o_coef, coef.data(), (size_t)nreal * sizeof(Coef));
-  std::memcpy(host.data() + o_nt, ntask_r.data(), (size_t)nreal * 4);
-  UFC_CUDA(c, cudaMemcpyAsync(desc, host.data(), host.size(), cudaMemcpyHostToDevice, c->stream));
-  UFC_CUDA(c, cudaStreamSynchronize(c->stream));   // (host staging leaves scope)
-  const int gk = kappa_fwd_grid(c, npix), gm = moments_grid(c->num_sms, npix);
-  const size_t map_b = batch_map_stride(S, nside);
-  const size_t kap_b = ((size_t)npix * 4 + 255) / 256 * 256;
-  BatchArgs& ba = L.ba;
-  ba.items = reinterpret_cast<const BatchItem*>(desc);
-  ba.nitems = nitems;
-  ba.chunk = chunk;
-  ba.ntasks = task;
-  ba.coef = reinterpret_cast<const Coef*>(desc + o_coef);
-  ba.ntask_r = reinterpret_cast<const int32_t*>(desc + o_nt);
+  UFC_CUDA(c, cudaMemcpyAsync(desc, host, sp.up_bytes, cudaMemcpyHostToDevice, c->stream));
+  UFC_CUDA(c, cudaEventRecord(c->batch_ev, c->stream));
+  UFC_CUDA(c, cudaMemsetAsync(desc + sp.done, 0, (size_t)nreal * 4, c->stream));
+  // the bands of the largest shift of all the boxes
+  batch_bands(nside, smax, a.bd);
+  ufc_status s = bin_prep(c, st, maps + sp.maps, sp.kappa, &a.tab, &a.lut_scale);
+  if (s) return s;
+  a.items = reinterpret_cast<const DirectItem*>(desc + sp.items);
+  a.nitems = nitems;
+  a.N = nside;
+  a.npix = npix;
+  a.ncell = (int64_t)S * npix;
+  a.cnt = (BinCounters*)c->counters;
+  s = launch_direct(c, a, c->batch_blocks_per_sm);
+  if (s) return s;
+  BatchArgs ba;
+  ba.coef = desc + sp.coef;
   ba.nreal = nreal;
   ba.S = S;
-  ba.N = nside;
   ba.npix = npix;
-  ba.counts = reinterpret_cast<int32_t*>(maps);
-  ba.kappa = reinterpret_cast<float*>(maps + map_b * nreal);
-  ba.ksum = reinterpret_cast<double*>(maps + (map_b + kap_b) * nreal);
-  ba.mpart = ba.ksum + (size_t)gk * nreal;
-  ba.gk = gk;
-  ba.gm = gm;
+  ba.counts = reinterpret_cast<int32_t*>(maps + sp.maps);
+  ba.kappa = reinterpret_cast<float*>(maps + sp.kappa);
+  ba.ksum = reinterpret_cast<double*>(maps + sp.part);
+  ba.mpart = ba.ksum + (size_t)sp.gk * nreal;
+  ba.gk = sp.gk;
+  ba.gm = sp.gm;
   ba.moments = moments;
   ba.pdf = pdf;
   ba.stats = stats;
-  ba.state = state;
   ba.nbins = nbins;
   ba.d = 6 + nbins;
-  ba.queue = reinterpret_cast<unsigned long long*>(desc + o_q);
-  ba.done = reinterpret_cast<unsigned int*>(desc + o_q + 16);
-  if (map_b != (size_t)S * npix * 4)      // maps are indexed as [nreal][S][npix]
-    return set_err(c, UFC_ERR_UNSUPPORTED, "persistent batch: map size not a multiple of 256 B");
-  L.pp = make_pdf_param(lo, hi, nbins);
-  L.zero_maps = map_b * nreal;
-  L.q_off = o_q;
-  L.q_bytes = 16 + (size_t)nreal * 4;
-  L.grid = std::min(bps, 2) * c->num_sms;
-  L.smem = std::max((nbins + 3) * 4, 2 * welford_run(6 + nbins) * (6 + nbins) * 8);
-  c->batch_launch.resize(sizeof L);
-  std::memcpy(c->batch_launch.data(), &L, sizeof L);
-  // (static plus dynamic shared memory may pass the 48 KB default)
-  UFC_CUDA(c, cudaFuncSetAttribute(k_batch_persistent, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   L.smem));
-  return UFC_OK;
-}
-
-// The launch itself (capturable): clear the maps and the queue, run the kernel.
-ufc_status batch_persistent_enqueue(ufc_ctx* c, char* maps, char* desc) {
-  if (c->batch_launch.size() != sizeof(BatchLaunch))
-    return set_err(c, UFC_ERR_ARG, "persistent batch: no prepared launch");
-  BatchLaunch L;
-  std::memcpy(&L, c->batch_launch.data(), sizeof L);
-  UFC_CUDA(c, cudaMemsetAsync(maps, 0, L.zero_maps, c->stream));
-  UFC_CUDA(c, cudaMemsetAsync(desc + L.q_off, 0, L.q_bytes, c->stream));
+  ba.done = reinterpret_cast<unsigned int*>(desc + sp.done);
   {
-    ProfScope ps_(c, "k_batch_persistent");
-    k_batch_persistent<<<L.grid, kBT, L.smem, c->stream>>>(L.ba, L.st, L.bd, L.pp);
+    ProfScope ps_(c, "k_batch_kappa");
+    k_batch_kappa<<<dim3(sp.gk, nreal), kKV, 0, c->stream>>>(ba);
+  }
+  {
+    ProfScope ps_(c, "k_batch_moments");
+    k_batch_moments<<<dim3(sp.gm, nreal), kMT, (nbins + 3) * 4, c->stream>>>(
+        ba, make_pdf_param(lo, hi, nbins));
   }
   UFC_CUDA(c, cudaGetLastError());
-  return UFC_OK;
+  return run_welford_update(c, stats, nreal, 6 + nbins, state);
 }
 
 }  // namespace ufc
