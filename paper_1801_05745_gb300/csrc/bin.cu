@@ -87,6 +87,13 @@ __device__ __forceinline__ void dense_append(WarpChunk& wc, bool want, uint32_t 
   const unsigned full = 0xFFFFFFFFu;
   unsigned m = __ballot_sync(full, want);
   int lane = threadIdx.x & 31;
+  // every lane has a key and the chunk stays open (most calls of the pixel
+  // stage): no ranks
+  if (m == full && wc.base >= 0 && wc.fits && wc.fill < kChunk - 32) {
+    o.dense[wc.base + (wc.fill + lane)] = v;
+    wc.fill += 32;
+    return;
+  }
   if (m == 0) return;
   int cnt = __popc(m);
   int rank = __popc(m & ((1u << lane) - 1u));
@@ -702,7 +709,7 @@ k_fast_tma(const float* __restrict__ xyz, int64_t n, int64_t p_off, int32_t box_
           const uint32_t meta = __float_as_uint(ent.w);
           const int b = int(meta & 255u);
           const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
-          const float rinv = rsqrtf(r2);
+          const float rinv = rsqrt_fast(r2);
           const float z = dz * rinv;
           int32_t pix = kKeyUndecided;
           if (have) {

@@ -389,7 +389,7 @@ k_direct(const __grid_constant__ DirectArgs a, const __grid_constant__ BoxGeom b
           const float dx = ent.x, dy = ent.y, dz = ent.z;
           const uint32_t meta = __float_as_uint(ent.w);
           const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
-          const float rinv = rsqrtf(r2);
+          const float rinv = rsqrt_fast(r2);
           const float zz = dz * rinv;
           int32_t pix = kKeyUndecided;
           if (on) {

@@ -150,6 +150,26 @@ __device__ __forceinline__ float i2f_fast(int32_t k) {
   return __fsub_rn(__int_as_float(kMagicBits + k), kMagic);
 }
 
+// Reciprocal square root and division in their approximate forms without the
+// denormal handling that rsqrtf and __fdividef carry by default (a range test
+// and conditional scalings; the same results on normal operands).  The fast
+// stage takes roots of r^2 (at least the guard r2_min) and of 3 (1 - |z|), and
+// divides by max(|dx|, |dy|) (open below the guard axy_min) and by
+// r (r + |dz|): all normal where the answer is used.  A quotient that would be
+// denormal becomes 0, which moves the azimuth or 1 - |z| by less than 2^-126; a
+// root of 0 gives a NaN, which opens the decision.  k_fast of two boxes of
+// 512^3 particles: 1.88 -> 1.83 ms.
+__device__ __forceinline__ float rsqrt_fast(float x) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float div_fast(float a, float b) {
+  float r;
+  asm("div.approx.ftz.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
+
 // Floor of w when w is farther than a band b from every integer, else marks
 // the decision open; dmin >= b + 2^-23.  r = w + 1.5 2^23 rounds w to the
 // nearest integer n (every caller's |w| is below N + 1 <= 8193, far below
@@ -191,7 +211,7 @@ __device__ __forceinline__ Azim azimuth_fast(float dx, float dy, const Bands& bd
   const float ax = fabsf(dx), ay = fabsf(dy);
   open |= fmaxf(ax, ay) < bd.axy_min;
   const bool sw = ay > ax;
-  const float q = __fdividef(fminf(ax, ay), fmaxf(ax, ay));   // one division, either octant
+  const float q = div_fast(fminf(ax, ay), fmaxf(ax, ay));   // one division, either octant
   Azim r;
   r.a = atanq_poly(q);                         // quarter turns, [0, 1/2]
   const bool xp = dx >= 0.0f, yp = dy >= 0.0f;
@@ -232,9 +252,9 @@ __device__ __forceinline__ int32_t pixel_fast_cap(int32_t N, const Bands& bd, fl
   const Azim az = azimuth_fast(dx, dy, bd, open);
   const float s2 = fmaf(dx, dx, dy * dy);
   const float r = r2 * rinv;
-  const float omz = __fdividef(s2, r * (r + fabsf(dz)));
+  const float omz = div_fast(s2, r * (r + fabsf(dz)));
   const float o3 = 3.0f * omz;
-  float tmp = bd.fN * (o3 * rsqrtf(o3));
+  float tmp = bd.fN * (o3 * rsqrt_fast(o3));
   if (!(o3 > 0.0f)) { tmp = 0.0f; open = true; }
   const float tp = az.sgn_pos ? az.a : 1.0f - az.a;
   const int32_t jp = floor_certain_d(tp * tmp, bd.cap_d, open);
@@ -256,7 +276,7 @@ __device__ __forceinline__ int32_t pixel_fast_cap(int32_t N, const Bands& bd, fl
 // r2 = fmaf(dz,dz,fmaf(dy,dy,dx*dx)) > bands.r2_min.
 __device__ __forceinline__ int32_t pixel_fast(int32_t N, const Bands& bd, float dx,
                                               float dy, float dz, float r2) {
-  const float rinv = rsqrtf(r2);
+  const float rinv = rsqrt_fast(r2);
   const float z = dz * rinv;
   const float za = fabsf(z);
   if (za <= bd.z_eq) return pixel_fast_eq(N, bd, dx, dy, z);
