@@ -23,9 +23,9 @@ LIB = os.path.join(BUILD, "libufalcon_gb300.so")
 CUDA_HOME = os.environ.get("CUDA_HOME", "/usr/local/cuda")
 NVCC = os.path.join(CUDA_HOME, "bin", "nvcc")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-CU = ["bin.cu", "direct.cu", "stats.cu", "sht.cu", "capi.cu"]
+CU = ["bin.cu", "direct.cu", "stats.cu", "sht.cu", "sht_ring.cu", "capi.cu"]
 CPP = ["cosmo.cpp", "welford.cpp"]
-HEADERS = ["common.cuh", "direct.cuh", "packed.cuh", "pixel.cuh", "ctx.h"]
+HEADERS = ["common.cuh", "direct.cuh", "packed.cuh", "pixel.cuh", "sht_common.cuh", "ctx.h"]
 
 
 def _stale(target: str, deps: list[str]) -> bool:

@@ -9,11 +9,8 @@
 //                      one-dimensional tables from which every recurrence
 //                      coefficient and normalisation is a product.
 //   k_ring_transform : per ring, F_m = sum_j map_j e^{-i m phi_j}
-//                      = e^{-i m phi_0} X_{m mod n}, X the ring's DFT (radix-2
-//                      FFT in shared memory in double-float for power-of-two
-//                      rings, twiddles and phases from the root table;
-//                      radix-4 split and direct DFTs otherwise); F stored
-//                      m-major.
+//                      = e^{-i m phi_0} X_{m mod n}, X the ring's DFT
+//                      (sht_ring.cu); F stored m-major.
 //   k_lmm            : lambda_mm(z) of every north/south ring pair for every m,
 //                      as mantissa x 2^exponent (no underflow near the poles).
 //   k_legendre       : per (m, chunk of ring pairs) the recurrence over l of
@@ -27,116 +24,13 @@
 #include <cmath>
 #include <cstring>
 
-#include "common.cuh"
-#include "ctx.h"
-#include "packed.cuh"
+#include "sht_common.cuh"
 
 namespace ufc {
 
-constexpr int kShtMaxNside = 1024;     // shared-memory FFT of the 4 nside-pixel rings
 constexpr int kLegChunkL = 32;         // l values per reduction round
 static_assert(kLegChunkL == 32, "the block reduction gives each degree of a round one lane");
 
-struct Ring {
-  int64_t start;   // first pixel
-  int32_t n;       // pixels
-  double z, s;     // cos and sin of the colatitude
-  double phi0_pi;  // azimuth of the first pixel / pi
-};
-
-// Ring r (0-based, north to south) of the RING scheme.
-__host__ __device__ inline Ring ring_geom(int32_t N, int32_t r) {
-  const int64_t npix = 12ll * N * N;
-  const int32_t i = r + 1;
-  Ring g;
-  if (i < N) {
-    g.n = 4 * i;
-    g.start = 2ll * i * (i - 1);
-    const double t = (double)((int64_t)i * i) / (3.0 * (double)((int64_t)N * N));
-    g.z = 1.0 - t;
-    g.s = sqrt(t * (2.0 - t));
-    g.phi0_pi = 1.0 / (4.0 * i);
-  } else if (i <= 3 * N) {
-    g.n = 4 * N;
-    g.start = 2ll * N * (N - 1) + 4ll * N * (i - N);
-    g.z = 4.0 / 3.0 - 2.0 * (double)i / (3.0 * (double)N);
-    g.s = sqrt((1.0 - g.z) * (1.0 + g.z));
-    g.phi0_pi = ((i - N + 1) % 2) / (4.0 * N);
-  } else {
-    const int32_t k = 4 * N - i;
-    g.n = 4 * k;
-    g.start = npix - 2ll * k * (k + 1);
-    const double t = (double)((int64_t)k * k) / (3.0 * (double)((int64_t)N * N));
-    g.z = -(1.0 - t);
-    g.s = sqrt(t * (2.0 - t));
-    g.phi0_pi = 1.0 / (4.0 * k);
-  }
-  return g;
-}
-
-__device__ __forceinline__ bool is_pow2(int v) { return (v & (v - 1)) == 0; }
-
-// Double-float arithmetic on the FP32 pipe (GB300 runs FP64 at 1/64 of the
-// FP32 rate): a value is h + l with |l| <= ulp(h)/2, about 48 bits.  Every
-// step is a correctly rounded FP32 intrinsic, so that no contraction changes
-// the error-free transformations (Dekker/Knuth two-sum, FMA two-product).
-struct dfl { float h, l; };
-__device__ __forceinline__ dfl df_from_d(double x) {
-  const float h = __double2float_rn(x);
-  return {h, __double2float_rn(x - (double)h)};
-}
-__device__ __forceinline__ double df_to_d(dfl a) { return (double)a.h + (double)a.l; }
-// h + l with |h| >= |l| renormalised (fast two-sum)
-__device__ __forceinline__ dfl df_norm(float h, float l) {
-  const float s = __fadd_rn(h, l);
-  return {s, __fadd_rn(l, __fsub_rn(h, s))};
-}
-// a * b: the exact product of the high parts plus the cross terms
-__device__ __forceinline__ dfl df_mul(dfl a, dfl b) {
-  const float p = __fmul_rn(a.h, b.h);
-  float e = __fmaf_rn(a.h, b.h, -p);
-  e = __fmaf_rn(a.h, b.l, e);
-  e = __fmaf_rn(a.l, b.h, e);
-  return df_norm(p, e);
-}
-// a + b (two-sum of the high parts)
-__device__ __forceinline__ dfl df_add(dfl a, dfl b) {
-  const float s = __fadd_rn(a.h, b.h);
-  const float bb = __fsub_rn(s, a.h);
-  const float err = __fadd_rn(__fsub_rn(a.h, __fsub_rn(s, bb)), __fsub_rn(b.h, bb));
-  return df_norm(s, __fadd_rn(err, __fadd_rn(a.l, b.l)));
-}
-__device__ __forceinline__ dfl df_neg(dfl a) { return {-a.h, -a.l}; }
-__device__ __forceinline__ dfl df_scale(dfl a, float p2) { return {a.h * p2, a.l * p2}; }  // exact
-// acc += a * b, the low part left unnormalised (renormalised by df_add)
-__device__ __forceinline__ void df_mac(dfl& acc, dfl a, dfl b) {
-  const float p = __fmul_rn(a.h, b.h);
-  const float pe = __fmaf_rn(a.h, b.h, -p);
-  const float s = __fadd_rn(acc.h, p);
-  const float bb = __fsub_rn(s, acc.h);
-  const float se = __fadd_rn(__fsub_rn(acc.h, __fsub_rn(s, bb)), __fsub_rn(p, bb));
-  const float cross = __fmaf_rn(a.h, b.l, __fmul_rn(a.l, b.h));
-  acc.h = s;
-  acc.l = __fadd_rn(acc.l, __fadd_rn(se, __fadd_rn(pe, cross)));
-}
-
-// Complex numbers with double-float parts, (re.h, re.l, im.h, im.l) in a float4.
-__device__ __forceinline__ float4 cdf_pack(dfl re, dfl im) { return make_float4(re.h, re.l, im.h, im.l); }
-// a * b
-__device__ __forceinline__ float4 cdf_mul(float4 a, float4 b) {
-  const dfl ar{a.x, a.y}, ai{a.z, a.w}, br{b.x, b.y}, bi{b.z, b.w};
-  return cdf_pack(df_add(df_mul(ar, br), df_neg(df_mul(ai, bi))),
-                  df_add(df_mul(ar, bi), df_mul(ai, br)));
-}
-__device__ __forceinline__ float4 cdf_add(float4 a, float4 b) {
-  return cdf_pack(df_add(dfl{a.x, a.y}, dfl{b.x, b.y}), df_add(dfl{a.z, a.w}, dfl{b.z, b.w}));
-}
-__device__ __forceinline__ float4 cdf_sub(float4 a, float4 b) {
-  return cdf_pack(df_add(dfl{a.x, a.y}, dfl{-b.x, -b.y}), df_add(dfl{a.z, a.w}, dfl{-b.z, -b.w}));
-}
-__device__ __forceinline__ float4 cdf_conj(float4 a) { return make_float4(a.x, a.y, -a.z, -a.w); }
-
-__device__ __forceinline__ dfx dfx_set(dfl a, dfl b) { return {x2_pack(a.h, b.h), x2_pack(a.l, b.l)}; }
 // v * f, the exact product of the high parts plus the cross terms (not
 // renormalised); nv = -v.h
 __device__ __forceinline__ dfx dfx_mul_raw(dfx v, dfx f) {
@@ -286,142 +180,6 @@ __device__ __forceinline__ bool leg_negligible(int lmax, int m, float c, float s
   if (!(fm > Ls)) return false;
   const float D = sqrtf((fm - Ls) * (fm + Ls)), R = sqrtf((L - fm) * (L + fm));
   return fm * logf((fm * c + D) / (s * R)) - L * logf((L * c + D) / R) > 130.0f * 0.69314718f;
-}
-
-// One block per ring.  Shared memory: twiddles w_k = e^{-2 pi i k / n} and the
-// ring's values (real, or complex for the FFT).
-__global__ void __launch_bounds__(512)
-k_ring_transform(const float* __restrict__ map, const float4* __restrict__ T, int32_t N,
-                 int32_t lmax, int32_t nrings, float4* __restrict__ F) {
-  extern __shared__ __align__(16) double2 sh[];
-  const int r = blockIdx.x;
-  const Ring g = ring_geom(N, r);
-  const int n = g.n;
-  if (is_pow2(n)) {
-    // radix-2 decimation-in-time FFT in double-float on the FP32 pipe
-    // (an FP64 instruction costs the FP32 pipe's time for about 64):
-    // bit-reversed load, then the stages; twiddles from the root table
-    float4* xd = reinterpret_cast<float4*>(sh);   // [n]
-    float4* wd = xd + n;                          // [n/2] e^{-2 pi i k / n}
-    const int ts = 8 * N / n;
-    for (int k = threadIdx.x; k < n / 2; k += blockDim.x) wd[k] = T[k * ts];
-    int bits = 0;
-    while ((1 << bits) < n) ++bits;
-    for (int j = threadIdx.x; j < n; j += blockDim.x) {
-      const int rj = __brev(j) >> (32 - bits);
-      xd[rj] = make_float4(map[g.start + j], 0.f, 0.f, 0.f);
-    }
-    __syncthreads();
-    for (int len = 2; len <= n; len <<= 1) {
-      const int half = len >> 1, step = n / len;
-      for (int t = threadIdx.x; t < n / 2; t += blockDim.x) {
-        const int grp = t / half, pos = t - grp * half;
-        const int a = grp * len + pos, b = a + half;
-        const float4 p = cdf_mul(wd[pos * step], xd[b]);
-        const float4 xa = xd[a];
-        xd[a] = cdf_add(xa, p);
-        xd[b] = cdf_sub(xa, p);
-      }
-      __syncthreads();
-    }
-    // F_m = e^{-i m phi_0} X_{m mod n} (phi_0 = 0 or pi/n)
-    const bool shifted = g.phi0_pi != 0.0;
-    const int ps = 4 * N / n;
-    for (int m = threadIdx.x; m <= lmax; m += blockDim.x) {
-      float4 X = xd[m & (n - 1)];
-      if (shifted) X = cdf_mul(T[(m * ps) & (8 * N - 1)], X);
-      F[(size_t)m * nrings + r] = X;
-    }
-    return;
-  }
-  // non power-of-two ring (a polar ring, n = 4 i): one radix-4 split,
-  // X_k = sum_{r<4} w_n^{rk} Y_r(k mod i) with Y_r(q) = sum_{a<i} x_{4a+r}
-  // w_n^{4aq} the length-i DFTs of the four sub-sequences (real input:
-  // Y_r(i-q) = conj Y_r(q), so q <= i/2), then k <= min(n/2, lmax) (real
-  // input: X_{n-k} = conj X_k).  Double-float on the FP32 pipe; the map
-  // values are FP32.  The twiddles w_n^k come from FP64 sincospi for the
-  // first quarter k < i only (w_n^{k + q i} = (-i)^q w_n^k), and the phase
-  // e^{-i m phi_0} = w_{2n}^m (phi_0 = pi/n) is w_n^{m/2}, times w_{2n} for
-  // odd m.
-  float4* wf = reinterpret_cast<float4*>(sh);             // [n] w_n^k
-  double2* x = sh + n;
-  float* xr = reinterpret_cast<float*>(x);                // [n] the ring's values
-  const int ni = n / 4, nq = ni / 2 + 1;
-  float4* Y = reinterpret_cast<float4*>(x + n / 4 + 1);   // [4][nq] after xr
-  float4* Xf = reinterpret_cast<float4*>(x);              // [n/2 + 1], once xr and Y are read
-  for (int jj = threadIdx.x; jj < n; jj += blockDim.x) xr[jj] = map[g.start + jj];
-  for (int k = threadIdx.x; k < ni; k += blockDim.x) {
-    double sn, cs;
-    sincospi(-2.0 * (double)k / (double)n, &sn, &cs);
-    const dfl c = df_from_d(cs), sv = df_from_d(sn);
-    wf[k] = cdf_pack(c, sv);                              // (c, s)
-    wf[k + ni] = cdf_pack(sv, dfl{-c.h, -c.l});           // -i (c + i s)
-    wf[k + 2 * ni] = cdf_pack(dfl{-c.h, -c.l}, dfl{-sv.h, -sv.l});
-    wf[k + 3 * ni] = cdf_pack(dfl{-sv.h, -sv.l}, c);
-  }
-  __syncthreads();
-  for (int o = threadIdx.x; o < 4 * nq; o += blockDim.x) {
-    const int r = o / nq, q = o - r * nq;
-    const int step = 4 * q;                  // < n since q <= i/2
-    dfl ar{0.f, 0.f}, ai{0.f, 0.f};
-    int idx = 0;
-    for (int a = 0; a < ni; ++a) {
-      const dfl v{xr[4 * a + r], 0.f};
-      const float4 tw = wf[idx];
-      df_mac(ar, v, dfl{tw.x, tw.y});
-      df_mac(ai, v, dfl{tw.z, tw.w});
-      idx += step;
-      idx -= idx >= n ? n : 0;
-    }
-    ar = df_add(ar, dfl{0.f, 0.f});
-    ai = df_add(ai, dfl{0.f, 0.f});
-    Y[o] = make_float4(ar.h, ar.l, ai.h, ai.l);
-  }
-  __syncthreads();
-  const int kmax = min(n / 2, lmax);
-  float4 out[4];
-#pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    const int k = threadIdx.x + u * (int)blockDim.x;
-    if (k > kmax) continue;
-    int q = k % ni;
-    const bool cj = q > ni / 2;
-    if (cj) q = ni - q;
-    dfl xre{0.f, 0.f}, xim{0.f, 0.f};
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const float4 yv = Y[r * nq + q];
-      const dfl yr{yv.x, yv.y}, yi = cj ? dfl{-yv.z, -yv.w} : dfl{yv.z, yv.w};
-      const float4 tw = wf[(r * k) % n];
-      const dfl tr{tw.x, tw.y}, ti{tw.z, tw.w};
-      df_mac(xre, tr, yr);                   // Re(w Y)
-      df_mac(xre, df_neg(ti), yi);
-      df_mac(xim, tr, yi);                   // Im(w Y)
-      df_mac(xim, ti, yr);
-    }
-    out[u] = cdf_pack(df_add(xre, dfl{0.f, 0.f}), df_add(xim, dfl{0.f, 0.f}));
-  }
-  __syncthreads();                           // xr and Y are read; X overwrites them
-#pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    const int k = threadIdx.x + u * (int)blockDim.x;
-    if (k <= kmax) Xf[k] = out[u];
-  }
-  __syncthreads();
-  // F_m = e^{-i m phi_0} X_{m mod n}, m = 0..lmax
-  float4 h1;                                 // w_{2n} = e^{-i pi / n}
-  {
-    double sn, cs;
-    sincospi(-1.0 / (double)n, &sn, &cs);
-    h1 = cdf_pack(df_from_d(cs), df_from_d(sn));
-  }
-  for (int m = threadIdx.x; m <= lmax; m += blockDim.x) {
-    const int k = m % n;
-    const float4 X = k <= n / 2 ? Xf[k] : cdf_conj(Xf[n - k]);
-    float4 ph = wf[(m >> 1) % n];
-    if (m & 1) ph = cdf_mul(ph, h1);
-    F[(size_t)m * nrings + r] = cdf_mul(ph, X);
-  }
 }
 
 // lambda_mm = cm_m sin(theta)^m of every ring pair p (north ring p) for
@@ -795,8 +553,7 @@ __global__ void k_alm2cl(const double2* __restrict__ alm, int32_t lmax, double* 
 //                      pair) with the even/odd split of the mirror rings;
 //   k_ring_synth     : map_j = sum_{|m| <= lmax} G_m e^{i m phi_j}, folding
 //                      m onto the ring's n frequencies and an inverse DFT
-//                      (double-float radix-2 FFT with root-table twiddles for
-//                      power-of-two rings, radix-4 split otherwise).
+//                      (sht_ring.cu).
 //
 // k_legendre_synth: block (chunk, m), a thread two adjacent ring pairs in
 // packed double-float, the recurrence and the exponents as in k_legendre; the
@@ -928,159 +685,6 @@ k_legendre_synth(const double2* __restrict__ alm, const float2* __restrict__ mu,
   }
 }
 
-// One block per ring: H_k = sum over m = k mod n (0 <= m <= lmax) of
-// G_m e^{i m phi_0} plus, for the negative frequencies, the conjugates of
-// the terms with m = -k mod n (1 <= m <= lmax); then map_j = sum_k H_k
-// e^{2 pi i k j / n} (inverse radix-2 FFT for power-of-two rings, direct
-// sum otherwise).  Each H_k is summed by one thread in increasing m.
-__global__ void __launch_bounds__(512)
-k_ring_synth(const float4* __restrict__ G, const float4* __restrict__ T, int32_t N,
-             int32_t lmax, int32_t nrings, float* __restrict__ map) {
-  extern __shared__ __align__(16) double2 sh[];
-  const int r = blockIdx.x;
-  const Ring g = ring_geom(N, r);
-  const int n = g.n;
-  if (is_pow2(n)) {
-    // double-float on the FP32 pipe; twiddles e^{+2 pi i k / n} and phases
-    // e^{+i m phi_0} (phi_0 = 0 or pi/n) are conjugates of root-table
-    // entries; H_k into bit-reversed order, then the inverse FFT stages
-    float4* hd = reinterpret_cast<float4*>(sh);   // [n]
-    float4* wd = hd + n;                          // [n/2]
-    const int ts = 8 * N / n, ps = 4 * N / n;
-    const bool shifted = g.phi0_pi != 0.0;
-    for (int k = threadIdx.x; k < n / 2; k += blockDim.x) wd[k] = cdf_conj(T[k * ts]);
-    int bits = 0;
-    while ((1 << bits) < n) ++bits;
-    auto term = [&](int m) {                    // G_m e^{i m phi_0}
-      float4 t = G[(size_t)m * nrings + r];
-      if (shifted) t = cdf_mul(cdf_conj(T[(m * ps) & (8 * N - 1)]), t);
-      return t;
-    };
-    for (int k = threadIdx.x; k < n; k += blockDim.x) {
-      float4 h = make_float4(0.f, 0.f, 0.f, 0.f);
-      for (int m = k; m <= lmax; m += n) h = cdf_add(h, term(m));            // m = k mod n
-      for (int m = (n - k) % n; m <= lmax; m += n)                           // -m = k mod n
-        if (m != 0) h = cdf_add(h, cdf_conj(term(m)));
-      hd[__brev(k) >> (32 - bits)] = h;
-    }
-    __syncthreads();
-    for (int len = 2; len <= n; len <<= 1) {
-      const int half = len >> 1, step = n / len;
-      for (int t = threadIdx.x; t < n / 2; t += blockDim.x) {
-        const int grp = t / half, pos = t - grp * half;
-        const int a = grp * len + pos, b = a + half;
-        const float4 p = cdf_mul(wd[pos * step], hd[b]);
-        const float4 xa = hd[a];
-        hd[a] = cdf_add(xa, p);
-        hd[b] = cdf_sub(xa, p);
-      }
-      __syncthreads();
-    }
-    for (int j = threadIdx.x; j < n; j += blockDim.x) map[g.start + j] = __fadd_rn(hd[j].x, hd[j].y);
-    return;
-  }
-  {
-    // non power-of-two ring (polar, n = 4 i), from the Hermitian half
-    // (H_{n-k} = conj H_k, the map being real) with one radix-4 split:
-    // map_{4a+r} = Re sum_{q<i} Z_r(q) w^{4aq}, Z_r(q) = sum_{t<4} H_{q+it}
-    // w^{r(q+it)}, and Z_r(i-q) = conj Z_r(q), so
-    // map_{4a+r} = Re Z_r(0) + 2 sum_{0<q<i/2} Re(Z_r(q) w^{4aq})
-    //              + [i even] (-1)^a Re Z_r(i/2).
-    // Double-float on the FP32 pipe.  The twiddles w^k = e^{+2 pi i k / n}
-    // come from FP64 sincospi for k < i only (w^{k + q i} = i^q w^k); the
-    // phases e^{+i m phi_0} = e^{+i pi m / n} are w^{m/2}, times e^{+i pi / n}
-    // for odd m.
-    float4* wf = reinterpret_cast<float4*>(sh);   // [n] (re.h, re.l, im.h, im.l)
-    float4* hf = wf + n;                          // [n/2 + 1]
-    const int ni = n / 4, nq = ni / 2 + 1, half = n / 2;
-    float4* Z = hf + half + 1;                    // [4][nq]
-    for (int k = threadIdx.x; k < ni; k += blockDim.x) {
-      double sn, cs;
-      sincospi(2.0 * (double)k / (double)n, &sn, &cs);
-      const dfl c = df_from_d(cs), sv = df_from_d(sn);
-      wf[k] = cdf_pack(c, sv);
-      wf[k + ni] = cdf_pack(dfl{-sv.h, -sv.l}, c);                    // i (c + i s)
-      wf[k + 2 * ni] = cdf_pack(dfl{-c.h, -c.l}, dfl{-sv.h, -sv.l});
-      wf[k + 3 * ni] = cdf_pack(sv, dfl{-c.h, -c.l});
-    }
-    float4 h1;                                    // e^{+i pi / n}
-    {
-      double sn, cs;
-      sincospi(1.0 / (double)n, &sn, &cs);
-      h1 = cdf_pack(df_from_d(cs), df_from_d(sn));
-    }
-    __syncthreads();
-    auto term = [&](int m) {                      // G_m e^{i m phi_0}
-      float4 ph = wf[(m >> 1) % n];
-      if (m & 1) ph = cdf_mul(ph, h1);
-      return cdf_mul(ph, G[(size_t)m * nrings + r]);
-    };
-    for (int k = threadIdx.x; k <= half; k += blockDim.x) {
-      float4 h = make_float4(0.f, 0.f, 0.f, 0.f);
-      for (int m = k; m <= lmax; m += n) h = cdf_add(h, term(m));          // m = k mod n
-      for (int m = (n - k) % n; m <= lmax; m += n)                         // -m = k mod n
-        if (m != 0) h = cdf_add(h, cdf_conj(term(m)));
-      hf[k] = h;
-    }
-    __syncthreads();
-    for (int o = threadIdx.x; o < 4 * nq; o += blockDim.x) {
-      const int r = o / nq, q = o - r * nq;
-      dfl zr{0.f, 0.f}, zi{0.f, 0.f};
-#pragma unroll
-      for (int t = 0; t < 4; ++t) {
-        const int k = q + ni * t;
-        const bool cj = k > half;
-        const float4 hv = hf[cj ? n - k : k];
-        const dfl hr{hv.x, hv.y}, hi = cj ? dfl{-hv.z, -hv.w} : dfl{hv.z, hv.w};
-        const float4 tw = wf[(r * k) % n];
-        const dfl tr{tw.x, tw.y}, ti{tw.z, tw.w};
-        df_mac(zr, tr, hr);                    // Re(H w)
-        df_mac(zr, df_neg(ti), hi);
-        df_mac(zi, tr, hi);                    // Im(H w)
-        df_mac(zi, ti, hr);
-      }
-      zr = df_add(zr, dfl{0.f, 0.f});
-      zi = df_add(zi, dfl{0.f, 0.f});
-      Z[o] = make_float4(zr.h, zr.l, zi.h, zi.l);
-    }
-    __syncthreads();
-    const int qe = (ni + 1) / 2;                 // q in [1, qe): the doubled terms
-    for (int jj = threadIdx.x; jj < n; jj += blockDim.x) {
-      const int a = jj >> 2, r = jj & 3;
-      const float4* Zr = Z + r * nq;
-      const int step = (4 * a) % n;              // w^{4aq}: index 4 a q mod n
-      dfl acc0{0.f, 0.f}, acc1{0.f, 0.f};
-      int idx = step;
-      int q = 1;
-      for (; q + 1 < qe; q += 2) {
-        int idx1 = idx + step;
-        idx1 -= idx1 >= n ? n : 0;
-        const float4 z0 = Zr[q], t0 = wf[idx], z1 = Zr[q + 1], t1 = wf[idx1];
-        df_mac(acc0, dfl{z0.x, z0.y}, dfl{t0.x, t0.y});       // Re(Z w)
-        df_mac(acc0, dfl{-z0.z, -z0.w}, dfl{t0.z, t0.w});
-        df_mac(acc1, dfl{z1.x, z1.y}, dfl{t1.x, t1.y});
-        df_mac(acc1, dfl{-z1.z, -z1.w}, dfl{t1.z, t1.w});
-        idx = idx1 + step;
-        idx -= idx >= n ? n : 0;
-      }
-      if (q < qe) {
-        const float4 z0 = Zr[q], t0 = wf[idx];
-        df_mac(acc0, dfl{z0.x, z0.y}, dfl{t0.x, t0.y});
-        df_mac(acc0, dfl{-z0.z, -z0.w}, dfl{t0.z, t0.w});
-      }
-      dfl sum = df_add(acc0, acc1);
-      sum = df_add(sum, sum);                    // the conjugate half
-      const float4 z0 = Zr[0];
-      sum = df_add(sum, dfl{z0.x, z0.y});
-      if ((ni & 1) == 0) {                       // the self-conjugate q = i/2
-        const float4 zn = Zr[ni / 2];
-        sum = df_add(sum, (a & 1) ? dfl{-zn.x, -zn.y} : dfl{zn.x, zn.y});
-      }
-      map[g.start + jj] = (float)df_to_d(sum);
-    }
-  }
-}
-
 // a_lm b_l with the Gaussian beam b_l = exp(-l(l+1) sigma^2 / 2).
 __global__ void k_alm_beam(const double2* __restrict__ in, int32_t lmax, double sigma,
                            double2* __restrict__ out) {
@@ -1179,13 +783,8 @@ ufc_status run_map2alm(ufc_ctx* c, const float* map, int nside, int lmax, double
   ShtSpace sp;
   const ufc_status s = sht_space(c, nside, lmax, nchunk, sp);
   if (s) return s;
-  const int smem = 2 * 4 * nside * (int)sizeof(double2);
-  UFC_CUDA(c, cudaFuncSetAttribute(k_ring_transform, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   smem));
-  {
-    ProfScope ps_(c, "k_ring_transform");
-    k_ring_transform<<<nrings, 512, smem, c->stream>>>(map, sp.tb.roots, nside, lmax, nrings, sp.ring);
-  }
+  const ufc_status sr = launch_ring_transform(c, map, sp.tb.roots, nside, lmax, sp.ring);
+  if (sr) return sr;
   double2* alm = reinterpret_cast<double2*>(alm_out);
   {
     ProfScope ps_(c, "k_legendre");
@@ -1242,14 +841,8 @@ ufc_status run_alm2map(ufc_ctx* c, const double* alm, int nside, int lmax, float
     else UFC_SYN(64);
 #undef UFC_SYN
   }
-  const int smem = 2 * 4 * nside * (int)sizeof(double2);
-  UFC_CUDA(c, cudaFuncSetAttribute(k_ring_synth, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-  {
-    ProfScope ps_(c, "k_ring_synth");
-    k_ring_synth<<<nrings, 512, smem, c->stream>>>(sp.ring, sp.tb.roots, nside, lmax, nrings, map);
-  }
   UFC_CUDA(c, cudaGetLastError());
-  return UFC_OK;
+  return launch_ring_synth(c, sp.ring, sp.tb.roots, nside, lmax, map);
 }
 
 ufc_status run_alm_beam(ufc_ctx* c, const double* in, int lmax, double sigma, double* out) {
