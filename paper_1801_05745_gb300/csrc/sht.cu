@@ -28,8 +28,8 @@
 
 namespace ufc {
 
-constexpr int kLegChunkL = 32;         // l values per reduction round
-static_assert(kLegChunkL == 32, "the block reduction gives each degree of a round one lane");
+constexpr int kLegChunkL = 64;         // l values per round (two barriers, or one): 32 cost
+                                       // 1.5% more
 
 // v * f, the exact product of the high parts plus the cross terms (not
 // renormalised); nv = -v.h
@@ -158,12 +158,19 @@ __global__ void k_sht_tables(int32_t N, int32_t lmax, float4* __restrict__ T,
   }
 }
 
-// alpha_l without its sign (+ + - - of (l - m) mod 4).  m0 = SW_m SL_m.
-__device__ __forceinline__ double sht_alpha(const ShtTables& t, int l, int m, double m0,
-                                            double sl_m1) {
+// Per-order factors of alpha and a, formed once per block (a division per
+// coefficient instead kept the FP64 pipe 9 to 13% busy).
+struct OrderConst { double even, odd, step; };
+__device__ __forceinline__ OrderConst order_const(const ShtTables& t, int m) {
+  const double m0 = t.sw[m] * t.sl[m], s1 = t.sl[m + 1];
+  return {1.0 / m0, m0 / s1, s1 * t.inv_z};
+}
+// alpha_l, with the sign + + - - of (l - m) mod 4.
+__device__ __forceinline__ double sht_alpha(const ShtTables& t, int l, int m, OrderConst oc) {
   const int d = l - m, k = d >> 1;
-  return (d & 1) ? t.sv[k] * t.sv[m + k] * t.sl[l] * (m0 / sl_m1)
-                 : t.sw[k] * t.sw[m + k] * t.sl[l] / m0;
+  const double a = (d & 1) ? t.sv[k] * t.sv[m + k] * t.sl[l] * oc.odd
+                           : t.sw[k] * t.sw[m + k] * t.sl[l] * oc.even;
+  return (d & 2) ? -a : a;
 }
 
 // True when |lambda_lm| < 2^-128 for every l <= lmax on the ring with cos and
@@ -233,13 +240,13 @@ __device__ __forceinline__ double warp_sum_dd(double v) {
   return v;
 }
 
-// Coefficients of one round of 32 degrees from l0 = m + 32 i, duplicated for
+// Coefficients of one round of degrees, duplicated for
 // the packed instructions (h, h, l, l); 0 above lmax.  One thread per degree.
-__device__ __forceinline__ float4 leg_coef(const ShtTables& t, int l, int lmax, int m, double m0,
-                                           double sl_m1) {
+__device__ __forceinline__ float4 leg_coef(const ShtTables& t, int l, int lmax, int m,
+                                           OrderConst oc) {
   if (l >= lmax) return make_float4(0.f, 0.f, 0.f, 0.f);   // (the step from lmax is not used)
-  const double al = sht_alpha(t, l, m, m0, sl_m1);
-  const double a = sl_m1 * t.inv_z * al * al;
+  const double al = sht_alpha(t, l, m, oc);
+  const double a = oc.step * al * al;
   const dfl f = df_from_d(((l - m) & 1) ? -a : a);
   return make_float4(f.h, f.h, f.l, f.l);
 }
@@ -274,7 +281,8 @@ constexpr int kLegMinExp = -120;       // terms of pairs at or below this expone
 // block's result: an FP64 instruction costs the FP32 pipe's time for about 64).
 // Output: alm (nchunk = 1) or part[chunk], with the factor alpha_l w.
 //
-// Measured at Nside 1024, lmax 3071 (9.7e9 triples): 13.4 ms with G = 2 and
+// Measured at Nside 1024, lmax 3071 (9.7e9 triples): 13.0 ms; in rounds of 32
+// degrees and with a division per coefficient 13.4 ms with G = 2 and
 // 128 threads, 4 blocks per SM (128 registers); G = 4 with 128 threads and 2
 // blocks 16.6 ms, G = 2 with 256 threads and 2 blocks 14.2 ms, with 64 threads
 // and 8 blocks 13.6 ms: 16 warps per SM hide the recurrence's chain of
@@ -299,7 +307,7 @@ k_legendre(const float4* __restrict__ F, const float2* __restrict__ mu,
   const unsigned full = 0xFFFFFFFFu;
   const size_t base = (size_t)m * (2 * lmax + 1 - m) / 2;  // index of (l = 0, m)
   double2* dst = out + (size_t)chunk * nalm + base;
-  const double sl_m1 = tb.sl[m + 1], m0 = tb.sw[m] * tb.sl[m];
+  const OrderConst oc = order_const(tb, m);
   // the block's most equatorial pair decides whether there is any work
   const int p_hi = min((chunk + 1) * 2 * G * NT, npairs) - 1;
   {
@@ -406,7 +414,7 @@ k_legendre(const float4* __restrict__ F, const float2* __restrict__ mu,
     }
   };
   if (threadIdx.x < kLegChunkL)
-    cs[0][threadIdx.x] = leg_coef(tb, m + threadIdx.x, lmax, m, m0, sl_m1);
+    cs[0][threadIdx.x] = leg_coef(tb, m + threadIdx.x, lmax, m, oc);
   __syncthreads();
   int buf = 0;
   for (int l0 = m; l0 <= lmax; l0 += kLegChunkL, buf ^= 1) {
@@ -486,19 +494,21 @@ k_legendre(const float4* __restrict__ F, const float2* __restrict__ mu,
       }
     }
     if (threadIdx.x < kLegChunkL)                         // the next round's coefficients
-      cs[buf ^ 1][threadIdx.x] = leg_coef(tb, l0 + kLegChunkL + threadIdx.x, lmax, m, m0, sl_m1);
+      cs[buf ^ 1][threadIdx.x] = leg_coef(tb, l0 + kLegChunkL + threadIdx.x, lmax, m, oc);
     __syncthreads();
     // the group sums of each degree: warp j adds rows j, j + NW, ...
     // (lane t: conflict-free rows), then the warps' partials per degree
-    if (lane < cnt) {
+#pragma unroll
+    for (int t = lane; t < kLegChunkL; t += 32) {
+      if (t >= cnt) break;
       dfl sr{0.f, 0.f}, si{0.f, 0.f};
       for (int row = warp; row < NT / 4; row += NW) {
         if (!live_s[row >> 3]) continue;                  // (uniform)
-        const float4 v = red[row][lane];
+        const float4 v = red[row][t];
         sr = df_add(sr, dfl{v.x, v.y});
         si = df_add(si, dfl{v.z, v.w});
       }
-      red2[warp][lane] = make_float4(sr.h, sr.l, si.h, si.l);
+      red2[warp][t] = make_float4(sr.h, sr.l, si.h, si.l);
     }
     __syncthreads();
     if (threadIdx.x < cnt) {
@@ -510,8 +520,7 @@ k_legendre(const float4* __restrict__ F, const float2* __restrict__ mu,
         sr = df_add(sr, dfl{v.x, v.y});
         si = df_add(si, dfl{v.z, v.w});
       }
-      const double al = w * sht_alpha(tb, l, m, m0, sl_m1);
-      const double f = ((l - m) & 2) ? -al : al;
+      const double f = w * sht_alpha(tb, l, m, oc);
       dst[l] = make_double2(f * df_to_d(sr), f * df_to_d(si));
     }
   }
@@ -562,7 +571,9 @@ __global__ void k_alm2cl(const double2* __restrict__ alm, int32_t lmax, double* 
 // negligible), so nothing is reduced across threads.  A warp whose pairs are
 // all negligible up to lmax (leg_negligible) writes zeros, and none of its
 // terms is formed before one of its pairs has e > -120.  Bound by the FP32
-// pipe: 18 + 24 packed operations per degree and pair of ring pairs.
+// pipe: 18 + 24 packed operations per degree and pair of ring pairs (FMA pipe
+// 71% busy).  Nside 512, lmax 1535: 1.47 ms with blocks of 128 threads, 1.51 with
+// 256 or 64 (2.96 ms before the one-coefficient recurrence and the packed pairs).
 template <int NT>
 __global__ void __launch_bounds__(NT)
 k_legendre_synth(const double2* __restrict__ alm, const float2* __restrict__ mu,
@@ -574,7 +585,7 @@ k_legendre_synth(const double2* __restrict__ alm, const float2* __restrict__ mu,
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const unsigned full = 0xFFFFFFFFu;
   const size_t base = (size_t)m * (2 * lmax + 1 - m) / 2;
-  const double sl_m1 = tb.sl[m + 1], m0 = tb.sw[m] * tb.sl[m];
+  const OrderConst oc = order_const(tb, m);
   const int first = chunk * 2 * NT + warp * 64;           // the warp's first pair
   const int p = first + 2 * lane;
   const bool have = p < npairs;                           // (npairs is even)
@@ -612,13 +623,12 @@ k_legendre_synth(const double2* __restrict__ alm, const float2* __restrict__ mu,
     for (int t = threadIdx.x; t < 2 * kLegChunkL; t += NT) {
       const int l = l0 + (t & (kLegChunkL - 1));
       if (t < kLegChunkL) {
-        cs[b][t] = leg_coef(tb, l, lmax, m, m0, sl_m1);
+        cs[b][t] = leg_coef(tb, l, lmax, m, oc);
       } else {
         float4 re = zero, im = zero;
         if (l <= lmax) {
           const double2 a = alm[base + l];
-          const double al = sht_alpha(tb, l, m, m0, sl_m1);
-          const double f = ((l - m) & 2) ? -al : al;
+          const double f = sht_alpha(tb, l, m, oc);
           const dfl x = df_from_d(f * a.x), y = df_from_d(f * a.y);
           re = make_float4(x.h, x.h, x.l, x.l);
           im = make_float4(y.h, y.h, y.l, y.l);
@@ -685,21 +695,19 @@ k_legendre_synth(const double2* __restrict__ alm, const float2* __restrict__ mu,
   }
 }
 
-// a_lm b_l with the Gaussian beam b_l = exp(-l(l+1) sigma^2 / 2).
-__global__ void k_alm_beam(const double2* __restrict__ in, int32_t lmax, double sigma,
-                           double2* __restrict__ out) {
-  const int64_t nalm = (int64_t)(lmax + 1) * (lmax + 2) / 2;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nalm;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    // m from the m-major index: block m starts at s(m) = m (2 lmax + 3 - m) / 2
-    // (the entry l = m); take the largest m with s(m) <= i
-    const double q = 2.0 * lmax + 3.0;
-    int m = (int)((q - sqrt(fmax(q * q - 8.0 * (double)i, 0.0))) / 2.0);
-    m = m < 0 ? 0 : (m > lmax ? lmax : m);
-    while (m > 0 && (int64_t)m * (2 * lmax + 3 - m) / 2 > i) --m;
-    while (m < lmax && (int64_t)(m + 1) * (2 * lmax + 2 - m) / 2 <= i) ++m;
-    const int l = (int)(i - (int64_t)m * (2 * lmax + 1 - m) / 2);
-    const double b = exp(-0.5 * (double)l * (l + 1) * sigma * sigma);
+// a_lm b_l with the Gaussian beam b_l = exp(-l(l+1) sigma^2 / 2).  A thread
+// takes one degree and every gridDim.y-th order, so that the FP64 exponential
+// (and the index of a coefficient) is not formed per coefficient: 92 us at lmax
+// 1535 when it was, for 38 MB of traffic.  Consecutive threads take consecutive
+// coefficients of one order.
+__global__ void __launch_bounds__(256)
+k_alm_beam(const double2* __restrict__ in, int32_t lmax, double sigma,
+           double2* __restrict__ out) {
+  const int l = blockIdx.x * blockDim.x + threadIdx.x;
+  if (l > lmax) return;
+  const double b = exp(-0.5 * (double)l * (l + 1) * sigma * sigma);
+  for (int m = blockIdx.y; m <= l; m += gridDim.y) {
+    const size_t i = (size_t)m * (2 * lmax + 1 - m) / 2 + l;
     const double2 a = in[i];
     out[i] = make_double2(a.x * b, a.y * b);
   }
@@ -831,13 +839,12 @@ ufc_status run_alm2map(ufc_ctx* c, const double* alm, int nside, int lmax, float
   if (s) return s;
   {
     ProfScope ps_(c, "k_legendre_synth");
-    const int nt = npairs > 256 ? 256 : (npairs > 128 ? 128 : 64);
+    const int nt = npairs > 128 ? 128 : 64;
     const dim3 grid((npairs + 2 * nt - 1) / (2 * nt), lmax + 1);
 #define UFC_SYN(NT)                                                                                \
   k_legendre_synth<NT><<<grid, NT, 0, c->stream>>>(reinterpret_cast<const double2*>(alm), sp.mu,   \
                                                    sp.ex, sp.tb, lmax, nrings, npairs, sp.ring)
-    if (nt == 256) UFC_SYN(256);
-    else if (nt == 128) UFC_SYN(128);
+    if (nt == 128) UFC_SYN(128);
     else UFC_SYN(64);
 #undef UFC_SYN
   }
@@ -852,8 +859,10 @@ ufc_status run_alm_beam(ufc_ctx* c, const double* in, int lmax, double sigma, do
   if ((reinterpret_cast<uintptr_t>(in) & 15) || (reinterpret_cast<uintptr_t>(out) & 15))
     return set_err(c, UFC_ERR_ARG, "a_lm buffers must be 16-byte aligned");
   ProfScope ps_(c, "k_alm_beam");
-  k_alm_beam<<<2 * c->num_sms, 256, 0, c->stream>>>(reinterpret_cast<const double2*>(in), lmax,
-                                                    sigma, reinterpret_cast<double2*>(out));
+  const int nl = lmax / 256 + 1;                       // blocks of 256 degrees
+  const int slices = std::min(lmax + 1, std::max(1, 8 * c->num_sms / nl));
+  k_alm_beam<<<dim3(nl, slices), 256, 0, c->stream>>>(reinterpret_cast<const double2*>(in), lmax,
+                                                      sigma, reinterpret_cast<double2*>(out));
   UFC_CUDA(c, cudaGetLastError());
   return UFC_OK;
 }
