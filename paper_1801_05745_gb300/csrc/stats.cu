@@ -58,6 +58,16 @@ __device__ __forceinline__ long long warp_sum_ll(long long v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xFFFFFFFFu, v, o);
   return v;
 }
+// Sum of v[0], v[stride], ..., v[(n - 1) stride] by one warp in a fixed
+// order: lane l adds elements l, l + 32, ... in turn, then a butterfly; every
+// lane ends with the same value (each pairwise sum is formed by both lanes).
+__device__ __forceinline__ double warp_sum_fixed(const double* v, int n, int stride) {
+  double s = 0.0;
+  for (int i = threadIdx.x & 31; i < n; i += 32) s += __ldcg(v + (size_t)i * stride);
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
+  return s;
+}
+
 // Block sum of a double in fixed order (lane order, then warp order).
 template <int NT>
 __device__ __forceinline__ double block_sum_d(double v, double* sh) {
@@ -298,271 +308,419 @@ k_kappa_finish(const double* __restrict__ part, float ch, float cl, int npix,
 }
 
 // --------------------------------------------------------- adjoint -----
-// One pass (k_adj_main) over tiles of 4 pixels per thread (2560 or 3072
-// pixels, the block sizes below), one block per SM.  Phase 1:
-// e_p = sum_b A_b n_bp - C unrounded (double-float, the shells in order, as
-// the forward pass), e_p^2, the power sums P1..P3 = sum_p e_p^k and
-// Q = sum_p g_p, and the tile's maxima of |e|, e^2, |g|.  Each quantity is
-// quantised (quant2: two integers, 43 bits relative to the scale) with a
-// power-of-two scale from the block's running maximum over the tiles it has
-// seen; when a tile raises a maximum, the 64-bit accumulators are first
+// One read of the counts (k_adj_main) in tiles of 2 NT pixels, two adjacent
+// pixels per thread, a few blocks per SM so that one block's arithmetic overlaps
+// another's loads.
+//
+// Bound by the latency that is left: 60 shells at Nside 1024 take 750 us for 3.0 GB
+// read once (4.0 TB/s, 60% of the copy rate; 53% issue, FMA pipe 49%), with waits
+// for loads and the barriers around phase 2; 140 shells at Nside 512 595 us (3.0
+// TB/s).  Two reads with 64-bit integer multiply-adds took 1080 and 1370 us.  A
+// batch of 8 shells in flight while 8 are added (80 registers, three blocks per
+// SM) against none: 930; 4 shells: 765; two blocks with 16: 830.  256-pixel tiles for
+// every shell count: 780.  Phase 2's pixels split over idle warps: 875 (its sums take
+// the shared memory that the loads in flight use as L1).
+//
+// Phase 1: e_p = sum_b A_b n_bp - C unrounded (double-float, the shells in order,
+// the operations of the forward pass, two pixels side by side in packed
+// registers), e_p^2, the power sums P1..P3 = sum_p e_p^k and Q = sum_p g_p, and
+// the tile's maxima of |e|, e^2, |g|.  The counts' low bytes stay in shared
+// memory.
+//
+// Quantisation: each quantity as two integers (quant2: 43 bits relative to the
+// scale) with a power-of-two scale from the block's running maximum over the
+// tiles it has seen; when a tile raises a maximum, the sums so far are first
 // flushed at the old scale into the block's 128-bit fixed-point rows, which
 // take every flush at its own scale exactly.  Every pixel is therefore
-// quantised at least as finely as a single scale from the global maxima
-// would.  Phase 2: warp w of NW owns shells w, w + NW, w + 2 NW (of the
-// launch's window) and each lane a
-// column of the tile's pixels, accumulating q n in 64-bit integers (the
-// tile's counts read a second time, mostly from L2).  A bound on the
-// accumulated magnitudes (pixels per lane x tile maximum count x 2^22 per
-// tile) triggers a flush before any 64-bit sum could overflow.  A launch
-// covers 3 NW shells (60 at 640 threads, 72 at 768); more shells take one
-// launch per window (phase 1 reads all shells in each).  With EXT, e comes from summed subvolume partials E_p (e =
-// E_p - C, the same double-float subtraction as k_kappa_finish) and the
-// counts, those of one subvolume, enter phase 1 only through their maximum:
-// the per-shell sums are then that subvolume's share, and they add over
-// subvolumes.
-// Block sizes (4 pixels per thread, 3 shells per warp): 640 threads (2560-
-// pixel tiles, 60 shells per launch) for maps of up to 60 shells, 768 (3072-
-// pixel tiles, 72 shells) above.  Measured at 60 shells, Nside 1024: 1024
-// threads 1.34 ms, 896 1.34, 832 1.30, 768 1.08, 704 1.20, 640 1.04 (12
-// shells unrolled in phase 1); the tiles in flight of the smaller blocks
-// (152 x 2560 pixels x 60 shells x 4 B = 93 MB) stay in L2 for phase 2.
-constexpr int kAdjThreadsSmall = 640;
-constexpr int kAdjThreadsLarge = 768;
-constexpr int kAdjSpw = 3;                // shells per warp in phase 2
+// quantised at least as finely as a single scale from the global maxima would.
+//
+// Phase 2: the per-shell sums sum_p q_p n_bp are a matrix product, shells x
+// pixels times pixels x quantities, on the tensor cores: the integers as signed
+// 8-bit digits (three per integer, six per quantity, and one column of ones
+// for N_b), the counts byte by byte, both exactly as FP16, and FP32 sums of
+// products that stay integers below 2^22, so they are exact whatever the order
+// and the alignment inside the tensor core.  They are added to 64-bit sums in
+// shared memory every few steps.  Counts of 256 and more take further passes
+// over the tile (from L2) with their higher bytes, the last one signed.  (mma.sync:
+// 16 or 24 columns are far too few for a tcgen05 tile to matter; the product
+// takes 16 multiply-adds per count, a percent of the tensor cores' rate.)  With
+// 64-bit integer multiply-adds in place of it, a warp per three shells, the
+// counts were read a second time and phase 2 took as long as phase 1.
+//
+// With EXT, e comes from summed subvolume partials E_p (e = E_p - C, the same
+// double-float subtraction as k_kappa_finish) and the counts, those of one
+// subvolume, enter phase 2 only: the per-shell sums are then that subvolume's
+// share, and they add over subvolumes.
+// columns: digits of e and e^2 (6 each), ones, digits of g (6), padded to 8
+__host__ __device__ constexpr int adj_cols(bool g) { return g ? 24 : 16; }
+__host__ __device__ constexpr int adj_lda(int nt) { return 2 * nt + 32; }    // bytes per count row
+__host__ __device__ constexpr int adj_ldb(int nt) { return 2 * nt + 32; }    // halves per column
+// (row strides of 8 and 16 words modulo 32: the fragments' loads meet no bank
+// conflict)
+__host__ __device__ constexpr int adj_batch(int nt) { return nt < 256 ? 16 : 8; }  // shells a fetch
+__host__ __device__ constexpr int adj_rows(int nt, int S) {       // whole pairs of batches
+  return (S + 2 * adj_batch(nt) - 1) / (2 * adj_batch(nt)) * (2 * adj_batch(nt));
+}
+__host__ __device__ inline size_t adj_smem(int nt, int S, bool g) {
+  const size_t mp = adj_rows(nt, S), nc = adj_cols(g);
+  return mp * adj_lda(nt) + nc * adj_ldb(nt) * 2 + mp * nc * 8 + (size_t)S * sizeof(AdjRow) +
+         mp * sizeof(float4);
+}
+
+__device__ __forceinline__ void mma_f16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2,
+                                        uint32_t a3, uint32_t b0, uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+      "{%0,%1,%2,%3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+// Two integers u < 1024 in the halves of w (0x6400 | u is the FP16 number
+// 1024 + u), minus 1024 + off: exact.
+__device__ __forceinline__ uint32_t half2_minus(uint32_t w, uint32_t bias) {
+  uint32_t r;
+  asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(w), "r"(bias));
+  return r;
+}
+constexpr uint32_t kHalf1024 = 0x64006400u;   // 1024, 1024
+constexpr uint32_t kHalf1152 = 0x64806480u;   // 1152, 1152
 
 template <bool USE_G, int NT, bool EXT>
-__global__ void __launch_bounds__(NT, 1)
-k_adj_main(const int32_t* __restrict__ counts, Coef cf, const float* __restrict__ g,
-           double* __restrict__ rows_out, double* __restrict__ sumpart,
-           unsigned long long* range_flag, int s0, float* __restrict__ kappa_out,
-           double* __restrict__ ksum_out, const double* __restrict__ ext,
-           unsigned long long* __restrict__ pdf, int npdf) {
-  if (kappa_out) clear_pdf(pdf, npdf);
+__global__ void __launch_bounds__(NT, USE_G || NT < 256 ? 2 : 3)
+k_adj_main(const int32_t* __restrict__ counts, const __grid_constant__ Coef cf,
+           const float* __restrict__ g, double* __restrict__ rows_out,
+           double* __restrict__ sumpart, unsigned long long* range_flag,
+           float* __restrict__ kappa_out, double* __restrict__ ksum_out,
+           const double* __restrict__ ext, unsigned long long* __restrict__ pdf, int npdf) {
   extern __shared__ __align__(16) uint8_t adj_sm[];
-  constexpr int T = NT, NW = T / 32, TP = 4 * T;
-  int* q_s = reinterpret_cast<int*>(adj_sm);                 // [6][TP] quantised e, e^2, g
-  float* ef_s = reinterpret_cast<float*>(adj_sm);            // the same memory: e, e^2 as floats
-  float* ps_s = reinterpret_cast<float*>(adj_sm + 24 * TP);   // [8][T] this thread's power sums
-  AdjRow* rows = reinterpret_cast<AdjRow*>(adj_sm + 24 * TP + 32 * T);  // [nshell]
-  __shared__ float ah_s[kMaxShells], al_s[kMaxShells];
+  constexpr int NW = NT / 32, P = 2 * NT, NC = adj_cols(USE_G);
+  constexpr int LDA = adj_lda(NT), LDB = adj_ldb(NT);
+  if (kappa_out) clear_pdf(pdf, npdf);
+  const int S = cf.nshell, npix = cf.npix, np2 = npix >> 1;
+  const int mt_n = (S + 15) >> 4, mp = adj_rows(NT, S);      // tiles of 16 shells; rows held
+  uint8_t* An = adj_sm;                                      // [mp][LDA] a byte of the counts
+  uint16_t* Bq = reinterpret_cast<uint16_t*>(An + (size_t)mp * LDA);            // [NC][LDB]
+  long long* sums = reinterpret_cast<long long*>(Bq + (size_t)NC * LDB);        // [mp][NC]
+  AdjRow* rows = reinterpret_cast<AdjRow*>(sums + (size_t)mp * NC);           // [S]
+  float4* coef = reinterpret_cast<float4*>(rows + S);                           // [mp] A_b, twice
   __shared__ float mred[3][NW];
-  __shared__ int nred[NW];
+  __shared__ unsigned nred[NW];
   __shared__ double red[NW];
-  const int S = cf.nshell, npix = cf.npix, ng = npix >> 2;
-  const int w = threadIdx.x >> 5, ln = threadIdx.x & 31;
-  for (int i = threadIdx.x; i < S; i += T) { ah_s[i] = cf.ah[i]; al_s[i] = cf.al[i]; rows[i] = AdjRow{}; }
+  const int tid = threadIdx.x, w = tid >> 5, ln = tid & 31;
+  for (int i = tid; i < mp; i += NT)                         // 0 above the last shell
+    coef[i] = i < S ? make_float4(cf.ah[i], cf.ah[i], cf.al[i], cf.al[i])
+                    : make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int i = tid; i < S; i += NT) rows[i] = AdjRow{};
+  for (int i = tid; i < mp * NC; i += NT) sums[i] = 0;
+  // the column of ones, and zeros in the padding
+  for (int i = tid; i < P / 2; i += NT) {
+    reinterpret_cast<uint32_t*>(Bq + 12 * LDB)[i] = 0x3C003C00u;               // 1, 1
+    for (int k = USE_G ? 19 : 13; k < NC; ++k) reinterpret_cast<uint32_t*>(Bq + k * LDB)[i] = 0u;
+  }
   // running maxima of |e|, e^2, |g| over this block's tiles, in shared
   // memory: thread 0 updates them after a barrier that every thread's read
   // of them for the tile has passed
   __shared__ float Ms[3];
-  if (threadIdx.x == 0) Ms[0] = Ms[1] = Ms[2] = 0.f;
+  if (tid == 0) Ms[0] = Ms[1] = Ms[2] = 0.f;
   auto scale = [](float M) { return M > 0.f ? min(120, 21 - ilog2f(M)) : 0; };
-  for (int k = 0; k < 8; ++k) ps_s[k * T + threadIdx.x] = 0.f;
-  __syncthreads();                         // ah_s, al_s, rows and Ms before any use
-  constexpr int NQ = USE_G ? 6 : 4;
-  long long acc[kAdjSpw][NQ + 1];
-#pragma unroll
-  for (int k = 0; k < kAdjSpw; ++k)
-#pragma unroll
-    for (int j = 0; j <= NQ; ++j) acc[k][j] = 0;
+  // the 64-bit sums into the rows (thread t takes shells t, t + NT, ...)
   auto flush = [&](int s1, int s2, int s3) {
+    for (int b = tid; b < S; b += NT) {
+      AdjRow& row = rows[b];
+      long long* v = sums + (size_t)b * NC;
 #pragma unroll
-    for (int k = 0; k < kAdjSpw; ++k) {
-      const int b = s0 + w + NW * k;
-      long long a[NQ + 1];
-#pragma unroll
-      for (int j = 0; j <= NQ; ++j) { a[j] = warp_sum_ll(acc[k][j]); acc[k][j] = 0; }
-      if (ln == 0 && b < S) {
-        AdjRow& row = rows[b];
-        i128_add(row.s[0], a[0], kFrac1 - s1);
-        i128_add(row.s[0], a[1], kFrac1 - s1 - 22);
-        i128_add(row.s[1], a[2], kFrac2 - s2);
-        i128_add(row.s[1], a[3], kFrac2 - s2 - 22);
+      for (int k = 0; k < 3; ++k) {
+        i128_add(row.s[0], v[k], kFrac1 - s1 + 8 * k);
+        i128_add(row.s[0], v[3 + k], kFrac1 - s1 - 22 + 8 * k);
+        i128_add(row.s[1], v[6 + k], kFrac2 - s2 + 8 * k);
+        i128_add(row.s[1], v[9 + k], kFrac2 - s2 - 22 + 8 * k);
         if (USE_G) {
-          i128_add(row.s[2], a[4], kFrac3 - s3);
-          i128_add(row.s[2], a[5], kFrac3 - s3 - 22);
+          i128_add(row.s[2], v[13 + k], kFrac3 - s3 + 8 * k);
+          i128_add(row.s[2], v[16 + k], kFrac3 - s3 - 22 + 8 * k);
         }
-        row.n += a[NQ];
+      }
+      row.n += v[12];
+      for (int k = 0; k < NC; ++k) v[k] = 0;
+    }
+  };
+  // digits of the integers h0, h1 of the thread's two pixels into columns col,
+  // col + 1, col + 2: h = d0 + 2^8 d1 + 2^16 d2, |d| <= 128
+  auto digits = [&](int col, int h0, int h1) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      h0 += 128;
+      h1 += 128;
+      const uint32_t u = k < 2 ? (uint32_t)(h0 & 255) | (uint32_t)(h1 & 255) << 16
+                               : (uint32_t)h0 | (uint32_t)h1 << 16;      // d2 + 128 in [0, 255]
+      reinterpret_cast<uint32_t*>(Bq + (size_t)(col + k) * LDB)[tid] =
+          half2_minus(u | kHalf1024, kHalf1152);
+      h0 >>= 8;
+      h1 >>= 8;
+    }
+  };
+  // phase 2 with the byte plane in An (shift 8 plane; u_off 128 when its bytes
+  // are signed), counts below `most` in it
+  auto product = [&](int plane, bool sgn, unsigned most) {
+    const int gq = ln >> 2, c = ln & 3;
+    const uint32_t flip = sgn ? 0x80808080u : 0u, bias = sgn ? kHalf1152 : kHalf1024;
+    const int steps = max(1, 1024 / (int)max(1u, min(most, 255u)));   // of 32 pixels per sum
+    for (int mt = w; mt < mt_n; mt += NW) {
+      const uint8_t* r0 = An + (size_t)(16 * mt + gq) * LDA + 8 * c;
+      const uint8_t* r1 = r0 + 8 * LDA;
+      long long* dst = sums + (size_t)(16 * mt + gq) * NC + 2 * c;
+      for (int k0 = 0; k0 < P / 32; k0 += steps) {
+        float acc[NC / 8][4];
+#pragma unroll
+        for (int j = 0; j < NC / 8; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
+        const int k1 = min(k0 + steps, P / 32);
+        for (int k = k0; k < k1; ++k) {
+          uint2 x = *reinterpret_cast<const uint2*>(r0 + 32 * k);
+          uint2 y = *reinterpret_cast<const uint2*>(r1 + 32 * k);
+          x.x ^= flip; x.y ^= flip; y.x ^= flip; y.y ^= flip;
+          // bytes 0, 1 and 2, 3 as FP16 pairs
+          auto lo = [&](uint32_t v) { return half2_minus(__byte_perm(v, 0x64, 0x4140), bias); };
+          auto hi = [&](uint32_t v) { return half2_minus(__byte_perm(v, 0x64, 0x4342), bias); };
+          const uint32_t a0 = lo(x.x), a1 = lo(y.x), a2 = hi(x.x), a3 = hi(y.x);
+          const uint32_t e0 = lo(x.y), e1 = lo(y.y), e2 = hi(x.y), e3 = hi(y.y);
+#pragma unroll
+          for (int j = 0; j < NC / 8; ++j) {
+            const uint4 q = *reinterpret_cast<const uint4*>(Bq + (size_t)(8 * j + gq) * LDB +
+                                                            32 * k + 8 * c);
+            mma_f16(acc[j], a0, a1, a2, a3, q.x, q.y);
+            mma_f16(acc[j], e0, e1, e2, e3, q.z, q.w);
+          }
+        }
+#pragma unroll
+        for (int j = 0; j < NC / 8; ++j) {
+          auto add = [&](long long* p, float v) {
+            *p += (long long)__float2int_rn(v) * (1ll << (8 * plane));
+          };
+          add(dst + 8 * j, acc[j][0]);
+          add(dst + 8 * j + 1, acc[j][1]);
+          add(dst + 8 * NC + 8 * j, acc[j][2]);
+          add(dst + 8 * NC + 8 * j + 1, acc[j][3]);
+        }
       }
     }
   };
-  const int4* c4 = reinterpret_cast<const int4*>(counts);
   const f2 mc{-cf.ch, -cf.cl};
-  const int ntile = (npix + TP - 1) / TP;
-  double bound = 0.0;                      // bound on |any 64-bit sum|, uniform
+  const int ntile = (npix + P - 1) / P;
+  // power sums: the tile's two pixels first, then into the running sums, of
+  // which the threads of a narrow block (more tiles each) have two in turn, so
+  // that none takes more than some tens of additions per million pixels
+  constexpr int kA = NT < 256 ? 2 : 1;
+  f2 pw[kA][4];
+#pragma unroll
+  for (int i = 0; i < 4 * kA; ++i) pw[i >> 2][i & 3] = f2{0.f, 0.f};
   f2 ks{0.f, 0.f};                         // this thread's sum of the FP32 map (kappa_out)
+  // the counts in batches of kB shells, the next one's loads in flight while one
+  // is added; the first batch of the next tile is fetched before phase 2
+  constexpr int kB = adj_batch(NT);
+  // (q: row b0 of the thread's pixels; whole tiles and batches without tests)
+  const uint32_t stride = (uint32_t)npix * 4u;
+  auto row = [&](const char* q, int u) {
+    return reinterpret_cast<const int2*>(q + (size_t)stride * (uint32_t)u);
+  };
+  auto fetch = [&](int2 (&v)[kB], const char* q, int b0, int tile) {
+    if ((tile + 1) * NT <= np2 && b0 + kB <= S) {            // (uniform)
+#pragma unroll
+      for (int u = 0; u < kB; ++u) v[u] = __ldcs(row(q, u));
+    } else {
+      const bool in = tile * NT + tid < np2;
+#pragma unroll
+      for (int u = 0; u < kB; ++u)
+        v[u] = in && b0 + u < S ? __ldcs(row(q, u)) : make_int2(0, 0);
+    }
+  };
+  const char* base = reinterpret_cast<const char*>(counts) + 8 * (size_t)tid;
+  auto tile_at = [&](int tile) { return base + (size_t)tile * (8 * NT); };
+  int2 v0[kB], v1[kB];
+  fetch(v0, tile_at(blockIdx.x), 0, blockIdx.x);
+  __syncthreads();
   for (int tile = blockIdx.x; tile < ntile; tile += gridDim.x) {
-    // phase 1: e of 4 adjacent pixels per thread (the shells in order, as in
-    // the forward pass), the power sums and the tile's maxima; e and e^2
-    // wait in shared memory until the tile's scale is known
-    const int gi = tile * T + threadIdx.x;   // group of 4 pixels
-    const bool have = gi < ng;
-    f2 a[4] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
-    int nmx = 0;
-    if (have) {
-      // shells unrolled for loads in flight (fewer with g, whose registers
-      // would spill more)
-      constexpr int kU1 = USE_G ? 6 : 12;
-#pragma unroll kU1
-      for (int b = 0; b < S; ++b) {
-        const int4 n = c4[(size_t)b * ng + gi];
-        nmx = max(nmx, max(max(n.x, n.y), max(n.z, n.w)));
+    // phase 1 (past the map's end: counts of 0)
+    const int gi = tile * NT + tid;        // pair of pixels
+    const bool have = gi < np2;
+    const int2* src = reinterpret_cast<const int2*>(counts) + gi;
+    uint8_t* arow = An + 2 * tid;
+    dfx a{0ull, 0ull};
+    unsigned nor = 0u;
+    const u64 two23 = x2_pack(8388608.0f, 8388608.0f);
+    auto add = [&](const int2 (&v)[kB], int b0) {
+#pragma unroll
+      for (int u = 0; u < kB; ++u) {
+        const int2 n = v[u];
+        nor |= (unsigned)n.x | (unsigned)n.y;
+        *reinterpret_cast<uint16_t*>(arow + (size_t)(b0 + u) * LDA) =
+            (uint16_t)__byte_perm(n.x, n.y, 0x0040);
         if constexpr (!EXT) {
-          const float h = ah_s[b], l = al_s[b];
-          f2_mac(a[0], h, l, float(n.x));
-          f2_mac(a[1], h, l, float(n.y));
-          f2_mac(a[2], h, l, float(n.z));
-          f2_mac(a[3], h, l, float(n.w));
+          const float4 cb = coef[b0 + u];
+          const u64 ah = x2_pack(cb.x, cb.y), al = x2_pack(cb.z, cb.w);
+          // float(n) for n < 2^23 (larger ones: below)
+          const u64 fb = x2_pack(__int_as_float(n.x | 0x4B000000),
+                                 __int_as_float(n.y | 0x4B000000));
+          const u64 f = x2_sub(fb, two23);
+          const u64 pn = x2_mul(ah, x2_sub(two23, fb));      // -ah n
+          const u64 pe = x2_fma(ah, f, pn);
+          const u64 sm = x2_sub(a.h, pn), bb = x2_sub(sm, a.h);
+          const u64 er = x2_sub(x2_sub(a.h, x2_sub(sm, bb)), x2_add(pn, bb));
+          a.h = sm;
+          a.l = x2_add(a.l, x2_add(er, x2_fma(al, f, pe)));
         }
       }
-      if constexpr (EXT) {
-        const double2 d01 = reinterpret_cast<const double2*>(ext)[2 * gi];
-        const double2 d23 = reinterpret_cast<const double2*>(ext)[2 * gi + 1];
-        a[0] = d_to_f2(d01.x);
-        a[1] = d_to_f2(d01.y);
-        a[2] = d_to_f2(d23.x);
-        a[3] = d_to_f2(d23.y);
+    };
+#pragma unroll 1
+    for (int b0 = 0; b0 < mp; b0 += 2 * kB) {
+      const char* q = tile_at(tile) + (size_t)stride * (uint32_t)b0;
+      fetch(v1, q + (size_t)stride * kB, b0 + kB, tile);
+      add(v0, b0);
+      const bool more = b0 + 2 * kB < mp;                    // else the next tile's first batch
+      const int nt = more ? tile : tile + (int)gridDim.x;
+      fetch(v0, more ? q + (size_t)stride * (2 * kB) : tile_at(nt), more ? b0 + 2 * kB : 0, nt);
+      add(v1, b0 + kB);
+    }
+    f2 av[2];
+    {
+      const float2 h = x2_get(a.h), l = x2_get(a.l);
+      av[0] = f2{h.x, l.x};
+      av[1] = f2{h.y, l.y};
+    }
+    if constexpr (EXT) {
+      if (have) {
+        const double2 d = reinterpret_cast<const double2*>(ext)[gi];
+        av[0] = d_to_f2(d.x);
+        av[1] = d_to_f2(d.y);
+      }
+    } else if (nor & 0xFF800000u) {        // rare: counts of 2^23 and more, or negative
+      av[0] = av[1] = f2{0.f, 0.f};
+      for (int b = 0; b < S; ++b) {
+        const int2 n = src[(size_t)b * np2];
+        f2_mac(av[0], coef[b].x, coef[b].z, float(n.x));
+        f2_mac(av[1], coef[b].x, coef[b].z, float(n.y));
       }
     }
-    const float4 gv4 = (USE_G && have) ? reinterpret_cast<const float4*>(g)[gi]
-                                       : make_float4(0.f, 0.f, 0.f, 0.f);
-    const float gs[4] = {gv4.x, gv4.y, gv4.z, gv4.w};
-    float t1 = 0.f, t2 = 0.f, t3 = 0.f;
-    float kv[4];
+    const float2 gv = (USE_G && have) ? reinterpret_cast<const float2*>(g)[gi] : make_float2(0.f, 0.f);
+    const float gs[2] = {gv.x, gv.y};
+    f2 e[2], e2[2];
+    float kv[2], t1 = 0.f, t2 = 0.f, t3 = 0.f;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      f2 e = f2_add(f2_norm(a[i].h, a[i].l), mc);
-      kv[i] = __fadd_rn(e.h, e.l);             // the FP32 map, as the forward pass rounds it
-      f2 e2 = f2_mul(e, e);
-      if (!have) { e = f2{0.f, 0.f}; e2 = f2{0.f, 0.f}; }
-      t1 = fmaxf(t1, fabsf(e.h));
-      t2 = fmaxf(t2, fabsf(e2.h));
+    for (int i = 0; i < 2; ++i) {
+      e[i] = f2_add(f2_norm(av[i].h, av[i].l), mc);
+      kv[i] = __fadd_rn(e[i].h, e[i].l);       // the FP32 map, as the forward pass rounds it
+      e2[i] = f2_mul(e[i], e[i]);
+      if (!have) { e[i] = f2{0.f, 0.f}; e2[i] = f2{0.f, 0.f}; }
+      t1 = fmaxf(t1, fabsf(e[i].h));
+      t2 = fmaxf(t2, fabsf(e2[i].h));
       t3 = fmaxf(t3, fabsf(gs[i]));
-      const int px = 4 * threadIdx.x + i;
-      ef_s[px] = e.h;
-      ef_s[TP + px] = e.l;
-      ef_s[2 * TP + px] = e2.h;
-      ef_s[3 * TP + px] = e2.l;
-    }
-    if (kappa_out && have) {                   // (uniform) the map itself, with its sum
-      reinterpret_cast<float4*>(kappa_out)[gi] = make_float4(kv[0], kv[1], kv[2], kv[3]);
-      ks = f2_add(ks, f2_add(f2_two_sum(kv[0], kv[1]), f2_two_sum(kv[2], kv[3])));
     }
     if (have) {
-      f2 p1{ps_s[threadIdx.x], ps_s[T + threadIdx.x]};
-      f2 p2{ps_s[2 * T + threadIdx.x], ps_s[3 * T + threadIdx.x]};
-      f2 p3{ps_s[4 * T + threadIdx.x], ps_s[5 * T + threadIdx.x]};
-      f2 qg{ps_s[6 * T + threadIdx.x], ps_s[7 * T + threadIdx.x]};
+      const f2 d[4] = {f2_add(e[0], e[1]), f2_add(e2[0], e2[1]),
+                       f2_add(f2_mul(e2[0], e[0]), f2_mul(e2[1], e[1])), f2_two_sum(gs[0], gs[1])};
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int px = 4 * threadIdx.x + i;
-        const f2 e{ef_s[px], ef_s[TP + px]};
-        const f2 e2{ef_s[2 * TP + px], ef_s[3 * TP + px]};
-        p1 = f2_add(p1, e);
-        p2 = f2_add(p2, e2);
-        p3 = f2_add(p3, f2_mul(e2, e));
-        qg = f2_add(qg, f2{gs[i], 0.f});
+      for (int k = 0; k < 4; ++k) {
+        const f2 t = f2_add(pw[kA - 1][k], d[k]);
+        if (kA > 1) pw[kA - 1][k] = pw[0][k];
+        pw[0][k] = t;
       }
-      ps_s[threadIdx.x] = p1.h; ps_s[T + threadIdx.x] = p1.l;
-      ps_s[2 * T + threadIdx.x] = p2.h; ps_s[3 * T + threadIdx.x] = p2.l;
-      ps_s[4 * T + threadIdx.x] = p3.h; ps_s[5 * T + threadIdx.x] = p3.l;
-      ps_s[6 * T + threadIdx.x] = qg.h; ps_s[7 * T + threadIdx.x] = qg.l;
     }
+    if (kappa_out && have) {                   // (uniform) the map itself, with its sum
+      reinterpret_cast<float2*>(kappa_out)[gi] = make_float2(kv[0], kv[1]);
+      ks = f2_add(ks, f2_two_sum(kv[0], kv[1]));
+    }
+    nor = __reduce_or_sync(0xFFFFFFFFu, nor);
     for (int o = 16; o > 0; o >>= 1) {
-      nmx = max(nmx, __shfl_xor_sync(0xFFFFFFFFu, nmx, o));
       t1 = fmaxf(t1, __shfl_xor_sync(0xFFFFFFFFu, t1, o));
       t2 = fmaxf(t2, __shfl_xor_sync(0xFFFFFFFFu, t2, o));
       t3 = fmaxf(t3, __shfl_xor_sync(0xFFFFFFFFu, t3, o));
     }
-    if (ln == 0) { nred[w] = nmx; mred[0][w] = t1; mred[1][w] = t2; mred[2][w] = t3; }
+    if (ln == 0) { nred[w] = nor; mred[0][w] = t1; mred[1][w] = t2; mred[2][w] = t3; }
     __syncthreads();
-    int NMX = 0;
+    unsigned NOR = 0u;                         // every count <= NOR (as unsigned)
     float T1 = 0.f, T2 = 0.f, T3 = 0.f;
+#pragma unroll
     for (int i = 0; i < NW; ++i) {
-      NMX = max(NMX, nred[i]);
+      NOR |= nred[i];
       T1 = fmaxf(T1, mred[0][i]);
       T2 = fmaxf(T2, mred[1][i]);
       T3 = fmaxf(T3, mred[2][i]);
     }
     const float M1 = Ms[0], M2 = Ms[1], M3 = Ms[2];
     const bool grow = T1 > M1 || T2 > M2 || T3 > M3;   // (uniform) a coarser scale
-    const double inc = double(TP / 32) * double(NMX) * 4194304.0;   // per lane, this tile
-    if (grow || bound + inc > 2305843009213693952.0) {              // 2^61
-      flush(scale(M1), scale(M2), scale(M3));                       // at the old scale
-      bound = 0.0;
-    }
-    bound += inc;
+    if (grow) flush(scale(M1), scale(M2), scale(M3));  // at the old scale
     const float N1 = fmaxf(M1, T1), N2 = fmaxf(M2, T2), N3 = fmaxf(M3, T3);
-    if (grow && threadIdx.x == 0 && (N1 >= 16384.0f || N3 >= 16384.0f || N2 >= 268435456.0f))
+    if (grow && tid == 0 && (N1 >= 16384.0f || N3 >= 16384.0f || N2 >= 268435456.0f))
       atomicAdd(range_flag, 1ull);
     const int s1 = scale(N1), s2 = scale(N2), s3 = scale(N3);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int px = 4 * threadIdx.x + i;
-      const f2 e{ef_s[px], ef_s[TP + px]};
-      const f2 e2{ef_s[2 * TP + px], ef_s[3 * TP + px]};
-      int h, l;
-      quant2(e, s1, h, l);
-      q_s[px] = h;
-      q_s[TP + px] = l;
-      quant2(e2, s2, h, l);
-      q_s[2 * TP + px] = h;
-      q_s[3 * TP + px] = l;
+    {
+      int h0, l0, h1, l1;
+      quant2(e[0], s1, h0, l0);
+      quant2(e[1], s1, h1, l1);
+      digits(0, h0, h1);
+      digits(3, l0, l1);
+      quant2(e2[0], s2, h0, l0);
+      quant2(e2[1], s2, h1, l1);
+      digits(6, h0, h1);
+      digits(9, l0, l1);
       if (USE_G) {
-        quant2(f2{gs[i], 0.f}, s3, h, l);
-        q_s[4 * TP + px] = h;
-        q_s[5 * TP + px] = l;
+        quant2(f2{gs[0], 0.f}, s3, h0, l0);
+        quant2(f2{gs[1], 0.f}, s3, h1, l1);
+        digits(13, h0, h1);
+        digits(16, l0, l1);
       }
     }
-    __syncthreads();                       // q_s complete; every thread has read Ms
-    if (grow && threadIdx.x == 0) { Ms[0] = N1; Ms[1] = N2; Ms[2] = N3; }
-    // phase 2: lane ln takes pixels ln, ln + 32, ... of the tile (L2 re-reads)
-    const int base = tile * TP;
-    const int valid = min(TP, npix - base);
-#pragma unroll 16
-    for (int pi = ln; pi < valid; pi += 32) {          // 48 count loads in flight per lane
-      int qv[NQ];
-#pragma unroll
-      for (int j = 0; j < NQ; ++j) qv[j] = q_s[j * TP + pi];
-#pragma unroll
-      for (int k = 0; k < kAdjSpw; ++k) {
-        const int b = s0 + w + NW * k;
-        if (b < S) {
-          const long long n = counts[(size_t)b * npix + base + pi];
-#pragma unroll
-          for (int j = 0; j < NQ; ++j) acc[k][j] += (long long)qv[j] * n;
-          acc[k][NQ] += n;
+    __syncthreads();                       // bytes and digits complete; every thread has read Ms
+    if (grow && tid == 0) { Ms[0] = N1; Ms[1] = N2; Ms[2] = N3; }
+    // phase 2: the low bytes, then (rare) the higher ones
+    product(0, false, NOR);
+    for (int plane = 1; plane < 4 && NOR >> (8 * plane); ++plane) {
+      __syncthreads();
+      if (have)
+        for (int b = 0; b < S; ++b) {
+          const int2 n = src[(size_t)b * np2];
+          *reinterpret_cast<uint16_t*>(arow + (size_t)b * LDA) =
+              (uint16_t)(((unsigned)n.x >> (8 * plane) & 255u) |
+                         ((unsigned)n.y >> (8 * plane) & 255u) << 8);
         }
-      }
+      __syncthreads();
+      product(plane, plane == 3, 255u);
     }
-    __syncthreads();                       // q_s and nred are rewritten by the next tile
+    __syncthreads();                       // the next tile rewrites the bytes, digits and maxima
   }
-  __syncthreads();
   flush(scale(Ms[0]), scale(Ms[1]), scale(Ms[2]));
-  __syncthreads();
   double* dst = rows_out + (size_t)blockIdx.x * 4 * S;
-  const int s_end = min(S, s0 + kAdjSpw * NW);   // the shells of this launch: [s0, s_end)
-  for (int b = s0 + threadIdx.x; b < s_end; b += T) {
+  for (int b = tid; b < S; b += NT) {      // (this thread's own rows)
     dst[4 * b + 0] = i128_to_d(rows[b].s[0], kFrac1);
     dst[4 * b + 1] = i128_to_d(rows[b].s[1], kFrac2);
     dst[4 * b + 2] = USE_G ? i128_to_d(rows[b].s[2], kFrac3) : 0.0;
     dst[4 * b + 3] = (double)rows[b].n;
   }
-  const f2 p1{ps_s[threadIdx.x], ps_s[T + threadIdx.x]}, p2{ps_s[2 * T + threadIdx.x], ps_s[3 * T + threadIdx.x]};
-  const f2 p3{ps_s[4 * T + threadIdx.x], ps_s[5 * T + threadIdx.x]}, qg{ps_s[6 * T + threadIdx.x], ps_s[7 * T + threadIdx.x]};
   if (kappa_out) {                         // (uniform)
-    const double vk = block_sum_d<T>(f2_to_d(ks), red);
-    if (threadIdx.x == 0) ksum_out[blockIdx.x] = vk;
+    const double vk = block_sum_d<NT>(f2_to_d(ks), red);
+    if (tid == 0) ksum_out[blockIdx.x] = vk;
   }
-  const double v1 = block_sum_d<T>(f2_to_d(p1), red);
-  if (threadIdx.x == 0) sumpart[4 * blockIdx.x + 0] = v1;
-  const double v2 = block_sum_d<T>(f2_to_d(p2), red);
-  if (threadIdx.x == 0) sumpart[4 * blockIdx.x + 1] = v2;
-  const double v3 = block_sum_d<T>(f2_to_d(p3), red);
-  if (threadIdx.x == 0) sumpart[4 * blockIdx.x + 2] = v3;
-  const double v4 = block_sum_d<T>(f2_to_d(qg), red);
-  if (threadIdx.x == 0) sumpart[4 * blockIdx.x + 3] = v4;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const double own = f2_to_d(pw[0][k]) + (kA > 1 ? f2_to_d(pw[kA - 1][k]) : 0.0);
+    const double v = block_sum_d<NT>(own, red);
+    if (tid == 0) sumpart[4 * blockIdx.x + k] = v;
+  }
+}
+
+// out[k] = the sum of quantity k (4 S row entries, then 4 power sums) over the
+// blocks of k_adj_main, one warp each in a fixed order; out[4 S + 4] = the range
+// flag, which is cleared.
+__global__ void __launch_bounds__(128)
+k_adj_reduce(const double* __restrict__ rows, const double* __restrict__ sums, int S, int nblk,
+             unsigned long long* range_flag, double* __restrict__ out) {
+  const int k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (k == 0 && threadIdx.x == 0) {
+    out[4 * S + 4] = (double)*range_flag;
+    *range_flag = 0ull;
+  }
+  if (k >= 4 * S + 4) return;
+  const double v = k < 4 * S ? warp_sum_fixed(rows + k, nblk, 4 * S)
+                             : warp_sum_fixed(sums + (k - 4 * S), nblk, 4);
+  if ((threadIdx.x & 31) == 0) out[k] = v;
 }
 
 // Per-block sums of an FP32 map (double-float per thread), the first pass of
@@ -597,16 +755,6 @@ struct PdfParam {
   float lo_dn, lo_up, hi_dn, hi_up;   // FP32 brackets of lo and hi
   int32_t nbins;
 };
-
-// Sum of v[0], v[stride], ..., v[(n - 1) stride] by one warp in a fixed
-// order: lane l adds elements l, l + 32, ... in turn, then a butterfly; every
-// lane ends with the same value (each pairwise sum is formed by both lanes).
-__device__ __forceinline__ double warp_sum_fixed(const double* v, int n, int stride) {
-  double s = 0.0;
-  for (int i = threadIdx.x & 31; i < n; i += 32) s += __ldcg(v + (size_t)i * stride);
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
-  return s;
-}
 
 // PDF slot of one FP32 value by the FP64 definition: floor((k - lo) * scale),
 // under/overflow and NaN.  A call of its own: inlined, the compiler evaluates
@@ -1164,47 +1312,54 @@ static ufc_status adjoint_sums(ufc_ctx* c, const int32_t* counts, int S, int nsi
   if (ext && (reinterpret_cast<uintptr_t>(ext) & 15))
     return set_err(c, UFC_ERR_ARG, "partial_dev must be 16-byte aligned");
   const int npix = 12 * nside * nside;
-  const int grid2 = c->num_sms;                            // one block per SM
+  // threads per block and blocks per SM: 512-pixel tiles where two blocks' shared
+  // memory fits an SM (up to 128 shells, 96 with g), 256-pixel tiles above
+  // (Nside 512, wide against narrow tiles: 100 shells 366 and 450 us, 128 shells
+  // 421 and 482, 90 with g 349 and 402; 140 shells, one wide block per SM, 657 and
+  // 529)
+  const size_t sm_bytes = (size_t)c->smem_optin;             // (per block; an SM holds 1 KB more)
+  const bool wide = 2 * (adj_smem(256, S, g != nullptr) + 1024) <= sm_bytes + 1024;
+  const int nt = wide ? 256 : 128;
+  const size_t smem2 = adj_smem(nt, S, g != nullptr);
+  const int per_sm = std::max(1, std::min(g || !wide ? 2 : 3, (int)((sm_bytes + 1024) / (smem2 + 1024))));
+  const int grid2 = std::min(per_sm * c->num_sms, (npix + 2 * nt - 1) / (2 * nt));
   const size_t nrow = (size_t)grid2 * 4 * S, nsum = (size_t)grid2 * 4;
   const int mgrid = moments_grid(c->num_sms, npix);
   const size_t nmap = kappa ? (size_t)grid2 + 3 * (size_t)mgrid : 0;   // map sums, moment partials
-  double* part = (double*)ws_get(c, kSlotPartials, (nrow + nsum + nmap) * 8);
+  const size_t nout = 4 * (size_t)S + 5;
+  double* part = (double*)ws_get(c, kSlotPartials, (nrow + nsum + nmap + nout) * 8);
   if (!part) return UFC_ERR_ALLOC;
   double* rows = part;
   double* sums = part + nrow;
   double* ksum = sums + nsum;
   double* mpart = ksum + grid2;
+  double* dout = part + nrow + nsum + nmap;
   BinCounters* bc = reinterpret_cast<BinCounters*>(c->counters);
-  UFC_CUDA(c, cudaMemsetAsync(&bc->range, 0, sizeof(unsigned long long), c->stream));
-  // q_s, the threads' power sums, rows; one launch per window of shells
-  // (a launch's warps own 3 shells each); every launch recomputes e from all
-  // shells and writes the same power sums
-  const bool small = S <= kAdjSpw * (kAdjThreadsSmall / 32);
-  const int nt = small ? kAdjThreadsSmall : kAdjThreadsLarge;
-  const int win = kAdjSpw * (nt / 32);
-  const size_t smem2 = (size_t)24 * 4 * nt + (size_t)32 * nt + (size_t)S * sizeof(AdjRow);
   {
     ProfScope ps_(c, "k_adj_main");
 #define UFC_ADJ(G, NT_, X)                                                                        \
   do {                                                                                            \
     UFC_CUDA(c, cudaFuncSetAttribute(k_adj_main<G, NT_, X>,                                       \
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2));   \
-    for (int s0 = 0; s0 < S; s0 += win)                                                           \
-      k_adj_main<G, NT_, X><<<grid2, NT_, smem2, c->stream>>>(                                    \
-          counts, cf, g, rows, sums, &bc->range, s0, s0 == 0 ? kappa : nullptr, ksum, ext,        \
-          (unsigned long long*)pdf, nbins + 3);                                                   \
+    k_adj_main<G, NT_, X><<<grid2, NT_, smem2, c->stream>>>(                                      \
+        counts, cf, g, rows, sums, &bc->range, kappa, ksum, ext, (unsigned long long*)pdf,        \
+        nbins + 3);                                                                               \
   } while (0)
 #define UFC_ADJ_X(G, NT_)                                                                         \
   do {                                                                                            \
     if (ext) UFC_ADJ(G, NT_, true);                                                               \
     else UFC_ADJ(G, NT_, false);                                                                  \
   } while (0)
-    if (g && small) UFC_ADJ_X(true, kAdjThreadsSmall);
-    else if (g) UFC_ADJ_X(true, kAdjThreadsLarge);
-    else if (small) UFC_ADJ_X(false, kAdjThreadsSmall);
-    else UFC_ADJ_X(false, kAdjThreadsLarge);
+    if (g && wide) UFC_ADJ_X(true, 256);
+    else if (g) UFC_ADJ_X(true, 128);
+    else if (wide) UFC_ADJ_X(false, 256);
+    else UFC_ADJ_X(false, 128);
 #undef UFC_ADJ_X
 #undef UFC_ADJ
+  }
+  {
+    ProfScope ps_(c, "k_adj_reduce");
+    k_adj_reduce<<<(int)(nout + 3) / 4, 128, 0, c->stream>>>(rows, sums, S, grid2, &bc->range, dout);
   }
   UFC_CUDA(c, cudaGetLastError());
   if (kappa) {                             // moments and PDF of the map just written
@@ -1212,23 +1367,13 @@ static ufc_status adjoint_sums(ufc_ctx* c, const int32_t* counts, int S, int nsi
                                   true);
     if (s) return s;
   }
-  std::vector<double> hp(nrow + nsum);
-  unsigned long long range_hits = 0;
-  UFC_CUDA(c, cudaMemcpyAsync(hp.data(), part, hp.size() * 8, cudaMemcpyDeviceToHost, c->stream));
-  UFC_CUDA(c, cudaMemcpyAsync(&range_hits, &bc->range, 8, cudaMemcpyDeviceToHost, c->stream));
+  double hp[4 * kMaxShells + 5];
+  UFC_CUDA(c, cudaMemcpyAsync(hp, dout, nout * 8, cudaMemcpyDeviceToHost, c->stream));
   UFC_CUDA(c, cudaStreamSynchronize(c->stream));
-  if (range_hits)
+  if (hp[4 * S + 4] != 0.0)
     return set_err(c, UFC_ERR_UNSUPPORTED,
                    "adjoint needs |kappa_p| < 2^14 and |g_p| < 2^14 (fixed-point range)");
-  for (int k = 0; k < 4 * S + 4; ++k) out[k] = 0.0;
-  for (int i = 0; i < grid2; ++i) {        // blocks in order: a fixed summation order
-    const double* r = hp.data() + (size_t)i * 4 * S;
-    for (int k = 0; k < 4 * S; ++k) out[k] += r[k];
-  }
-  for (int i = 0; i < grid2; ++i) {
-    const double* r = hp.data() + nrow + 4 * (size_t)i;
-    for (int k = 0; k < 4; ++k) out[4 * S + k] += r[k];
-  }
+  std::memcpy(out, hp, (4 * (size_t)S + 4) * 8);
   return UFC_OK;
 }
 
