@@ -71,6 +71,7 @@ struct WarpChunk {
   int32_t fill;
   bool fits;      // the whole chunk lies below the capacity (always, with the
                   // workspace's sizes; a chunk that did not would be dropped)
+  int32_t lim;    // 32 keys fit and leave the chunk open while fill < lim (0: none)
 };
 
 __device__ __forceinline__ uint32_t dense_key(int32_t key, int32_t npix, const KeyOut& o) {
@@ -89,7 +90,7 @@ __device__ __forceinline__ void dense_append(WarpChunk& wc, bool want, uint32_t 
   int lane = threadIdx.x & 31;
   // every lane has a key and the chunk stays open (most calls of the pixel
   // stage): no ranks
-  if (m == full && wc.base >= 0 && wc.fits && wc.fill < kChunk - 32) {
+  if (m == full && wc.fill < wc.lim) {
     o.dense[wc.base + (wc.fill + lane)] = v;
     wc.fill += 32;
     return;
@@ -103,6 +104,7 @@ __device__ __forceinline__ void dense_append(WarpChunk& wc, bool want, uint32_t 
     wc.base = (int64_t)__shfl_sync(full, b, 0);
     wc.fill = 0;
     wc.fits = wc.base + kChunk <= o.dense_cap;
+    wc.lim = wc.fits ? kChunk - 32 : 0;
   }
   int room = kChunk - wc.fill;
   if (want && rank < room && wc.fits) o.dense[wc.base + (wc.fill + rank)] = v;
@@ -114,6 +116,7 @@ __device__ __forceinline__ void dense_append(WarpChunk& wc, bool want, uint32_t 
     if (want && rank >= room && nfits) o.dense[nb + (rank - room)] = v;
     wc.base = nb;
     wc.fits = nfits;
+    wc.lim = nfits ? kChunk - 32 : 0;
     wc.fill = cnt - room;
   } else {
     wc.fill += cnt;
@@ -323,6 +326,7 @@ __device__ __forceinline__ void fast_particle(bool have, float x, float y, float
   fc.n_keyed += key >= 0;
 }
 
+template <bool LUT>
 __device__ __forceinline__ void fast_init_shared(FastShared& fs, const BoxGeom& bg,
                                                  const ShellTable& st, const uint16_t* lut) {
   if (threadIdx.x < 3) {
@@ -337,9 +341,11 @@ __device__ __forceinline__ void fast_init_shared(FastShared& fs, const BoxGeom& 
     fs.lo2[st.nshell + 1] = INFINITY;
     fs.hi2[st.nshell + 1] = INFINITY;
   }
-  const uint4* src = reinterpret_cast<const uint4*>(lut);
-  uint4* dst = reinterpret_cast<uint4*>(fs.lut);
-  for (int i = threadIdx.x; i < kLut / 8; i += blockDim.x) dst[i] = src[i];
+  if (LUT) {
+    const uint4* src = reinterpret_cast<const uint4*>(lut);
+    uint4* dst = reinterpret_cast<uint4*>(fs.lut);
+    for (int i = threadIdx.x; i < kLut / 8; i += blockDim.x) dst[i] = src[i];
+  }
 }
 
 template <int MODE>
@@ -367,7 +373,7 @@ k_fast(const float* __restrict__ xyz, int64_t n, int64_t p_off, int32_t box_id, 
        int32_t npix, KeyOut o, Queues qs) {
   extern __shared__ uint32_t hist_s[];
   __shared__ FastShared fs;
-  fast_init_shared(fs, bg, st, tab->lut);
+  fast_init_shared<true>(fs, bg, st, tab->lut);
   if (MODE == kModeDense && o.smem_hist)
     for (int i = threadIdx.x; i < o.nbuckets; i += blockDim.x) hist_s[i] = 0;
   __syncthreads();
@@ -463,11 +469,11 @@ __device__ __noinline__ int32_t key_exact_slow(const ShellTable& st, int32_t lo,
 // every chunk and works through it alone, 32 particles at a time:
 //   A: radius, shell (lookup table) and zone; the belt and cap particles are
 //      appended, with their FP32 observer-relative coordinates, to two
-//      circular pending lists of the warp in shared memory (ballots);
+//      pending lists of the warp in shared memory (ballots);
 //   B: whenever a list holds 32 entries, the warp computes their pixels
-//      together, so the pixel code always runs on full warps; keys go to the
-//      dense array through the warp's chunk, bucket counts to 16-bit shared
-//      counters (an overflow at 65536 is carried to the global histogram).
+//      together (the newest 32), so the pixel code always runs on full warps; keys
+//      go to the dense array through the warp's chunk, bucket counts to 16-bit
+//      shared counters (a count that reaches 32768 is moved to the global histogram).
 // A stage is free once every warp has finished A on it (the entries hold
 // copies); the last warp to finish issues the copy that refills it, so the
 // steady state has no block-wide barrier.  The lists carry over from chunk to
@@ -475,6 +481,12 @@ __device__ __noinline__ int32_t key_exact_slow(const ShellTable& st, int32_t lo,
 // number modulo 4096, and the lists are drained at least every kWAgeFlush
 // chunks.  Particle p of the launch is
 // element p_off + p of the caller's array (chunked launches of ufc_bin_host).
+//
+// Bound by instruction issue: 6.4 warp instructions per particle (per lane: 204) in a box half of
+// whose particles are keyed, 75% of the issue slots (ALU pipe 58%, FMA 28%, DRAM 25%);
+// two boxes of 512^3 particles at Nside 512 take 1.61 ms (1.80 with circular lists, a table
+// of shell bounds with range tests after it, and the image loop of the periodic path).  Of a
+// box's time about 0.42 are classification and streaming, the rest pixels and emission.
 constexpr int kWThreads = 768;
 constexpr int kWChunk = 3840;                  // particles per chunk (45 KB)
 constexpr int kWStages = 2;                    // the stage index of the ring loop is k & 1
@@ -490,20 +502,41 @@ static_assert(kWAgeFlush < 4096, "chunk tags are 12-bit");
 
 constexpr int kWSmemBase = kWStages * kWChunk * 12 + kWWarps * 2 * kWList * 16;   // ring + lists
 
-// One increment of a 16-bit counter held in half of a 32-bit word; true when it wrapped the
-// half, which hist16_carry then settles (the low half's carry undone, 65536 added globally).
+// One increment of a 16-bit counter held in half of a 32-bit word; true when it reached
+// 32768, which hist16_carry then moves to the global count (the other half of the range
+// holds what other warps add before that).
 __device__ __forceinline__ bool hist16_add(uint32_t* h32, uint32_t bucket) {
-  const uint32_t shift = (bucket & 1u) << 4;
-  const uint32_t old = atomicAdd(h32 + (bucket >> 1), 1u << shift);
-  return ((old >> shift) & 0xFFFFu) == 0xFFFFu;
+  const uint32_t inc = (bucket & 1u) ? 0x10000u : 1u;
+  const uint32_t old = atomicAdd(h32 + (bucket >> 1), inc);
+  return ((old + inc) & ~old & 0x80008000u) != 0u;
 }
 
 __device__ __forceinline__ void hist16_carry(uint32_t* h32, uint32_t* ghist, uint32_t bucket) {
-  if ((bucket & 1u) == 0u) atomicSub(h32 + (bucket >> 1), 1u << 16);
-  atomicAdd(ghist + bucket, 65536u);
+  atomicSub(h32 + (bucket >> 1), 0x8000u << ((bucket & 1u) << 4));
+  atomicAdd(ghist + bucket, 32768u);
 }
 
-template <int MODE>
+// The lookup table as the kernel below wants it: the shell itself where a bin lies in one
+// of the box's shells for certain, kLutOut where it is outside for certain, and the flag
+// kLutScan (any lower bound of the edge in the low bits, plus 1) where the edges have to be
+// scanned and for the bins of radii below the near guard.
+constexpr uint32_t kLutOut = 0x4000u;
+__device__ __forceinline__ void fill_lut_classified(uint16_t* lut, const uint16_t* src,
+                                                    int near_bin, int lo, int hi) {
+  auto conv = [&](uint32_t e, int bin) -> uint32_t {
+    if ((e & kLutScan) || bin <= near_bin) return e | kLutScan;
+    const int a = int(e) - 1;
+    return a >= lo && a < hi ? uint32_t(a) : kLutOut;
+  };
+  const uint32_t* s2 = reinterpret_cast<const uint32_t*>(src);
+  uint32_t* d2 = reinterpret_cast<uint32_t*>(lut);
+  for (int i = threadIdx.x; i < kLut / 2; i += blockDim.x) {
+    const uint32_t w = s2[i];
+    d2[i] = conv(w & 0xFFFFu, 2 * i) | conv(w >> 16, 2 * i + 1) << 16;
+  }
+}
+
+template <int MODE, bool SH>
 __global__ void __launch_bounds__(kWThreads, 1)
 k_fast_tma(const float* __restrict__ xyz, int64_t n, int64_t p_off, int32_t box_id, BoxGeom bg,
            ShellTable st, const BinTables* __restrict__ tab, float lut_scale, Bands bd, int32_t N,
@@ -516,9 +549,15 @@ k_fast_tma(const float* __restrict__ xyz, int64_t n, int64_t p_off, int32_t box_
   __shared__ __align__(8) uint64_t bar[kWStages];
   __shared__ int done_s[kWStages];
   __shared__ int abort_s;
-  fast_init_shared(fs, bg, st, tab->lut);
+  const int lo = bg.shell_lo, hi = bg.shell_hi;
+  // bin of a squared radius: the nearest integer to v, exact
+  auto lut_bin = [&](float r2) {
+    return __float_as_int(fminf(r2 * lut_scale, float(kLut - 1)) + 8388608.0f) - 0x4B000000;
+  };
+  fast_init_shared<false>(fs, bg, st, tab->lut);
+  fill_lut_classified(fs.lut, tab->lut, lut_bin(bd.r2_min), lo, hi);
   const int nwords = (o.nbuckets + 1) >> 1;
-  if (MODE == kModeDense && o.smem_hist)
+  if (SH)
     for (int i = threadIdx.x; i < nwords; i += blockDim.x) h32[i] = 0u;
   if (threadIdx.x == 0) {
     for (int s = 0; s < kWStages; ++s) {
@@ -530,9 +569,6 @@ k_fast_tma(const float* __restrict__ xyz, int64_t n, int64_t p_off, int32_t box_
   }
   __syncthreads();
 
-  const int lo = bg.shell_lo, hi = bg.shell_hi;
-  const int n1 = 2 * bg.R + 1;
-  const bool carry = bg.nimg == 1;             // (always: see the loop over images)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const unsigned lt_mask = (1u << lane) - 1u;
   float4* list_eq = lists + (2 * warp) * kWList;
@@ -560,8 +596,8 @@ k_fast_tma(const float* __restrict__ xyz, int64_t n, int64_t p_off, int32_t box_
 
   FastCtx fc{{-1, 0}, {-1, 0}, 0, 0};
   uint32_t* ghist = o.hist;
-  int he = 0, ne = 0, hc = 0, nc = 0;          // heads and lengths of the two lists
-  int ii = 0, jj = 0, kk = 0;                  // current image
+  uint32_t n_keyed = 0;                        // the warp's keys of stage B
+  int ne = 0, nc = 0;                          // lengths of the two lists
   bool aborted = false;
   int64_t k = 0;
   const float sx = fs.shf[0], sy = fs.shf[1], sz = fs.shf[2];
@@ -582,98 +618,82 @@ k_fast_tma(const float* __restrict__ xyz, int64_t n, int64_t p_off, int32_t box_
     const bool fullc = cq < nfull;
     const int nvalid = last ? 0 : (fullc ? kWChunk : tail_n);
     const int nsmem = fullc ? kWChunk : tail_smem;      // particles inside the bulk copy
-    const float* buf = ring + s * 3 * kWChunk;
-    const uint32_t kqtag = uint32_t(kq & 4095) << 20;
-    const int nimg = last ? 1 : bg.nimg;
-    const bool drain_all = last || !carry || ((k & (kWAgeFlush - 1)) == kWAgeFlush - 1);
+    const bool drain_all = last || (k & (kWAgeFlush - 1)) == kWAgeFlush - 1;
     const int ng = last ? 0 : kWGroups;                  // groups of 32 particles to classify
     const int nsteps = ng + (drain_all ? 1 : 0);         // + a drain step
-    ii = jj = kk = 0;
-    // (one pass: boxes with periodic images take the direct path.  The loop
-    // over images and the drain after each stay because the code the compiler
-    // makes without them is slower, k_fast of two boxes of 512^3: 2.02 ms
-    // without either, 1.87 ms without the drain, 1.80 ms with both)
+    const int j0 = warp * kWPerWarp + lane;
+    const float* buf = ring + s * 3 * kWChunk + 3 * j0;
+    uint32_t tag = uint32_t(kq & 4095) << 20 | uint32_t(j0) << 8;   // chunk, offset in it
+    const uint64_t qbase = qpack(box_id, 0, p_off + base);   // + offset in the chunk
 #pragma unroll 1
-    for (int img = 0; img < nimg; ++img) {
-      if (img) {
-        if (++kk == n1) { kk = 0; if (++jj == n1) { jj = 0; ++ii; } }
-      }
-      const uint64_t qbase = qpack(box_id, img, p_off + base);   // + offset in the chunk
-#pragma unroll 1
-      for (int h = 0; h < nsteps; ++h) {
-        if (h < ng) {
-          // ---- A: classify 32 particles of this warp's slice
-          const int j = warp * kWPerWarp + 32 * h + lane;
-          bool have;
-          float x, y, zc;
-          if (fullc) {                           // every particle inside the bulk copy
-            have = true;
-            x = buf[3 * j];
-            y = buf[3 * j + 1];
-            zc = buf[3 * j + 2];
-          } else {
-            have = j < nvalid;
-            x = 0.f; y = 0.f; zc = 0.f;
-            if (j < nsmem) {
-              x = buf[3 * j];
-              y = buf[3 * j + 1];
-              zc = buf[3 * j + 2];
-            } else if (have) {                   // ragged tail outside the bulk copy
-              x = __ldg(xyz + 3 * (base + j));
-              y = __ldg(xyz + 3 * (base + j) + 1);
-              zc = __ldg(xyz + 3 * (base + j) + 2);
-            }
+    for (int h = 0; h < nsteps; ++h, buf += 96, tag += 32u << 8) {
+      if (h < ng) {
+        // ---- A: classify 32 particles of this warp's slice
+        const int j = j0 + 32 * h;
+        float x, y, zc;
+        if (fullc) {                             // every particle inside the bulk copy
+          x = buf[0];
+          y = buf[1];
+          zc = buf[2];
+        } else {
+          x = INFINITY; y = 0.f; zc = 0.f;       // no particle: sorted out with the scans
+          if (j < nsmem) {
+            x = buf[0];
+            y = buf[1];
+            zc = buf[2];
+          } else if (j < nvalid) {               // ragged tail outside the bulk copy
+            x = __ldg(xyz + 3 * (base + j));
+            y = __ldg(xyz + 3 * (base + j) + 1);
+            zc = __ldg(xyz + 3 * (base + j) + 2);
           }
-          const float dx = (x + sx) + lx;
-          const float dy = (y + sy) + ly;
-          const float dz = (zc + sz) + lz;
-          const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
-          // classification without branches but for the rare edge scan:
-          // outside, undecided (c1), belt (c2) or cap (c3)
-          const bool fin = r2 <= 3.0e38f;                // false for NaN and overflow
-          const bool near = !(r2 >= bd.r2_min);          // near the observer (r == 0 is invalid)
-          const float v = fminf(r2 * lut_scale, float(kLut - 1));
-          const int bin = __float_as_int(v + 8388608.0f) - 0x4B000000;
-          const uint32_t e = fs.lut[bin];
-          int a = int(e & 0x7FFFu) - 1;
-          bool band = false;
-          // rare: scan the edges (finite r2 ends at +inf); a warp-uniform
-          // test first, so that the common case is one vote and a branch
-          if (__any_sync(0xFFFFFFFFu, (e & kLutScan) && fin)) {
-            if ((e & kLutScan) && fin) {
+        }
+        const float dx = (x + sx) + lx;
+        const float dy = (y + sy) + ly;
+        const float dz = (zc + sz) + lz;
+        const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
+        // outside, undecided (c1), belt (c2) or cap (c3): the table's entry decides the shell
+        // but for the bins that hold an edge or the near guard, and for a NaN or an overflow
+        // (one vote and a branch for these)
+        uint32_t a = fs.lut[lut_bin(r2)];
+        bool in = a < kLutOut, und = false;
+        const bool fin = r2 <= 3.0e38f;                  // false for NaN and overflow
+        const bool scan = a >= kLutScan || !fin;
+        if (__any_sync(0xFFFFFFFFu, scan)) {
+          if (scan) {
+            // NaN or overflowing r2 goes to the queue as well: the FP64 stage returns the
+            // invalid key for non-finite coordinates and decides a finite overflow
+            in = false;
+            und = j < nvalid && (!fin || !(r2 >= bd.r2_min));   // (near the observer: r == 0 is invalid)
+            if (fin && !und) {
+              int e = int(a & 0x7FFFu) - 1;              // ends at the +inf sentinel
               for (;;) {
-                if (r2 < fs.lo2[a + 1]) break;
-                if (r2 < fs.hi2[a + 1]) { band = true; break; }
-                ++a;
+                if (r2 < fs.lo2[e + 1]) break;
+                if (r2 < fs.hi2[e + 1]) { und = true; break; }
+                ++e;
               }
+              in = !und && e >= lo && e < hi;
+              a = uint32_t(e);
             }
           }
-          const bool inshell = uint32_t(a - lo) < uint32_t(hi - lo);
-          const float dz2 = dz * dz;
-          const bool eqz = dz2 <= bd.z_eq2 * r2;
-          const bool capz = dz2 > bd.z_cap2 * r2;
-          const bool dec = have && fin && !near && !band && inshell;
-          const bool c2 = dec && eqz;
-          const bool c3 = dec && capz;
-          // NaN or overflowing r2 (rare) goes to the queue as well: the FP64
-          // stage returns the invalid key for non-finite coordinates and
-          // decides a finite overflow
-          const bool c1 = have && (fin ? (near || band || (inshell && !eqz && !capz)) : true);
-          const uint32_t meta = uint32_t(a & 255) | (uint32_t(j) << 8) | kqtag;
-          const float4 ent = make_float4(dx, dy, dz, __uint_as_float(meta));
-          const unsigned meq = __ballot_sync(0xFFFFFFFFu, c2);
-          const unsigned mcap = __ballot_sync(0xFFFFFFFFu, c3);
-          if (c2) list_eq[(he + ne + __popc(meq & lt_mask)) & (kWList - 1)] = ent;
-          if (c3) list_cap[(hc + nc + __popc(mcap & lt_mask)) & (kWList - 1)] = ent;
-          ne += __popc(meq);
-          nc += __popc(mcap);
-          // undecided images wait in queue 1; outside/invalid are final
-          bool pushed = true;                    // (a warp-uniform test first, as above)
-          if (__any_sync(0xFFFFFFFFu, c1))
-            pushed = queue_push(fc.qc, c1, qbase + uint64_t(j), qs.q1, qs.cap1, &qs.cnt->q1);
+        }
+        const float dz2 = dz * dz;
+        const bool c2 = in && dz2 <= bd.z_eq2 * r2;
+        const bool c3 = in && dz2 > bd.z_cap2 * r2;
+        const bool c1 = und || (in && !c2 && !c3);
+        const float4 ent = make_float4(dx, dy, dz, __uint_as_float(tag | a));
+        const unsigned meq = __ballot_sync(0xFFFFFFFFu, c2);
+        const unsigned mcap = __ballot_sync(0xFFFFFFFFu, c3);
+        if (c2) list_eq[ne + __popc(meq & lt_mask)] = ent;
+        if (c3) list_cap[nc + __popc(mcap & lt_mask)] = ent;
+        ne += __popc(meq);
+        nc += __popc(mcap);
+        // undecided images wait in queue 1; outside/invalid are final
+        bool pushed = true;                      // (a warp-uniform test first, as above)
+        if (__any_sync(0xFFFFFFFFu, c1)) {
+          pushed = queue_push(fc.qc, c1, qbase + uint64_t(j), qs.q1, qs.cap1, &qs.cnt->q1);
           if (!pushed) {
-            const int32_t kx = key_exact_slow(st, lo, hi, N, npix, x, y, zc, bg.sh64[0][ii],
-                                              bg.sh64[1][jj], bg.sh64[2][kk]);
+            const int32_t kx = key_exact_slow(st, lo, hi, N, npix, x, y, zc, bg.sh64[0][0],
+                                              bg.sh64[1][0], bg.sh64[2][0]);
             if (kx == kKeyInvalid) ++fc.n_invalid;
             if (kx >= 0) {
               ++fc.n_keyed;
@@ -684,78 +704,66 @@ k_fast_tma(const float* __restrict__ xyz, int64_t n, int64_t p_off, int32_t box_
                 if ((int64_t)at < o.dense_cap) o.dense[at] = dk;
               }
             }
-            if (MODE == kModeKeys && have) o.keys[p_off + base + j] = kx;
-          } else if (MODE == kModeKeys && have && !c2 && !c3) {
-            o.keys[p_off + base + j] = c1 ? kKeyUndecided
-                : ((!fin && !(isfinite(x) && isfinite(y) && isfinite(zc))) ? kKeyInvalid : kKeyOutside);
+            if (MODE == kModeKeys) o.keys[p_off + base + j] = kx;
           }
         }
-        __syncwarp();
-        // ---- B: pixels of full groups of 32 pending entries (in the drain
-        // step, also of the partial rest)
-        const bool tail = h == ng;
-        // one instantiation per zone, so that a group runs only its zone's
-        // pixel code
-        auto group_b = [&](auto zone_tag, int take) {
-          constexpr int ZONE = decltype(zone_tag)::value;
-          const float4* L = ZONE == 0 ? list_eq : list_cap;
-          const int head = ZONE == 0 ? he : hc;
-          const bool have = lane < take;
-          float4 ent = make_float4(0.f, 0.f, 0.f, 0.f);
-          if (have) ent = L[(head + lane) & (kWList - 1)];
-          if constexpr (ZONE == 0) { he = (he + take) & (kWList - 1); ne -= take; }
-          else { hc = (hc + take) & (kWList - 1); nc -= take; }
-          const float dx = ent.x, dy = ent.y, dz = ent.z;
-          const uint32_t meta = __float_as_uint(ent.w);
-          const int b = int(meta & 255u);
-          const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
-          const float rinv = rsqrt_fast(r2);
-          const float z = dz * rinv;
-          int32_t pix = kKeyUndecided;
-          if (have) {
-            if constexpr (ZONE == 0) pix = pixel_fast_eq(N, bd, dx, dy, z);
-            else pix = pixel_fast_cap(N, bd, dx, dy, dz, r2, rinv, z);
-          }
-          const bool ok = have && pix != kKeyUndecided;
-          // the entry's particle (launch-local index pl): chunk from the
-          // 12-bit tag, offset in the chunk; computed only where needed
-          auto local_index = [&]() -> int64_t {
-            const int64_t ke = kq - ((kq - int64_t(meta >> 20)) & 4095);
-            return (blockIdx.x + ke * gridDim.x) * kWChunk + int64_t((meta >> 8) & 4095u);
-          };
-          const int32_t key = b * npix + pix;
-          if (__any_sync(0xFFFFFFFFu, have && !ok)) {   // rare: a warp-uniform test first
-            // queue full: left to the exact pass
-            queue_push_mark(
-                fc.qc, have && !ok, [&]() { return qpack(box_id, 0, p_off + local_index()); },
-                qs.q1, qs.cap1, &qs.cnt->q1, qs.ovf, qs.ovf_base, &qs.cnt->ovf);
-          }
-          if (MODE == kModeKeys) {
-            if (have) o.keys[p_off + local_index()] = ok ? key : kKeyUndecided;
-          } else {
-            uint32_t dk = 0u, bucket = 0u;
-            bool wrapped = false;
-            if (ok) {
-              const uint32_t blk = uint32_t(pix >> 13) / 3u;       // pix / 24576
-              bucket = uint32_t(b - o.shell0) * uint32_t(o.nblk) + blk;
-              dk = (bucket << kOffBits) | (uint32_t(pix) - blk * uint32_t(kBlockPix));
-              if (UFC_IDX_OK(bucket, o.nbuckets, 1)) {
-                if (o.smem_hist) wrapped = hist16_add(h32, bucket);
-                else atomicAdd(ghist + bucket, 1u);
-              }
-            }
-            // rare (one increment in 65536 per counter): a warp-uniform test first
-            if (__any_sync(0xFFFFFFFFu, wrapped) && wrapped) hist16_carry(h32, ghist, bucket);
-            dense_append(fc.wc, ok, dk, o);
-          }
-          fc.n_keyed += ok;
-        };
-        const int take_e = ne >= 32 ? 32 : ((tail && drain_all) ? ne : 0);
-        if (take_e) group_b(std::integral_constant<int, 0>{}, take_e);
-        const int take_c = nc >= 32 ? 32 : ((tail && drain_all) ? nc : 0);
-        if (take_c) group_b(std::integral_constant<int, 1>{}, take_c);
-        __syncwarp();
+        if (MODE == kModeKeys && pushed && j < nvalid && !c2 && !c3)
+          o.keys[p_off + base + j] = c1 ? kKeyUndecided : kKeyOutside;
       }
+      __syncwarp();
+      // ---- B: pixels of full groups of 32 pending entries, the newest first (in the drain
+      // step, also of the partial rest); one instantiation per zone, so that a group runs
+      // only its zone's pixel code
+      auto group_b = [&](auto zone_tag, int& len) {
+        constexpr int ZONE = decltype(zone_tag)::value;
+        const int take = min(len, 32);
+        len -= take;
+        const bool have = lane < take;           // (a lane without one reads an old entry)
+        const float4 ent = (ZONE == 0 ? list_eq : list_cap)[len + lane];
+        const float dx = ent.x, dy = ent.y, dz = ent.z;
+        const uint32_t meta = __float_as_uint(ent.w);
+        const int b = int(meta & 255u);
+        const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
+        const float rinv = rsqrt_fast(r2);
+        const float z = dz * rinv;
+        int32_t pix;
+        if constexpr (ZONE == 0) pix = pixel_fast_eq(N, bd, dx, dy, z);
+        else pix = pixel_fast_cap(N, bd, dx, dy, dz, r2, rinv, z);
+        const bool ok = have && pix != kKeyUndecided;
+        // the entry's particle (launch-local index pl): chunk from the
+        // 12-bit tag, offset in the chunk; computed only where needed
+        auto local_index = [&]() -> int64_t {
+          const int64_t ke = kq - ((kq - int64_t(meta >> 20)) & 4095);
+          return (blockIdx.x + ke * gridDim.x) * kWChunk + int64_t((meta >> 8) & 4095u);
+        };
+        const unsigned m = __ballot_sync(0xFFFFFFFFu, ok);
+        n_keyed += __popc(m);
+        if (m != 0xFFFFFFFFu) {                  // rare: a warp-uniform test first
+          // queue full: left to the exact pass
+          queue_push_mark(
+              fc.qc, have && !ok, [&]() { return qpack(box_id, 0, p_off + local_index()); },
+              qs.q1, qs.cap1, &qs.cnt->q1, qs.ovf, qs.ovf_base, &qs.cnt->ovf);
+        }
+        if (MODE == kModeKeys) {
+          if (have) o.keys[p_off + local_index()] = ok ? b * npix + pix : kKeyUndecided;
+        } else {
+          const uint32_t blk = uint32_t(pix >> 13) / 3u;         // pix / 24576
+          const uint32_t bucket = uint32_t(b - o.shell0) * uint32_t(o.nblk) + blk;
+          const uint32_t dk = (bucket << kOffBits) | (uint32_t(pix) - blk * uint32_t(kBlockPix));
+          bool wrapped = false;
+          if (ok && UFC_IDX_OK(bucket, o.nbuckets, 1)) {
+            if (SH) wrapped = hist16_add(h32, bucket);
+            else atomicAdd(ghist + bucket, 1u);
+          }
+          // rare (one increment in 32768 per counter): a warp-uniform test first
+          if (SH && __any_sync(0xFFFFFFFFu, wrapped) && wrapped) hist16_carry(h32, ghist, bucket);
+          dense_append(fc.wc, ok, dk, o);
+        }
+      };
+      const int need = h < ng ? 32 : 1;
+      if (ne >= need) group_b(std::integral_constant<int, 0>{}, ne);
+      if (nc >= need) group_b(std::integral_constant<int, 1>{}, nc);
+      __syncwarp();
     }
     if (last) break;
     // this warp is done with stage s; the last warp refills it
@@ -782,12 +790,12 @@ k_fast_tma(const float* __restrict__ xyz, int64_t n, int64_t p_off, int32_t box_
   // ---- end: close the warp's chunks, counters, bucket counts
   if (MODE == kModeDense) dense_close(fc.wc, o);
   queue_close(fc.qc, qs.q1, qs.cap1);
-  const unsigned long long ni = warp_sum(fc.n_invalid), nk = warp_sum(fc.n_keyed);
+  const unsigned long long ni = warp_sum(fc.n_invalid), nk = warp_sum(fc.n_keyed) + n_keyed;
   if (lane == 0) {
     if (ni) atomicAdd(&qs.cnt->invalid, ni);
     if (nk) atomicAdd(&qs.cnt->keyed, nk);
   }
-  if (MODE == kModeDense && o.smem_hist) {
+  if (SH) {
     __syncthreads();
     for (int i = threadIdx.x; i < o.nbuckets; i += blockDim.x) {
       const uint32_t v = (h32[i >> 1] >> ((i & 1) << 4)) & 0xFFFFu;
@@ -1767,13 +1775,14 @@ ufc_status run_keys_pipeline(ufc_ctx* c, int mode_req, const float* const* xyz,
       ProfScope ps_(c, "k_fast");
       if (tma) {
         qs.ovf_base = bp.bit_base[k];
-#define UFC_LAUNCH_TMA(M)                                                                        \
-  UFC_CUDA(c, cudaFuncSetAttribute(k_fast_tma<M>, cudaFuncAttributeMaxDynamicSharedMemorySize,    \
-                                   tma_smem));                                                   \
-  k_fast_tma<M><<<c->num_sms, kWThreads, tma_smem, c->stream>>>(                                 \
+#define UFC_LAUNCH_TMA(...)                                                                      \
+  UFC_CUDA(c, cudaFuncSetAttribute(k_fast_tma<__VA_ARGS__>,                                      \
+                                   cudaFuncAttributeMaxDynamicSharedMemorySize, tma_smem));      \
+  k_fast_tma<__VA_ARGS__><<<c->num_sms, kWThreads, tma_smem, c->stream>>>(                                 \
       src, cnt, p0, k, bp.box[k], st, tab, lut_scale, bd, nside, (int32_t)npix, o, qs)
-        if (plan.mode == kModeDense) { UFC_LAUNCH_TMA(kModeDense); }
-        else { UFC_LAUNCH_TMA(kModeKeys); }
+        if (plan.mode == kModeDense && plan.smem_hist) { UFC_LAUNCH_TMA(kModeDense, true); }
+        else if (plan.mode == kModeDense) { UFC_LAUNCH_TMA(kModeDense, false); }
+        else { UFC_LAUNCH_TMA(kModeKeys, false); }
 #undef UFC_LAUNCH_TMA
       } else {
         const int ssm = plan.mode == kModeDense ? smem : 0;

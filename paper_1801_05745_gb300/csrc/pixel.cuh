@@ -181,7 +181,7 @@ __device__ __forceinline__ int32_t floor_certain_d(float w, float dmin, bool& op
   const float n = __fsub_rn(r, kMagic);
   const float d = __fsub_rn(w, n);
   open |= !(fabsf(d) >= dmin);
-  return (__float_as_int(r) - kMagicBits) - (d < 0.0f ? 1 : 0);
+  return (__float_as_int(r) - kMagicBits) + (__float_as_int(d) >> 31);   // (d = -0 is open)
 }
 
 // atan(q) * 2/pi for q in [0, 1] as q * P(q^2), P of degree 8 with
@@ -203,27 +203,28 @@ __device__ __forceinline__ float atanq_poly(float q) {
   return q * p;
 }
 
-// Azimuth of the fast stage: t = base + sgn * a (exact-real identity of the
+// Azimuth of the fast stage: t = base + sa, sa = +-a (exact-real identity of the
 // quadrant/octant cases of the FP64 procedure), a in [0, 1/2] quarter turns.
-struct Azim { float a, sa; int32_t base; bool sgn_pos; };
+struct Azim { float a, sa; int32_t base; uint32_t neg; };
 
 __device__ __forceinline__ Azim azimuth_fast(float dx, float dy, const Bands& bd, bool& open) {
   const float ax = fabsf(dx), ay = fabsf(dy);
   open |= fmaxf(ax, ay) < bd.axy_min;
-  const bool sw = ay > ax;
   const float q = div_fast(fminf(ax, ay), fmaxf(ax, ay));   // one division, either octant
   Azim r;
   r.a = atanq_poly(q);                         // quarter turns, [0, 1/2]
-  const bool xp = dx >= 0.0f, yp = dy >= 0.0f;
-  // (base, sgn): Q0 (0,+)|(1,-)  Q1 (2,-)|(1,+)  Q2 (2,+)|(3,-)  Q3 (4,-)|(3,+),
-  // one nibble (base | sgn << 3) per (xp, yp, sw) in a 32-bit table:
-  // base = xp ? (yp ? (sw ? 1 : 0) : (sw ? 3 : 4)) : (yp ? (sw ? 1 : 2) : (sw ? 3 : 2)),
-  // sgn = (xp == yp) != sw
-  const uint32_t idx = (xp ? 4u : 0u) | (yp ? 2u : 0u) | (sw ? 1u : 0u);
-  const uint32_t nib = (0x18B4923Au >> (4u * idx)) & 15u;
-  r.base = int32_t(nib & 7u);
-  r.sgn_pos = nib >= 8u;
-  r.sa = r.sgn_pos ? r.a : -r.a;
+  // (base, sgn): Q0 (0,+)|(1,-)  Q1 (2,-)|(1,+)  Q2 (2,+)|(3,-)  Q3 (4,-)|(3,+)
+  // from the sign bits of dx, dy and ax - ay: base = 1 in the octants next to the
+  // y axis, else 0 or 2 by dx; mirrored to 4 - base for negative dy; the sign is the
+  // product of the three.  A zero coordinate of either sign gives a = 0: in the belt
+  // the two readings are the same pixel (base 0 and 4 agree modulo 4 N), in a cap
+  // both leave the decision open.
+  const uint32_t ux = __float_as_uint(dx), uy = __float_as_uint(dy);
+  const uint32_t uw = __float_as_uint(ax - ay);
+  r.neg = (ux ^ uy ^ uw) & 0x80000000u;
+  r.sa = __uint_as_float(__float_as_uint(r.a) ^ r.neg);
+  const int32_t b0 = int32_t(uw) < 0 ? 1 : int32_t((ux >> 30) & 2u);
+  r.base = int32_t(uy) < 0 ? 4 - b0 : b0;
   return r;
 }
 
@@ -256,7 +257,7 @@ __device__ __forceinline__ int32_t pixel_fast_cap(int32_t N, const Bands& bd, fl
   const float o3 = 3.0f * omz;
   float tmp = bd.fN * (o3 * rsqrt_fast(o3));
   if (!(o3 > 0.0f)) { tmp = 0.0f; open = true; }
-  const float tp = az.sgn_pos ? az.a : 1.0f - az.a;
+  const float tp = az.neg ? 1.0f - az.a : az.a;
   const int32_t jp = floor_certain_d(tp * tmp, bd.cap_d, open);
   const int32_t jm = floor_certain_d((1.0f - tp) * tmp, bd.cap_d, open);
   int32_t ir = jp + jm + 1;
