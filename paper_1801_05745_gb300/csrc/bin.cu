@@ -69,9 +69,9 @@ struct Queues {
 struct WarpChunk {
   int64_t base;   // start of the warp's current chunk (-1: none)
   int32_t fill;
-  bool fits;      // the whole chunk lies below the capacity (always, with the
-                  // workspace's sizes; a chunk that did not would be dropped)
-  int32_t lim;    // 32 keys fit and leave the chunk open while fill < lim (0: none)
+  int32_t lim;    // 32 keys fit and leave the chunk open while fill < lim; 0: no chunk, or
+                  // one that does not lie below the capacity as a whole and is dropped
+                  // (never, with the workspace's sizes)
 };
 
 __device__ __forceinline__ uint32_t dense_key(int32_t key, int32_t npix, const KeyOut& o) {
@@ -103,11 +103,10 @@ __device__ __forceinline__ void dense_append(WarpChunk& wc, bool want, uint32_t 
     if (lane == 0) b = atomicAdd(o.dense_count, (unsigned long long)kChunk);
     wc.base = (int64_t)__shfl_sync(full, b, 0);
     wc.fill = 0;
-    wc.fits = wc.base + kChunk <= o.dense_cap;
-    wc.lim = wc.fits ? kChunk - 32 : 0;
+    wc.lim = wc.base + kChunk <= o.dense_cap ? kChunk - 32 : 0;
   }
   int room = kChunk - wc.fill;
-  if (want && rank < room && wc.fits) o.dense[wc.base + (wc.fill + rank)] = v;
+  if (want && rank < room && wc.lim) o.dense[wc.base + (wc.fill + rank)] = v;
   if (cnt >= room) {
     unsigned long long b = 0;
     if (lane == 0) b = atomicAdd(o.dense_count, (unsigned long long)kChunk);
@@ -115,7 +114,6 @@ __device__ __forceinline__ void dense_append(WarpChunk& wc, bool want, uint32_t 
     const bool nfits = nb + kChunk <= o.dense_cap;
     if (want && rank >= room && nfits) o.dense[nb + (rank - room)] = v;
     wc.base = nb;
-    wc.fits = nfits;
     wc.lim = nfits ? kChunk - 32 : 0;
     wc.fill = cnt - room;
   } else {
@@ -266,7 +264,7 @@ __device__ __forceinline__ int32_t shell_lut(const FastShared& fs, int32_t lo, i
 struct FastCtx {
   WarpChunk wc;
   QChunk qc;
-  unsigned long long n_invalid, n_keyed;
+  uint32_t n_invalid, n_keyed;   // of one lane in one launch
 };
 
 // One particle (warp-collective: every lane calls it).
@@ -463,44 +461,54 @@ __device__ __noinline__ int32_t key_exact_slow(const ShellTable& st, int32_t lo,
   return key_exact(st, lo, hi, N, npix, x, y, zc, shx, shy, shz);
 }
 
-// Fast stage fed by bulk copies, warp-autonomous.  Persistent blocks; a ring
-// of kWStages chunks of kWChunk particles streams in by cp.async.bulk
-// (16-byte aligned xyz).  Each warp owns a slice of kWPerWarp particles of
-// every chunk and works through it alone, 32 particles at a time:
-//   A: radius, shell (lookup table) and zone; the belt and cap particles are
-//      appended, with their FP32 observer-relative coordinates, to two
-//      pending lists of the warp in shared memory (ballots);
-//   B: whenever a list holds 32 entries, the warp computes their pixels
-//      together (the newest 32), so the pixel code always runs on full warps; keys
-//      go to the dense array through the warp's chunk, bucket counts to 16-bit
-//      shared counters (a count that reaches 32768 is moved to the global histogram).
-// A stage is free once every warp has finished A on it (the entries hold
-// copies); the last warp to finish issues the copy that refills it, so the
-// steady state has no block-wide barrier.  The lists carry over from chunk to
-// chunk; an entry keeps its offset in its chunk and the chunk's sequence
-// number modulo 4096, and the lists are drained at least every kWAgeFlush
-// chunks.  Particle p of the launch is
-// element p_off + p of the caller's array (chunked launches of ufc_bin_host).
+// Fast stage fed by asynchronous copies, warp-autonomous.  Persistent blocks; every warp
+// streams its own pieces of kWPiece particles (16-byte aligned xyz) through kWStages slots of
+// shared memory with cp.async, so no warp waits for another, and works through a piece 32
+// particles at a time:
+//   A: radius, shell (lookup table) and zone; the belt and cap particles are appended, with
+//      their FP32 observer-relative coordinates, to two pending lists of the warp in shared
+//      memory (ballots);
+//   B: whenever a list holds 32 entries, the warp computes the pixels of the newest 32
+//      together, so the pixel code always runs on full warps; keys go to the dense array
+//      through the warp's chunk, bucket counts to 16-bit shared counters (a count that
+//      reaches 32768 is moved to the global histogram).
+// The lists carry over from piece to piece; an entry keeps its offset in its piece and the
+// piece's sequence number modulo 2^17, and the lists are drained at least every 2^16 pieces.
+// Particle p of the launch is element p_off + p of the caller's array (chunked launches of
+// ufc_bin_host).
 //
-// Bound by instruction issue: 6.4 warp instructions per particle (per lane: 204) in a box half of
-// whose particles are keyed, 75% of the issue slots (ALU pipe 58%, FMA 28%, DRAM 25%);
-// two boxes of 512^3 particles at Nside 512 take 1.61 ms (1.80 with circular lists, a table
-// of shell bounds with range tests after it, and the image loop of the periodic path).  Of a
-// box's time about 0.42 are classification and streaming, the rest pixels and emission.
+// Bound by instruction issue: about 6.3 warp instructions per particle in a box half of whose
+// particles are keyed, three quarters of the issue slots (ALU pipe 58%, FMA 28%, DRAM 25%).
+// Two boxes of 512^3 particles at Nside 512 take 1.57 ms; 1.61 when the block shared bulk
+// copies of 3840 particles behind mbarriers (ring bookkeeping per chunk), 1.80 with circular
+// lists, range tests on the shell after the table and the periodic path's image loop as well.
+// Of a box whose particles are all keyed, 0.4 of the time is classification and streaming.
+// Other shapes: 4 slots per warp 1.64 ms, 640 threads 1.71, 800 threads (spills) 1.73.
 constexpr int kWThreads = 768;
-constexpr int kWChunk = 3840;                  // particles per chunk (45 KB)
-constexpr int kWStages = 2;                    // the stage index of the ring loop is k & 1
-static_assert(kWStages == 2, "the ring loop takes the stage of chunk k as k & 1");
 constexpr int kWWarps = kWThreads / 32;        // 24
-constexpr int kWPerWarp = kWChunk / kWWarps;   // 160
-constexpr int kWGroups = kWPerWarp / 32;
+constexpr int kWPiece = 128;                   // particles per copy of one warp (1536 bytes)
+constexpr int kWStages = 2;
+constexpr int kWGroups = kWPiece / 32;
 constexpr int kWList = 64;                     // entries of one pending list
-constexpr int kWAgeFlush = 1024;
-static_assert(kWPerWarp % 32 == 0 && kWChunk <= 4096 && kMaxShells <= 256,
-              "entry metadata: 8-bit shell, 12-bit offset, 12-bit chunk tag");
-static_assert(kWAgeFlush < 4096, "chunk tags are 12-bit");
+constexpr int kWTagBits = 17;
+static_assert(kWPiece == 128 && kMaxShells <= 256 && 8 + 7 + kWTagBits == 32,
+              "entry metadata: 8-bit shell, 7-bit offset, 17-bit piece tag");
 
-constexpr int kWSmemBase = kWStages * kWChunk * 12 + kWWarps * 2 * kWList * 16;   // ring + lists
+constexpr int kWSmemBase = kWWarps * (kWStages * kWPiece * 12 + 2 * kWList * 16);   // slots, lists
+
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async4(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
 
 // One increment of a 16-bit counter held in half of a 32-bit word; true when it reached
 // 32768, which hist16_carry then moves to the global count (the other half of the range
@@ -538,17 +546,15 @@ __device__ __forceinline__ void fill_lut_classified(uint16_t* lut, const uint16_
 
 template <int MODE, bool SH>
 __global__ void __launch_bounds__(kWThreads, 1)
-k_fast_tma(const float* __restrict__ xyz, int64_t n, int64_t p_off, int32_t box_id, BoxGeom bg,
+k_fast_stream(const float* __restrict__ xyz, int64_t n, int64_t p_off, int32_t box_id, BoxGeom bg,
            ShellTable st, const BinTables* __restrict__ tab, float lut_scale, Bands bd, int32_t N,
            int32_t npix, KeyOut o, Queues qs) {
   extern __shared__ __align__(128) uint8_t dyn[];
-  float* ring = reinterpret_cast<float*>(dyn);                          // [kWStages][3 kWChunk]
-  float4* lists = reinterpret_cast<float4*>(dyn + kWStages * kWChunk * 12);  // [warps][2][kWList]
+  float* slots = reinterpret_cast<float*>(dyn);           // [warps][kWStages][3 kWPiece]
+  float4* lists = reinterpret_cast<float4*>(dyn + kWWarps * kWStages * kWPiece * 12);
+                                                          // [warps][2][kWList]
   uint32_t* h32 = reinterpret_cast<uint32_t*>(dyn + kWSmemBase);          // 16-bit counters
   __shared__ FastShared fs;
-  __shared__ __align__(8) uint64_t bar[kWStages];
-  __shared__ int done_s[kWStages];
-  __shared__ int abort_s;
   const int lo = bg.shell_lo, hi = bg.shell_hi;
   // bin of a squared radius: the nearest integer to v, exact
   auto lut_bin = [&](float r2) {
@@ -559,94 +565,62 @@ k_fast_tma(const float* __restrict__ xyz, int64_t n, int64_t p_off, int32_t box_
   const int nwords = (o.nbuckets + 1) >> 1;
   if (SH)
     for (int i = threadIdx.x; i < nwords; i += blockDim.x) h32[i] = 0u;
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < kWStages; ++s) {
-      mbar_init(&bar[s], 1);
-      done_s[s] = 0;
-    }
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    abort_s = 0;
-  }
   __syncthreads();
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const unsigned lt_mask = (1u << lane) - 1u;
   float4* list_eq = lists + (2 * warp) * kWList;
   float4* list_cap = list_eq + kWList;
-  const int64_t nchunks = (n + kWChunk - 1) / kWChunk;
-  const int64_t mine = nchunks > blockIdx.x ? (nchunks - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
-  const int64_t nfull = n / kWChunk;                   // chunks of kWChunk particles
-  const int tail_n = int(n - nfull * kWChunk);         // particles of the last, partial chunk
-  const int tail_smem = int(((uint32_t(tail_n) * 12u) & ~15u) / 12u);   // of them inside its copy
-  auto chunk_bytes = [&](int64_t c) -> uint32_t {
-    const int64_t rest = n - c * kWChunk;
-    const int64_t cnt = rest < kWChunk ? rest : (int64_t)kWChunk;
-    return uint32_t((cnt * 12) & ~15ll);       // bulk copies move multiples of 16 bytes
+  float* slot0 = slots + warp * (kWStages * 3 * kWPiece);
+  // the warp's pieces: first, first + stride, ...; the last piece of all may be partial
+  const int64_t first = int64_t(blockIdx.x) * kWWarps + warp, stride = int64_t(gridDim.x) * kWWarps;
+  const int64_t npiece = (n + kWPiece - 1) / kWPiece;
+  const uint32_t mine = npiece > first ? uint32_t((npiece - first + stride - 1) / stride) : 0u;
+  const int tail_n = int(n - (npiece - 1) * kWPiece);      // particles of the last piece
+  // valid particles of the warp's last piece
+  const int last_n = mine > 0 && first + int64_t(mine - 1) * stride == npiece - 1 ? tail_n : kWPiece;
+  const float* src = xyz + first * (3 * kWPiece) + 4 * lane;
+  // the t-th piece of this warp into a slot (always one copy group per lane)
+  auto issue = [&](uint32_t t, float* slot, const float* q) {
+    if (t + 1u < mine || (t + 1u == mine && last_n == kWPiece)) {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) cp_async16(slot + 128 * c + 4 * lane, q + 128 * c);
+    } else if (t + 1u == mine) {                           // word by word up to the end
+      for (int c = lane; c < 3 * last_n; c += 32) cp_async4(slot + c, q - 4 * lane + c);
+    }
+    cp_async_commit();
   };
-  auto issue = [&](int64_t k) {                // k-th chunk of this block into stage k % kWStages
-    const int64_t c = blockIdx.x + k * gridDim.x;
-    const int s = int(k % kWStages);
-    const uint32_t bytes = chunk_bytes(c);
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    mbar_expect_tx(&bar[s], bytes);
-    if (bytes) bulk_g2s(ring + s * 3 * kWChunk, xyz + c * kWChunk * 3, bytes, &bar[s]);
-  };
-  if (threadIdx.x == 0)
-    for (int64_t kk = 0; kk < mine && kk < kWStages; ++kk) issue(kk);
+#pragma unroll
+  for (int t = 0; t < kWStages; ++t)
+    issue(t, slot0 + t * 3 * kWPiece, src + t * stride * (3 * kWPiece));
 
   FastCtx fc{{-1, 0}, {-1, 0}, 0, 0};
   uint32_t* ghist = o.hist;
   uint32_t n_keyed = 0;                        // the warp's keys of stage B
   int ne = 0, nc = 0;                          // lengths of the two lists
-  bool aborted = false;
-  int64_t k = 0;
   const float sx = fs.shf[0], sy = fs.shf[1], sz = fs.shf[2];
   const float lx = fs.shlo[0], ly = fs.shlo[1], lz = fs.shlo[2];
-  for (; k <= mine; ++k) {
-    const bool last = k == mine;               // the final pass only drains the lists
-    const int s = int(k & 1);                  // stage (two stages)
-    if (!last) {
-      if (!mbar_wait(&bar[s], uint32_t(k >> 1) & 1u)) {   // every lane waits (bounded)
-        aborted = true;
-        abort_s = 1;
-      }
-      if (__any_sync(0xFFFFFFFFu, aborted) || abort_s) { aborted = true; break; }
-    }
-    const int64_t kq = last ? (k > 0 ? k - 1 : 0) : k;   // chunk of the newest entries
-    const int64_t cq = blockIdx.x + kq * gridDim.x;
-    const int64_t base = cq * kWChunk;
-    const bool fullc = cq < nfull;
-    const int nvalid = last ? 0 : (fullc ? kWChunk : tail_n);
-    const int nsmem = fullc ? kWChunk : tail_smem;      // particles inside the bulk copy
-    const bool drain_all = last || (k & (kWAgeFlush - 1)) == kWAgeFlush - 1;
-    const int ng = last ? 0 : kWGroups;                  // groups of 32 particles to classify
-    const int nsteps = ng + (drain_all ? 1 : 0);         // + a drain step
-    const int j0 = warp * kWPerWarp + lane;
-    const float* buf = ring + s * 3 * kWChunk + 3 * j0;
-    uint32_t tag = uint32_t(kq & 4095) << 20 | uint32_t(j0) << 8;   // chunk, offset in it
-    const uint64_t qbase = qpack(box_id, 0, p_off + base);   // + offset in the chunk
+  // first particle of the warp's t-th piece
+  auto piece_at = [&](uint32_t t) { return (first + int64_t(t) * stride) * kWPiece; };
+#pragma unroll 1
+  for (uint32_t t = 0; t < mine; ++t) {
+    float* slot = slot0 + (t & (kWStages - 1)) * (3 * kWPiece);
+    cp_async_wait<kWStages - 1>();             // this lane's copies of piece t; then all lanes'
+    const bool last = t + 1u == mine;
+    const int nvalid = last ? last_n : kWPiece;
+    if (last)                                  // no particle: sorted out with the edge scans
+      for (int c = 3 * last_n + lane; c < 3 * kWPiece; c += 32) slot[c] = INFINITY;
+    __syncwarp();
+    const bool drain_all = last || (t & 0xFFFFu) == 0xFFFFu;
+    const int nsteps = kWGroups + (drain_all ? 1 : 0);         // + a drain step
+    const float* buf = slot + 3 * lane;
+    uint32_t tag = t << 15 | uint32_t(lane) << 8;              // piece, offset in it
 #pragma unroll 1
     for (int h = 0; h < nsteps; ++h, buf += 96, tag += 32u << 8) {
-      if (h < ng) {
+      if (h < kWGroups) {
         // ---- A: classify 32 particles of this warp's slice
-        const int j = j0 + 32 * h;
-        float x, y, zc;
-        if (fullc) {                             // every particle inside the bulk copy
-          x = buf[0];
-          y = buf[1];
-          zc = buf[2];
-        } else {
-          x = INFINITY; y = 0.f; zc = 0.f;       // no particle: sorted out with the scans
-          if (j < nsmem) {
-            x = buf[0];
-            y = buf[1];
-            zc = buf[2];
-          } else if (j < nvalid) {               // ragged tail outside the bulk copy
-            x = __ldg(xyz + 3 * (base + j));
-            y = __ldg(xyz + 3 * (base + j) + 1);
-            zc = __ldg(xyz + 3 * (base + j) + 2);
-          }
-        }
+        const int j = 32 * h + lane;
+        const float x = buf[0], y = buf[1], zc = buf[2];
         const float dx = (x + sx) + lx;
         const float dy = (y + sy) + ly;
         const float dz = (zc + sz) + lz;
@@ -690,7 +664,8 @@ k_fast_tma(const float* __restrict__ xyz, int64_t n, int64_t p_off, int32_t box_
         // undecided images wait in queue 1; outside/invalid are final
         bool pushed = true;                      // (a warp-uniform test first, as above)
         if (__any_sync(0xFFFFFFFFu, c1)) {
-          pushed = queue_push(fc.qc, c1, qbase + uint64_t(j), qs.q1, qs.cap1, &qs.cnt->q1);
+          pushed = queue_push_f(fc.qc, c1, [&]() { return qpack(box_id, 0, p_off + piece_at(t) + j); },
+                                qs.q1, qs.cap1, &qs.cnt->q1);
           if (!pushed) {
             const int32_t kx = key_exact_slow(st, lo, hi, N, npix, x, y, zc, bg.sh64[0][0],
                                               bg.sh64[1][0], bg.sh64[2][0]);
@@ -704,11 +679,11 @@ k_fast_tma(const float* __restrict__ xyz, int64_t n, int64_t p_off, int32_t box_
                 if ((int64_t)at < o.dense_cap) o.dense[at] = dk;
               }
             }
-            if (MODE == kModeKeys) o.keys[p_off + base + j] = kx;
+            if (MODE == kModeKeys) o.keys[p_off + piece_at(t) + j] = kx;
           }
         }
         if (MODE == kModeKeys && pushed && j < nvalid && !c2 && !c3)
-          o.keys[p_off + base + j] = c1 ? kKeyUndecided : kKeyOutside;
+          o.keys[p_off + piece_at(t) + j] = c1 ? kKeyUndecided : kKeyOutside;
       }
       __syncwarp();
       // ---- B: pixels of full groups of 32 pending entries, the newest first (in the drain
@@ -730,11 +705,11 @@ k_fast_tma(const float* __restrict__ xyz, int64_t n, int64_t p_off, int32_t box_
         if constexpr (ZONE == 0) pix = pixel_fast_eq(N, bd, dx, dy, z);
         else pix = pixel_fast_cap(N, bd, dx, dy, dz, r2, rinv, z);
         const bool ok = have && pix != kKeyUndecided;
-        // the entry's particle (launch-local index pl): chunk from the
-        // 12-bit tag, offset in the chunk; computed only where needed
+        // the entry's particle (launch-local index): piece from the tag, offset in the
+        // piece; computed only where needed
         auto local_index = [&]() -> int64_t {
-          const int64_t ke = kq - ((kq - int64_t(meta >> 20)) & 4095);
-          return (blockIdx.x + ke * gridDim.x) * kWChunk + int64_t((meta >> 8) & 4095u);
+          const uint32_t te = t - ((t - (meta >> 15)) & ((1u << kWTagBits) - 1u));
+          return piece_at(te) + int64_t((meta >> 8) & 127u);
         };
         const unsigned m = __ballot_sync(0xFFFFFFFFu, ok);
         n_keyed += __popc(m);
@@ -760,32 +735,13 @@ k_fast_tma(const float* __restrict__ xyz, int64_t n, int64_t p_off, int32_t box_
           dense_append(fc.wc, ok, dk, o);
         }
       };
-      const int need = h < ng ? 32 : 1;
+      const int need = h < kWGroups ? 32 : 1;
       if (ne >= need) group_b(std::integral_constant<int, 0>{}, ne);
       if (nc >= need) group_b(std::integral_constant<int, 1>{}, nc);
       __syncwarp();
     }
-    if (last) break;
-    // this warp is done with stage s; the last warp refills it
-    if (lane == 0) {
-      __threadfence_block();
-      const int prev = atomicAdd(&done_s[s], 1);
-      if (prev == kWWarps - 1) {
-        atomicExch(&done_s[s], 0);
-        if (k + kWStages < mine) issue(k + kWStages);
-      }
-    }
-    __syncwarp();
-  }
-  if (aborted) {
-    // a wait ran out: report, then wait (bounded) for the copies that may
-    // still be in flight into this block's shared memory, and leave
-    if (lane == 0) {
-      atomicAdd(&qs.cnt->timeouts, 1ull);
-      for (int64_t q = k; q < mine && q < k + kWStages; ++q)
-        mbar_wait(&bar[q % kWStages], uint32_t((q / kWStages) & 1));
-    }
-    return;
+    src += stride * (3 * kWPiece);             // (every lane has read the slot)
+    issue(t + kWStages, slot, src + (kWStages - 1) * stride * (3 * kWPiece));
   }
   // ---- end: close the warp's chunks, counters, bucket counts
   if (MODE == kModeDense) dense_close(fc.wc, o);
@@ -1775,15 +1731,15 @@ ufc_status run_keys_pipeline(ufc_ctx* c, int mode_req, const float* const* xyz,
       ProfScope ps_(c, "k_fast");
       if (tma) {
         qs.ovf_base = bp.bit_base[k];
-#define UFC_LAUNCH_TMA(...)                                                                      \
-  UFC_CUDA(c, cudaFuncSetAttribute(k_fast_tma<__VA_ARGS__>,                                      \
+#define UFC_LAUNCH_STREAM(...)                                                                      \
+  UFC_CUDA(c, cudaFuncSetAttribute(k_fast_stream<__VA_ARGS__>,                                      \
                                    cudaFuncAttributeMaxDynamicSharedMemorySize, tma_smem));      \
-  k_fast_tma<__VA_ARGS__><<<c->num_sms, kWThreads, tma_smem, c->stream>>>(                                 \
+  k_fast_stream<__VA_ARGS__><<<c->num_sms, kWThreads, tma_smem, c->stream>>>(                                 \
       src, cnt, p0, k, bp.box[k], st, tab, lut_scale, bd, nside, (int32_t)npix, o, qs)
-        if (plan.mode == kModeDense && plan.smem_hist) { UFC_LAUNCH_TMA(kModeDense, true); }
-        else if (plan.mode == kModeDense) { UFC_LAUNCH_TMA(kModeDense, false); }
-        else { UFC_LAUNCH_TMA(kModeKeys, false); }
-#undef UFC_LAUNCH_TMA
+        if (plan.mode == kModeDense && plan.smem_hist) { UFC_LAUNCH_STREAM(kModeDense, true); }
+        else if (plan.mode == kModeDense) { UFC_LAUNCH_STREAM(kModeDense, false); }
+        else { UFC_LAUNCH_STREAM(kModeKeys, false); }
+#undef UFC_LAUNCH_STREAM
       } else {
         const int ssm = plan.mode == kModeDense ? smem : 0;
 #define UFC_LAUNCH_PLAIN(M)                                                                      \
