@@ -524,26 +524,6 @@ __device__ __forceinline__ void hist16_carry(uint32_t* h32, uint32_t* ghist, uin
   atomicAdd(ghist + bucket, 32768u);
 }
 
-// The lookup table as the kernel below wants it: the shell itself where a bin lies in one
-// of the box's shells for certain, kLutOut where it is outside for certain, and the flag
-// kLutScan (any lower bound of the edge in the low bits, plus 1) where the edges have to be
-// scanned and for the bins of radii below the near guard.
-constexpr uint32_t kLutOut = 0x4000u;
-__device__ __forceinline__ void fill_lut_classified(uint16_t* lut, const uint16_t* src,
-                                                    int near_bin, int lo, int hi) {
-  auto conv = [&](uint32_t e, int bin) -> uint32_t {
-    if ((e & kLutScan) || bin <= near_bin) return e | kLutScan;
-    const int a = int(e) - 1;
-    return a >= lo && a < hi ? uint32_t(a) : kLutOut;
-  };
-  const uint32_t* s2 = reinterpret_cast<const uint32_t*>(src);
-  uint32_t* d2 = reinterpret_cast<uint32_t*>(lut);
-  for (int i = threadIdx.x; i < kLut / 2; i += blockDim.x) {
-    const uint32_t w = s2[i];
-    d2[i] = conv(w & 0xFFFFu, 2 * i) | conv(w >> 16, 2 * i + 1) << 16;
-  }
-}
-
 template <int MODE, bool SH>
 __global__ void __launch_bounds__(kWThreads, 1)
 k_fast_stream(const float* __restrict__ xyz, int64_t n, int64_t p_off, int32_t box_id, BoxGeom bg,
@@ -556,12 +536,8 @@ k_fast_stream(const float* __restrict__ xyz, int64_t n, int64_t p_off, int32_t b
   uint32_t* h32 = reinterpret_cast<uint32_t*>(dyn + kWSmemBase);          // 16-bit counters
   __shared__ FastShared fs;
   const int lo = bg.shell_lo, hi = bg.shell_hi;
-  // bin of a squared radius: the nearest integer to v, exact
-  auto lut_bin = [&](float r2) {
-    return __float_as_int(fminf(r2 * lut_scale, float(kLut - 1)) + 8388608.0f) - 0x4B000000;
-  };
   fast_init_shared<false>(fs, bg, st, tab->lut);
-  fill_lut_classified(fs.lut, tab->lut, lut_bin(bd.r2_min), lo, hi);
+  fill_lut_classified(fs.lut, tab->lut, lut_bin(bd.r2_min, lut_scale), lo, hi);
   const int nwords = (o.nbuckets + 1) >> 1;
   if (SH)
     for (int i = threadIdx.x; i < nwords; i += blockDim.x) h32[i] = 0u;
@@ -628,7 +604,7 @@ k_fast_stream(const float* __restrict__ xyz, int64_t n, int64_t p_off, int32_t b
         // outside, undecided (c1), belt (c2) or cap (c3): the table's entry decides the shell
         // but for the bins that hold an edge or the near guard, and for a NaN or an overflow
         // (one vote and a branch for these)
-        uint32_t a = fs.lut[lut_bin(r2)];
+        uint32_t a = fs.lut[lut_bin(r2, lut_scale)];
         bool in = a < kLutOut, und = false;
         const bool fin = r2 <= 3.0e38f;                  // false for NaN and overflow
         const bool scan = a >= kLutScan || !fin;

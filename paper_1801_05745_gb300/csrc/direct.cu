@@ -101,7 +101,8 @@ struct DirectImages {                          // after DirectShared, with image
   float shf[3][kMaxImg1D], shlo[3][kMaxImg1D];
   int count;
   uint32_t mask[(kDMaxImg + 31) / 32];         // images kept, one bit each
-  uint16_t list[kDMaxImg];                     // in increasing order, the same in every block
+  uint16_t list[kDMaxImg];                     // in increasing order, the same in every block:
+                                               // the image's place per axis, 5 bits each
 };
 
 // Key of an image the FP32 stage left open: the double-float stage, then the
@@ -119,11 +120,10 @@ __device__ __noinline__ int2 key_late(const BinTables* t, int32_t lo, int32_t hi
 // Each warp takes its tasks alone (task w, w + warps, ...), 32 particles at a
 // time:
 //   A: radius, shell (lookup table) and zone in FP32; belt and cap particles are
-//      appended, with their observer-relative coordinates, to two circular
-//      pending lists of the warp in shared memory (ballots), undecided ones to
-//      a third;
-//   B: whenever a list holds 32 entries, the warp computes their pixels
-//      together and adds them to the item's count map (atomics in L2);
+//      appended, with their observer-relative coordinates, to two pending
+//      lists of the warp in shared memory (ballots), undecided ones to a third;
+//   B: whenever a list holds 32 entries, the warp computes the pixels of the
+//      newest 32 together and adds them to the item's count map (atomics in L2);
 //   C: whenever 32 undecided images wait, their keys by the double-float and
 //      FP64 stages, out of line.
 // Without images (IMG false) a task is a.task particles of one item, read
@@ -139,14 +139,17 @@ __device__ __noinline__ int2 key_late(const BinTables* t, int32_t lo, int32_t hi
 // 0 stays in the list for non-finite and overflowing coordinates, which count
 // once per particle.
 //
-// What bounds it: issue slots (7.2 warp instructions per particle) and, at small
-// sizes, latency; 24 warps per SM (32 of 64 registers spill: 940 against 775 us
-// for the batched case below).
-// Measured: 64^3 particles with four image layers (729 images, 10 shells,
-// Nside 64) 1910 us with every image of every particle tested, in chunks of
-// 3840 particles that left half of the SMs idle, now 442 us; two boxes of 64^3
-// in one launch of 20 us instead of two of 27, a late stage of 16 + 13 + 7 us
-// and their queues; 150 realisations of 2 x 64^3 particles 775 us.
+// What bounds it: without images the scattered atomics (150 realisations of 2 x 64^3
+// particles: 106 G/s, 0.7 per SM and cycle; issue 44%, the particles' loads wait behind
+// them, and neither loads two groups ahead nor the next task's particles fetched into L2
+// changed that); with images the issue slots; at small sizes latency.  24 warps per SM (32
+// of 64 registers spill: 940 against 775 us for the batched case then).
+// Measured: 64^3 particles with four image layers (729 images, 10 shells, Nside 64) 1910 us
+// with every image of every particle tested, in chunks of 3840 particles that left half of
+// the SMs idle; 442 us with the image list; 288 us with one comparison per table entry, lists
+// as stacks and the images' places per axis kept in the list (no divisions per step).  Two
+// boxes of 64^3 in one launch of 20 us instead of two of 27, a late stage of 16 + 13 + 7 us
+// and their queues; 150 realisations of 2 x 64^3 particles 743 us.
 template <bool IMG>
 __global__ void __launch_bounds__(kDT, 2)
 k_direct(const __grid_constant__ DirectArgs a, const __grid_constant__ BoxGeom bg, int box) {
@@ -163,11 +166,8 @@ k_direct(const __grid_constant__ DirectArgs a, const __grid_constant__ BoxGeom b
     fs.hi2[i] = tab->st.hi2[i];
   }
   if (threadIdx.x == 0) fs.lo2[S + 1] = fs.hi2[S + 1] = INFINITY;
-  {
-    const uint4* src = reinterpret_cast<const uint4*>(tab->lut);
-    uint4* dst = reinterpret_cast<uint4*>(fs.lut);
-    for (int i = threadIdx.x; i < kLut / 8; i += kDT) dst[i] = src[i];
-  }
+  // (all shells: the items of a launch have their own ranges)
+  fill_lut_classified(fs.lut, tab->lut, lut_bin(a.bd.r2_min, a.lut_scale), 0, S);
   if (IMG) {
     const int n1 = 2 * bg.R + 1;
     for (int i = threadIdx.x; i < 3 * kMaxImg1D; i += kDT) {
@@ -208,7 +208,11 @@ k_direct(const __grid_constant__ DirectArgs a, const __grid_constant__ BoxGeom b
       for (int k = lane; k < w; k += 32) before += __popc(im.mask[k]);
       before = __reduce_add_sync(full, before);
       const unsigned m = im.mask[w];
-      if (m >> lane & 1u) im.list[before + __popc(m & lt_mask)] = (uint16_t)(32 * w + lane);
+      if (m >> lane & 1u) {
+        const int i = 32 * w + lane;
+        im.list[before + __popc(m & lt_mask)] =
+            (uint16_t)(i / (n1 * n1) << 10 | (i / n1) % n1 << 5 | i % n1);
+      }
       if (w == nword - 1 && lane == 0) im.count = before + __popc(m);
     }
   }
@@ -218,13 +222,12 @@ k_direct(const __grid_constant__ DirectArgs a, const __grid_constant__ BoxGeom b
   float4* list_eq = fs.lists[warp][0];
   float4* list_cap = fs.lists[warp][1];
   uint64_t* und = fs.und[warp];
-  int he = 0, ne = 0, hc = 0, nc = 0;          // heads and lengths of the two lists
+  int ne = 0, nc = 0;                          // lengths of the two lists
   int hu = 0, nu = 0;                          // of the undecided images
-  unsigned n_keyed = 0, n_invalid = 0, n_ref = 0, n_ex = 0;
+  unsigned n_keyed = 0, n_invalid = 0, n_ref = 0, n_ex = 0;   // of this lane
+  unsigned n_group = 0;                        // keys of the pixel stage (whole warp)
   const int64_t nw = (int64_t)gridDim.x * kDWarps;
   int it = -1;                                 // current item
-  const float* xyz = nullptr;
-  int64_t n = 0, task0 = 0;
   int32_t* cmap = nullptr;
   int lo = 0, hi = 0;
   float sx = 0.f, sy = 0.f, sz = 0.f, lx = 0.f, ly = 0.f, lz = 0.f;
@@ -264,6 +267,10 @@ k_direct(const __grid_constant__ DirectArgs a, const __grid_constant__ BoxGeom b
     nu -= take;
     __syncwarp();
   };
+  auto image_tag = [&](uint32_t img) {         // the image's number, in an undecided entry
+    const uint32_t n1 = uint32_t(2 * bg.R + 1);
+    return uint64_t(((img >> 10) * n1 + ((img >> 5) & 31u)) * n1 + (img & 31u)) << 47;
+  };
   auto push = [&](bool want, uint64_t e) {     // (the whole warp calls it)
     const unsigned m = __ballot_sync(full, want);
     if (want) und[(hu + nu + __popc(m & lt_mask)) & (kDUnd - 1)] = e;
@@ -276,9 +283,6 @@ k_direct(const __grid_constant__ DirectArgs a, const __grid_constant__ BoxGeom b
       ++it;
       while (!IMG && it + 1 < a.nitems && item(it + 1).task0 <= t) ++it;
       const DirectItem& d = item(it);
-      xyz = d.xyz;
-      n = d.n;
-      task0 = d.task0;
       cmap = d.counts;
       lo = d.shell_lo;
       hi = d.shell_hi;
@@ -290,16 +294,17 @@ k_direct(const __grid_constant__ DirectArgs a, const __grid_constant__ BoxGeom b
     int64_t p0;                                // first particle of the task
     int cnt;                                   // particles
     int nsteps, i0 = 0;                        // groups of 32, or images from i0 on
+    const DirectItem& ti = item(it);
     if (IMG) {
       const int64_t g = t / a.nslice;
       const int sl = int(t - g * a.nslice);
       p0 = 32 * g;
-      cnt = int(min((int64_t)32, n - p0));
+      cnt = int(min((int64_t)32, ti.n - p0));
       i0 = int((int64_t)nimg * sl / a.nslice);
       nsteps = int((int64_t)nimg * (sl + 1) / a.nslice) - i0;
     } else {
-      p0 = (t - task0) * a.task;
-      cnt = int(min((int64_t)a.task, n - p0));
+      p0 = (t - ti.task0) * a.task;
+      cnt = int(min((int64_t)a.task, ti.n - p0));
       nsteps = (cnt + 31) >> 5;
     }
     // the late stage is called outside the loop over the steps, with nothing of
@@ -308,109 +313,102 @@ k_direct(const __grid_constant__ DirectArgs a, const __grid_constant__ BoxGeom b
     int h = 0;
 #pragma unroll 1
     do {
-      float x = 0.f, y = 0.f, z = 0.f;
+      float x = INFINITY, y = 0.f, z = 0.f;    // no particle: sorted out with the edge scans
       const int j0 = IMG ? lane : 32 * h + lane;
-      bool have = j0 < cnt;
-      const float* q = xyz + 3 * (p0 + j0);
-      if (have) { x = __ldg(q); y = __ldg(q + 1); z = __ldg(q + 2); }
+      const float* q = ti.xyz + 3 * (p0 + j0);
+      if (j0 < cnt) { x = __ldg(q); y = __ldg(q + 1); z = __ldg(q + 2); }
 #pragma unroll 1
       for (;;) {
         const bool tail = h == nsteps || nu >= 32;       // drains the lists
         if (!tail) {
           // ---- A
-          int img = 0;
-          float x1 = 0.f, y1 = 0.f, z1 = 0.f;    // the next group's particle
-          bool have1 = false;
+          uint32_t img = 0;                      // the image's place per axis
+          float x1 = INFINITY, y1 = 0.f, z1 = 0.f;   // the next group's particle
           if (IMG) {
-            const int n1 = 2 * bg.R + 1;
             img = im.list[i0 + h];
-            const int ii = img / (n1 * n1), jj = (img / n1) % n1, kk = img % n1;
+            const uint32_t ii = img >> 10, jj = (img >> 5) & 31u, kk = img & 31u;
             sx = im.shf[0][ii]; sy = im.shf[1][jj]; sz = im.shf[2][kk];
             lx = im.shlo[0][ii]; ly = im.shlo[1][jj]; lz = im.shlo[2][kk];
           } else {
-            have1 = 32 * (h + 1) + lane < cnt;
             q += 96;
-            if (have1) { x1 = __ldg(q); y1 = __ldg(q + 1); z1 = __ldg(q + 2); }
+            if (32 * (h + 1) + lane < cnt) { x1 = __ldg(q); y1 = __ldg(q + 1); z1 = __ldg(q + 2); }
           }
           const float dx = (x + sx) + lx;
           const float dy = (y + sy) + ly;
           const float dz = (z + sz) + lz;
           const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
+          uint32_t b = fs.lut[lut_bin(r2, a.lut_scale)];
+          bool in = b - uint32_t(lo) < uint32_t(hi - lo), open = false;
           const bool fin = r2 <= 3.0e38f;                // false for NaN and overflow
-          const bool near = !(r2 >= a.bd.r2_min);        // near the observer (r == 0 is invalid)
-          const float v = fminf(r2 * a.lut_scale, float(kLut - 1));
-          const int bin = __float_as_int(v + 8388608.0f) - 0x4B000000;
-          const uint32_t e = fs.lut[bin];
-          int b = int(e & 0x7FFFu) - 1;
-          bool band = false;
-          if (__any_sync(full, (e & kLutScan) && fin)) { // rare: scan the edges
-            if ((e & kLutScan) && fin) {
-              for (;;) {                                 // (ends at the +inf sentinel)
-                if (r2 < fs.lo2[b + 1]) break;
-                if (r2 < fs.hi2[b + 1]) { band = true; break; }
-                ++b;
+          const bool scan = b >= kLutScan || !fin;
+          if (__any_sync(full, scan)) {                  // rare: scan the edges
+            if (scan) {
+              in = false;
+              const bool have = (IMG ? lane : 32 * h + lane) < cnt;
+              // (non-finite or overflowing coordinates once per particle, with image 0)
+              open = have && (fin ? !(r2 >= a.bd.r2_min)   // near the observer (r == 0 is invalid)
+                                  : (!IMG || img == 0u));
+              if (fin && !open) {
+                int e = int(b & 0x7FFFu) - 1;
+                for (;;) {                               // (ends at the +inf sentinel)
+                  if (r2 < fs.lo2[e + 1]) break;
+                  if (r2 < fs.hi2[e + 1]) { open = true; break; }
+                  ++e;
+                }
+                in = !open && e >= lo && e < hi;
+                b = uint32_t(e);
               }
             }
           }
-          const bool inshell = uint32_t(b - lo) < uint32_t(hi - lo);
           const float dz2 = dz * dz;
-          const bool eqz = dz2 <= a.bd.z_eq2 * r2;
-          const bool capz = dz2 > a.bd.z_cap2 * r2;
-          const bool dec = have && fin && !near && !band && inshell;
-          const bool c2 = dec && eqz, c3 = dec && capz;
-          const bool c1 = have && (fin ? (near || band || (inshell && !eqz && !capz))
-                                       : (!IMG || img == 0));
+          const bool c2 = in && dz2 <= a.bd.z_eq2 * r2;
+          const bool c3 = in && dz2 > a.bd.z_cap2 * r2;
+          const bool c1 = open || (in && !c2 && !c3);
           // entry: coordinates, shell, and particle (offset, or lane and image)
-          const uint32_t meta = uint32_t(b & 255) |
-                                (IMG ? uint32_t(lane) << 8 | uint32_t(img) << 13
-                                     : uint32_t(32 * h + lane) << 8);
+          const uint32_t meta = b | (IMG ? uint32_t(lane) << 8 | img << 13
+                                         : uint32_t(32 * h + lane) << 8);
           const float4 ent = make_float4(dx, dy, dz, __uint_as_float(meta));
           const unsigned meq = __ballot_sync(full, c2), mcap = __ballot_sync(full, c3);
-          if (c2) list_eq[(he + ne + __popc(meq & lt_mask)) & (kDList - 1)] = ent;
-          if (c3) list_cap[(hc + nc + __popc(mcap & lt_mask)) & (kDList - 1)] = ent;
+          if (c2) list_eq[ne + __popc(meq & lt_mask)] = ent;
+          if (c3) list_cap[nc + __popc(mcap & lt_mask)] = ent;
           ne += __popc(meq);
           nc += __popc(mcap);
           if (__any_sync(full, c1))
-            push(c1, uint64_t(IMG ? img : it) << 47 | uint64_t(p0 + (IMG ? lane : 32 * h + lane)));
-          if (!IMG) { x = x1; y = y1; z = z1; have = have1; }
+            push(c1, (IMG ? image_tag(img) : uint64_t(it) << 47) |
+                         uint64_t(p0 + (IMG ? lane : 32 * h + lane)));
+          if (!IMG) { x = x1; y = y1; z = z1; }
           ++h;
         }
         __syncwarp();
         // ---- B
-        auto group_b = [&](auto zone_tag, int take) {
+        auto group_b = [&](auto zone_tag, int& len) {    // the newest 32 (or the rest)
           constexpr int ZONE = decltype(zone_tag)::value;
-          const float4* L = ZONE == 0 ? list_eq : list_cap;
-          const int head = ZONE == 0 ? he : hc;
-          const bool on = lane < take;
-          float4 ent = make_float4(0.f, 0.f, 0.f, 0.f);
-          if (on) ent = L[(head + lane) & (kDList - 1)];
-          if constexpr (ZONE == 0) { he = (he + take) & (kDList - 1); ne -= take; }
-          else { hc = (hc + take) & (kDList - 1); nc -= take; }
+          const int take = min(len, 32);
+          len -= take;
+          const bool on = lane < take;           // (a lane without one reads an old entry)
+          const float4 ent = (ZONE == 0 ? list_eq : list_cap)[len + lane];
           const float dx = ent.x, dy = ent.y, dz = ent.z;
           const uint32_t meta = __float_as_uint(ent.w);
           const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
           const float rinv = rsqrt_fast(r2);
           const float zz = dz * rinv;
-          int32_t pix = kKeyUndecided;
-          if (on) {
-            if constexpr (ZONE == 0) pix = pixel_fast_eq(a.N, a.bd, dx, dy, zz);
-            else pix = pixel_fast_cap(a.N, a.bd, dx, dy, dz, r2, rinv, zz);
-          }
+          int32_t pix;
+          if constexpr (ZONE == 0) pix = pixel_fast_eq(a.N, a.bd, dx, dy, zz);
+          else pix = pixel_fast_cap(a.N, a.bd, dx, dy, dz, r2, rinv, zz);
           const bool ok = on && pix != kKeyUndecided;
           const int32_t key = int(meta & 255u) * a.npix + pix;
           if (ok && UFC_IDX_OK(key, a.ncell, 2)) atomicAdd(cmap + key, 1);
-          n_keyed += ok;
-          if (__any_sync(full, on && !ok)) {
-            const uint64_t eu = IMG ? uint64_t(meta >> 13) << 47 |
-                                          uint64_t(p0 + ((meta >> 8) & 31u))
+          const unsigned m = __ballot_sync(full, ok);
+          n_group += __popc(m);
+          if (m != full) {
+            const uint64_t eu = IMG ? image_tag(meta >> 13) | uint64_t(p0 + ((meta >> 8) & 31u))
                                     : uint64_t(it) << 47 | uint64_t(p0 + (meta >> 8));
             push(on && !ok, eu);
           }
         };
-        const int take_e = ne >= 32 ? 32 : (tail ? ne : 0);
-        if (take_e) group_b(std::integral_constant<int, 0>{}, take_e);
-        const int take_c = nc >= 32 ? 32 : (tail ? nc : 0);
-        if (take_c) group_b(std::integral_constant<int, 1>{}, take_c);
+        const int need = tail ? 1 : 32;
+        if (ne >= need) group_b(std::integral_constant<int, 0>{}, ne);
+        if (nc >= need) group_b(std::integral_constant<int, 1>{}, nc);
         __syncwarp();
         if (tail) break;
       }
@@ -420,7 +418,7 @@ k_direct(const __grid_constant__ DirectArgs a, const __grid_constant__ BoxGeom b
     } while (h < nsteps);
   }
   if (nu) settle(nu);
-  n_keyed = __reduce_add_sync(full, n_keyed);
+  n_keyed = __reduce_add_sync(full, n_keyed) + n_group;
   n_invalid = __reduce_add_sync(full, n_invalid);
   n_ref = __reduce_add_sync(full, n_ref);
   n_ex = __reduce_add_sync(full, n_ex);

@@ -17,6 +17,35 @@ constexpr int kLutBits = 13;
 constexpr int kLut = 1 << kLutBits;
 constexpr uint16_t kLutScan = 0x8000;
 
+// A block's copy of the table with one comparison per particle: the shell itself where a bin
+// lies in one of the shells [lo, hi) for certain, kLutOut where it is outside for certain, and
+// the flag kLutScan (with the edge to scan from in the low bits) for the other bins and for
+// those of radii below the near guard.
+constexpr uint32_t kLutOut = 0x4000u;
+__device__ __forceinline__ void fill_lut_classified(uint16_t* lut, const uint16_t* src,
+                                                    int near_bin, int lo, int hi) {
+  auto conv = [&](uint32_t e, int bin) -> uint32_t {
+    const uint32_t a = e - 1u;
+    const uint32_t r = a - uint32_t(lo) < uint32_t(hi - lo) ? a : kLutOut;
+    return (e & kLutScan) || bin <= near_bin ? e | kLutScan : r;
+  };
+  const uint4* s8 = reinterpret_cast<const uint4*>(src);
+  uint4* d8 = reinterpret_cast<uint4*>(lut);
+#pragma unroll 2
+  for (int i = threadIdx.x; i < kLut / 8; i += blockDim.x) {
+    const uint4 w = s8[i];
+    auto two = [&](uint32_t e, int bin) {
+      return conv(e & 0xFFFFu, bin) | conv(e >> 16, bin + 1) << 16;
+    };
+    d8[i] = make_uint4(two(w.x, 8 * i), two(w.y, 8 * i + 2), two(w.z, 8 * i + 4),
+                       two(w.w, 8 * i + 6));
+  }
+}
+// The bin of a squared radius (the nearest integer, exact).
+__device__ __forceinline__ int lut_bin(float r2, float scale) {
+  return __float_as_int(fminf(r2 * scale, float(kLut - 1)) + 8388608.0f) - 0x4B000000;
+}
+
 // Tables of one call in device memory, written by k_bin_prep.
 struct BinTables {
   ShellTable st;

@@ -1,4 +1,4 @@
-"""The dense path's first stage at the edges of its form: pieces of 128 particles
+"""The FP32 stages of the dense and the direct path at the edges of their form: pieces of 128 particles
 with every kind of remainder (none, less than a piece, not a multiple of 4),
 fewer pieces than warps, several shell edges in one bin of the lookup table,
 particles at and around the observer, outside every shell, and non-finite or
@@ -39,11 +39,11 @@ def test_keys_and_counts_at_the_edges(orc, n, nside, nshell):
         x[-16:, 0], x[-16:, 1], x[-16:, 2] = 1000.0 + e, 1000.0, 1000.0
     ba, bo = both_boxes(api, orc, L, [1000.0] * 3, n, 0, nshell)
     dev = torch.from_numpy(x).cuda()
-    if nside >= 64:                                                # (the dense path's least)
-        counts = ctx.bin([dev], [ba], chi, nside, path="dense").cpu().numpy()
+    ref, inv = orc.bin_counts(x, bo, chi, nside)
+    for path in ["direct"] + (["dense"] if nside >= 64 else []):   # (the dense path's least)
+        counts = ctx.bin([dev], [ba], chi, nside, path=path).cpu().numpy()
         info = ctx.bin_info()
-        ref, inv = orc.bin_counts(x, bo, chi, nside)
-        assert np.array_equal(counts, ref)
+        assert np.array_equal(counts, ref), path
         assert info["invalid"] == inv and info["keyed"] == int(ref.sum())
     keys = ctx.keys(dev, ba, chi, nside).cpu().numpy()
     assert np.array_equal(keys, orc.keys(x, bo, chi, nside))
