@@ -854,7 +854,7 @@ __device__ __forceinline__ int pdf_slot(float k, const PdfParam& pp) {
 
 // One block's share of the moment pass: block vb of a grid of nb blocks of
 // kMT threads (every thread calls it).  Central power sums about `mean` into
-// out[0..2] (valid in thread 0); PDF counts into the shared histogram.  Two
+// out[0..2] (global; red holds 3 kMT / 32); PDF counts into the shared histogram.  Two
 // of a thread's pixels at a time, side by side in packed double-float.
 __device__ __forceinline__ void moments_block(const float* __restrict__ kappa, int npix,
                                               double mean, const PdfParam& pp, int vb, int nb,
@@ -895,13 +895,32 @@ __device__ __forceinline__ void moments_block(const float* __restrict__ kappa, i
     const float k0 = kappa[p], k1 = both ? kappa[p + step] : k0;
     add_pair(k0, k1, both);
   }
-  auto total = [](dfx a) {                             // the halves, in FP64
-    const float2 h = x2_get(a.h), l = x2_get(a.l);
-    return ((double)h.x + (double)l.x) + ((double)h.y + (double)l.y);
-  };
-  out[0] = block_sum_d<kMT>(total(a2), red);
-  out[1] = block_sum_d<kMT>(total(a3), red);
-  out[2] = block_sum_d<kMT>(total(a4), red);
+  // Over the lanes in double-float, over the warps in FP64, in fixed orders.  (FP64
+  // additions over the lanes kept the FP64 pipe 79% busy in a batch of small maps: 150
+  // maps of Nside 64, 174 us then, 119 now.)
+  const int w = threadIdx.x >> 5, ln = threadIdx.x & 31;
+  dfx q[3] = {a2, a3, a4};
+  double v[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    q[k] = dfx_norm(q[k].h, q[k].l);
+    for (int o = 16; o > 0; o >>= 1) {
+      const dfx r{__shfl_down_sync(0xFFFFFFFFu, q[k].h, o), __shfl_down_sync(0xFFFFFFFFu, q[k].l, o)};
+      q[k] = dfx_add_raw(q[k], r);
+      q[k] = dfx_norm(q[k].h, q[k].l);
+    }
+    const float2 h = x2_get(q[k].h), l = x2_get(q[k].l);
+    v[k] = ((double)h.x + (double)l.x) + ((double)h.y + (double)l.y);   // (used in lane 0)
+  }
+  __syncthreads();
+  if (ln == 0)
+    for (int k = 0; k < 3; ++k) red[kMT / 32 * k + w] = v[k];
+  __syncthreads();
+  if (threadIdx.x < 3) {
+    double t = 0.0;
+    for (int i = 0; i < kMT / 32; ++i) t += red[kMT / 32 * threadIdx.x + i];
+    out[threadIdx.x] = t;
+  }
 }
 
 // moments[10] from the partial sums, by a block of kMT threads (fixed orders:
@@ -940,8 +959,8 @@ __device__ __forceinline__ void moments_final_block(const double* ksum_part, int
 
 // Blocks of the moment pass: 4 per SM (32 warps), no more than there are
 // pixels for at four per thread (the loads a thread has in flight; a block of
-// fewer pixels pays its prologue and its PDF's global atomics for little).  What bounds the pass is the
-// latency of a pixel's chain (load, shared-memory histogram, double-float
+// fewer pixels pays its prologue and its PDF's global atomics for little).  What
+// bounds the pass is the latency of a pixel's chain (load, shared-memory histogram, double-float
 // sums): with 2 blocks per SM and one pixel at a time it took 200 us for the
 // 12.6 M pixels of Nside 1024.
 static int moments_grid(int num_sms, int npix) {
@@ -956,7 +975,7 @@ k_moments(const float* __restrict__ kappa, int npix, const double* __restrict__ 
           unsigned long long* __restrict__ pdf /*[nbins+3]*/, double* __restrict__ m,
           unsigned int* __restrict__ ticket) {
   extern __shared__ unsigned int hist[];   // [nbins + 3]
-  __shared__ double red[kMT / 32];
+  __shared__ double red[3 * kMT / 32];
   __shared__ double mean_s;
   __shared__ bool last_s;
   for (int i = threadIdx.x; i < pp.nbins + 3; i += blockDim.x) hist[i] = 0;
@@ -965,14 +984,11 @@ k_moments(const float* __restrict__ kappa, int npix, const double* __restrict__ 
     if (threadIdx.x == 0) mean_s = s / double(npix);
   }
   __syncthreads();
-  double o[3];
-  moments_block(kappa, npix, mean_s, pp, blockIdx.x, gridDim.x, hist, red, o);
-  if (threadIdx.x == 0) {
-    part[3 * blockIdx.x + 0] = o[0];
-    part[3 * blockIdx.x + 1] = o[1];
-    part[3 * blockIdx.x + 2] = o[2];
+  moments_block(kappa, npix, mean_s, pp, blockIdx.x, gridDim.x, hist, red, part + 3 * blockIdx.x);
+  if (threadIdx.x < 32) {
     __threadfence();                       // this block's sums before its ticket
-    last_s = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    __syncwarp();
+    if (threadIdx.x == 0) last_s = atomicAdd(ticket, 1u) == gridDim.x - 1;
   }
   __syncthreads();
   for (int i = threadIdx.x; i < pp.nbins + 3; i += blockDim.x)
@@ -1157,7 +1173,7 @@ k_batch_kappa(const __grid_constant__ BatchArgs ba) {
 __global__ void __launch_bounds__(kMT)
 k_batch_moments(const __grid_constant__ BatchArgs ba, const __grid_constant__ PdfParam pp) {
   extern __shared__ unsigned int hist[];   // [nbins + 3]
-  __shared__ double red[kMT / 32];
+  __shared__ double red[3 * kMT / 32];
   __shared__ double mean_s;
   __shared__ bool last_s;
   const int r = blockIdx.y;
@@ -1170,14 +1186,8 @@ k_batch_moments(const __grid_constant__ BatchArgs ba, const __grid_constant__ Pd
     if (threadIdx.x == 0) mean_s = s / double(ba.npix);
   }
   __syncthreads();
-  double o[3];
-  moments_block(ba.kappa + (size_t)r * ba.npix, ba.npix, mean_s, pp, blockIdx.x, ba.gm, hist, red, o);
-  if (threadIdx.x == 0) {
-    mp[3 * blockIdx.x + 0] = o[0];
-    mp[3 * blockIdx.x + 1] = o[1];
-    mp[3 * blockIdx.x + 2] = o[2];
-  }
-  __syncthreads();
+  moments_block(ba.kappa + (size_t)r * ba.npix, ba.npix, mean_s, pp, blockIdx.x, ba.gm, hist, red,
+                mp + 3 * blockIdx.x);
   for (int i = threadIdx.x; i < ba.nbins + 3; i += blockDim.x)
     if (hist[i]) atomicAdd((unsigned long long*)pd + i, (unsigned long long)hist[i]);
   __threadfence();                         // sums and PDF before this block's count
