@@ -108,12 +108,19 @@ constexpr int kShtTab = 4 * kShtMaxNside + 2;     // entries of the one-dimensio
 // C(2k, k) / 4^k, integers under 2^53), above by the asymptotic series of
 // Gamma(x + 1/4) / Gamma(x + 3/4), x = k + 1/4, in 1/x^2 (from the Bernoulli
 // polynomials at 1/4; the first term left out is below 2^-75 at x = 24).
-__device__ __forceinline__ double sht_w(int k) {
-  if (k < 24) {
-    double c = 1.0;
-    for (int j = 1; j <= k; ++j) c = c * (double)(2 * (2 * j - 1)) / (double)j;
-    return ldexp(c, -2 * k);
+struct Binomials { double c[24]; };             // C(2k, k)
+constexpr Binomials make_binomials() {
+  Binomials b{};
+  long long c = 1;
+  for (int k = 0; k < 24; ++k) {
+    b.c[k] = (double)c;
+    c = c * (2 * (2 * k + 1)) / (k + 1);
   }
+  return b;
+}
+__constant__ const Binomials kBinom = make_binomials();
+__device__ __forceinline__ double sht_w(int k) {
+  if (k < 24) return ldexp(kBinom.c[k], -2 * k);
   const double x = (double)k + 0.25, y = 1.0 / (x * x);
   double p = 7426362705.0 / 1099511627776.0;
   p = fma(p, y, -20898423.0 / 8589934592.0);
@@ -125,36 +132,47 @@ __device__ __forceinline__ double sht_w(int k) {
   return fma(p * y, r, r);
 }
 
-// All tables of one call (a grid over the longest of them).  Unit roots
-// e^{-2 pi i j / (8N)}, j < 8N, as double-float complex numbers (FP64
-// sincospi, split once).  Every power-of-two ring (n = 4N, or n = 4i
-// with i a power of two) has n | 8N: its FFT twiddles are T[k 8N/n] and the
-// phase of its first pixel, e^{-i m phi_0} with phi_0 = pi/n, is
-// T[m 4N/n mod 8N].
-__global__ void k_sht_tables(int32_t N, int32_t lmax, float4* __restrict__ T,
-                             double* __restrict__ tab, float4* __restrict__ pair) {
-  const int n8 = 8 * N;
-  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < max(n8, lmax + 2);
-       j += gridDim.x * blockDim.x) {
-    if (j < n8) {
-      double sn, cs;
-      sincospi(-2.0 * (double)j / (double)n8, &sn, &cs);
-      T[j] = cdf_pack(df_from_d(cs), df_from_d(sn));
-    }
-    if (j < lmax + 2) {
-      const double w = sht_w(j), l2 = 2.0 * j + 1.0;
-      tab[j] = sqrt(w);
-      tab[kShtTab + j] = sqrt(1.0 / (l2 * w));
-      tab[2 * kShtTab + j] = sqrt(l2);
-      const double c = sqrt(l2 * w * 0.079577471545947667884);     // 1 / (4 pi)
-      tab[3 * kShtTab + j] = (j & 1) ? -c : c;
-    }
-    if (j < 2 * N) {
-      const Ring g = ring_geom(N, j);
-      const int i = j + 1;                                        // (whole numbers below 2^22)
-      pair[j] = make_float4((float)(i < N ? 3 * N * N - i * i : 2 * N * (2 * N - i)), (float)g.z,
-                            (float)g.s, 0.f);
-    }
+// All tables of one call.  Unit roots e^{-2 pi i j / (8N)}, j < 8N, as double-float
+// complex numbers (FP64 sincospi, split once).  Every power-of-two ring (n = 4N, or
+// n = 4i with i a power of two) has n | 8N: its FFT twiddles are T[k 8N/n] and the
+// phase of its first pixel, e^{-i m phi_0} with phi_0 = pi/n, is T[m 4N/n mod 8N].
+// Each FP64 chain has threads of its own (the kernel is latency: one thread per index
+// with all of them, and the binomials of w by a loop of divisions, took 21 us at Nside
+// 64, 8 now).
+__global__ void __launch_bounds__(64)
+k_sht_tables(int32_t N, int32_t lmax, float4* __restrict__ T, double* __restrict__ tab,
+             float4* __restrict__ pair) {
+  const int n8 = 8 * N, nl = (lmax + 2 + 31) / 32 * 32;              // (whole warps per part)
+  int j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j < n8) {
+    double sn, cs;
+    sincospi(-2.0 * (double)j / (double)n8, &sn, &cs);
+    T[j] = cdf_pack(df_from_d(cs), df_from_d(sn));
+    return;
+  }
+  j -= n8;
+  if (j < 2 * N) {
+    const Ring g = ring_geom(N, j);
+    const int i = j + 1;                                             // (whole numbers below 2^22)
+    pair[j] = make_float4((float)(i < N ? 3 * N * N - i * i : 2 * N * (2 * N - i)), (float)g.z,
+                          (float)g.s, 0.f);
+    return;
+  }
+  j -= 2 * N;
+  const int part = j / nl;
+  j -= part * nl;
+  if (part > 3 || j >= lmax + 2) return;
+  const double l2 = 2.0 * j + 1.0;
+  if (part == 2) {
+    tab[2 * kShtTab + j] = sqrt(l2);
+    return;
+  }
+  const double w = sht_w(j);
+  if (part == 0) tab[j] = sqrt(w);
+  else if (part == 1) tab[kShtTab + j] = sqrt(1.0 / (l2 * w));
+  else {
+    const double c = sqrt(l2 * w * 0.079577471545947667884);         // 1 / (4 pi)
+    tab[3 * kShtTab + j] = (j & 1) ? -c : c;
   }
 }
 
@@ -760,8 +778,8 @@ static ufc_status sht_space(ufc_ctx* c, int nside, int lmax, int nchunk, ShtSpac
   o.part = reinterpret_cast<double2*>(ws + o_part);
   {
     ProfScope ps_(c, "k_sht_tables");
-    const int n = std::max(8 * nside, lmax + 2);
-    k_sht_tables<<<(n + 127) / 128, 128, 0, c->stream>>>(nside, lmax, roots, tab, pair);
+    const int n = 10 * nside + 4 * ((lmax + 2 + 31) / 32 * 32);
+    k_sht_tables<<<(n + 63) / 64, 64, 0, c->stream>>>(nside, lmax, roots, tab, pair);
   }
   {
     ProfScope ps_(c, "k_lmm");
