@@ -144,7 +144,9 @@ class UfcError(RuntimeError):
 
 
 def _np_ptr(a: np.ndarray):
-    return a.ctypes.data_as(P)
+    p = P(a.ctypes.data)
+    p._arr = a                       # alive as long as the pointer (callers pass temporaries)
+    return p
 
 
 def _check(status: int, ctx=None, what=""):
@@ -231,6 +233,10 @@ class Context:
         if st != UFC_OK:
             raise UfcError(f"ufc_create({device}) failed with status {st}")
         self.h = h
+        torch.cuda.init()
+        # (the handle alone: a Stream object per call took a third of a small map's host time
+        # together with the casts that the argument types make unnecessary)
+        self._raw_stream = torch._C._cuda_getCurrentRawStream
 
     def close(self):
         if self.h:
@@ -244,9 +250,7 @@ class Context:
             pass
 
     def _stream(self):
-        import torch
-        s = torch.cuda.current_stream(self.device).cuda_stream
-        _lib.ufc_set_stream(self.h, P(s))
+        _lib.ufc_set_stream(self.h, self._raw_stream(self.device))
 
     def _ck(self, st, what):
         _check(st, self.h, what)
@@ -324,14 +328,13 @@ class Context:
         if counts is None:
             counts = torch.empty((S, npix), dtype=torch.int32, device=f"cuda:{self.device}")
         assert counts.dtype == torch.int32 and counts.is_contiguous() and counts.numel() == S * npix
-        ptrs = (P * len(xs))(*[P(x.data_ptr()) for x in xs])
+        ptrs = (P * len(xs))(*[x.data_ptr() for x in xs])
         ns = (I64 * len(xs))(*[x.numel() // 3 for x in xs])
         arr = (Box * len(boxes))(*boxes)
         self._stream()
         flags = _bin_flags(accumulate, path)
-        self._ck(_lib.ufc_bin(self.h, ctypes.cast(ptrs, P), ctypes.cast(ns, P), ctypes.cast(arr, P),
-                              len(boxes), _np_ptr(chi), S, nside, flags, P(counts.data_ptr())),
-                 "ufc_bin")
+        self._ck(_lib.ufc_bin(self.h, ptrs, ns, arr, len(boxes), _np_ptr(chi), S, nside, flags,
+                              P(counts.data_ptr())), "ufc_bin")
         return counts
 
     def bin_host(self, xyz_list, boxes, chi_edges, nside: int, counts=None, accumulate=False,

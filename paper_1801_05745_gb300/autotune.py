@@ -18,10 +18,18 @@ import threading
 _lock = threading.Lock()
 
 
+_default: dict = {}  # $HOME -> the default path (every binning call asks for it)
+
+
 def cache_path() -> str:
-    return os.environ.get("UFC_AUTOTUNE_CACHE",
-                          os.path.join(os.path.expanduser("~"), ".cache", "ufalcon_gb300",
-                                       "autotune.json"))
+    p = os.environ.get("UFC_AUTOTUNE_CACHE")
+    if p is not None:
+        return p
+    home = os.environ.get("HOME")
+    if home not in _default or home is None:
+        _default[home] = os.path.join(os.path.expanduser("~"), ".cache", "ufalcon_gb300",
+                                      "autotune.json")
+    return _default[home]
 
 
 _memo: dict = {}     # path -> (mtime, contents): the cache file is read once per change
@@ -70,9 +78,9 @@ def tune_key(gpu_name: str, nside: int, nshell: int, n_total: int) -> str:
 
 def cached_bin_path(ctx, nside: int, nshell: int, n_total: int):
     """The cached binning path ('direct' or 'dense') for this shape, or None."""
-    key = tune_key(_gpu_name(ctx.device), nside, nshell, n_total)
     with _lock:
-        e = _load().get(key)
+        d = _load()
+    e = d.get(tune_key(_gpu_name(ctx.device), nside, nshell, n_total)) if d else None
     return e["path"] if e else None
 
 
