@@ -173,14 +173,25 @@ __device__ __forceinline__ int log2_of(int v) { return 31 - __clz(v); }   // v a
 __device__ __forceinline__ int bit_rev(int k, int b) { return (int)(__brev((unsigned)k) >> (32 - b)); }
 
 // Unit roots w_n^k of a ring of n = 4i pixels that is not a power of two: the
-// first quarter k < i in shared memory (FP64 sincospi, split once), the rest by
-// exact quadrant rotations (w_n^{k + i} = -i w_n^k).
+// first quarter k < i in shared memory, the rest by exact quadrant rotations
+// (w_n^{k + i} = -i w_n^k).  k < 32 and the multiples of 32 by FP64 sincospi
+// (split once), the others as the double-float product of two of these; wf[i] =
+// w_{2n}.  (FP64 runs at 1/64 of the FP32 rate: with a sincospi per root, and w_2n
+// and the ring's geometry by every thread, its pipe was 42% busy and the 2047 rings of
+// Nside 512 took 380 us to synthesise, 324 now; the transform of Nside 64 24 us, 13
+// now.)  Every thread calls it; ends with a barrier.
 __device__ __forceinline__ void fill_quarter(float4* wf, int i) {
-  for (int k = threadIdx.x; k < i; k += kRingThreads) {
+  const int nd = min(i, 32) + (i - 1) / 32;              // roots formed directly, then w_2n
+  for (int t = threadIdx.x; t <= nd; t += kRingThreads) {
+    const int k = t < 32 && t < i ? t : (t - min(i, 32) + 1) * 32;
     double sn, cs;
-    sincospi(-0.5 * (double)k / (double)i, &sn, &cs);
-    wf[k] = cdf_pack(df_from_d(cs), df_from_d(sn));
+    sincospi(t == nd ? -0.25 / (double)i : -0.5 * (double)k / (double)i, &sn, &cs);
+    wf[t == nd ? i : k] = cdf_pack(df_from_d(cs), df_from_d(sn));
   }
+  __syncthreads();
+  for (int k = 32 + threadIdx.x; k < i; k += kRingThreads)
+    if (k & 31) wf[k] = cx_to4(cx_mul(cx_of(wf[k & ~31]), cx_of(wf[k & 31])));
+  __syncthreads();
 }
 __device__ __forceinline__ cx quarter_root(const float4* wf, int i, int k) {   // 0 <= k < 4i
   int q = 0;
@@ -200,10 +211,14 @@ __device__ __forceinline__ cx quarter_phase(const float4* wf, int i, int m, cx h
   const cx p = quarter_root(wf, i, (m >> 1) % (4 * i));
   return (m & 1) ? cx_mul(p, h1) : p;
 }
-__device__ __forceinline__ cx half_step(int n) {             // w_{2n}
-  double sn, cs;
-  sincospi(-1.0 / (double)n, &sn, &cs);
-  return cx_of(cdf_pack(df_from_d(cs), df_from_d(sn)));
+// First pixel and number of pixels of ring r, and whether its first pixel lies half a
+// step from azimuth 0 (ring_geom, whole numbers only).
+struct RingSpan { int32_t start, n; bool shifted; };
+__device__ __forceinline__ RingSpan ring_span(int N, int r) {
+  const int i = r + 1, k = 4 * N - i;
+  if (i < N) return {2 * i * (i - 1), 4 * i, true};
+  if (i <= 3 * N) return {2 * N * (N - 1) + 4 * N * (i - N), 4 * N, ((i - N + 1) & 1) != 0};
+  return {12 * N * N - 2 * k * (k + 1), 4 * k, true};
 }
 
 // One block per ring.
@@ -212,7 +227,7 @@ k_ring_transform(const float* __restrict__ map, const float4* __restrict__ T, in
                  int32_t lmax, int32_t nrings, float4* __restrict__ F) {
   extern __shared__ __align__(16) cxs sh[];
   const int r = blockIdx.x;
-  const Ring g = ring_geom(N, r);
+  const RingSpan g = ring_span(N, r);
   const int n = g.n, L = n / 2, N8 = 8 * N;
   const float* px = map + g.start;
   // X_k from Z_k and Z_{L-k}
@@ -233,7 +248,7 @@ k_ring_transform(const float* __restrict__ map, const float4* __restrict__ T, in
       X[k] = cx_st(real_dft(cx_ld(Z[bit_rev(k & (L - 1), b)]),
                             cx_ld(Z[bit_rev((L - k) & (L - 1), b)]), cx_of(__ldg(T + k * ts))));
     __syncthreads();
-    const bool shifted = g.phi0_pi != 0.0;                   // phi_0 = pi / n or 0
+    const bool shifted = g.shifted;                          // phi_0 = pi / n or 0
     for (int m = threadIdx.x; m <= lmax; m += kRingThreads) {
       const int k = m & (n - 1);
       cx v = k <= L ? cx_ld(X[k]) : cx_conj(cx_ld(X[n - k]));
@@ -246,9 +261,8 @@ k_ring_transform(const float* __restrict__ map, const float4* __restrict__ T, in
   cxs* B = sh;                                               // chirp, then Z [2i]
   cxs* U = sh + M;                                           // even z, then X [2i + 1]
   cxs* V = sh + 2 * M;                                       // odd z
-  float4* wf = reinterpret_cast<float4*>(sh + 3 * M);        // [i]
+  float4* wf = reinterpret_cast<float4*>(sh + 3 * M);        // [i + 1]
   fill_quarter(wf, i);
-  __syncthreads();
   for (int a = threadIdx.x; a < M; a += kRingThreads) {
     cx u{0ull, 0ull}, v{0ull, 0ull}, c{0ull, 0ull};
     if (a < i) {
@@ -284,7 +298,7 @@ k_ring_transform(const float* __restrict__ map, const float4* __restrict__ T, in
     U[k] = cx_st(real_dft(cx_ld(B[k == L ? 0 : k]), cx_ld(B[k == 0 ? 0 : L - k]),
                           quarter_root(wf, i, k)));
   __syncthreads();
-  const cx h1 = half_step(n);
+  const cx h1 = cx_of(wf[i]);
   for (int m = threadIdx.x; m <= lmax; m += kRingThreads) {
     const int k = m % n;
     const cx v = k <= L ? cx_ld(U[k]) : cx_conj(cx_ld(U[n - k]));
@@ -304,7 +318,7 @@ k_ring_synth(const float4* __restrict__ G, const float4* __restrict__ T, int32_t
              int32_t lmax, int32_t nrings, float* __restrict__ map) {
   extern __shared__ __align__(16) cxs sh[];
   const int r = blockIdx.x;
-  const Ring g = ring_geom(N, r);
+  const RingSpan g = ring_span(N, r);
   const int n = g.n, L = n / 2, N8 = 8 * N;
   float* px = map + g.start;
   auto fold = [&](cxs* H, auto term) {                       // H_k, k <= L
@@ -323,7 +337,7 @@ k_ring_synth(const float4* __restrict__ G, const float4* __restrict__ T, int32_t
     cxs* Z = sh;                                             // [L]
     cxs* H = sh + L;                                         // [L + 1]
     const int b = log2_of(L), ts = N8 / n, ps = 4 * N / n;
-    const bool shifted = g.phi0_pi != 0.0;
+    const bool shifted = g.shifted;
     fold(H, [&](int m) {
       const cx v = cx_of(G[(size_t)m * nrings + r]);
       return shifted ? cx_mul(v, cx_conj(cx_of(__ldg(T + ((m * ps) & (N8 - 1)))))) : v;
@@ -347,10 +361,9 @@ k_ring_synth(const float4* __restrict__ G, const float4* __restrict__ T, int32_t
   cxs* B = sh;                                               // H [2i + 1], then the chirp
   cxs* U = sh + M;
   cxs* V = sh + 2 * M;
-  float4* wf = reinterpret_cast<float4*>(sh + 3 * M);        // [i]
+  float4* wf = reinterpret_cast<float4*>(sh + 3 * M);        // [i + 1]
   fill_quarter(wf, i);
-  const cx h1 = half_step(n);
-  __syncthreads();
+  const cx h1 = cx_of(wf[i]);
   fold(B, [&](int m) {
     return cx_mul(cx_of(G[(size_t)m * nrings + r]), cx_conj(quarter_phase(wf, i, m, h1)));
   });
@@ -392,7 +405,7 @@ k_ring_synth(const float4* __restrict__ G, const float4* __restrict__ T, int32_t
   }
 }
 
-// Shared memory: three buffers of M <= 2N complex numbers and N - 1 roots (the
+// Shared memory: three buffers of M <= 2N complex numbers and N roots (the
 // belt rings' 4N + 1 complex numbers fit in that).
 static int ring_smem(int nside) { return 7 * nside * (int)sizeof(float4); }
 
