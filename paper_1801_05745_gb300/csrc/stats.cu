@@ -852,15 +852,18 @@ __device__ __forceinline__ int pdf_slot(float k, const PdfParam& pp) {
   return pdf_slot_exact(k, pp.lo, pp.hi, pp.scale, pp.nbins);
 }
 
+__device__ __forceinline__ float2 mean_pair(double mean) {
+  const float h = (float)mean;
+  return make_float2(h, (float)(mean - (double)h));
+}
 // One block's share of the moment pass: block vb of a grid of nb blocks of
 // kMT threads (every thread calls it).  Central power sums about `mean` into
-// out[0..2] (global; red holds 3 kMT / 32); PDF counts into the shared histogram.  Two
+// out[0..2] (global; red holds 6 kMT / 32, 16-byte aligned); PDF counts into the shared histogram.  Two
 // of a thread's pixels at a time, side by side in packed double-float.
 __device__ __forceinline__ void moments_block(const float* __restrict__ kappa, int npix,
-                                              double mean, const PdfParam& pp, int vb, int nb,
+                                              float2 mean, const PdfParam& pp, int vb, int nb,
                                               unsigned int* hist, double* red, double* out) {
-  const float mh = (float)mean;
-  const float ml = (float)(mean - (double)mh);
+  const float mh = mean.x, ml = mean.y;
   const u64 nmh = x2_pack(-mh, -mh), nml = x2_pack(-ml, -ml);
   dfx a2{0ull, 0ull}, a3{0ull, 0ull}, a4{0ull, 0ull};
   auto acc = [](dfx& a, dfx x) { a = dfx_add_raw(a, x); };
@@ -895,12 +898,13 @@ __device__ __forceinline__ void moments_block(const float* __restrict__ kappa, i
     const float k0 = kappa[p], k1 = both ? kappa[p + step] : k0;
     add_pair(k0, k1, both);
   }
-  // Over the lanes in double-float, over the warps in FP64, in fixed orders.  (FP64
-  // additions over the lanes kept the FP64 pipe 79% busy in a batch of small maps: 150
-  // maps of Nside 64, 174 us then, 119 now.)
+  // Over the lanes in double-float, over the halves and warps in FP64 by the lanes of
+  // one warp, in fixed orders.  (FP64 kept its pipe 79% busy in a batch of small maps when
+  // it added the lanes, 74% when every warp converted its sums: 150 maps of Nside 64 took
+  // 174 us, then 119, now 70.)
   const int w = threadIdx.x >> 5, ln = threadIdx.x & 31;
+  float4* part = reinterpret_cast<float4*>(red);       // [3][kMT / 32]
   dfx q[3] = {a2, a3, a4};
-  double v[3];
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     q[k] = dfx_norm(q[k].h, q[k].l);
@@ -910,16 +914,15 @@ __device__ __forceinline__ void moments_block(const float* __restrict__ kappa, i
       q[k] = dfx_norm(q[k].h, q[k].l);
     }
     const float2 h = x2_get(q[k].h), l = x2_get(q[k].l);
-    v[k] = ((double)h.x + (double)l.x) + ((double)h.y + (double)l.y);   // (used in lane 0)
+    if (ln == 0) part[kMT / 32 * k + w] = make_float4(h.x, l.x, h.y, l.y);
   }
   __syncthreads();
-  if (ln == 0)
-    for (int k = 0; k < 3; ++k) red[kMT / 32 * k + w] = v[k];
-  __syncthreads();
-  if (threadIdx.x < 3) {
-    double t = 0.0;
-    for (int i = 0; i < kMT / 32; ++i) t += red[kMT / 32 * threadIdx.x + i];
-    out[threadIdx.x] = t;
+  static_assert(3 * kMT / 32 <= 32, "one warp adds the warps' sums");
+  if (w == 0) {
+    const float4 p = ln < 3 * kMT / 32 ? part[ln] : make_float4(0.f, 0.f, 0.f, 0.f);
+    double v = ((double)p.x + (double)p.y) + ((double)p.z + (double)p.w);
+    for (int o = kMT / 64; o > 0; o >>= 1) v += __shfl_down_sync(0xFFFFFFFFu, v, o);
+    if (ln < 3 * kMT / 32 && ln % (kMT / 32) == 0) out[ln / (kMT / 32)] = v;
   }
 }
 
@@ -975,13 +978,13 @@ k_moments(const float* __restrict__ kappa, int npix, const double* __restrict__ 
           unsigned long long* __restrict__ pdf /*[nbins+3]*/, double* __restrict__ m,
           unsigned int* __restrict__ ticket) {
   extern __shared__ unsigned int hist[];   // [nbins + 3]
-  __shared__ double red[3 * kMT / 32];
-  __shared__ double mean_s;
+  __shared__ __align__(16) double red[6 * kMT / 32];
+  __shared__ float2 mean_s;                // the mean as a double-float
   __shared__ bool last_s;
   for (int i = threadIdx.x; i < pp.nbins + 3; i += blockDim.x) hist[i] = 0;
   if (threadIdx.x < 32) {
     const double s = warp_sum_fixed(ksum_part, nksum, 1);   // fixed order
-    if (threadIdx.x == 0) mean_s = s / double(npix);
+    if (threadIdx.x == 0) mean_s = mean_pair(s / double(npix));
   }
   __syncthreads();
   moments_block(kappa, npix, mean_s, pp, blockIdx.x, gridDim.x, hist, red, part + 3 * blockIdx.x);
@@ -1173,8 +1176,8 @@ k_batch_kappa(const __grid_constant__ BatchArgs ba) {
 __global__ void __launch_bounds__(kMT)
 k_batch_moments(const __grid_constant__ BatchArgs ba, const __grid_constant__ PdfParam pp) {
   extern __shared__ unsigned int hist[];   // [nbins + 3]
-  __shared__ double red[3 * kMT / 32];
-  __shared__ double mean_s;
+  __shared__ __align__(16) double red[6 * kMT / 32];
+  __shared__ float2 mean_s;                // the mean as a double-float
   __shared__ bool last_s;
   const int r = blockIdx.y;
   const double* ks = ba.ksum + (size_t)r * ba.gk;
@@ -1183,7 +1186,7 @@ k_batch_moments(const __grid_constant__ BatchArgs ba, const __grid_constant__ Pd
   for (int i = threadIdx.x; i < ba.nbins + 3; i += blockDim.x) hist[i] = 0;
   if (threadIdx.x < 32) {
     const double s = warp_sum_fixed(ks, ba.gk, 1);          // fixed order, as k_moments
-    if (threadIdx.x == 0) mean_s = s / double(ba.npix);
+    if (threadIdx.x == 0) mean_s = mean_pair(s / double(ba.npix));
   }
   __syncthreads();
   moments_block(ba.kappa + (size_t)r * ba.npix, ba.npix, mean_s, pp, blockIdx.x, ba.gm, hist, red,
