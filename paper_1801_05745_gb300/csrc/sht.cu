@@ -141,7 +141,7 @@ __device__ __forceinline__ double sht_w(int k) {
 // 64, 8 now).
 __global__ void __launch_bounds__(64)
 k_sht_tables(int32_t N, int32_t lmax, float4* __restrict__ T, double* __restrict__ tab,
-             float4* __restrict__ pair) {
+             float4* __restrict__ pair, double* __restrict__ sin_d) {
   const int n8 = 8 * N, nl = (lmax + 2 + 31) / 32 * 32;              // (whole warps per part)
   int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j < n8) {
@@ -156,6 +156,7 @@ k_sht_tables(int32_t N, int32_t lmax, float4* __restrict__ T, double* __restrict
     const int i = j + 1;                                             // (whole numbers below 2^22)
     pair[j] = make_float4((float)(i < N ? 3 * N * N - i * i : 2 * N * (2 * N - i)), (float)g.z,
                           (float)g.s, 0.f);
+    sin_d[j] = g.s;
     return;
   }
   j -= 2 * N;
@@ -213,27 +214,44 @@ __device__ __forceinline__ bool leg_negligible(int lmax, int m, float c, float s
 // starts from sin(theta)^{m0} by repeated squaring, as (mantissa in [1/2, 1),
 // binary exponent) so that nothing underflows, and steps through its run by
 // products with sin(theta).  Long runs share the squarings, short ones the
-// chip: 64 orders fill it at Nside 1024 (0.14 ms), and small maps take the
+// chip: 64 orders fill it at Nside 1024 (0.09 ms), and small maps take the
 // longest run that still gives every SM a block.
+//
+// Bound by the FP64 pipe: per coefficient two products and the split, six
+// instructions of it; exponents, the range test and the widening of the high part
+// are integer operations on the bits, and sin(theta) comes from the tables.  (With
+// frexp, an FP64 comparison and ring_geom per thread 69 us at Nside 512, lmax 1535,
+// and 14 us at Nside 64, lmax 150; now 37 and 8.)
 struct MantExp { double m; int e; };
+// x > 0 (normal) as mantissa in [1/2, 1) and exponent
+__device__ __forceinline__ MantExp me_split(double x) {
+  const int hi = __double2hiint(x);
+  return {__hiloint2double((hi & 0x000FFFFF) | 0x3FE00000, __double2loint(x)), (hi >> 20) - 1022};
+}
 __device__ __forceinline__ MantExp me_mul(MantExp a, MantExp b) {
-  int d;
-  const double x = frexp(a.m * b.m, &d);
-  return {x, a.e + b.e + d};
+  const MantExp r = me_split(a.m * b.m);
+  return {r.m, a.e + b.e + r.e};
+}
+// double-float of |x| in [1/2, 1): the high part is a normal FP32 number
+__device__ __forceinline__ float2 split_unit(double x) {
+  const float h = __double2float_rn(x);
+  const unsigned b = __float_as_uint(h);
+  const double hd = __hiloint2double(
+      (int)((b & 0x80000000u) | (((b & 0x7FFFFFFFu) >> 3) + (896u << 20))), (int)(b << 29));
+  return make_float2(h, __double2float_rn(x - hd));
 }
 __global__ void __launch_bounds__(256)
-k_lmm(int32_t N, int32_t lmax, int32_t npairs, int32_t run, const double* __restrict__ cm,
-      float2* __restrict__ mu, int32_t* __restrict__ ex) {
+k_lmm(int32_t lmax, int32_t npairs, int32_t run, const double* __restrict__ cm,
+      const double* __restrict__ sin_d, float2* __restrict__ mu, int32_t* __restrict__ ex) {
   const int nrun = lmax / run + 1;
   const int64_t total = (int64_t)npairs * nrun;
   for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total;
        t += (int64_t)gridDim.x * blockDim.x) {
     const int p = int(t % npairs), j = int(t / npairs);
-    const Ring g = ring_geom(N, p);
+    const double sn = sin_d[p];                 // in (0, 1]
     const int m0 = run * j, mend = min(lmax, m0 + run - 1);
     MantExp r{0.5, 1};                          // 1
-    MantExp b;
-    b.m = frexp(g.s, &b.e);
+    MantExp b = me_split(sn);
     for (int k = m0; k; k >>= 1) {              // s^{m0}
       if (k & 1) r = me_mul(r, b);
       b = me_mul(b, b);
@@ -242,13 +260,14 @@ k_lmm(int32_t N, int32_t lmax, int32_t npairs, int32_t run, const double* __rest
     int e = r.e;
     for (int m = m0; m <= mend; ++m) {
       if (m > m0) {
-        v *= g.s;
-        if (v < 0x1p-500) { v *= 0x1p500; e -= 500; }
+        v *= sn;
+        if (__double2hiint(v) < 0x20B00000) { v *= 0x1p500; e -= 500; }   // below 2^-500
       }
-      int d;
-      const dfl f = df_from_d(frexp(cm[m] * v, &d));
-      mu[(size_t)m * npairs + p] = make_float2(f.h, f.l);
-      ex[(size_t)m * npairs + p] = e + d;
+      const double c = cm[m] * v;               // (of either sign, never 0)
+      const int hi = __double2hiint(c);
+      mu[(size_t)m * npairs + p] = split_unit(
+          __hiloint2double((hi & (int)0x800FFFFF) | 0x3FE00000, __double2loint(c)));
+      ex[(size_t)m * npairs + p] = e + ((hi >> 20) & 0x7FF) - 1022;
     }
   }
 }
@@ -761,6 +780,7 @@ static ufc_status sht_space(ufc_ctx* c, int nside, int lmax, int nchunk, ShtSpac
   const size_t o_roots = piece((size_t)8 * nside * sizeof(float4));
   const size_t o_tab = piece((size_t)4 * kShtTab * sizeof(double));
   const size_t o_pair = piece(npairs * sizeof(float4));
+  const size_t o_sin = piece(npairs * sizeof(double));
   const size_t o_ring = piece((size_t)(lmax + 1) * nrings * sizeof(float4));
   const size_t o_mu = piece((size_t)(lmax + 1) * npairs * sizeof(float2));
   const size_t o_ex = piece((size_t)(lmax + 1) * npairs * sizeof(int32_t));
@@ -770,6 +790,7 @@ static ufc_status sht_space(ufc_ctx* c, int nside, int lmax, int nchunk, ShtSpac
   float4* roots = reinterpret_cast<float4*>(ws + o_roots);
   double* tab = reinterpret_cast<double*>(ws + o_tab);
   float4* pair = reinterpret_cast<float4*>(ws + o_pair);
+  double* sin_d = reinterpret_cast<double*>(ws + o_sin);
   o.tb = ShtTables{roots, tab, tab + kShtTab, tab + 2 * kShtTab, tab + 3 * kShtTab, pair,
                    1.0 / (3.0 * (double)nside * (double)nside)};
   o.ring = reinterpret_cast<float4*>(ws + o_ring);
@@ -779,7 +800,8 @@ static ufc_status sht_space(ufc_ctx* c, int nside, int lmax, int nchunk, ShtSpac
   {
     ProfScope ps_(c, "k_sht_tables");
     const int n = 10 * nside + 4 * ((lmax + 2 + 31) / 32 * 32);
-    k_sht_tables<<<(n + 63) / 64, 64, 0, c->stream>>>(nside, lmax, roots, tab, pair);
+    k_sht_tables<<<(n + 63) / 64, 64, 0, c->stream>>>(nside, lmax, roots, tab, pair,
+                                                        sin_d);
   }
   {
     ProfScope ps_(c, "k_lmm");
@@ -787,7 +809,7 @@ static ufc_status sht_space(ufc_ctx* c, int nside, int lmax, int nchunk, ShtSpac
     while (run > 4 && (int64_t)npairs * (lmax / run + 1) < 256ll * c->num_sms) run /= 2;
     const int64_t lt = (int64_t)npairs * (lmax / run + 1);
     k_lmm<<<(int)std::min<int64_t>((lt + 255) / 256, 8 * c->num_sms), 256, 0, c->stream>>>(
-        nside, lmax, (int)npairs, run, o.tb.cm, o.mu, o.ex);
+        lmax, (int)npairs, run, o.tb.cm, sin_d, o.mu, o.ex);
   }
   UFC_CUDA(c, cudaGetLastError());
   return UFC_OK;
