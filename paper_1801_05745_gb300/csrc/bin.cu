@@ -81,12 +81,11 @@ __device__ __forceinline__ uint32_t dense_key(int32_t key, int32_t npix, const K
   return (uint32_t((b - o.shell0) * o.nblk + blk) << kOffBits) | uint32_t(pix - blk * kBlockPix);
 }
 
-// Appends the keys of lanes with `want` to the warp's chunk of the dense
+// Appends the keys of lanes with `want` (ballot m) to the warp's chunk of the dense
 // array (all 32 lanes call this together).
-__device__ __forceinline__ void dense_append(WarpChunk& wc, bool want, uint32_t v,
+__device__ __forceinline__ void dense_append(WarpChunk& wc, unsigned m, bool want, uint32_t v,
                                              const KeyOut& o) {
   const unsigned full = 0xFFFFFFFFu;
-  unsigned m = __ballot_sync(full, want);
   int lane = threadIdx.x & 31;
   // every lane has a key and the chunk stays open (most calls of the pixel
   // stage): no ranks
@@ -319,7 +318,7 @@ __device__ __forceinline__ void fast_particle(bool have, float x, float y, float
         else atomicAdd(o.hist + bucket, 1u);
       }
     }
-    dense_append(fc.wc, key >= 0, dkey, o);
+    dense_append(fc.wc, __ballot_sync(0xFFFFFFFFu, key >= 0), key >= 0, dkey, o);
   }
   fc.n_keyed += key >= 0;
 }
@@ -708,7 +707,7 @@ k_fast_stream(const float* __restrict__ xyz, int64_t n, int64_t p_off, int32_t b
           }
           // rare (one increment in 32768 per counter): a warp-uniform test first
           if (SH && __any_sync(0xFFFFFFFFu, wrapped) && wrapped) hist16_carry(h32, ghist, bucket);
-          dense_append(fc.wc, ok, dk, o);
+          dense_append(fc.wc, m, ok, dk, o);
         }
       };
       const int need = h < kWGroups ? 32 : 1;
@@ -745,7 +744,7 @@ __device__ __forceinline__ void emit_late(int32_t key, int64_t p, int32_t npix,
   } else {
     uint32_t dk = key >= 0 ? dense_key(key, npix, o) : 0u;
     if (key >= 0 && UFC_IDX_OK(dk >> kOffBits, o.nbuckets, 1)) atomicAdd(o.hist + (dk >> kOffBits), 1u);
-    dense_append(wc, key >= 0, dk, o);
+    dense_append(wc, __ballot_sync(0xFFFFFFFFu, key >= 0), key >= 0, dk, o);
   }
 }
 
