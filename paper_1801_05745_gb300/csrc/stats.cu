@@ -390,7 +390,7 @@ k_kappa_finish(const double* __restrict__ part, float ch, float cl, int npix,
 //
 // Bound by the latency that is left: 60 shells at Nside 1024 take 750 us for 3.0 GB
 // read once (4.0 TB/s, 60% of the copy rate; 53% issue, FMA pipe 49%), with waits
-// for loads and the barriers around phase 2; 140 shells at Nside 512 595 us (3.0
+// for loads and the barriers around phase 2; 140 shells at Nside 512 554 us (3.2
 // TB/s).  Two reads with 64-bit integer multiply-adds took 1080 and 1370 us.  A
 // batch of 8 shells in flight while 8 are added (80 registers, three blocks per
 // SM) against none: 930; 4 shells: 765; two blocks with 16: 830.  256-pixel tiles for
@@ -434,11 +434,11 @@ __host__ __device__ constexpr int adj_ldb(int nt) { return 2 * nt + 32; }    // 
 // (row strides of 8 and 16 words modulo 32: the fragments' loads meet no bank
 // conflict)
 __host__ __device__ constexpr int adj_batch(int nt) { return nt < 256 ? 16 : 8; }  // shells a fetch
-__host__ __device__ constexpr int adj_rows(int nt, int S) {       // whole pairs of batches
-  return (S + 2 * adj_batch(nt) - 1) / (2 * adj_batch(nt)) * (2 * adj_batch(nt));
+__host__ __device__ constexpr int adj_rows(int S) {               // whole batches, or pairs
+  return (S + 15) / 16 * 16;
 }
 __host__ __device__ inline size_t adj_smem(int nt, int S, bool g) {
-  const size_t mp = adj_rows(nt, S), nc = adj_cols(g);
+  const size_t mp = adj_rows(S), nc = adj_cols(g);
   return mp * adj_lda(nt) + nc * adj_ldb(nt) * 2 + mp * nc * 8 + (size_t)S * sizeof(AdjRow) +
          mp * sizeof(float4);
 }
@@ -473,7 +473,7 @@ k_adj_main(const int32_t* __restrict__ counts, const __grid_constant__ Coef cf,
   constexpr int LDA = adj_lda(NT), LDB = adj_ldb(NT);
   if (kappa_out) clear_pdf(pdf, npdf);
   const int S = cf.nshell, npix = cf.npix, np2 = npix >> 1;
-  const int mt_n = (S + 15) >> 4, mp = adj_rows(NT, S);      // tiles of 16 shells; rows held
+  const int mt_n = (S + 15) >> 4, mp = adj_rows(S);      // tiles of 16 shells; rows held
   uint8_t* An = adj_sm;                                      // [mp][LDA] a byte of the counts
   uint16_t* Bq = reinterpret_cast<uint16_t*>(An + (size_t)mp * LDA);            // [NC][LDB]
   long long* sums = reinterpret_cast<long long*>(Bq + (size_t)NC * LDB);        // [mp][NC]
@@ -590,14 +590,17 @@ k_adj_main(const int32_t* __restrict__ counts, const __grid_constant__ Coef cf,
   for (int i = 0; i < 4 * kA; ++i) pw[i >> 2][i & 3] = f2{0.f, 0.f};
   f2 ks{0.f, 0.f};                         // this thread's sum of the FP32 map (kappa_out)
   // the counts in batches of kB shells, the next one's loads in flight while one
-  // is added; the first batch of the next tile is fetched before phase 2
+  // is added (in a second set of registers, or in the same one by one: the first
+  // is faster in wide blocks, where the second spills at 80 registers, 750 against 800
+  // us for 60 shells at Nside 1024; the second in narrow ones, 595 against 554 us
+  // for 140 shells at Nside 512); the first batch of the next tile before phase 2
   constexpr int kB = adj_batch(NT);
   // (q: row b0 of the thread's pixels; whole tiles and batches without tests)
   const uint32_t stride = (uint32_t)npix * 4u;
   auto row = [&](const char* q, int u) {
     return reinterpret_cast<const int2*>(q + (size_t)stride * (uint32_t)u);
   };
-  auto fetch = [&](int2 (&v)[kB], const char* q, int b0, int tile) {
+  auto fetch = [&](int2* v, const char* q, int b0, int tile) {
     if ((tile + 1) * NT <= np2 && b0 + kB <= S) {            // (uniform)
 #pragma unroll
       for (int u = 0; u < kB; ++u) v[u] = __ldcs(row(q, u));
@@ -610,7 +613,8 @@ k_adj_main(const int32_t* __restrict__ counts, const __grid_constant__ Coef cf,
   };
   const char* base = reinterpret_cast<const char*>(counts) + 8 * (size_t)tid;
   auto tile_at = [&](int tile) { return base + (size_t)tile * (8 * NT); };
-  int2 v0[kB], v1[kB];
+  constexpr bool kTurn = NT < 256;
+  int2 v0[kB], v1[kTurn ? 1 : kB];
   fetch(v0, tile_at(blockIdx.x), 0, blockIdx.x);
   __syncthreads();
   for (int tile = blockIdx.x; tile < ntile; tile += gridDim.x) {
@@ -621,29 +625,53 @@ k_adj_main(const int32_t* __restrict__ counts, const __grid_constant__ Coef cf,
     uint8_t* arow = An + 2 * tid;
     dfx a{0ull, 0ull};
     unsigned nor = 0u;
-    auto add = [&](const int2 (&v)[kB], int b0) {
-#pragma unroll
-      for (int u = 0; u < kB; ++u) {
-        const int2 n = v[u];
-        nor |= (unsigned)n.x | (unsigned)n.y;
-        *reinterpret_cast<uint16_t*>(arow + (size_t)(b0 + u) * LDA) =
-            (uint16_t)__byte_perm(n.x, n.y, 0x0040);
-        if constexpr (!EXT) {
-          const float4 cb = coef[b0 + u];
-          const u64 ah = x2_pack(cb.x, cb.y), al = x2_pack(cb.z, cb.w);
-          kappa_mac(a, ah, al, kappa_bits(n.x, n.y));          // (larger counts: below)
-        }
+    auto take = [&](int2 n, int b) {
+      nor |= (unsigned)n.x | (unsigned)n.y;
+      *reinterpret_cast<uint16_t*>(arow + (size_t)b * LDA) =
+          (uint16_t)__byte_perm(n.x, n.y, 0x0040);
+      if constexpr (!EXT) {                    // (counts of 2^23 and more: below)
+        const float4 cb = coef[b];
+        kappa_mac(a, x2_pack(cb.x, cb.y), x2_pack(cb.z, cb.w), kappa_bits(n.x, n.y));
       }
     };
+    if constexpr (kTurn) {
+      // a register takes the row kB further on as soon as its counts are used
+      const char* q = tile_at(tile);
 #pragma unroll 1
-    for (int b0 = 0; b0 < mp; b0 += 2 * kB) {
-      const char* q = tile_at(tile) + (size_t)stride * (uint32_t)b0;
-      fetch(v1, q + (size_t)stride * kB, b0 + kB, tile);
-      add(v0, b0);
-      const bool more = b0 + 2 * kB < mp;                    // else the next tile's first batch
-      const int nt = more ? tile : tile + (int)gridDim.x;
-      fetch(v0, more ? q + (size_t)stride * (2 * kB) : tile_at(nt), more ? b0 + 2 * kB : 0, nt);
-      add(v1, b0 + kB);
+      for (int b0 = 0; b0 < mp; b0 += kB) {
+        const bool more = b0 + kB < mp;                      // else the next tile's first batch
+        const int nb0 = more ? b0 + kB : 0, nt = more ? tile : tile + (int)gridDim.x;
+        q = more ? q + (size_t)stride * kB : tile_at(nt);
+        if ((nt + 1) * NT <= np2 && nb0 + kB <= S) {         // (uniform)
+#pragma unroll
+          for (int u = 0; u < kB; ++u) {
+            const int2 n = v0[u];
+            v0[u] = __ldcs(row(q, u));
+            take(n, b0 + u);
+          }
+        } else {
+          const bool in = nt * NT + tid < np2;
+#pragma unroll
+          for (int u = 0; u < kB; ++u) {
+            const int2 n = v0[u];
+            v0[u] = in && nb0 + u < S ? __ldcs(row(q, u)) : make_int2(0, 0);
+            take(n, b0 + u);
+          }
+        }
+      }
+    } else {
+#pragma unroll 1
+      for (int b0 = 0; b0 < mp; b0 += 2 * kB) {
+        const char* q = tile_at(tile) + (size_t)stride * (uint32_t)b0;
+        fetch(v1, q + (size_t)stride * kB, b0 + kB, tile);
+#pragma unroll
+        for (int u = 0; u < kB; ++u) take(v0[u], b0 + u);
+        const bool more = b0 + 2 * kB < mp;                  // else the next tile's first batch
+        const int nt = more ? tile : tile + (int)gridDim.x;
+        fetch(v0, more ? q + (size_t)stride * (2 * kB) : tile_at(nt), more ? b0 + 2 * kB : 0, nt);
+#pragma unroll
+        for (int u = 0; u < kB; ++u) take(v1[u], b0 + kB + u);
+      }
     }
     f2 av[2];
     {
@@ -1392,9 +1420,9 @@ static ufc_status adjoint_sums(ufc_ctx* c, const int32_t* counts, int S, int nsi
   const int npix = 12 * nside * nside;
   // threads per block and blocks per SM: 512-pixel tiles where two blocks' shared
   // memory fits an SM (up to 128 shells, 96 with g), 256-pixel tiles above
-  // (Nside 512, wide against narrow tiles: 100 shells 366 and 450 us, 128 shells
-  // 421 and 482, 90 with g 349 and 402; 140 shells, one wide block per SM, 657 and
-  // 529)
+  // (Nside 512, wide against narrow tiles: 100 shells 366 and 405 us, 128 shells
+  // 421 and 451, 90 with g 349 and 397; 140 shells, one wide block per SM, 657
+  // and 515)
   const size_t sm_bytes = (size_t)c->smem_optin;             // (per block; an SM holds 1 KB more)
   const bool wide = 2 * (adj_smem(256, S, g != nullptr) + 1024) <= sm_bytes + 1024;
   const int nt = wide ? 256 : 128;
