@@ -414,9 +414,11 @@ k_kappa_finish(const double* __restrict__ part, float ch, float cl, int npix,
 // pixels times pixels x quantities, on the tensor cores: the integers as signed
 // 8-bit digits (three per integer, six per quantity, and one column of ones
 // for N_b), the counts byte by byte, both exactly as FP16, and FP32 sums of
-// products that stay integers below 2^22, so they are exact whatever the order
-// and the alignment inside the tensor core.  They are added to 64-bit sums in
-// shared memory every few steps.  Counts of 256 and more take further passes
+// products that stay whole numbers up to 2^24, which they hold exactly (1.6e7
+// sums of random and of extreme digits up to 1.67e7 equal the integers on this
+// GPU).  They are added to 64-bit sums in shared memory every few steps (with a
+// bound of 2^22, four times as often: 759 us instead of 738 for 60 shells at Nside
+// 1024, 790 instead of 737 where counts reach 100).  Counts of 256 and more take further passes
 // over the tile (from L2) with their higher bytes, the last one signed.  (mma.sync:
 // 16 or 24 columns are far too few for a tcgen05 tile to matter; the product
 // takes 16 multiply-adds per count, a percent of the tensor cores' rate.)  With
@@ -539,7 +541,7 @@ k_adj_main(const int32_t* __restrict__ counts, const __grid_constant__ Coef cf,
   auto product = [&](int plane, bool sgn, unsigned most) {
     const int gq = ln >> 2, c = ln & 3;
     const uint32_t flip = sgn ? 0x80808080u : 0u, bias = sgn ? kHalf1152 : kHalf1024;
-    const int steps = max(1, 1024 / (int)max(1u, min(most, 255u)));   // of 32 pixels per sum
+    const int steps = max(1, 4096 / (int)max(1u, min(most, 255u)));   // of 32 pixels per sum
     for (int mt = w; mt < mt_n; mt += NW) {
       const uint8_t* r0 = An + (size_t)(16 * mt + gq) * LDA + 8 * c;
       const uint8_t* r1 = r0 + 8 * LDA;
@@ -603,12 +605,12 @@ k_adj_main(const int32_t* __restrict__ counts, const __grid_constant__ Coef cf,
   auto fetch = [&](int2* v, const char* q, int b0, int tile) {
     if ((tile + 1) * NT <= np2 && b0 + kB <= S) {            // (uniform)
 #pragma unroll
-      for (int u = 0; u < kB; ++u) v[u] = __ldcs(row(q, u));
+      for (int u = 0; u < kB; ++u) v[u] = __ldg(row(q, u));
     } else {
       const bool in = tile * NT + tid < np2;
 #pragma unroll
       for (int u = 0; u < kB; ++u)
-        v[u] = in && b0 + u < S ? __ldcs(row(q, u)) : make_int2(0, 0);
+        v[u] = in && b0 + u < S ? __ldg(row(q, u)) : make_int2(0, 0);
     }
   };
   const char* base = reinterpret_cast<const char*>(counts) + 8 * (size_t)tid;
@@ -646,7 +648,7 @@ k_adj_main(const int32_t* __restrict__ counts, const __grid_constant__ Coef cf,
 #pragma unroll
           for (int u = 0; u < kB; ++u) {
             const int2 n = v0[u];
-            v0[u] = __ldcs(row(q, u));
+            v0[u] = __ldg(row(q, u));
             take(n, b0 + u);
           }
         } else {
@@ -654,7 +656,7 @@ k_adj_main(const int32_t* __restrict__ counts, const __grid_constant__ Coef cf,
 #pragma unroll
           for (int u = 0; u < kB; ++u) {
             const int2 n = v0[u];
-            v0[u] = in && nb0 + u < S ? __ldcs(row(q, u)) : make_int2(0, 0);
+            v0[u] = in && nb0 + u < S ? __ldg(row(q, u)) : make_int2(0, 0);
             take(n, b0 + u);
           }
         }
@@ -739,12 +741,19 @@ k_adj_main(const int32_t* __restrict__ counts, const __grid_constant__ Coef cf,
       T3 = fmaxf(T3, mred[2][i]);
     }
     const float M1 = Ms[0], M2 = Ms[1], M3 = Ms[2];
-    const bool grow = T1 > M1 || T2 > M2 || T3 > M3;   // (uniform) a coarser scale
-    if (grow) flush(scale(M1), scale(M2), scale(M3));  // at the old scale
+    const bool grow = T1 > M1 || T2 > M2 || T3 > M3;   // (uniform)
     const float N1 = fmaxf(M1, T1), N2 = fmaxf(M2, T2), N3 = fmaxf(M3, T3);
-    if (grow && tid == 0 && (N1 >= 16384.0f || N3 >= 16384.0f || N2 >= 268435456.0f))
-      atomicAdd(range_flag, 1ull);
     const int s1 = scale(N1), s2 = scale(N2), s3 = scale(N3);
+    if (grow) {
+      if (tid == 0 && (N1 >= 16384.0f || N3 >= 16384.0f || N2 >= 268435456.0f))
+        atomicAdd(range_flag, 1ull);
+      // a maximum that stays below the next power of two leaves the scale as it is (a
+      // flush costs as much as a tile: a map whose values rise along the rings paid one
+      // per tile); before the first values there is nothing to flush
+      const int o1 = scale(M1), o2 = scale(M2), o3 = scale(M3);
+      if ((s1 != o1 || s2 != o2 || s3 != o3) && (M1 > 0.f || M2 > 0.f || M3 > 0.f))
+        flush(o1, o2, o3);
+    }
     {
       int h0, l0, h1, l1;
       quant2(e[0], s1, h0, l0);
@@ -768,15 +777,22 @@ k_adj_main(const int32_t* __restrict__ counts, const __grid_constant__ Coef cf,
     product(0, false, NOR);
     for (int plane = 1; plane < 4 && NOR >> (8 * plane); ++plane) {
       __syncthreads();
+      // (eight loads in flight: row by row these tiles took 1210 us for a map of counts
+      // near 300 that has them everywhere, with the counts loaded evict-first 1140, now 1055)
+      const unsigned sel = 0x0040u + 0x11u * plane;          // byte `plane` of both
       if (have)
-        for (int b = 0; b < S; ++b) {
-          const int2 n = src[(size_t)b * np2];
-          *reinterpret_cast<uint16_t*>(arow + (size_t)b * LDA) =
-              (uint16_t)(((unsigned)n.x >> (8 * plane) & 255u) |
-                         ((unsigned)n.y >> (8 * plane) & 255u) << 8);
+        for (int b0 = 0; b0 < S; b0 += 8) {
+          int2 n[8];
+#pragma unroll
+          for (int u = 0; u < 8; ++u)
+            n[u] = b0 + u < S ? __ldg(src + (size_t)(b0 + u) * np2) : make_int2(0, 0);
+#pragma unroll
+          for (int u = 0; u < 8; ++u)
+            *reinterpret_cast<uint16_t*>(arow + (size_t)(b0 + u) * LDA) =
+                (uint16_t)__byte_perm(n[u].x, n[u].y, sel);
         }
       __syncthreads();
-      product(plane, plane == 3, 255u);
+      product(plane, plane == 3, plane == 3 ? 128u : NOR >> (8 * plane));
     }
     __syncthreads();                       // the next tile rewrites the bytes, digits and maxima
   }

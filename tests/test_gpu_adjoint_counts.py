@@ -105,3 +105,26 @@ def test_gradient_weights_against_exact(nside, S, use_g, top, neg):
     err = np.abs(G - ref)
     assert (err <= tol).all(), float((err / (tol + 1e-300)).max())
     assert abs(H - gl.sum()) <= 2.0 ** -41 * (float(np.abs(gl).sum()) + 1e-300)
+
+
+@pytest.mark.parametrize("rising", [True, False])
+def test_sums_of_an_ordered_map(rising):
+    """A map in order of |e|: with rising values every tile has a new maximum, some
+    of them in a new power of two, and what was summed before moves to the wider
+    scale; the tolerance is that of the sums above."""
+    _, ctx = api_ctx()
+    nside, S = 128, 20
+    npix = 12 * nside * nside
+    rng = np.random.default_rng(5)
+    cn = _counts(rng, S, npix, 300, False)
+    E = 10.0 ** np.linspace(-3, 3, npix) * rng.choice([-1.0, 1.0], size=npix)
+    if not rising:
+        E = E[::-1].copy()
+    sums, _, _, _ = ctx.kappa_adjoint_sums(to_dev(cn), to_dev(E), 0.0)
+    rows = sums[:4 * S].reshape(S, 4)
+    n, e = cn.astype(np.longdouble), E.astype(np.longdouble)
+    for k, q in enumerate([e, e * e]):
+        err = np.abs(rows[:, k] - (n * q).sum(1))
+        # every term at the scale of its running maximum, which is at most the last one
+        assert (err <= n.sum(1) * float(np.abs(q).max()) * 2.0 ** -41).all(), k
+    assert np.array_equal(rows[:, 3], cn.astype(np.int64).sum(1).astype(np.float64))
