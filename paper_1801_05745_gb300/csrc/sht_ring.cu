@@ -178,7 +178,7 @@ __device__ __forceinline__ int bit_rev(int k, int b) { return (int)(__brev((unsi
 // (split once), the others as the double-float product of two of these; wf[i] =
 // w_{2n}.  (FP64 runs at 1/64 of the FP32 rate: with a sincospi per root, and w_2n
 // and the ring's geometry by every thread, its pipe was 42% busy and the 2047 rings of
-// Nside 512 took 380 us to synthesise, 324 now; the transform of Nside 64 24 us, 13
+// Nside 512 took 380 us to synthesise, 324 without; the transform of Nside 64 24 us, 13
 // now.)  Every thread calls it; ends with a barrier.
 __device__ __forceinline__ void fill_quarter(float4* wf, int i) {
   const int nd = min(i, 32) + (i - 1) / 32;              // roots formed directly, then w_2n
@@ -311,8 +311,11 @@ k_ring_transform(const float* __restrict__ map, const float4* __restrict__ T, in
 // the terms with m = -k mod n (1 <= m <= lmax), for k <= L (H_{n-k} = conj
 // H_k); then the inverse of the real DFT, map_j = sum_k H_k e^{2 pi i k j / n}:
 // Z_k = E_k + i O_k with E_k = H_k + conj H_{L-k}, O_k = (H_k - conj H_{L-k})
-// e^{2 pi i k / n}, and z = the inverse DFT of Z.  Each H_k is summed by one
-// thread in increasing m.
+// e^{2 pi i k / n}, and z = the inverse DFT of Z.  The terms of H_k are dealt to
+// as many threads as a short ring leaves free, each adding its own in increasing
+// m, and the parts added in order.  (One thread per H_k left the rings next to the
+// poles, 3 to 9 sums of hundreds of dependent loads, as the tail of the kernel: 350
+// us at Nside 512, lmax 1535, now 134.)
 __global__ void __launch_bounds__(kRingThreads, 2)
 k_ring_synth(const float4* __restrict__ G, const float4* __restrict__ T, int32_t N,
              int32_t lmax, int32_t nrings, float* __restrict__ map) {
@@ -321,12 +324,27 @@ k_ring_synth(const float4* __restrict__ G, const float4* __restrict__ T, int32_t
   const RingSpan g = ring_span(N, r);
   const int n = g.n, L = n / 2, N8 = 8 * N;
   float* px = map + g.start;
+  __shared__ cxs part_s[kRingThreads];
   auto fold = [&](cxs* H, auto term) {                       // H_k, k <= L
-    for (int k = threadIdx.x; k <= L; k += kRingThreads) {
+    auto some = [&](int k, int p, int np) {                  // part p of np
       cx h{0ull, 0ull};
-      for (int m = k; m <= lmax; m += n) h = cx_add(h, term(m));
-      for (int m = k ? n - k : n; m <= lmax; m += n) h = cx_add(h, cx_conj(term(m)));
-      H[k] = cx_st(h);
+      for (int m = k + p * n; m <= lmax; m += np * n) h = cx_add(h, term(m));
+      for (int m = (k ? n - k : n) + p * n; m <= lmax; m += np * n)
+        h = cx_add(h, cx_conj(term(m)));
+      return h;
+    };
+    const int np = kRingThreads / (L + 1);                   // (uniform)
+    if (np < 2) {
+      for (int k = threadIdx.x; k <= L; k += kRingThreads) H[k] = cx_st(some(k, 0, 1));
+      return;
+    }
+    if (threadIdx.x < (L + 1) * np)
+      part_s[threadIdx.x] = cx_st(some(threadIdx.x % (L + 1), threadIdx.x / (L + 1), np));
+    __syncthreads();
+    if (threadIdx.x <= L) {
+      cx h = cx_ld(part_s[threadIdx.x]);
+      for (int p = 1; p < np; ++p) h = cx_add(h, cx_ld(part_s[p * (L + 1) + threadIdx.x]));
+      H[threadIdx.x] = cx_st(h);
     }
   };
   auto z_of = [](cx hk, cx hl, cx w) {                       // H_k, H_{L-k}, e^{2 pi i k / n}
