@@ -478,7 +478,7 @@ __device__ __noinline__ int32_t key_exact_slow(const ShellTable& st, int32_t lo,
 //
 // Bound by instruction issue: about 6.3 warp instructions per particle in a box half of whose
 // particles are keyed, three quarters of the issue slots (ALU pipe 58%, FMA 28%, DRAM 25%).
-// Two boxes of 512^3 particles at Nside 512 take 1.57 ms; 1.61 when the block shared bulk
+// Two boxes of 512^3 particles at Nside 512 take 1.55 ms; 1.61 when the block shared bulk
 // copies of 3840 particles behind mbarriers (ring bookkeeping per chunk), 1.80 with circular
 // lists, range tests on the shell after the table and the periodic path's image loop as well.
 // Of a box whose particles are all keyed, 0.4 of the time is classification and streaming.
@@ -612,7 +612,7 @@ k_fast_stream(const float* __restrict__ xyz, int64_t n, int64_t p_off, int32_t b
             // NaN or overflowing r2 goes to the queue as well: the FP64 stage returns the
             // invalid key for non-finite coordinates and decides a finite overflow
             in = false;
-            und = j < nvalid && (!fin || !(r2 >= bd.r2_min));   // (near the observer: r == 0 is invalid)
+            und = j < nvalid && (!fin || !(r2 >= bd.r2_min));   // (near: r == 0 is invalid)
             if (fin && !und) {
               int e = int(a & 0x7FFFu) - 1;              // ends at the +inf sentinel
               for (;;) {
@@ -649,7 +649,8 @@ k_fast_stream(const float* __restrict__ xyz, int64_t n, int64_t p_off, int32_t b
               ++fc.n_keyed;
               if (MODE == kModeDense) {            // rare: straight to the global histogram
                 const uint32_t dk = dense_key(kx, npix, o);
-                if (UFC_IDX_OK(dk >> kOffBits, o.nbuckets, 1)) atomicAdd(ghist + (dk >> kOffBits), 1u);
+                if (UFC_IDX_OK(dk >> kOffBits, o.nbuckets, 1))
+                  atomicAdd(ghist + (dk >> kOffBits), 1u);
                 const unsigned long long at = atomicAdd(o.dense_count, 1ull);
                 if ((int64_t)at < o.dense_cap) o.dense[at] = dk;
               }
@@ -1374,7 +1375,7 @@ struct BinPlan {
 };
 
 // Particles per staged chunk of ufc_bin_host (402 MB); a multiple of 4, so
-// that every chunk starts 16-byte aligned for the bulk copies.
+// that every chunk starts 16-byte aligned for the asynchronous copies.
 constexpr int64_t kHostChunk = 1ll << 25;
 
 // Workspace of one binning call of total_img particle images in
@@ -1694,7 +1695,7 @@ ufc_status run_keys_pipeline(ufc_ctx* c, int mode_req, const float* const* xyz,
     smem = plan.smem_hist ? plan.nbuckets * 4 : 0;
   }
   // fast stage: one launch per box, or per staged chunk for host input
-  const int tma_smem = kWSmemBase +
+  const int stream_smem = kWSmemBase +
                        (plan.mode == kModeDense && plan.smem_hist ? ((plan.nbuckets + 1) / 2) * 4 : 0);
   for (int k = 0; k < nbox; ++k) {
     const int64_t step = xyz_host ? kHostChunk : std::max<int64_t>(n[k], 1);
@@ -1702,14 +1703,14 @@ ufc_status run_keys_pipeline(ufc_ctx* c, int mode_req, const float* const* xyz,
       const int64_t cnt = std::min(step, n[k] - p0);
       const float* src = xyz[k] + 3 * p0;
       if (xyz_host && (s = stage(k, p0, cnt))) return s;
-      const bool tma = (reinterpret_cast<uintptr_t>(src) & 15) == 0;
+      const bool aligned = (reinterpret_cast<uintptr_t>(src) & 15) == 0;
       ProfScope ps_(c, "k_fast");
-      if (tma) {
+      if (aligned) {
         qs.ovf_base = bp.bit_base[k];
 #define UFC_LAUNCH_STREAM(...)                                                                      \
   UFC_CUDA(c, cudaFuncSetAttribute(k_fast_stream<__VA_ARGS__>,                                      \
-                                   cudaFuncAttributeMaxDynamicSharedMemorySize, tma_smem));      \
-  k_fast_stream<__VA_ARGS__><<<c->num_sms, kWThreads, tma_smem, c->stream>>>(                                 \
+                                   cudaFuncAttributeMaxDynamicSharedMemorySize, stream_smem));   \
+  k_fast_stream<__VA_ARGS__><<<c->num_sms, kWThreads, stream_smem, c->stream>>>(                 \
       src, cnt, p0, k, bp.box[k], st, tab, lut_scale, bd, nside, (int32_t)npix, o, qs)
         if (plan.mode == kModeDense && plan.smem_hist) { UFC_LAUNCH_STREAM(kModeDense, true); }
         else if (plan.mode == kModeDense) { UFC_LAUNCH_STREAM(kModeDense, false); }

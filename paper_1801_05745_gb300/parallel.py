@@ -20,7 +20,7 @@ from __future__ import annotations
 def shard_range(n: int, rank: int, world: int, align: int = 1) -> tuple[int, int]:
     """[start, stop) of rank's contiguous share of n particles; every start is
     a multiple of `align` (4 keeps a shard of 12-byte particles on 16-byte
-    boundaries, which the binning's bulk copies need)."""
+    boundaries, which the binning's 16-byte copies need)."""
     units, rest = divmod(n, align)
     base, extra = divmod(units, world)
     start = (rank * base + min(rank, extra)) * align
