@@ -931,16 +931,25 @@ __device__ __forceinline__ void moments_block(const float* __restrict__ kappa, i
   };
   const int step = nb * kMT;
   int p = vb * kMT + threadIdx.x;
-  for (; p < npix - 3 * step; p += 4 * step) {         // four loads in flight
-    const float k0 = kappa[p], k1 = kappa[p + step], k2 = kappa[p + 2 * step],
-                k3 = kappa[p + 3 * step];
-    add_pair(k0, k1, true);
-    add_pair(k2, k3, true);
-  }
-  for (; p < npix; p += 2 * step) {
-    const bool both = p < npix - step;
-    const float k0 = kappa[p], k1 = both ? kappa[p + step] : k0;
-    add_pair(k0, k1, both);
+  if ((reinterpret_cast<uintptr_t>(kappa) & 15) == 0) {      // (12 nside^2 is a multiple of 4)
+    // four adjacent pixels per load, the next load in flight
+    const float4* k4 = reinterpret_cast<const float4*>(kappa);
+    const int ng = npix >> 2;
+    float4 v = p < ng ? k4[p] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+    for (; p < ng; p += step) {
+      const float4 w = v;
+      if (p + step < ng) v = k4[p + step];
+      add_pair(w.x, w.y, true);
+      add_pair(w.z, w.w, true);
+    }
+  } else {
+#pragma unroll 1
+    for (; p < npix; p += 2 * step) {
+      const bool both = p < npix - step;
+      const float k0 = kappa[p], k1 = both ? kappa[p + step] : k0;
+      add_pair(k0, k1, both);
+    }
   }
   // Over the lanes in double-float, over the halves and warps in FP64 by the lanes of
   // one warp, in fixed orders.  (FP64 kept its pipe 79% busy in a batch of small maps when
@@ -1009,7 +1018,8 @@ __device__ __forceinline__ void moments_final_block(const double* ksum_part, int
 // fewer pixels pays its prologue and its PDF's global atomics for little).  What
 // bounds the pass is the latency of a pixel's chain (load, shared-memory histogram, double-float
 // sums): with 2 blocks per SM and one pixel at a time it took 200 us for the
-// 12.6 M pixels of Nside 1024.
+// 12.6 M pixels of Nside 1024, with four scalar loads in flight 59, with four
+// pixels per load and the next load in flight 51 (6 blocks per SM 53, 8 55).
 static int moments_grid(int num_sms, int npix) {
   return std::min(4 * num_sms, (npix + 4 * kMT - 1) / (4 * kMT));
 }
