@@ -573,7 +573,7 @@ def main():
     bin_ms = sum(prof[k][0] for k in bin_kernels if k in prof) / args.steps
     bin_bytes = 12.0 * n_local + 4.0 * w.nshell * npix
     kap_ms = sum(prof[k][0] for k in ("k_kappa_partial", "k_adj_main", "k_moments",
-                                      "k_moments_final") if k in prof)
+                                      "k_adj_reduce") if k in prof)
     adj_launch = prof.get("k_adj_main", (0.0, 1))
     roof = {
         "bound": "hbm", "kernel": "k_fast",
