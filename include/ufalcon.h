@@ -562,7 +562,9 @@ ufc_status ufc_stats_vector(ufc_ctx *ctx, const double *moments_dev,
 
 /* A Welford state for d-dimensional vectors is 1 + d + d*d doubles:
  * count, mean[d], M2[d][d].  ufc_welford_update adds the nvec vectors
- * v_dev [nvec][d] in order (Welford/Chan update in FP64, device memory);
+ * v_dev [nvec][d] in order (Welford/Chan update in FP64, device memory; it
+ * uses nothing of the context but its stream: no workspace, and updates of
+ * different states may overlap with each other and with any other call);
  * ufc_welford_merge adds state b into state a (Chan et al. pairwise
  * formula); ufc_welford_finalize writes mean, cov = M2/(n - ddof) and
  * corr = cov_ij / sqrt(cov_ii cov_jj) (0 where a variance is 0), all device

@@ -844,11 +844,8 @@ ufc_status ufc_batched_stats(ufc_ctx* c, int32_t nreal, int32_t nbox, const floa
                             moments, pdf, stats, state);
   ufc_status s = reserve_bin_workspace(c, nbox, max_img, nshell, nside);
   if (s) return s;
-  // per-block partial sums of the kappa and moment kernels, and the new mean of
-  // the Welford update
-  if (!ws_get(c, kSlotPartials, (size_t)20 * c->num_sms * 8) ||
-      !ws_get(c, kSlotWelford, (size_t)d * 8))
-    return UFC_ERR_ALLOC;
+  // per-block partial sums of the kappa and moment kernels
+  if (!ws_get(c, kSlotPartials, (size_t)20 * c->num_sms * 8)) return UFC_ERR_ALLOC;
   // small maps: realisation r runs on lane r mod nlane, the lanes concurrently
   // (lane 0 is this context with the caller's scratch maps; the others have
   // their own count and kappa maps, workspace and stream)

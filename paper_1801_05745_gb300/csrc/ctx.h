@@ -18,7 +18,7 @@ struct ufc_ctx {
   int num_sms = 0;
   int smem_optin = 0;            // shared memory per block with opt-in (bytes)
   // grow-only device buffers, one per slot
-  static constexpr int kSlots = 19;
+  static constexpr int kSlots = 18;
   void* buf[kSlots] = {};
   size_t cap[kSlots] = {};
   void* counters = nullptr;      // ufc::BinCounters of the last binning call
@@ -78,7 +78,6 @@ enum Slot {
   kSlotLaneMap,    // a lane's count map and kappa map (ufc_batched_stats)
   kSlotBatchMaps,  // batched call: per-realisation maps and partial sums
   kSlotBatchDesc,  // batched call: items, coefficients and counters
-  kSlotWelford,    // the new mean of a Welford update
 };
 
 inline ufc_status set_err(ufc_ctx* c, ufc_status s, const char* fmt, ...) {

@@ -1076,8 +1076,13 @@ __global__ void k_stats_vector(const double* __restrict__ m, const unsigned long
 // of kWfRun vectors into the other of two buffers while the run before is
 // added.  (The chains are the same whatever the blocks: the result does not
 // depend on how the vectors are split over calls.)  Every block reads the old
-// mean; the blocks of the first column leave the new one in `mean_new`, and the
-// last block to finish (ticket, left at 0) copies it into the state.
+// mean and count, so they are written last: by a second launch, k_welford_mean,
+// which forms the mean's chain once more.  The update then keeps nothing outside
+// the caller's state: updates of different states may overlap on different
+// streams, and a captured one allocates nothing.  The batched call, which has
+// scratch of its own anyway, passes a place for the new mean and a count of
+// finished blocks (0 at launch) instead, and the last block to finish copies the
+// mean: 200 vectors' chain, formed again, takes some 20 us of latency.
 //
 // FP64 at 1/64 of the FP32 rate bounds it: one block of 1024 threads took 12 us
 // for one vector of 206 components and 2 ms for 150 (the tail of a batched
@@ -1085,6 +1090,29 @@ __global__ void k_stats_vector(const double* __restrict__ m, const unsigned long
 constexpr int kWfTile = 16;
 constexpr int kWfThreads = kWfTile * kWfTile + 32;
 constexpr int kWfRun = 16;
+// One run of the chain of component `comp` by one warp (comp per lane, all lanes
+// call it): vectors r0 .. r0 + kWfRun - 1, the mean m carried on, out(q, dold, dnew)
+// for each.
+template <class Out>
+__device__ __forceinline__ void welford_run(const double* __restrict__ v, int nvec, int d, int comp,
+                                            double n0, int r0, double& m, Out&& out) {
+  // the run's values first (their loads in flight together) and 1 / n of
+  // its vectors, one per lane; the chain is then three operations a vector
+  const double rn = 1.0 / (n0 + double(r0 + ((int)threadIdx.x & (kWfRun - 1)) + 1));
+  double x[kWfRun];
+#pragma unroll
+  for (int q = 0; q < kWfRun; ++q)
+    x[q] = comp < d && r0 + q < nvec ? v[(size_t)(r0 + q) * d + comp] : 0.0;
+#pragma unroll
+  for (int q = 0; q < kWfRun; ++q) {
+    const double r = __shfl_sync(0xFFFFFFFFu, rn, q);
+    const double a = x[q] - m;
+    const double mq = __fma_rn(a, r, m);
+    if (r0 + q < nvec) m = mq;
+    out(q, a, x[q] - mq);
+  }
+}
+
 __global__ void __launch_bounds__(kWfThreads)
 k_welford_update(const double* __restrict__ v, int nvec, int d, double* __restrict__ st,
                  double* __restrict__ mean_new, unsigned int* __restrict__ ticket) {
@@ -1103,22 +1131,10 @@ k_welford_update(const double* __restrict__ v, int nvec, int d, double* __restri
   const bool mine = !maker && i < d && j < d;
   double acc = mine ? M2[(size_t)i * d + j] : 0.0;
   auto make = [&](int r0, int buf) {                 // (the maker warp)
-    // the run's values first (their loads in flight together) and 1 / n of
-    // its vectors, one per lane; the chain is then three operations a vector
-    const double rn = 1.0 / (n0 + double(r0 + (lane & (kWfRun - 1)) + 1));
-    double x[kWfRun];
-#pragma unroll
-    for (int q = 0; q < kWfRun; ++q)
-      x[q] = comp < d && r0 + q < nvec ? v[(size_t)(r0 + q) * d + comp] : 0.0;
-#pragma unroll
-    for (int q = 0; q < kWfRun; ++q) {
-      const double r = __shfl_sync(0xFFFFFFFFu, rn, q);
-      const double a = x[q] - m;
-      const double mq = __fma_rn(a, r, m);
-      if (r0 + q < nvec) m = mq;
+    welford_run(v, nvec, d, comp, n0, r0, m, [&](int q, double a, double b) {
       if (lane < kWfTile) dold[buf][q][lane] = a;
-      else dnew[buf][q][lane - kWfTile] = x[q] - mq;
-    }
+      else dnew[buf][q][lane - kWfTile] = b;
+    });
   };
   if (maker) make(0, 0);
   __syncthreads();
@@ -1133,6 +1149,7 @@ k_welford_update(const double* __restrict__ v, int nvec, int d, double* __restri
     __syncthreads();
   }
   if (mine) M2[(size_t)i * d + j] = acc;
+  if (!mean_new) return;                             // (uniform) k_welford_mean follows
   if (maker && blockIdx.x == 0 && lane < kWfTile && comp < d) mean_new[comp] = m;
   __threadfence();                                   // the means before the ticket
   __syncthreads();
@@ -1141,10 +1158,70 @@ k_welford_update(const double* __restrict__ v, int nvec, int d, double* __restri
   if (!last_s) return;
   __threadfence();
   for (int k = t; k < d; k += kWfThreads) mean[k] = __ldcg(mean_new + k);
-  if (t == 0) {
-    st[0] = n0 + double(nvec);
-    *ticket = 0u;
+  if (t == 0) st[0] = n0 + double(nvec);
+}
+
+// The mean and the count after k_welford_update: one cluster, so that the count
+// is written after every block has read it.
+constexpr int kWfCluster = 8;
+__global__ void __cluster_dims__(kWfCluster, 1, 1) __launch_bounds__(256)
+k_welford_mean(const double* __restrict__ v, int nvec, int d, double* __restrict__ st) {
+  const double n0 = st[0];
+  const int lane = threadIdx.x & 31, nth = gridDim.x * blockDim.x;
+  for (int c0 = blockIdx.x * blockDim.x + threadIdx.x - lane; c0 < d; c0 += nth) {
+    const int comp = c0 + lane;
+    double m = comp < d ? st[1 + comp] : 0.0;
+    for (int r0 = 0; r0 < nvec; r0 += kWfRun)
+      welford_run(v, nvec, d, comp, n0, r0, m, [](int, double, double) {});
+    if (comp < d) st[1 + comp] = m;
   }
+  asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::
+                   : "memory");
+  if (blockIdx.x == 0 && threadIdx.x == 0) st[0] = n0 + double(nvec);
+}
+
+// One vector into a state of up to kWfOne components (a map at a time) by one
+// cluster in one launch: the operations of the two kernels above.  A second launch
+// costs such a caller more than the arithmetic on 8 SMs: bin, kappa, vector and
+// update of a map of Nside 64 took 128 us before, 132 with two launches.
+constexpr int kWfOne = 256, kWfOneThreads = 512;
+__global__ void __cluster_dims__(kWfCluster, 1, 1) __launch_bounds__(kWfOneThreads)
+k_welford_one(const double* __restrict__ v, int d, double* __restrict__ st) {
+  __shared__ double dold[kWfOne], dnew[kWfOne], rn_s;
+  constexpr int kV = 8;                              // elements in flight per thread
+  const int t = threadIdx.x, step = kWfCluster * kWfOneThreads;
+  const double n0 = st[0];
+  double* M2 = st + 1 + d;
+  double x = 0.0, m = 0.0;
+  if (t < d) { x = v[t]; m = st[1 + t]; }
+  int k = blockIdx.x * kWfOneThreads + t;
+  double acc[kV];
+#pragma unroll
+  for (int u = 0; u < kV; ++u) acc[u] = k + u * step < d * d ? M2[k + u * step] : 0.0;
+  if (t == 0) rn_s = 1.0 / (n0 + 1.0);
+  __syncthreads();
+  double mq = 0.0;
+  if (t < d) {
+    const double a = x - m;
+    mq = __fma_rn(a, rn_s, m);
+    dold[t] = a;
+    dnew[t] = x - mq;
+  }
+  __syncthreads();
+  for (; k < d * d; k += kV * step) {
+#pragma unroll
+    for (int u = 0; u < kV; ++u) {
+      const int q = k + u * step;
+      if (q < d * d) M2[q] = __fma_rn(dold[q / d], dnew[q % d], acc[u]);
+      const int nq = q + kV * step;
+      acc[u] = nq < d * d ? M2[nq] : 0.0;
+    }
+  }
+  asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::
+                   : "memory");
+  if (blockIdx.x != 0) return;
+  if (t < d) st[1 + t] = mq;
+  if (t == 0) st[0] = n0 + 1.0;
 }
 
 __global__ void __launch_bounds__(1024)
@@ -1723,20 +1800,34 @@ ufc_status run_stats_vector(ufc_ctx* c, const double* m, const int64_t* pdf, int
   return UFC_OK;
 }
 
-ufc_status run_welford_update(ufc_ctx* c, const double* v, int nvec, int d, double* st) {
+// mean_new [d] and ticket (0 when the launch runs): scratch that no other call
+// uses meanwhile, or NULL both.
+static ufc_status launch_welford(ufc_ctx* c, const double* v, int nvec, int d, double* st,
+                                 double* mean_new, unsigned int* ticket) {
   if (!v || !st || nvec < 0 || d < 1 || d > 8192)
     return set_err(c, UFC_ERR_ARG, "welford_update: bad arguments");
   if (nvec == 0) return UFC_OK;
-  double* mean_new = (double*)ws_get(c, kSlotWelford, (size_t)d * 8);
-  if (!mean_new) return UFC_ERR_ALLOC;
+  if (nvec == 1 && d <= kWfOne) {
+    ProfScope ps_(c, "k_welford_update");
+    k_welford_one<<<kWfCluster, kWfOneThreads, 0, c->stream>>>(v, d, st);
+    UFC_CUDA(c, cudaGetLastError());
+    return UFC_OK;
+  }
   {
     ProfScope ps_(c, "k_welford_update");
     const int g = (d + kWfTile - 1) / kWfTile;
-    k_welford_update<<<dim3(g, g), kWfThreads, 0, c->stream>>>(
-        v, nvec, d, st, mean_new, &reinterpret_cast<BinCounters*>(c->counters)->ticket);
+    k_welford_update<<<dim3(g, g), kWfThreads, 0, c->stream>>>(v, nvec, d, st, mean_new, ticket);
+  }
+  if (!mean_new) {
+    ProfScope ps_(c, "k_welford_mean");
+    const int warps = (d + 32 * kWfCluster - 1) / (32 * kWfCluster);       // per block, at most 8
+    k_welford_mean<<<kWfCluster, 32 * std::min(warps, 8), 0, c->stream>>>(v, nvec, d, st);
   }
   UFC_CUDA(c, cudaGetLastError());
   return UFC_OK;
+}
+ufc_status run_welford_update(ufc_ctx* c, const double* v, int nvec, int d, double* st) {
+  return launch_welford(c, v, nvec, d, st, nullptr, nullptr);
 }
 ufc_status run_welford_merge(ufc_ctx* c, double* a, const double* b, int d) {
   if (!a || !b || d < 1 || d > 8192) return set_err(c, UFC_ERR_ARG, "welford_merge: bad arguments");
@@ -1765,15 +1856,16 @@ ufc_status batch_geometry(ufc_ctx* c, const double* chi, int nshell, const ufc_b
 void batch_bands(int nside, float smax, Bands& bd);
 
 // Workspace of a batched call: per realisation a count map, a kappa map and the
-// partial sums of the serial grids, then the items, the coefficients and the
-// finished-block counters.
+// partial sums of the serial grids, then the items, the coefficients, the
+// finished-block counters (one per realisation, one of the Welford update) and
+// the new Welford mean.
 struct BatchSpace {
   size_t maps, kappa, part;                  // offsets in the map buffer
   size_t maps_bytes;
-  size_t items, coef, done, up_bytes, desc_bytes;   // in the descriptor buffer
+  size_t items, coef, done, mean, up_bytes, desc_bytes;   // in the descriptor buffer
   int gk, gm;
 };
-static BatchSpace batch_space(const ufc_ctx* c, int nreal, int nbox, int S, int nside) {
+static BatchSpace batch_space(const ufc_ctx* c, int nreal, int nbox, int S, int nside, int d) {
   const int npix = 12 * nside * nside;
   auto up = [](size_t b) { return (b + 255) / 256 * 256; };
   BatchSpace o;
@@ -1787,7 +1879,8 @@ static BatchSpace batch_space(const ufc_ctx* c, int nreal, int nbox, int S, int 
   o.coef = up((size_t)nreal * nbox * sizeof(DirectItem));
   o.up_bytes = o.coef + (size_t)nreal * batch_coef_stride(S);
   o.done = up(o.up_bytes);
-  o.desc_bytes = o.done + (size_t)nreal * 4;
+  o.mean = up(o.done + (size_t)(nreal + 1) * 4);
+  o.desc_bytes = o.mean + (size_t)d * 8;
   return o;
 }
 // Whether the batched call of this shape runs stage by stage over all
@@ -1795,7 +1888,7 @@ static BatchSpace batch_space(const ufc_ctx* c, int nreal, int nbox, int S, int 
 // 65535 rows.
 bool batch_stages_ok(const ufc_ctx* c, int nreal, int nbox, int S, int nside, size_t max_bytes) {
   return (int64_t)nreal * nbox <= (1 << 17) && nreal <= 65535 &&
-         batch_space(c, nreal, nbox, S, nside).maps_bytes <= max_bytes;
+         batch_space(c, nreal, nbox, S, nside, 0).maps_bytes <= max_bytes;
 }
 
 // A batched call over all realisations at once.  The items and coefficients
@@ -1811,7 +1904,7 @@ ufc_status run_batch_stages(ufc_ctx* c, int nreal, int nbox, const float* const*
   if (cs != cudaStreamCaptureStatusNone)
     return set_err(c, UFC_ERR_UNSUPPORTED, "ufc_batched_stats cannot be captured into a graph");
   const int npix = 12 * nside * nside, nitems = nreal * nbox;
-  const BatchSpace sp = batch_space(c, nreal, nbox, S, nside);
+  const BatchSpace sp = batch_space(c, nreal, nbox, S, nside, 6 + nbins);
   char* maps = (char*)ws_get(c, kSlotBatchMaps, sp.maps_bytes);
   char* desc = (char*)ws_get(c, kSlotBatchDesc, sp.desc_bytes);
   if (!maps || !desc) return UFC_ERR_ALLOC;
@@ -1882,7 +1975,7 @@ ufc_status run_batch_stages(ufc_ctx* c, int nreal, int nbox, const float* const*
   }
   UFC_CUDA(c, cudaMemcpyAsync(desc, host, sp.up_bytes, cudaMemcpyHostToDevice, c->stream));
   UFC_CUDA(c, cudaEventRecord(c->batch_ev, c->stream));
-  UFC_CUDA(c, cudaMemsetAsync(desc + sp.done, 0, (size_t)nreal * 4, c->stream));
+  UFC_CUDA(c, cudaMemsetAsync(desc + sp.done, 0, (size_t)(nreal + 1) * 4, c->stream));
   // the bands of the largest shift of all the boxes
   batch_bands(nside, smax, a.bd);
   ufc_status s = bin_prep(c, st, maps + sp.maps, sp.kappa, &a.tab, &a.lut_scale);
@@ -1922,7 +2015,8 @@ ufc_status run_batch_stages(ufc_ctx* c, int nreal, int nbox, const float* const*
         ba, make_pdf_param(lo, hi, nbins));
   }
   UFC_CUDA(c, cudaGetLastError());
-  return run_welford_update(c, stats, nreal, 6 + nbins, state);
+  return launch_welford(c, stats, nreal, 6 + nbins, state, reinterpret_cast<double*>(desc + sp.mean),
+                        ba.done + nreal);
 }
 
 }  // namespace ufc

@@ -1,0 +1,111 @@
+"""Calls of one context that overlap on different streams, and under stream
+capture: a Welford update keeps nothing outside the caller's state, so it may
+run beside any other call, allocates nothing and can be captured before the
+context has made a first call."""
+import numpy as np
+import pytest
+
+from tests.gpu_common import api_ctx
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def _vectors(nvec, d, seed):
+    return torch.from_numpy(np.random.default_rng(seed).normal(1.0, 0.1, size=(nvec, d))).cuda()
+
+
+@pytest.mark.parametrize("d", [1, 206, 2049])
+def test_welford_update_keeps_nothing_in_the_context(d):
+    """No workspace, and the state of 17 + 2 vectors equals the host's chain."""
+    api, _ = api_ctx()
+    ctx = api.Context(0)
+    try:
+        held = ctx.workspace_bytes()
+        v = _vectors(19, d, d)
+        st = api.welford_state(d)
+        ctx.welford_update(v[:17], st)
+        ctx.welford_update(v[17:], st)
+        torch.cuda.synchronize()
+        assert ctx.workspace_bytes() == held
+        one = api.welford_state(d)
+        ctx.welford_update(v, one)
+        torch.cuda.synchronize()
+        assert torch.equal(st, one) and st[0].item() == 19.0
+        # a mean of 19 values near 1 by 19 rounded steps, M2 by 19 fused ones: each
+        # step errs by at most 2^-53 of values below 2 (a few steps for M2's sums)
+        host = np.zeros(1 + d + d * d)
+        api.welford_update_host(v.cpu().numpy(), host)
+        assert np.abs(st.cpu().numpy() - host).max() <= 19 * 4 * 2.0 ** -52
+    finally:
+        ctx.close()
+
+
+@pytest.mark.parametrize("d", [1, 15, 206, 256, 257])
+def test_one_vector_at_a_time_equals_all_at_once(d):
+    """One vector takes a launch of its own up to 256 components: the same bits."""
+    api, ctx = api_ctx()
+    v = _vectors(7, d, d + 1)
+    st, one = api.welford_state(d), api.welford_state(d)
+    ctx.welford_update(v, one)
+    for r in range(7):
+        ctx.welford_update(v[r:r + 1], st)
+    torch.cuda.synchronize()
+    assert torch.equal(st, one)
+
+
+@pytest.mark.parametrize("nvec", [1, 5])
+def test_first_welford_update_can_be_captured(nvec):
+    api, _ = api_ctx()
+    ctx = api.Context(0)
+    try:
+        v = _vectors(nvec, 206, 1)
+        st = api.welford_state(206)
+        ref = api.welford_state(206)
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            ctx.welford_update(v, st)
+        assert st.abs().max().item() == 0.0              # captured, not run
+        for _ in range(2):
+            graph.replay()
+            ctx.welford_update(v, ref)
+        torch.cuda.synchronize()
+        assert torch.equal(st, ref)
+    finally:
+        ctx.close()
+
+
+def test_welford_updates_overlap_with_each_other_and_with_moments():
+    """Updates of two states and moment passes of a map, enqueued in turn on
+    three streams without waiting: the same results as one after the other."""
+    api, ctx = api_ctx()
+    nside, rounds = 64, 24
+    kap = torch.from_numpy(np.random.default_rng(3).normal(0.0, 0.01, 12 * nside * nside)
+                           .astype(np.float32)).cuda()
+    va, vb = _vectors(40, 1030, 4), _vectors(33, 46, 5)
+    vc = _vectors(1, 206, 6)
+    sa, sb, ra, rb, sc, rc = (api.welford_state(d) for d in (1030, 46, 1030, 46, 206, 206))
+    m0, p0 = (t.clone() for t in ctx.map_stats(kap, nside, -0.05, 0.05, 64))
+    for _ in range(rounds):
+        ctx.welford_update(va, ra)
+        ctx.welford_update(vb, rb)
+        ctx.welford_update(vc, rc)
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream() for _ in range(3)]
+    out = []
+    for _ in range(rounds):
+        with torch.cuda.stream(streams[0]):
+            ctx.welford_update(va, sa)
+        with torch.cuda.stream(streams[1]):
+            ctx.welford_update(vb, sb)
+            ctx.welford_update(vc, sc)
+        with torch.cuda.stream(streams[2]):
+            out.append(ctx.map_stats(kap, nside, -0.05, 0.05, 64))
+    torch.cuda.synchronize()
+    assert torch.equal(sa, ra) and torch.equal(sb, rb) and torch.equal(sc, rc)
+    for m, p in out:
+        assert torch.equal(m, m0) and torch.equal(p, p0)
+    m, p = ctx.map_stats(kap, nside, -0.05, 0.05, 64)    # and the context still works
+    torch.cuda.synchronize()
+    assert torch.equal(m, m0) and torch.equal(p, p0)
