@@ -844,8 +844,9 @@ ufc_status ufc_batched_stats(ufc_ctx* c, int32_t nreal, int32_t nbox, const floa
                             moments, pdf, stats, state);
   ufc_status s = reserve_bin_workspace(c, nbox, max_img, nshell, nside);
   if (s) return s;
-  // per-block partial sums of the kappa and moment kernels
-  if (!ws_get(c, kSlotPartials, (size_t)20 * c->num_sms * 8)) return UFC_ERR_ALLOC;
+  // per-block partial sums of the kappa and moment kernels and the latter's count
+  const size_t part_bytes = ((size_t)20 * c->num_sms + 1) * 8;
+  if (!ws_get(c, kSlotPartials, part_bytes)) return UFC_ERR_ALLOC;
   // small maps: realisation r runs on lane r mod nlane, the lanes concurrently
   // (lane 0 is this context with the caller's scratch maps; the others have
   // their own count and kappa maps, workspace and stream)
@@ -865,7 +866,7 @@ ufc_status ufc_batched_stats(ufc_ctx* c, int32_t nreal, int32_t nbox, const floa
     s = reserve_bin_workspace(lane[k], nbox, max_img, nshell, nside);
     if (s) return set_err(c, s, "%s", lane[k]->err.c_str());
     char* m = (char*)ws_get(lane[k], kSlotLaneMap, map_bytes + (size_t)npix * 4 + 256);
-    if (!m || !ws_get(lane[k], kSlotPartials, (size_t)20 * c->num_sms * 8))
+    if (!m || !ws_get(lane[k], kSlotPartials, part_bytes))
       return set_err(c, UFC_ERR_ALLOC, "%s", lane[k]->err.c_str());
     lane_counts[k] = reinterpret_cast<int32_t*>(m);
     lane_kappa[k] = reinterpret_cast<float*>(m + ((map_bytes + 255) & ~(size_t)255));

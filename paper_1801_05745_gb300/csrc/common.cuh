@@ -95,10 +95,6 @@ struct BinCounters {
   // bounded device waits that ran out: last, so that a binning call's reset
   // (everything before it) keeps it until ufc_synchronize reports it
   unsigned long long timeouts;
-  // blocks of the running moment pass that have finished (the last one does the
-  // final step and clears it); also outside the reset
-  unsigned int ticket;
-  unsigned int pad_;
 };
 
 // ---- index checks of checked builds ----------------------------------------

@@ -82,11 +82,18 @@ __device__ __forceinline__ double block_sum_d(double v, double* sh) {
   return t;   // valid in thread 0
 }
 
-// Clears the PDF that the moment pass after this kernel adds to (block 0; pdf
-// may be NULL).  One launch less than a memset between the two passes.
-__device__ __forceinline__ void clear_pdf(unsigned long long* pdf, int n) {
-  if (pdf && blockIdx.x == 0)
-    for (int i = threadIdx.x; i < n; i += blockDim.x) pdf[i] = 0ull;
+// Clears the PDF that the moment pass after this kernel adds to and its count of
+// finished blocks (block 0; pdf may be NULL: no moment pass).  One launch less
+// than a memset between the two passes.
+struct MomentOut {
+  unsigned long long* pdf;
+  int npdf;
+  unsigned int* ticket;      // beside the pass's partial sums
+};
+__device__ __forceinline__ void clear_pdf(const MomentOut& o) {
+  if (!o.pdf || blockIdx.x != 0) return;
+  for (int i = threadIdx.x; i < o.npdf; i += blockDim.x) o.pdf[i] = 0ull;
+  if (threadIdx.x == 0 && o.ticket) *o.ticket = 0u;
 }
 
 struct Coef {
@@ -171,8 +178,8 @@ struct AdjRow { I128 s[3]; long long n; long long pad_; };
 // aligned.
 __global__ void __launch_bounds__(kKT)
 k_kappa_plain(const int32_t* __restrict__ counts, Coef cf, float* __restrict__ kappa,
-              double* __restrict__ ksum_part, unsigned long long* __restrict__ pdf, int npdf) {
-  clear_pdf(pdf, npdf);
+              double* __restrict__ ksum_part, MomentOut mo) {
+  clear_pdf(mo);
   __shared__ float ah_s[kMaxShells], al_s[kMaxShells];
   __shared__ double red[kKT / 32];
   const int S = cf.nshell;
@@ -320,9 +327,8 @@ __device__ __forceinline__ double kappa_vec_block(const int32_t* __restrict__ co
 
 __global__ void __launch_bounds__(kKV, 4)
 k_kappa_vec(const int32_t* __restrict__ counts, const __grid_constant__ Coef cf,
-            float* __restrict__ kappa, double* __restrict__ ksum_part,
-            unsigned long long* __restrict__ pdf, int npdf) {
-  clear_pdf(pdf, npdf);
+            float* __restrict__ kappa, double* __restrict__ ksum_part, MomentOut mo) {
+  clear_pdf(mo);
   __shared__ float4 cs[kMaxShells];
   __shared__ double red[kKV / 32];
   kappa_coef(cs, cf.nshell, [&](int i) { return make_float2(cf.ah[i], cf.al[i]); });
@@ -364,9 +370,8 @@ k_kappa_partial(const int32_t* __restrict__ counts, const __grid_constant__ Coef
 // the moment pass treats it exactly as a map from the counts.
 __global__ void __launch_bounds__(kKV)
 k_kappa_finish(const double* __restrict__ part, float ch, float cl, int npix,
-               float* __restrict__ kappa, double* __restrict__ ksum_part,
-               unsigned long long* __restrict__ pdf, int npdf) {
-  clear_pdf(pdf, npdf);
+               float* __restrict__ kappa, double* __restrict__ ksum_part, MomentOut mo) {
+  clear_pdf(mo);
   __shared__ double red[kKV / 32];
   const int ng = npix >> 2;
   const f2 mc{-ch, -cl};
@@ -469,11 +474,11 @@ k_adj_main(const int32_t* __restrict__ counts, const __grid_constant__ Coef cf,
            const float* __restrict__ g, double* __restrict__ rows_out,
            double* __restrict__ sumpart, unsigned long long* range_flag,
            float* __restrict__ kappa_out, double* __restrict__ ksum_out,
-           const double* __restrict__ ext, unsigned long long* __restrict__ pdf, int npdf) {
+           const double* __restrict__ ext, MomentOut mo) {
   extern __shared__ __align__(16) uint8_t adj_sm[];
   constexpr int NW = NT / 32, P = 2 * NT, NC = adj_cols(USE_G);
   constexpr int LDA = adj_lda(NT), LDB = adj_ldb(NT);
-  if (kappa_out) clear_pdf(pdf, npdf);
+  if (kappa_out) clear_pdf(mo);
   const int S = cf.nshell, npix = cf.npix, np2 = npix >> 1;
   const int mt_n = (S + 15) >> 4, mp = adj_rows(S);      // tiles of 16 shells; rows held
   uint8_t* An = adj_sm;                                      // [mp][LDA] a byte of the counts
@@ -837,9 +842,8 @@ k_adj_reduce(const double* __restrict__ rows, const double* __restrict__ sums, i
 // the moments of an arbitrary map (ufc_map_stats).  Needs a 16-byte aligned
 // map of a multiple of 4 values.
 __global__ void __launch_bounds__(kKV)
-k_map_sum(const float* __restrict__ map, int npix, double* __restrict__ ksum_part,
-          unsigned long long* __restrict__ pdf, int npdf) {
-  clear_pdf(pdf, npdf);
+k_map_sum(const float* __restrict__ map, int npix, double* __restrict__ ksum_part, MomentOut mo) {
+  clear_pdf(mo);
   __shared__ double red[kKV / 32];
   const int ng = npix >> 2;
   f2 ks{0.f, 0.f};
@@ -1024,8 +1028,8 @@ static int moments_grid(int num_sms, int npix) {
   return std::min(4 * num_sms, (npix + 4 * kMT - 1) / (4 * kMT));
 }
 
-// The last block to finish (ticket) turns the partial sums into the moments:
-// one launch less, and nothing waits.  The ticket is left at 0.
+// The last block to finish (ticket, cleared by the kernel before) turns the
+// partial sums into the moments: one launch less, and nothing waits.
 __global__ void __launch_bounds__(kMT)
 k_moments(const float* __restrict__ kappa, int npix, const double* __restrict__ ksum_part,
           int nksum, PdfParam pp, double* __restrict__ part /*[grid][3]*/,
@@ -1053,7 +1057,6 @@ k_moments(const float* __restrict__ kappa, int npix, const double* __restrict__ 
   if (!last_s) return;
   __threadfence();                         // every block's sums are visible
   moments_final_block(ksum_part, nksum, part, gridDim.x, npix, red, m);
-  if (threadIdx.x == 0) *ticket = 0u;
 }
 
 // Statistics vector of one map for the covariance (Eq. 10): the first six
@@ -1295,7 +1298,8 @@ k_batch_kappa(const __grid_constant__ BatchArgs ba) {
   __shared__ float4 cs[kMaxShells];
   __shared__ double red[kKV / 32];
   const int r = blockIdx.y, S = ba.S;
-  clear_pdf((unsigned long long*)ba.pdf + (size_t)(ba.nbins + 3) * r, ba.nbins + 3);
+  clear_pdf(MomentOut{(unsigned long long*)ba.pdf + (size_t)(ba.nbins + 3) * r, ba.nbins + 3,
+                      nullptr});
   const BatchCoef& cf = *reinterpret_cast<const BatchCoef*>(ba.coef + batch_coef_stride(S) * r);
   kappa_coef(cs, S, [&](int i) { return make_float2(cf.a[i].x, cf.a[i].y); });
   const double t = kappa_vec_block(ba.counts + (size_t)r * S * ba.npix, cs, S, ba.npix,
@@ -1378,17 +1382,26 @@ static int kappa_fwd_grid(const ufc_ctx* c, int npix) {   // blocks with work on
   return std::min(8 * c->num_sms, (npix / 4 + kKV - 1) / kKV);
 }
 static ufc_status launch_kappa_fwd(ufc_ctx* c, const int32_t* counts, const Coef& cf,
-                                   float* kappa, double* ksum, int grid, int64_t* pdf, int nbins) {
-  unsigned long long* pd = reinterpret_cast<unsigned long long*>(pdf);
+                                   float* kappa, double* ksum, int grid, const MomentOut& mo) {
   if ((reinterpret_cast<uintptr_t>(kappa) & 15) == 0) {
-    k_kappa_vec<<<grid, kKV, 0, c->stream>>>(counts, cf, kappa, ksum, pd, nbins + 3);
+    k_kappa_vec<<<grid, kKV, 0, c->stream>>>(counts, cf, kappa, ksum, mo);
   } else {
-    k_kappa_plain<<<grid, kKT, 0, c->stream>>>(counts, cf, kappa, ksum, pd, nbins + 3);
+    k_kappa_plain<<<grid, kKT, 0, c->stream>>>(counts, cf, kappa, ksum, mo);
   }
   UFC_CUDA(c, cudaGetLastError());
   return UFC_OK;
 }
 
+
+// Scratch of a map pass and the moment pass after it, in doubles: the block sums
+// of `grid` blocks, three sums for each of `mgrid`, and the moment pass's count of
+// finished blocks.  (Each pass's own, so that passes with different scratch may
+// overlap on different streams.)
+static size_t pass_doubles(int grid, int mgrid) { return (size_t)grid + 3 * (size_t)mgrid + 1; }
+static MomentOut moment_out(double* mpart, int mgrid, int64_t* pdf, int nbins) {
+  return MomentOut{reinterpret_cast<unsigned long long*>(pdf), nbins + 3,
+                   reinterpret_cast<unsigned int*>(mpart + 3 * mgrid)};
+}
 
 // Moments and PDF of an FP32 map whose per-block sums (grid of them) are in
 // ksum: the second pass over the map and the final reduction.
@@ -1417,7 +1430,7 @@ static PdfParam make_pdf_param(double lo, double hi, int nbins) {
   return pp;
 }
 
-// (the PDF has been cleared by the kernel that wrote ksum)
+// (the PDF and the count have been cleared by the kernel that wrote ksum)
 static ufc_status launch_moments(ufc_ctx* c, const float* kmap, int npix, const double* ksum,
                                  int grid, double lo, double hi, int nbins, double* mpart,
                                  double* moments, int64_t* pdf, bool timed) {
@@ -1425,9 +1438,10 @@ static ufc_status launch_moments(ufc_ctx* c, const float* kmap, int npix, const 
   const int smem = (nbins + 3) * 4;
   {
     ProfScope ps_(timed ? c : nullptr, "k_moments");
-    k_moments<<<moments_grid(c->num_sms, npix), kMT, smem, c->stream>>>(
-        kmap, npix, ksum, grid, pp, mpart, (unsigned long long*)pdf, moments,
-        &reinterpret_cast<BinCounters*>(c->counters)->ticket);
+    const int mgrid = moments_grid(c->num_sms, npix);
+    const MomentOut mo = moment_out(mpart, mgrid, pdf, nbins);
+    k_moments<<<mgrid, kMT, smem, c->stream>>>(kmap, npix, ksum, grid, pp, mpart, mo.pdf, moments,
+                                               mo.ticket);
   }
   UFC_CUDA(c, cudaGetLastError());
   return UFC_OK;
@@ -1445,11 +1459,12 @@ ufc_status run_map_stats(ufc_ctx* c, const float* map, int nside, double lo, dou
   if (reinterpret_cast<uintptr_t>(map) & 15) return set_err(c, UFC_ERR_ARG, "map_dev must be 16-byte aligned");
   const int npix = 12 * nside * nside;
   const int grid = kappa_fwd_grid(c, npix), mgrid = moments_grid(c->num_sms, npix);
-  double* ksum = (double*)ws_get(c, kSlotPartials, (size_t)(grid + 3 * mgrid) * 8);
+  double* ksum = (double*)ws_get(c, kSlotPartials, pass_doubles(grid, mgrid) * 8);
   if (!ksum) return UFC_ERR_ALLOC;
   {
     ProfScope ps_(c, "k_map_sum");
-    k_map_sum<<<grid, kKV, 0, c->stream>>>(map, npix, ksum, (unsigned long long*)pdf, nbins + 3);
+    k_map_sum<<<grid, kKV, 0, c->stream>>>(map, npix, ksum,
+                                           moment_out(ksum + grid, mgrid, pdf, nbins));
   }
   UFC_CUDA(c, cudaGetLastError());
   return launch_moments(c, map, npix, ksum, grid, lo, hi, nbins, ksum + grid, moments, pdf, true);
@@ -1476,7 +1491,7 @@ ufc_status run_kappa_stats(ufc_ctx* c, const int32_t* counts, int S, int nside,
     return set_err(c, UFC_ERR_ARG, "counts_dev must be 16-byte aligned");
   const int grid = kappa_fwd_grid(c, npix);
   const int mgrid = moments_grid(c->num_sms, npix);
-  double* ksum = (double*)ws_get(c, kSlotPartials, (size_t)(grid + 3 * mgrid) * 8);
+  double* ksum = (double*)ws_get(c, kSlotPartials, pass_doubles(grid, mgrid) * 8);
   if (!ksum) return UFC_ERR_ALLOC;
   double* mpart = ksum + grid;
   float* kmap = kappa;
@@ -1487,7 +1502,7 @@ ufc_status run_kappa_stats(ufc_ctx* c, const int32_t* counts, int S, int nside,
   if (!kmap) return UFC_OK;   // nothing requested
   {
     ProfScope ps_(c, "k_kappa");
-    s = launch_kappa_fwd(c, counts, cf, kmap, ksum, grid, pdf, nbins);
+    s = launch_kappa_fwd(c, counts, cf, kmap, ksum, grid, moment_out(mpart, mgrid, pdf, nbins));
     if (s) return s;
   }
   if (!want_stats) return UFC_OK;
@@ -1534,7 +1549,7 @@ static ufc_status adjoint_sums(ufc_ctx* c, const int32_t* counts, int S, int nsi
   const int grid2 = std::min(per_sm * c->num_sms, (npix + 2 * nt - 1) / (2 * nt));
   const size_t nrow = (size_t)grid2 * 4 * S, nsum = (size_t)grid2 * 4;
   const int mgrid = moments_grid(c->num_sms, npix);
-  const size_t nmap = kappa ? (size_t)grid2 + 3 * (size_t)mgrid : 0;   // map sums, moment partials
+  const size_t nmap = kappa ? pass_doubles(grid2, mgrid) : 0;   // map sums, moment partials
   const size_t nout = 4 * (size_t)S + 5;
   double* part = (double*)ws_get(c, kSlotPartials, (nrow + nsum + nmap + nout) * 8);
   if (!part) return UFC_ERR_ALLOC;
@@ -1544,6 +1559,7 @@ static ufc_status adjoint_sums(ufc_ctx* c, const int32_t* counts, int S, int nsi
   double* mpart = ksum + grid2;
   double* dout = part + nrow + nsum + nmap;
   BinCounters* bc = reinterpret_cast<BinCounters*>(c->counters);
+  const MomentOut mo = moment_out(mpart, mgrid, pdf, nbins);     // (used with kappa only)
   {
     ProfScope ps_(c, "k_adj_main");
 #define UFC_ADJ(G, NT_, X)                                                                        \
@@ -1551,8 +1567,7 @@ static ufc_status adjoint_sums(ufc_ctx* c, const int32_t* counts, int S, int nsi
     UFC_CUDA(c, cudaFuncSetAttribute(k_adj_main<G, NT_, X>,                                       \
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2));   \
     k_adj_main<G, NT_, X><<<grid2, NT_, smem2, c->stream>>>(                                      \
-        counts, cf, g, rows, sums, &bc->range, kappa, ksum, ext, (unsigned long long*)pdf,        \
-        nbins + 3);                                                                               \
+        counts, cf, g, rows, sums, &bc->range, kappa, ksum, ext, mo);                             \
   } while (0)
 #define UFC_ADJ_X(G, NT_)                                                                         \
   do {                                                                                            \
@@ -1688,13 +1703,13 @@ ufc_status run_kappa_stats_partial(ufc_ctx* c, const double* partial, int nside,
     return set_err(c, UFC_ERR_ARG, "PDF range needs finite lo < hi");
   const int npix = 12 * nside * nside;
   const int grid = kappa_fwd_grid(c, npix), mgrid = moments_grid(c->num_sms, npix);
-  double* ksum = (double*)ws_get(c, kSlotPartials, (size_t)(grid + 3 * mgrid) * 8);
+  double* ksum = (double*)ws_get(c, kSlotPartials, pass_doubles(grid, mgrid) * 8);
   if (!ksum) return UFC_ERR_ALLOC;
   const float ch = (float)C, cl = (float)(C - (double)ch);
   {
     ProfScope ps_(c, "k_kappa_finish");
     k_kappa_finish<<<grid, kKV, 0, c->stream>>>(partial, ch, cl, npix, kappa, ksum,
-                                                (unsigned long long*)pdf, nbins + 3);
+                                                moment_out(ksum + grid, mgrid, pdf, nbins));
   }
   UFC_CUDA(c, cudaGetLastError());
   return launch_moments(c, kappa, npix, ksum, grid, lo, hi, nbins, ksum + grid, moments, pdf, true);
@@ -1728,8 +1743,8 @@ ufc_status run_kappa_backward(ufc_ctx* c, const int32_t* counts, int S, int nsid
 }
 
 // ---- variant of ufc_kappa_stats that allocates nothing -------------------
-// Its per-block partial sums live in this file-scope device array instead of
-// the context workspace.  Every GPU that loads the library holds the array
+// Its per-block partial sums and its count of finished blocks live in this
+// file-scope device array instead of the context workspace.  Every GPU that loads the library holds the array
 // (kNoAllocScratch doubles = 32 KB) until the process exits; all calls on a
 // device share it, so calls that overlap on the GPU race on it.
 constexpr int kNoAllocScratch = 4096;
@@ -1772,17 +1787,17 @@ ufc_status run_kappa_stats_noalloc(ufc_ctx* c, const int32_t* counts, int S, int
   const int npix = 12 * nside * nside;
   const int grid = kappa_fwd_grid(c, npix);
   const int mgrid = moments_grid(c->num_sms, npix);
-  if (grid + 3 * mgrid > kNoAllocScratch)
+  if (pass_doubles(grid, mgrid) > (size_t)kNoAllocScratch)
     return set_err(c, UFC_ERR_CAPACITY,
-                   "scratch needs %d doubles, the fixed array holds %d", grid + 3 * mgrid,
+                   "scratch needs %zu doubles, the fixed array holds %d", pass_doubles(grid, mgrid),
                    kNoAllocScratch);
   double* ksum = nullptr;
   s = noalloc_scratch(c, &ksum);
   if (s) return s;
-  double* mpart = ksum + grid;   // every slot is written before it is read
+  double* mpart = ksum + grid;   // every slot is written before it is read, the count cleared
   Coef cf;
   make_coef(A, C, S, npix, cf);
-  s = launch_kappa_fwd(c, counts, cf, kappa, ksum, grid, pdf, nbins);
+  s = launch_kappa_fwd(c, counts, cf, kappa, ksum, grid, moment_out(mpart, mgrid, pdf, nbins));
   if (s) return s;
   // (no kernel-timing records here: recording them may allocate)
   return launch_moments(c, kappa, npix, ksum, grid, lo, hi, nbins, mpart, moments, pdf, false);

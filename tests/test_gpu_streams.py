@@ -1,7 +1,10 @@
 """Calls of one context that overlap on different streams, and under stream
 capture: a Welford update keeps nothing outside the caller's state, so it may
 run beside any other call, allocates nothing and can be captured before the
-context has made a first call."""
+context has made a first call; a moment pass counts its blocks in the scratch
+that holds its sums."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -109,3 +112,61 @@ def test_welford_updates_overlap_with_each_other_and_with_moments():
     m, p = ctx.map_stats(kap, nside, -0.05, 0.05, 64)    # and the context still works
     torch.cuda.synchronize()
     assert torch.equal(m, m0) and torch.equal(p, p0)
+
+
+def _noalloc(api, ctx, counts, A, C, lo, hi, nbins):
+    S, npix = counts.shape
+    kap = torch.empty(npix, dtype=torch.float32, device="cuda")
+    mom = torch.empty(10, dtype=torch.float64, device="cuda")
+    pdf = torch.empty(nbins + 3, dtype=torch.int64, device="cuda")
+    ctx._stream()
+    st = api._lib.ufc_kappa_stats_noalloc(
+        ctx.h, ctypes.c_void_p(counts.data_ptr()), S, int(round((npix / 12) ** 0.5)),
+        A.ctypes.data_as(ctypes.c_void_p), C, lo, hi, nbins, ctypes.c_void_p(kap.data_ptr()),
+        ctypes.c_void_p(mom.data_ptr()), ctypes.c_void_p(pdf.data_ptr()))
+    assert st == 0
+    return kap, mom, pdf
+
+
+def test_noalloc_call_overlaps_with_moment_passes_of_the_workspace():
+    """ufc_kappa_stats_noalloc (scratch of its own) on one stream, ufc_kappa_stats
+    (scratch in the workspace) on another: the results of both alone."""
+    api, ctx = api_ctx()
+    nside, S, nbins, lo, hi = 64, 5, 33, -0.5, 0.5
+    rng = np.random.default_rng(9)
+    counts = [torch.from_numpy(rng.poisson(3.0, (S, 12 * nside * nside)).astype(np.int32)).cuda()
+              for _ in range(2)]
+    A, C = np.linspace(0.01, 0.05, S), 0.4
+    ref = [_noalloc(api, ctx, counts[0], A, C, lo, hi, nbins),
+           ctx.kappa_stats(counts[1], A, C, lo, hi, nbins)]
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    out = []
+    for _ in range(40):
+        with torch.cuda.stream(streams[0]):
+            out.append((0, _noalloc(api, ctx, counts[0], A, C, lo, hi, nbins)))
+        with torch.cuda.stream(streams[1]):
+            out.append((1, ctx.kappa_stats(counts[1], A, C, lo, hi, nbins)))
+    torch.cuda.synchronize()
+    for which, got in out:
+        for a, b in zip(got, ref[which]):
+            assert torch.equal(a, b)
+
+
+def test_moment_passes_of_changing_sizes_clear_their_own_count():
+    """The count's place depends on the map's size, so a pass finds the sums of
+    passes of other sizes there: the results equal those of a new context."""
+    api, _ = api_ctx()
+    ctx = api.Context(0)
+    try:
+        for nside in (64, 16, 128, 1, 256, 32, 64, 2, 16):
+            kap = torch.from_numpy(np.random.default_rng(nside).normal(0.0, 0.01, 12 * nside ** 2)
+                                   .astype(np.float32)).cuda()
+            m, p = ctx.map_stats(kap, nside, -0.05, 0.05, 64)
+            new = api.Context(0)
+            m0, p0 = new.map_stats(kap, nside, -0.05, 0.05, 64)
+            torch.cuda.synchronize()
+            new.close()
+            assert torch.equal(m, m0) and torch.equal(p, p0)
+    finally:
+        ctx.close()
