@@ -1567,7 +1567,9 @@ ufc_status run_keys_pipeline(ufc_ctx* c, int mode_req, const float* const* xyz,
     UFC_CUDA(c, cudaStreamWaitEvent(c->stream, e, 0));
     return UFC_OK;
   };
-  BinTables* tab = nullptr;
+  BinTables* tab = (BinTables*)ws_get(c, kSlotTables, sizeof(BinTables));
+  if (!tab) return UFC_ERR_ALLOC;
+  BinCounters* cnt = (BinCounters*)c->counters;
   float lut_scale = 0.f;
 
   if (plan.mode == kModeDirect) {
@@ -1578,7 +1580,7 @@ ufc_status run_keys_pipeline(ufc_ctx* c, int mode_req, const float* const* xyz,
     const bool with_prep = clear && (reinterpret_cast<uintptr_t>(counts) & 15) == 0 &&
                            map_bytes % 16 == 0 && map_bytes <= (64ull << 20);
     if (clear && !with_prep) UFC_CUDA(c, cudaMemsetAsync(counts, 0, map_bytes, c->stream));
-    s = bin_prep(c, st, with_prep ? counts : nullptr, map_bytes, &tab, &lut_scale);
+    s = bin_prep(c, st, with_prep ? counts : nullptr, map_bytes, tab, cnt, &lut_scale);
     if (s) return s;
     DirectArgs a;
     std::memset(&a, 0, sizeof a);
@@ -1588,7 +1590,7 @@ ufc_status run_keys_pipeline(ufc_ctx* c, int mode_req, const float* const* xyz,
     a.N = nside;
     a.npix = (int32_t)npix;
     a.ncell = (int64_t)nshell * npix;
-    a.cnt = (BinCounters*)c->counters;
+    a.cnt = cnt;
     auto item = [&](int k, int64_t p0, int64_t cnt) {
       DirectItem d;
       std::memset(&d, 0, sizeof d);
@@ -1653,8 +1655,8 @@ ufc_status run_keys_pipeline(ufc_ctx* c, int mode_req, const float* const* xyz,
   qs.q1 = (uint64_t*)ws_get(c, kSlotQueue1, z.cap1 * 8);
   qs.q2 = (uint64_t*)ws_get(c, kSlotQueue2, z.cap2 * 8);
   if (!qs.q1 || !qs.q2) return UFC_ERR_ALLOC;
-  qs.cnt = (BinCounters*)c->counters;
-  s = bin_prep(c, st, nullptr, 0, &tab, &lut_scale);
+  qs.cnt = cnt;
+  s = bin_prep(c, st, nullptr, 0, tab, cnt, &lut_scale);
   if (s) return s;
   // overflow bits: one per particle
   int64_t nbits = 0;

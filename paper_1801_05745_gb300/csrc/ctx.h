@@ -77,7 +77,7 @@ enum Slot {
   kSlotOvf,        // one bit per particle image: left undecided when queue 1 was full
   kSlotLaneMap,    // a lane's count map and kappa map (ufc_batched_stats)
   kSlotBatchMaps,  // batched call: per-realisation maps and partial sums
-  kSlotBatchDesc,  // batched call: items, coefficients and counters
+  kSlotBatchDesc,  // batched call: items, coefficients, tables and counters
 };
 
 inline ufc_status set_err(ufc_ctx* c, ufc_status s, const char* fmt, ...) {

@@ -54,9 +54,7 @@ k_bin_prep(ShellTable st, float scale, BinTables* __restrict__ t,
 }
 
 ufc_status bin_prep(ufc_ctx* c, const ShellTable& st, void* zero, size_t zero_bytes,
-                    BinTables** tab, float* lut_scale) {
-  BinTables* t = (BinTables*)ws_get(c, kSlotTables, sizeof(BinTables));
-  if (!t) return UFC_ERR_ALLOC;
+                    BinTables* tab, BinCounters* cnt, float* lut_scale) {
   // bins 0 .. kLut-2 cover [0, hi2[nshell]]
   const double top = std::max((double)st.hi2[st.nshell], 1e-30);
   *lut_scale = (float)std::min((kLut - 2) / top, 1e30);
@@ -65,12 +63,11 @@ ufc_status bin_prep(ufc_ctx* c, const ShellTable& st, void* zero, size_t zero_by
       std::max(c->num_sms, (int)std::min<int64_t>(8 * c->num_sms, (nzero + 255) / 256));
   {
     ProfScope ps_(c, "k_bin_prep");
-    k_bin_prep<<<grid, 256, 0, c->stream>>>(st, *lut_scale, t, (unsigned long long*)c->counters,
+    k_bin_prep<<<grid, 256, 0, c->stream>>>(st, *lut_scale, tab, (unsigned long long*)cnt,
                                             (int)(offsetof(BinCounters, timeouts) / 8), (int4*)zero,
                                             nzero);
   }
   UFC_CUDA(c, cudaGetLastError());
-  *tab = t;
   return UFC_OK;
 }
 

@@ -81,11 +81,11 @@ struct DirectArgs {
   BinCounters* cnt;
 };
 
-// Tables of one call into the context's table slot, its counters cleared and
+// Tables of one call into `tab` (device), the counters `cnt` cleared and
 // `zero_bytes` of `zero` (16-byte aligned, a multiple of 16; may be NULL) set
 // to 0, by one launch on the context stream.
 ufc_status bin_prep(ufc_ctx* c, const ShellTable& st, void* zero, size_t zero_bytes,
-                    BinTables** tab, float* lut_scale);
+                    BinTables* tab, BinCounters* cnt, float* lut_scale);
 // Empties the particle bounds of box `box` again.
 ufc_status bin_prep_bounds(ufc_ctx* c, BinTables* tab, int box);
 // The direct path over a.nitems items (a.tab, a.bd, a.N, a.npix, a.cnt, the

@@ -1872,12 +1872,14 @@ void batch_bands(int nside, float smax, Bands& bd);
 
 // Workspace of a batched call: per realisation a count map, a kappa map and the
 // partial sums of the serial grids, then the items, the coefficients, the
-// finished-block counters (one per realisation, one of the Welford update) and
-// the new Welford mean.
+// finished-block counters (one per realisation, one of the Welford update), the
+// new Welford mean, and the binning's tables and counters: the call shares
+// nothing with the binning, kappa and moment calls of its context (which may run
+// on another stream meanwhile) and leaves ufc_bin_info as it was.
 struct BatchSpace {
   size_t maps, kappa, part;                  // offsets in the map buffer
   size_t maps_bytes;
-  size_t items, coef, done, mean, up_bytes, desc_bytes;   // in the descriptor buffer
+  size_t items, coef, done, mean, tab, cnt, up_bytes, desc_bytes;   // in the descriptor buffer
   int gk, gm;
 };
 static BatchSpace batch_space(const ufc_ctx* c, int nreal, int nbox, int S, int nside, int d) {
@@ -1895,7 +1897,9 @@ static BatchSpace batch_space(const ufc_ctx* c, int nreal, int nbox, int S, int 
   o.up_bytes = o.coef + (size_t)nreal * batch_coef_stride(S);
   o.done = up(o.up_bytes);
   o.mean = up(o.done + (size_t)(nreal + 1) * 4);
-  o.desc_bytes = o.mean + (size_t)d * 8;
+  o.tab = up(o.mean + (size_t)d * 8);
+  o.cnt = up(o.tab + sizeof(BinTables));
+  o.desc_bytes = o.cnt + sizeof(BinCounters);
   return o;
 }
 // Whether the batched call of this shape runs stage by stage over all
@@ -1993,14 +1997,15 @@ ufc_status run_batch_stages(ufc_ctx* c, int nreal, int nbox, const float* const*
   UFC_CUDA(c, cudaMemsetAsync(desc + sp.done, 0, (size_t)(nreal + 1) * 4, c->stream));
   // the bands of the largest shift of all the boxes
   batch_bands(nside, smax, a.bd);
-  ufc_status s = bin_prep(c, st, maps + sp.maps, sp.kappa, &a.tab, &a.lut_scale);
+  a.tab = reinterpret_cast<BinTables*>(desc + sp.tab);
+  a.cnt = reinterpret_cast<BinCounters*>(desc + sp.cnt);
+  ufc_status s = bin_prep(c, st, maps + sp.maps, sp.kappa, a.tab, a.cnt, &a.lut_scale);
   if (s) return s;
   a.items = reinterpret_cast<const DirectItem*>(desc + sp.items);
   a.nitems = nitems;
   a.N = nside;
   a.npix = npix;
   a.ncell = (int64_t)S * npix;
-  a.cnt = (BinCounters*)c->counters;
   s = launch_direct(c, a, c->batch_blocks_per_sm);
   if (s) return s;
   BatchArgs ba;

@@ -2,13 +2,14 @@
 capture: a Welford update keeps nothing outside the caller's state, so it may
 run beside any other call, allocates nothing and can be captured before the
 context has made a first call; a moment pass counts its blocks in the scratch
-that holds its sums."""
+that holds its sums; a batched call has its own tables and counters."""
 import ctypes
 
 import numpy as np
 import pytest
 
-from tests.gpu_common import api_ctx
+from paper_1801_05745_gb300 import synth
+from tests.gpu_common import api_ctx, to_dev
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -170,3 +171,68 @@ def test_moment_passes_of_changing_sizes_clear_their_own_count():
             assert torch.equal(m, m0) and torch.equal(p, p0)
     finally:
         ctx.close()
+
+
+def _batch(api, orc, nreal, n, nside, nshell):
+    z = np.linspace(0.1, 1.5, nshell + 1)
+    chi = orc.chi_edges(0.3, 0.7, 1, z)
+    split = int(np.argmin(np.abs(chi - 1000.0)))
+    xs, boxes = [], []
+    for r in range(nreal):
+        xs.append([to_dev(synth.particles_numpy(n, 2000.0, 5.0, 700 + 2 * r)),
+                   to_dev(synth.particles_numpy(n, 6400.0, 20.0, 701 + 2 * r))])
+        boxes.append([api.make_box(2000.0, [1000.0] * 3, n, 0, split),
+                      api.make_box(6400.0, [3200.0] * 3, n, split, nshell)])
+    A = np.tile(np.linspace(0.01, 0.05, nshell), (nreal, 1))
+    return chi, xs, boxes, A, np.full(nreal, 0.1)
+
+
+def test_batched_call_leaves_the_last_binning_calls_diagnostics(orc):
+    """ufc_bin_info tells of the last ufc_bin or ufc_keys call."""
+    api, ctx = api_ctx()
+    chi, xs, boxes, A, C = _batch(api, orc, 3, 20_000, 16, 6)
+    ctx.bin([xs[0][0][:1234]], boxes[0][:1], chi, 16)
+    info = ctx.bin_info()
+    assert info["keyed"] > 0
+    ctx.batched_stats(xs, boxes, chi, 16, A, C, -0.5, 0.5, 20, api.welford_state(26))
+    assert ctx.bin_info() == info
+
+
+def test_batched_call_overlaps_with_binning_and_kappa(orc):
+    """Batched calls on one stream, binning (dense and direct, with other shell
+    edges) and map statistics on two others: the results of each alone."""
+    api, ctx = api_ctx()
+    nside, nshell, nbins = 32, 8, 20
+    chi, xs, boxes, A, C = _batch(api, orc, 12, 60_000, nside, nshell)
+    chi2 = np.linspace(150.0, 900.0, 31)
+    x2 = to_dev(synth.particles_numpy(700_001, 2000.0, 5.0, 77))
+    b2 = [api.make_box(2000.0, [1000.0] * 3, 700_001, 0, 30)]
+    kap = torch.from_numpy(np.random.default_rng(1).normal(0.0, 0.1, 12 * 64 * 64)
+                           .astype(np.float32)).cuda()
+
+    def batched():
+        st = api.welford_state(6 + nbins)
+        return [*ctx.batched_stats(xs, boxes, chi, nside, A, C, -0.5, 0.5, nbins, st), st]
+
+    def others(path):
+        return [ctx.bin([x2], b2, chi2, 128, path=path)]
+
+    ref = [t.clone() for t in batched()]
+    torch.cuda.synchronize()
+    counts = {p: others(p)[0].clone() for p in ("dense", "direct")}
+    stats = [t.clone() for t in ctx.map_stats(kap, 64, -0.5, 0.5, 50)]
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream() for _ in range(3)]
+    got = []
+    for k in range(12):
+        with torch.cuda.stream(streams[0]):
+            got.append((batched(), ref))
+        with torch.cuda.stream(streams[1]):
+            p = ("dense", "direct")[k % 2]
+            got.append((others(p), [counts[p]]))
+        with torch.cuda.stream(streams[2]):
+            got.append((ctx.map_stats(kap, 64, -0.5, 0.5, 50), stats))
+    torch.cuda.synchronize()
+    for a, b in got:
+        for u, v in zip(a, b):
+            assert torch.equal(u, v)
