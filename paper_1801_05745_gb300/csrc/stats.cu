@@ -1876,6 +1876,9 @@ void batch_bands(int nside, float smax, Bands& bd);
 // new Welford mean, and the binning's tables and counters: the call shares
 // nothing with the binning, kappa and moment calls of its context (which may run
 // on another stream meanwhile) and leaves ufc_bin_info as it was.
+// A launch takes as many realisations as its grid has rows and the 17 bits of an
+// item's number in an undecided image's entry allow.
+constexpr int kBatchRows = 65535, kBatchItems = 1 << 17;
 struct BatchSpace {
   size_t maps, kappa, part;                  // offsets in the map buffer
   size_t maps_bytes;
@@ -1903,10 +1906,9 @@ static BatchSpace batch_space(const ufc_ctx* c, int nreal, int nbox, int S, int 
   return o;
 }
 // Whether the batched call of this shape runs stage by stage over all
-// realisations: item numbers have 17 bits in an undecided image's entry, grids
-// 65535 rows.
+// realisations.
 bool batch_stages_ok(const ufc_ctx* c, int nreal, int nbox, int S, int nside, size_t max_bytes) {
-  return (int64_t)nreal * nbox <= (1 << 17) && nreal <= 65535 &&
+  return nbox <= kBatchItems &&
          batch_space(c, nreal, nbox, S, nside, 0).maps_bytes <= max_bytes;
 }
 
@@ -1959,10 +1961,13 @@ ufc_status run_batch_stages(ufc_ctx* c, int nreal, int nbox, const float* const*
     total += n[i];
   }
   a.task = c->batch_chunk > 0 ? c->batch_chunk : direct_task(c, total);
+  const int per = std::min(kBatchRows, kBatchItems / nbox);      // realisations per launch
+  std::vector<int64_t> ntasks;                                   // of each launch
   std::vector<BoxGeom> bg(nbox);
   ShellTable st;
   float smax = 0.f;
   for (int r = 0; r < nreal; ++r) {
+    if (r % per == 0) ntasks.push_back(0);
     const ufc_status s = batch_geometry(c, r == 0 ? chi : nullptr, S, boxes + (size_t)r * nbox, nbox,
                                         st, bg.data());
     if (s) return s;
@@ -1973,7 +1978,7 @@ ufc_status run_batch_stages(ufc_ctx* c, int nreal, int nbox, const float* const*
       smax = std::max(smax, g.smax);
       d.xyz = xyz[i];
       d.n = n[i];
-      d.task0 = a.ntasks;
+      d.task0 = ntasks.back();
       d.counts = reinterpret_cast<int32_t*>(maps + sp.maps) + (size_t)r * S * npix;
       d.shell_lo = g.shell_lo;
       d.shell_hi = g.shell_hi;
@@ -1982,7 +1987,7 @@ ufc_status run_batch_stages(ufc_ctx* c, int nreal, int nbox, const float* const*
         d.shlo[ax] = g.shlo[ax][0];
         d.sh64[ax] = g.sh64[ax][0];
       }
-      a.ntasks += (n[i] + a.task - 1) / a.task;
+      ntasks.back() += (n[i] + a.task - 1) / a.task;
     }
     BatchCoef* cf = reinterpret_cast<BatchCoef*>(host + sp.coef + batch_coef_stride(S) * r);
     auto split = [](double x) {
@@ -2001,42 +2006,48 @@ ufc_status run_batch_stages(ufc_ctx* c, int nreal, int nbox, const float* const*
   a.cnt = reinterpret_cast<BinCounters*>(desc + sp.cnt);
   ufc_status s = bin_prep(c, st, maps + sp.maps, sp.kappa, a.tab, a.cnt, &a.lut_scale);
   if (s) return s;
-  a.items = reinterpret_cast<const DirectItem*>(desc + sp.items);
-  a.nitems = nitems;
   a.N = nside;
   a.npix = npix;
   a.ncell = (int64_t)S * npix;
-  s = launch_direct(c, a, c->batch_blocks_per_sm);
-  if (s) return s;
-  BatchArgs ba;
-  ba.coef = desc + sp.coef;
-  ba.nreal = nreal;
-  ba.S = S;
-  ba.npix = npix;
-  ba.counts = reinterpret_cast<int32_t*>(maps + sp.maps);
-  ba.kappa = reinterpret_cast<float*>(maps + sp.kappa);
-  ba.ksum = reinterpret_cast<double*>(maps + sp.part);
-  ba.mpart = ba.ksum + (size_t)sp.gk * nreal;
-  ba.gk = sp.gk;
-  ba.gm = sp.gm;
-  ba.moments = moments;
-  ba.pdf = pdf;
-  ba.stats = stats;
-  ba.nbins = nbins;
-  ba.d = 6 + nbins;
-  ba.done = reinterpret_cast<unsigned int*>(desc + sp.done);
-  {
-    ProfScope ps_(c, "k_batch_kappa");
-    k_batch_kappa<<<dim3(sp.gk, nreal), kKV, 0, c->stream>>>(ba);
-  }
-  {
-    ProfScope ps_(c, "k_batch_moments");
-    k_batch_moments<<<dim3(sp.gm, nreal), kMT, (nbins + 3) * 4, c->stream>>>(
-        ba, make_pdf_param(lo, hi, nbins));
+  double* const ksum = reinterpret_cast<double*>(maps + sp.part);
+  unsigned int* const done = reinterpret_cast<unsigned int*>(desc + sp.done);
+  for (int r0 = 0; r0 < nreal; r0 += per) {
+    const int nr = std::min(per, nreal - r0);
+    a.items = reinterpret_cast<const DirectItem*>(desc + sp.items) + (size_t)r0 * nbox;
+    a.nitems = nr * nbox;
+    a.ntasks = ntasks[r0 / per];
+    s = launch_direct(c, a, c->batch_blocks_per_sm);
+    if (s) return s;
+    BatchArgs ba;
+    ba.coef = desc + sp.coef + batch_coef_stride(S) * r0;
+    ba.nreal = nr;
+    ba.S = S;
+    ba.npix = npix;
+    ba.counts = reinterpret_cast<int32_t*>(maps + sp.maps) + (size_t)r0 * S * npix;
+    ba.kappa = reinterpret_cast<float*>(maps + sp.kappa) + (size_t)r0 * npix;
+    ba.ksum = ksum + (size_t)sp.gk * r0;
+    ba.mpart = ksum + (size_t)sp.gk * nreal + (size_t)3 * sp.gm * r0;
+    ba.gk = sp.gk;
+    ba.gm = sp.gm;
+    ba.moments = moments + (size_t)10 * r0;
+    ba.pdf = pdf + (size_t)(nbins + 3) * r0;
+    ba.stats = stats + (size_t)(6 + nbins) * r0;
+    ba.nbins = nbins;
+    ba.d = 6 + nbins;
+    ba.done = done + r0;
+    {
+      ProfScope ps_(c, "k_batch_kappa");
+      k_batch_kappa<<<dim3(sp.gk, nr), kKV, 0, c->stream>>>(ba);
+    }
+    {
+      ProfScope ps_(c, "k_batch_moments");
+      k_batch_moments<<<dim3(sp.gm, nr), kMT, (nbins + 3) * 4, c->stream>>>(
+          ba, make_pdf_param(lo, hi, nbins));
+    }
   }
   UFC_CUDA(c, cudaGetLastError());
   return launch_welford(c, stats, nreal, 6 + nbins, state, reinterpret_cast<double*>(desc + sp.mean),
-                        ba.done + nreal);
+                        done + nreal);
 }
 
 }  // namespace ufc
