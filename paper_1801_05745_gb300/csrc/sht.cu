@@ -141,9 +141,10 @@ __device__ __forceinline__ double sht_w(int k) {
 // 64, 8 now).
 __global__ void __launch_bounds__(64)
 k_sht_tables(int32_t N, int32_t lmax, float4* __restrict__ T, double* __restrict__ tab,
-             float4* __restrict__ pair, double* __restrict__ sin_d) {
+             float4* __restrict__ pair, double* __restrict__ sin_d, int* __restrict__ bad) {
   const int n8 = 8 * N, nl = (lmax + 2 + 31) / 32 * 32;              // (whole warps per part)
   int j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j == 0) *bad = 0;
   if (j < n8) {
     double sn, cs;
     sincospi(-2.0 * (double)j / (double)n8, &sn, &cs);
@@ -607,7 +608,12 @@ __global__ void k_alm2cl(const double2* __restrict__ alm, int32_t lmax, double* 
 // mantissas: terms 2^-30 below the current scale may lose bits, they are
 // negligible), so nothing is reduced across threads.  A warp whose pairs are
 // all negligible up to lmax (leg_negligible) writes zeros, and none of its
-// terms is formed before one of its pairs has e > -120.  Bound by the FP32
+// terms is formed before one of its pairs has e > -120.  These terms are 0 for
+// finite coefficients only, so one that is not finite sets *bad, with which
+// k_ring_synth makes every pixel a NaN: the sums of the equator's pair, which
+// leaves nothing out, are NaNs then.  (The imaginary part of order 0 does not
+// enter the map.  A test of every coefficient by every block, or by the equator's
+// thread at the end, made this kernel up to 12% slower at Nside 128.)  Bound by the FP32
 // pipe: 18 + 24 packed operations per degree and pair of ring pairs (FMA pipe
 // 71% busy).  Nside 512, lmax 1535: 1.47 ms with blocks of 128 threads, 1.51 with
 // 256 or 64 (2.96 ms before the one-coefficient recurrence and the packed pairs).
@@ -615,7 +621,7 @@ template <int NT>
 __global__ void __launch_bounds__(NT)
 k_legendre_synth(const double2* __restrict__ alm, const float2* __restrict__ mu,
                  const int32_t* __restrict__ ex, ShtTables tb, int32_t lmax, int32_t nrings,
-                 int32_t npairs, float4* __restrict__ G) {
+                 int32_t npairs, float4* __restrict__ G, int* __restrict__ bad) {
   __shared__ float4 cs[2][kLegChunkL];
   __shared__ float4 as[2][kLegChunkL][2];                 // alpha_l a_lm: real, imaginary
   const int chunk = blockIdx.x, m = blockIdx.y;
@@ -727,7 +733,9 @@ k_legendre_synth(const double2* __restrict__ alm, const float2* __restrict__ mu,
       return df_scale(k ? df_norm(h.y, l.y) : df_norm(h.x, l.x), sc);
     };
     const float4 ev = cdf_pack(part(ge[0]), part(ge[1])), od = cdf_pack(part(go[0]), part(go[1]));
-    G[(size_t)m * nrings + r] = cdf_add(ev, od);
+    const float4 sum = cdf_add(ev, od);
+    G[(size_t)m * nrings + r] = sum;
+    if (ps == r && (isnan(sum.x) || (m && isnan(sum.z)))) *bad = 1;   // (the equator)
     if (ps != r) G[(size_t)m * nrings + ps] = cdf_sub(ev, od);
   }
 }
@@ -771,6 +779,7 @@ struct ShtSpace {
   float2* mu;          // [lmax + 1][2N]
   int32_t* ex;
   double2* part;       // [nchunk][nalm]
+  int* bad;            // synthesis: a coefficient is not finite (cleared with the tables)
 };
 static ufc_status sht_space(ufc_ctx* c, int nside, int lmax, int nchunk, ShtSpace& o) {
   const size_t nrings = 4 * (size_t)nside - 1, npairs = 2 * (size_t)nside;
@@ -785,6 +794,7 @@ static ufc_status sht_space(ufc_ctx* c, int nside, int lmax, int nchunk, ShtSpac
   const size_t o_mu = piece((size_t)(lmax + 1) * npairs * sizeof(float2));
   const size_t o_ex = piece((size_t)(lmax + 1) * npairs * sizeof(int32_t));
   const size_t o_part = piece(nchunk > 1 ? nchunk * nalm * sizeof(double2) : 0);
+  const size_t o_bad = piece(sizeof(int));
   char* ws = (char*)ws_get(c, kSlotSht, at);
   if (!ws) return UFC_ERR_ALLOC;
   float4* roots = reinterpret_cast<float4*>(ws + o_roots);
@@ -797,11 +807,12 @@ static ufc_status sht_space(ufc_ctx* c, int nside, int lmax, int nchunk, ShtSpac
   o.mu = reinterpret_cast<float2*>(ws + o_mu);
   o.ex = reinterpret_cast<int32_t*>(ws + o_ex);
   o.part = reinterpret_cast<double2*>(ws + o_part);
+  o.bad = reinterpret_cast<int*>(ws + o_bad);
   {
     ProfScope ps_(c, "k_sht_tables");
     const int n = 10 * nside + 4 * ((lmax + 2 + 31) / 32 * 32);
     k_sht_tables<<<(n + 63) / 64, 64, 0, c->stream>>>(nside, lmax, roots, tab, pair,
-                                                        sin_d);
+                                                        sin_d, o.bad);
   }
   {
     ProfScope ps_(c, "k_lmm");
@@ -883,13 +894,14 @@ ufc_status run_alm2map(ufc_ctx* c, const double* alm, int nside, int lmax, float
     const dim3 grid((npairs + 2 * nt - 1) / (2 * nt), lmax + 1);
 #define UFC_SYN(NT)                                                                                \
   k_legendre_synth<NT><<<grid, NT, 0, c->stream>>>(reinterpret_cast<const double2*>(alm), sp.mu,   \
-                                                   sp.ex, sp.tb, lmax, nrings, npairs, sp.ring)
+                                                   sp.ex, sp.tb, lmax, nrings, npairs, sp.ring, \
+                                                   sp.bad)
     if (nt == 128) UFC_SYN(128);
     else UFC_SYN(64);
 #undef UFC_SYN
   }
   UFC_CUDA(c, cudaGetLastError());
-  return launch_ring_synth(c, sp.ring, sp.tb.roots, nside, lmax, map);
+  return launch_ring_synth(c, sp.ring, sp.tb.roots, nside, lmax, sp.bad, map);
 }
 
 ufc_status run_alm_beam(ufc_ctx* c, const double* in, int lmax, double sigma, double* out) {

@@ -112,10 +112,11 @@ __device__ __forceinline__ float4 cdf_conj(float4 a) { return make_float4(a.x, a
 __device__ __forceinline__ dfx dfx_set(dfl a, dfl b) { return {x2_pack(a.h, b.h), x2_pack(a.l, b.l)}; }
 
 // sht_ring.cu: F_m of every ring of a map ([lmax + 1][4N - 1]), and the map of
-// such coefficients; T: the 8N unit roots e^{-2 pi i j / (8N)}.
+// such coefficients (all NaN when *bad is set); T: the 8N unit roots
+// e^{-2 pi i j / (8N)}.
 ufc_status launch_ring_transform(ufc_ctx* c, const float* map, const float4* T, int nside, int lmax,
                                  float4* F);
 ufc_status launch_ring_synth(ufc_ctx* c, const float4* G, const float4* T, int nside, int lmax,
-                             float* map);
+                             const int* bad, float* map);
 
 }  // namespace ufc

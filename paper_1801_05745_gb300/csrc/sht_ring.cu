@@ -318,11 +318,12 @@ k_ring_transform(const float* __restrict__ map, const float4* __restrict__ T, in
 // us at Nside 512, lmax 1535, now 134.)
 __global__ void __launch_bounds__(kRingThreads, 2)
 k_ring_synth(const float4* __restrict__ G, const float4* __restrict__ T, int32_t N,
-             int32_t lmax, int32_t nrings, float* __restrict__ map) {
+             int32_t lmax, int32_t nrings, const int* __restrict__ bad, float* __restrict__ map) {
   extern __shared__ __align__(16) cxs sh[];
   const int r = blockIdx.x;
   const RingSpan g = ring_span(N, r);
   const int n = g.n, L = n / 2, N8 = 8 * N;
+  const float off = *bad ? NAN : 0.f;                        // added to every pixel
   float* px = map + g.start;
   __shared__ cxs part_s[kRingThreads];
   auto fold = [&](cxs* H, auto term) {                       // H_k, k <= L
@@ -368,8 +369,8 @@ k_ring_synth(const float4* __restrict__ G, const float4* __restrict__ T, int32_t
     for (int j = threadIdx.x; j < L; j += kRingThreads) {
       const cx v = cx_ld(Z[bit_rev(j, b)]);
       const float2 x = x2_get(x2_add(v.h, v.l));
-      px[2 * j] = x.x;
-      px[2 * j + 1] = x.y;
+      px[2 * j] = x.x + off;
+      px[2 * j + 1] = x.y + off;
     }
     return;
   }
@@ -416,10 +417,10 @@ k_ring_synth(const float4* __restrict__ G, const float4* __restrict__ T, int32_t
     const cx c = cx_scale(cx_conj(chirp(wf, i, a)), sc);
     const cx e = cx_mul(cx_ld(U[a]), c), o = cx_mul(cx_ld(V[a]), c);
     const float2 x = x2_get(x2_add(e.h, e.l)), y = x2_get(x2_add(o.h, o.l));
-    px[4 * a] = x.x;
-    px[4 * a + 1] = x.y;
-    px[4 * a + 2] = y.x;
-    px[4 * a + 3] = y.y;
+    px[4 * a] = x.x + off;
+    px[4 * a + 1] = x.y + off;
+    px[4 * a + 2] = y.x + off;
+    px[4 * a + 3] = y.y + off;
   }
 }
 
@@ -441,12 +442,12 @@ ufc_status launch_ring_transform(ufc_ctx* c, const float* map, const float4* T, 
 }
 
 ufc_status launch_ring_synth(ufc_ctx* c, const float4* G, const float4* T, int nside, int lmax,
-                             float* map) {
+                             const int* bad, float* map) {
   const int smem = ring_smem(nside), nrings = 4 * nside - 1;
   UFC_CUDA(c, cudaFuncSetAttribute(k_ring_synth, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
   {
     ProfScope ps_(c, "k_ring_synth");
-    k_ring_synth<<<nrings, kRingThreads, smem, c->stream>>>(G, T, nside, lmax, nrings, map);
+    k_ring_synth<<<nrings, kRingThreads, smem, c->stream>>>(G, T, nside, lmax, nrings, bad, map);
   }
   UFC_CUDA(c, cudaGetLastError());
   return UFC_OK;
