@@ -56,6 +56,7 @@ __device__ __forceinline__ cx cx_sub(cx a, cx b) {
 __device__ __forceinline__ cx cx_conj(cx a) {
   return {a.h ^ 0x8000000000000000ull, a.l ^ 0x8000000000000000ull};
 }
+__device__ __forceinline__ cx cx_real(cx a) { return {a.h & 0xFFFFFFFFull, a.l & 0xFFFFFFFFull}; }
 __device__ __forceinline__ cx cx_times_i(cx a) {  // (re, im) -> (-im, re)
   const float2 h = x2_get(a.h), l = x2_get(a.l);
   return {x2_pack(-h.y, h.x), x2_pack(-l.y, l.x)};
@@ -332,8 +333,8 @@ k_ring_synth(const float4* __restrict__ G, const float4* __restrict__ T, int32_t
       for (int m = k + p * n; m <= lmax; m += np * n) h = cx_add(h, term(m));
       for (int m = (k ? n - k : n) + p * n; m <= lmax; m += np * n)
         h = cx_add(h, cx_conj(term(m)));
-      return h;
-    };
+      return k ? h : cx_real(h);                             // (H_0: the conjugates cancel, and
+    };                                                       // Im G_0 does not enter the map)
     const int np = kRingThreads / (L + 1);                   // (uniform)
     if (np < 2) {
       for (int k = threadIdx.x; k <= L; k += kRingThreads) H[k] = cx_st(some(k, 0, 1));
