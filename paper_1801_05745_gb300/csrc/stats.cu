@@ -141,33 +141,36 @@ __device__ __forceinline__ void quant2(f2 v, int s, int& hi, int& lo) {
 
 // 128-bit two's-complement fixed-point accumulator (integer operations only).
 struct I128 { unsigned long long lo; long long hi; };
-// acc += v * 2^sh, sh in [-127, 62]; bits below 2^0 of the result are dropped.
-__device__ __forceinline__ void i128_add(I128& acc, long long v, int sh) {
-  unsigned long long lo;
-  long long hi;
-  if (sh >= 64) {
-    lo = 0ull;
-    hi = v << (sh - 64);
-  } else if (sh > 0) {
-    lo = (unsigned long long)v << sh;
-    hi = v >> (64 - sh);
-  } else if (sh == 0) {
-    lo = (unsigned long long)v;
-    hi = v < 0 ? -1ll : 0ll;
-  } else if (sh > -64) {
-    const long long t = v >> (-sh);
-    lo = (unsigned long long)t;
-    hi = t < 0 ? -1ll : 0ll;
-  } else {
-    lo = v < 0 ? ~0ull : 0ull;
-    hi = v < 0 ? -1ll : 0ll;
-  }
-  const unsigned long long nlo = acc.lo + lo;
-  acc.hi += hi + (nlo < acc.lo ? 1ll : 0ll);
+__device__ __forceinline__ void i128_add(I128& acc, I128 v) {
+  const unsigned long long nlo = acc.lo + v.lo;
+  acc.hi += v.hi + (nlo < acc.lo ? 1ll : 0ll);
   acc.lo = nlo;
 }
+// v * 2^sh rounded to the nearest whole number, |sh| < 128 (the adjoint's flush
+// passes kFrac - s - 22 with the scale s from 8, a maximum below 2^14, to 120).
+__device__ __forceinline__ I128 i128_shift(I128 v, int sh) {
+  if (sh < 0) i128_add(v, sh > -65 ? I128{1ull << (-sh - 1), 0ll} : I128{0ull, 1ll << (-sh - 65)});
+  if (sh >= 64) return {0ull, (long long)(v.lo << (sh - 64))};
+  if (sh > 0) return {v.lo << sh, (long long)((unsigned long long)v.hi << sh | v.lo >> (64 - sh))};
+  if (sh == 0) return v;
+  if (sh > -64) return {v.lo >> -sh | (unsigned long long)v.hi << (64 + sh), v.hi >> -sh};
+  return {(unsigned long long)(v.hi >> (-sh - 64)), v.hi >> 63};
+}
+// v[0] + 2^8 v[1] + 2^16 v[2] + 2^-22 (the same of v[3 .. 5]), times 2^22: exact.
+__device__ __forceinline__ I128 i128_digits(const long long* v) {
+  I128 r{0ull, 0ll};
+#pragma unroll
+  for (int k = 0; k < 6; ++k)
+    i128_add(r, i128_shift(I128{(unsigned long long)v[k], v[k] >> 63}, k < 3 ? 22 + 8 * k : 8 * (k - 3)));
+  return r;
+}
+// (by the magnitude: a small negative value has 64 high and many low bits set, and
+// converted as it is would keep 2^-53 of 2^64, not of itself)
 __device__ __forceinline__ double i128_to_d(I128 a, int frac_bits) {
-  return ldexp((double)a.hi * 18446744073709551616.0 + (double)a.lo, -frac_bits);
+  const bool neg = a.hi < 0;
+  if (neg) a = I128{0ull - a.lo, (long long)(0ull - (unsigned long long)a.hi - (a.lo ? 1ull : 0ull))};
+  const double m = (double)(unsigned long long)a.hi * 18446744073709551616.0 + (double)a.lo;
+  return ldexp(neg ? -m : m, -frac_bits);
 }
 // Fractional bits of the adjoint sums S1 (e n), S2 (e^2 n), T (g n); with
 // |e|, |g| < 2^14 and |e|^2 < 2^28 every sum fits the 128-bit range.
@@ -511,17 +514,13 @@ k_adj_main(const int32_t* __restrict__ counts, const __grid_constant__ Coef cf,
     for (int b = tid; b < S; b += NT) {
       AdjRow& row = rows[b];
       long long* v = sums + (size_t)b * NC;
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        i128_add(row.s[0], v[k], kFrac1 - s1 + 8 * k);
-        i128_add(row.s[0], v[3 + k], kFrac1 - s1 - 22 + 8 * k);
-        i128_add(row.s[1], v[6 + k], kFrac2 - s2 + 8 * k);
-        i128_add(row.s[1], v[9 + k], kFrac2 - s2 - 22 + 8 * k);
-        if (USE_G) {
-          i128_add(row.s[2], v[13 + k], kFrac3 - s3 + 8 * k);
-          i128_add(row.s[2], v[16 + k], kFrac3 - s3 - 22 + 8 * k);
-        }
-      }
+      // (the digits put together before the shift, which rounds once per flush: with a
+      // shift that drops bits for each digit, S2_b of a map near 1e-3 was 2 to 5 times
+      // less exact, with one for each integer on the fewer blocks of a larger tile
+      // 8e-15 at Nside 64, 40 shells)
+      i128_add(row.s[0], i128_shift(i128_digits(v), kFrac1 - s1 - 22));
+      i128_add(row.s[1], i128_shift(i128_digits(v + 6), kFrac2 - s2 - 22));
+      if (USE_G) i128_add(row.s[2], i128_shift(i128_digits(v + 13), kFrac3 - s3 - 22));
       row.n += v[12];
       for (int k = 0; k < NC; ++k) v[k] = 0;
     }
