@@ -781,20 +781,27 @@ k_adj_main(const int32_t* __restrict__ counts, const __grid_constant__ Coef cf,
     product(0, false, NOR);
     for (int plane = 1; plane < 4 && NOR >> (8 * plane); ++plane) {
       __syncthreads();
-      // (eight loads in flight: row by row these tiles took 1210 us for a map of counts
-      // near 300 that has them everywhere, with the counts loaded evict-first 1140, now 1055)
+      // (eight loads in flight, whole batches of rows without tests: 60 shells of counts
+      // near 300 at Nside 1024, which need this everywhere, take 0.99 ms, 1.08 with a test
+      // per row, 1.01 in the two reads with 64-bit multiply-adds that this form replaced)
       const unsigned sel = 0x0040u + 0x11u * plane;          // byte `plane` of both
-      if (have)
-        for (int b0 = 0; b0 < S; b0 += 8) {
+      if (have) {
+        const char* q = tile_at(tile);
+        for (int b0 = 0; b0 < S; b0 += 8, q += 8 * (size_t)stride) {
           int2 n[8];
+          if (b0 + 8 <= S) {
 #pragma unroll
-          for (int u = 0; u < 8; ++u)
-            n[u] = b0 + u < S ? __ldg(src + (size_t)(b0 + u) * np2) : make_int2(0, 0);
+            for (int u = 0; u < 8; ++u) n[u] = __ldg(row(q, u));
+          } else {
+#pragma unroll
+            for (int u = 0; u < 8; ++u) n[u] = b0 + u < S ? __ldg(row(q, u)) : make_int2(0, 0);
+          }
 #pragma unroll
           for (int u = 0; u < 8; ++u)
             *reinterpret_cast<uint16_t*>(arow + (size_t)(b0 + u) * LDA) =
                 (uint16_t)__byte_perm(n[u].x, n[u].y, sel);
         }
+      }
       __syncthreads();
       product(plane, plane == 3, plane == 3 ? 128u : NOR >> (8 * plane));
     }
