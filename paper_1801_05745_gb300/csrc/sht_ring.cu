@@ -307,6 +307,10 @@ k_ring_transform(const float* __restrict__ map, const float4* __restrict__ T, in
   }
 }
 
+// Complex numbers of shared memory that a ring with at least two threads per H_k
+// (L + 1 <= kRingThreads / 2, that is i <= 127) uses: three buffers of M <= 256
+// and i + 1 roots.
+constexpr int kPartUsed = 3 * 256 + 128;
 // One block per ring: H_k = sum over m = k mod n (0 <= m <= lmax) of
 // G_m e^{i m phi_0} plus, for the negative frequencies, the conjugates of
 // the terms with m = -k mod n (1 <= m <= lmax), for k <= L (H_{n-k} = conj
@@ -319,14 +323,17 @@ k_ring_transform(const float* __restrict__ map, const float4* __restrict__ T, in
 // us at Nside 512, lmax 1535, now 134.)
 __global__ void __launch_bounds__(kRingThreads, 2)
 k_ring_synth(const float4* __restrict__ G, const float4* __restrict__ T, int32_t N,
-             int32_t lmax, int32_t nrings, const int* __restrict__ bad, float* __restrict__ map) {
-  extern __shared__ __align__(16) cxs sh[];
+             int32_t lmax, int32_t nrings, int cap, const int* __restrict__ bad,
+             float* __restrict__ map) {
+  extern __shared__ __align__(16) cxs sh[];                  // [cap]
   const int r = blockIdx.x;
   const RingSpan g = ring_span(N, r);
   const int n = g.n, L = n / 2, N8 = 8 * N;
   const float off = *bad ? NAN : 0.f;                        // added to every pixel
   float* px = map + g.start;
-  __shared__ cxs part_s[kRingThreads];
+  // (free below the last kRingThreads numbers where a ring deals out its terms:
+  // it then uses at most kPartUsed of them, see ring_synth_cap)
+  cxs* part_s = sh + (cap - kRingThreads);
   auto fold = [&](cxs* H, auto term) {                       // H_k, k <= L
     auto some = [&](int k, int p, int np) {                  // part p of np
       cx h{0ull, 0ull};
@@ -427,11 +434,18 @@ k_ring_synth(const float4* __restrict__ G, const float4* __restrict__ T, int32_t
 
 // Shared memory: three buffers of M <= 2N complex numbers and N roots (the
 // belt rings' 4N + 1 complex numbers fit in that).
-static int ring_smem(int nside) { return 7 * nside * (int)sizeof(float4); }
+static int ring_cap(int nside) { return 7 * nside; }
+// The synthesis' partial sums lie at the end of that: a map too small to hold them
+// beside the buffers of the rings that deal out their terms has room for them
+// behind.  (A buffer of their own kept the second block of Nside 1024 off an SM:
+// 0.66 ms at lmax 3071, now 0.59.)
+static int ring_synth_cap(int nside) {
+  return std::max(ring_cap(nside), std::min(ring_cap(nside), kPartUsed) + kRingThreads);
+}
 
 ufc_status launch_ring_transform(ufc_ctx* c, const float* map, const float4* T, int nside, int lmax,
                                  float4* F) {
-  const int smem = ring_smem(nside), nrings = 4 * nside - 1;
+  const int smem = ring_cap(nside) * (int)sizeof(cxs), nrings = 4 * nside - 1;
   UFC_CUDA(c, cudaFuncSetAttribute(k_ring_transform, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    smem));
   {
@@ -444,11 +458,11 @@ ufc_status launch_ring_transform(ufc_ctx* c, const float* map, const float4* T, 
 
 ufc_status launch_ring_synth(ufc_ctx* c, const float4* G, const float4* T, int nside, int lmax,
                              const int* bad, float* map) {
-  const int smem = ring_smem(nside), nrings = 4 * nside - 1;
+  const int cap = ring_synth_cap(nside), smem = cap * (int)sizeof(cxs), nrings = 4 * nside - 1;
   UFC_CUDA(c, cudaFuncSetAttribute(k_ring_synth, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
   {
     ProfScope ps_(c, "k_ring_synth");
-    k_ring_synth<<<nrings, kRingThreads, smem, c->stream>>>(G, T, nside, lmax, nrings, bad, map);
+    k_ring_synth<<<nrings, kRingThreads, smem, c->stream>>>(G, T, nside, lmax, nrings, cap, bad, map);
   }
   UFC_CUDA(c, cudaGetLastError());
   return UFC_OK;
