@@ -920,7 +920,15 @@ __device__ __forceinline__ void moments_block(const float* __restrict__ kappa, i
   const float mh = mean.x, ml = mean.y;
   const u64 nmh = x2_pack(-mh, -mh), nml = x2_pack(-ml, -ml);
   dfx a2{0ull, 0ull}, a3{0ull, 0ull}, a4{0ull, 0ull};
+  // (the running sums are renormalised every four additions: low parts that grow
+  // over hundreds lose bits of their own, 1e-11 of mu4 of a two-valued map of Nside
+  // 4096, and each addition renormalised takes 5% longer)
   auto acc = [](dfx& a, dfx x) { a = dfx_add_raw(a, x); };
+  auto norm_all = [&]() {
+    a2 = dfx_norm(a2.h, a2.l);
+    a3 = dfx_norm(a3.h, a3.l);
+    a4 = dfx_norm(a4.h, a4.l);
+  };
   auto add_pair = [&](float k0, float k1, bool both) {
     // d = (k - mh) - ml: two exact sums, renormalised
     const u64 k = x2_pack(k0, k1);
@@ -947,18 +955,20 @@ __device__ __forceinline__ void moments_block(const float* __restrict__ kappa, i
     const int ng = npix >> 2;
     float4 v = p < ng ? k4[p] : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 1
-    for (; p < ng; p += step) {
+    for (int it = 0; p < ng; p += step, ++it) {
       const float4 w = v;
       if (p + step < ng) v = k4[p + step];
       add_pair(w.x, w.y, true);
       add_pair(w.z, w.w, true);
+      if (it & 1) norm_all();
     }
   } else {
 #pragma unroll 1
-    for (; p < npix; p += 2 * step) {
+    for (int it = 0; p < npix; p += 2 * step, ++it) {
       const bool both = p < npix - step;
       const float k0 = kappa[p], k1 = both ? kappa[p + step] : k0;
       add_pair(k0, k1, both);
+      if ((it & 3) == 3) norm_all();
     }
   }
   // Over the lanes in double-float, over the halves and warps in FP64 by the lanes of
