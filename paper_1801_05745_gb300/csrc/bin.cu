@@ -43,7 +43,6 @@ constexpr int kFastThreads = 512;
 
 struct KeyOut {
   int32_t* keys;               // KEYS
-  int32_t* counts;             // DIRECT
   uint32_t* dense;             // DENSE
   unsigned long long* dense_count;
   uint32_t* hist;              // DENSE: global bucket histogram
@@ -53,7 +52,6 @@ struct KeyOut {
   int32_t shell0;              // DENSE: first shell of the call's window; buckets
                                // count blocks from shell0 * nblk
   int32_t smem_hist;           // 1: histogram in shared memory
-  int64_t ncell;               // cells of the count map (checked builds' bound)
 };
 
 struct Queues {
@@ -1673,8 +1671,6 @@ ufc_status run_keys_pipeline(ufc_ctx* c, int mode_req, const float* const* xyz,
   KeyOut o;
   std::memset(&o, 0, sizeof o);
   o.keys = keys;
-  o.counts = counts;
-  o.ncell = (int64_t)nshell * npix;
   o.dense_count = &qs.cnt->dense;
   int smem = 0;
   if (plan.mode == kModeDense) {

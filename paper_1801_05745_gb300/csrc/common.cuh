@@ -140,7 +140,6 @@ __host__ __device__ inline uint64_t qpack(int box, int img, int64_t p) {
   return (uint64_t(box) << 60) | (uint64_t(img) << 47) | uint64_t(p);
 }
 __host__ __device__ inline int qbox(uint64_t e) { return int(e >> 60); }
-__host__ __device__ inline int qimg(uint64_t e) { return int((e >> 47) & 0x1FFF); }
 __host__ __device__ inline int64_t qidx(uint64_t e) { return int64_t(e & ((1ull << 47) - 1)); }
 
 }  // namespace ufc

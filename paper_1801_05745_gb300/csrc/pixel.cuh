@@ -285,21 +285,6 @@ __device__ __forceinline__ int32_t pixel_fast(int32_t N, const Bands& bd, float 
   return kKeyUndecided;
 }
 
-// Shell of r2 within edges [lo, hi] by the fast stage: returns the shell, -1
-// for certainly outside, or -2 for undecided.  Bands are ordered and
-// disjoint: lo2[e] <= hi2[e] <= lo2[e+1].
-__device__ __forceinline__ int32_t shell_fast(const float* lo2, const float* hi2,
-                                              int32_t lo, int32_t hi, float r2) {
-  if (r2 < lo2[lo]) return -1;                 // certainly below chi_lo
-  int32_t a = lo, b = hi + 1;                  // lo2[a] <= r2 < lo2[b] (b = hi+1: +inf)
-  while (b - a > 1) {
-    int32_t m = (a + b) >> 1;
-    if (r2 < lo2[m]) b = m; else a = m;
-  }
-  if (r2 < hi2[a]) return -2;                  // inside edge a's band
-  return (a < hi) ? a : -1;
-}
-
 // ======================= refine stage (double-float) ========================
 // Unevaluated sums hi + lo of two FP32 numbers (Dekker, Knuth).  Every
 // product and sum uses the _rn intrinsics so that no step is contracted.

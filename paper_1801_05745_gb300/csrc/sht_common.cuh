@@ -14,7 +14,6 @@ struct Ring {
   int64_t start;   // first pixel
   int32_t n;       // pixels
   double z, s;     // cos and sin of the colatitude
-  double phi0_pi;  // azimuth of the first pixel / pi
 };
 
 // Ring r (0-based, north to south) of the RING scheme.
@@ -28,13 +27,11 @@ __host__ __device__ inline Ring ring_geom(int32_t N, int32_t r) {
     const double t = (double)((int64_t)i * i) / (3.0 * (double)((int64_t)N * N));
     g.z = 1.0 - t;
     g.s = sqrt(t * (2.0 - t));
-    g.phi0_pi = 1.0 / (4.0 * i);
   } else if (i <= 3 * N) {
     g.n = 4 * N;
     g.start = 2ll * N * (N - 1) + 4ll * N * (i - N);
     g.z = 4.0 / 3.0 - 2.0 * (double)i / (3.0 * (double)N);
     g.s = sqrt((1.0 - g.z) * (1.0 + g.z));
-    g.phi0_pi = ((i - N + 1) % 2) / (4.0 * N);
   } else {
     const int32_t k = 4 * N - i;
     g.n = 4 * k;
@@ -42,7 +39,6 @@ __host__ __device__ inline Ring ring_geom(int32_t N, int32_t r) {
     const double t = (double)((int64_t)k * k) / (3.0 * (double)((int64_t)N * N));
     g.z = -(1.0 - t);
     g.s = sqrt(t * (2.0 - t));
-    g.phi0_pi = 1.0 / (4.0 * k);
   }
   return g;
 }
@@ -64,14 +60,6 @@ __device__ __forceinline__ dfl df_norm(float h, float l) {
   const float s = __fadd_rn(h, l);
   return {s, __fadd_rn(l, __fsub_rn(h, s))};
 }
-// a * b: the exact product of the high parts plus the cross terms
-__device__ __forceinline__ dfl df_mul(dfl a, dfl b) {
-  const float p = __fmul_rn(a.h, b.h);
-  float e = __fmaf_rn(a.h, b.h, -p);
-  e = __fmaf_rn(a.h, b.l, e);
-  e = __fmaf_rn(a.l, b.h, e);
-  return df_norm(p, e);
-}
 // a + b (two-sum of the high parts)
 __device__ __forceinline__ dfl df_add(dfl a, dfl b) {
   const float s = __fadd_rn(a.h, b.h);
@@ -79,35 +67,16 @@ __device__ __forceinline__ dfl df_add(dfl a, dfl b) {
   const float err = __fadd_rn(__fsub_rn(a.h, __fsub_rn(s, bb)), __fsub_rn(b.h, bb));
   return df_norm(s, __fadd_rn(err, __fadd_rn(a.l, b.l)));
 }
-__device__ __forceinline__ dfl df_neg(dfl a) { return {-a.h, -a.l}; }
 __device__ __forceinline__ dfl df_scale(dfl a, float p2) { return {a.h * p2, a.l * p2}; }  // exact
-// acc += a * b, the low part left unnormalised (renormalised by df_add)
-__device__ __forceinline__ void df_mac(dfl& acc, dfl a, dfl b) {
-  const float p = __fmul_rn(a.h, b.h);
-  const float pe = __fmaf_rn(a.h, b.h, -p);
-  const float s = __fadd_rn(acc.h, p);
-  const float bb = __fsub_rn(s, acc.h);
-  const float se = __fadd_rn(__fsub_rn(acc.h, __fsub_rn(s, bb)), __fsub_rn(p, bb));
-  const float cross = __fmaf_rn(a.h, b.l, __fmul_rn(a.l, b.h));
-  acc.h = s;
-  acc.l = __fadd_rn(acc.l, __fadd_rn(se, __fadd_rn(pe, cross)));
-}
 
 // Complex numbers with double-float parts, (re.h, re.l, im.h, im.l) in a float4.
 __device__ __forceinline__ float4 cdf_pack(dfl re, dfl im) { return make_float4(re.h, re.l, im.h, im.l); }
-// a * b
-__device__ __forceinline__ float4 cdf_mul(float4 a, float4 b) {
-  const dfl ar{a.x, a.y}, ai{a.z, a.w}, br{b.x, b.y}, bi{b.z, b.w};
-  return cdf_pack(df_add(df_mul(ar, br), df_neg(df_mul(ai, bi))),
-                  df_add(df_mul(ar, bi), df_mul(ai, br)));
-}
 __device__ __forceinline__ float4 cdf_add(float4 a, float4 b) {
   return cdf_pack(df_add(dfl{a.x, a.y}, dfl{b.x, b.y}), df_add(dfl{a.z, a.w}, dfl{b.z, b.w}));
 }
 __device__ __forceinline__ float4 cdf_sub(float4 a, float4 b) {
   return cdf_pack(df_add(dfl{a.x, a.y}, dfl{-b.x, -b.y}), df_add(dfl{a.z, a.w}, dfl{-b.z, -b.w}));
 }
-__device__ __forceinline__ float4 cdf_conj(float4 a) { return make_float4(a.x, a.y, -a.z, -a.w); }
 
 __device__ __forceinline__ dfx dfx_set(dfl a, dfl b) { return {x2_pack(a.h, b.h), x2_pack(a.l, b.l)}; }
 

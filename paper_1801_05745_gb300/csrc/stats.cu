@@ -54,10 +54,6 @@ __device__ __forceinline__ double warp_sum_d(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xFFFFFFFFu, v, o);
   return v;
 }
-__device__ __forceinline__ long long warp_sum_ll(long long v) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xFFFFFFFFu, v, o);
-  return v;
-}
 // Sum of v[0], v[stride], ..., v[(n - 1) stride] by one warp in a fixed
 // order: lane l adds elements l, l + 32, ... in turn, then a butterfly; every
 // lane ends with the same value (each pairwise sum is formed by both lanes).
@@ -1296,7 +1292,7 @@ __host__ __device__ inline size_t batch_coef_stride(int S) {
 }
 struct BatchArgs {
   const char* coef;         // [nreal] BatchCoef, batch_coef_stride(S) apart
-  int32_t nreal, S, npix;
+  int32_t S, npix;
   int32_t* counts;          // [nreal][S][npix]
   float* kappa;             // [nreal][npix]
   double* ksum;             // [nreal][gk]
@@ -2036,7 +2032,6 @@ ufc_status run_batch_stages(ufc_ctx* c, int nreal, int nbox, const float* const*
     if (s) return s;
     BatchArgs ba;
     ba.coef = desc + sp.coef + batch_coef_stride(S) * r0;
-    ba.nreal = nr;
     ba.S = S;
     ba.npix = npix;
     ba.counts = reinterpret_cast<int32_t*>(maps + sp.maps) + (size_t)r0 * S * npix;
