@@ -190,12 +190,49 @@ def cpu_baseline(w, parts_host, counts_host, A, C, dAC, seconds_budget=20.0):
     }
 
 
+# --------------------------------------------------- Legendre roofline ------
+def legendre_ops(nside: int, lmax: int) -> float:
+    """FP32 operations of k_legendre as it runs: warps of 64 ring pairs, 18 per
+    degree and pair for the recurrence from l = m on (none for the orders at which
+    the warp's most equatorial pair stays below 2^-128 up to lmax), and 23 for the
+    sums (two products of 4 or two multiply-adds of 12 over two groups of pairs,
+    and 7 of the lanes' sums) from the degree at which that pair passes 2^-120.
+    The sizes of lambda_lm come from the phase integral that the kernel uses."""
+    npairs = 2 * nside
+    p = np.arange(min(64, npairs) - 1, npairs, 64)      # the last pair of each warp
+    ring = p + 1
+    t = ring * ring / (3.0 * nside * nside)
+    z = np.where(ring < nside, 1.0 - t, 4.0 / 3.0 - 2.0 * ring / (3.0 * nside))
+    s = np.sqrt((1.0 - z) * (1.0 + z))
+    m = np.arange(lmax + 1)[:, None]
+
+    def below(l, bits):
+        """|lambda_lm| < 2^-(bits - 2) on the ring for every degree up to l"""
+        L = l + 0.5
+        with np.errstate(all="ignore"):
+            D = np.sqrt((m - L * s) * (m + L * s))
+            R = np.sqrt((L - m) * (L + m))
+            S = m * np.log((m * z + D) / (s * R)) - L * np.log((L * z + D) / R)
+            return (m > L * s) & (S > bits * np.log(2.0))
+
+    alive = ~below(np.full((lmax + 1, len(p)), lmax), 130)
+    first = np.broadcast_to(m, alive.shape).copy()      # by bisection in l
+    last = np.full_like(first, lmax)
+    while (first < last).any():
+        mid = (first + last) // 2
+        low = below(mid, 122)
+        first, last = np.where(low & (first < last), mid + 1, first), np.where(low, last, mid)
+    pairs = min(64, npairs)
+    return float((alive * pairs * (18.0 * (lmax + 1 - m) + 23.0 * (lmax + 1 - first))).sum())
+
+
 # ------------------------------------------------- batched vs serial leg ----
 def batched_leg(ctx, api, synth, dev, n_real: int, n_side: int, nbuf: int = 8,
                 nside: int | None = None):
     """Covariance of n_real realisations of the nested Nside-512 map, each box
-    holding Poisson(f n_side^3) particles, f ~ U(0.5, 1.5): one graph-captured
-    ufc_batched_stats call against the same maps one at a time through
+    holding Poisson(f n_side^3) particles, f ~ U(0.5, 1.5): one ufc_batched_stats
+    call (small maps stage by stage over all realisations, larger ones as one
+    captured graph) against the same maps one at a time through
     ufc_bin + ufc_kappa_stats + ufc_stats_vector + ufc_welford_update.
 
     Positions come from nbuf seeded buffers per box, 1.5 n_side^3 (+6 sigma)
@@ -748,14 +785,11 @@ def main():
                       "maps_per_s": 1e3 / ms_cl,
                       "kernels_ms_per_map": {k: round(v[0] / 3, 3) for k, v in cprof.items()},
                       "k_legendre_fp64_equiv_tflops": fp64 / (leg[0] / 3 * 1e-3) / 1e12 if leg[0] else None}
-        # k_legendre against the FP32 pipe: the double-float code's FP32
-        # operations per (l, m, ring pair) for l >= m + 2, as written (the
-        # recurrence step 18, two products of 4 or two multiply-adds of 12 into
-        # the sums over two groups of pairs, 7 of the lanes' sums), pairs left
-        # out as negligible included, against 128 FP32 lanes per SM at the
-        # maximum SM clock sampled during the main timed region
+        # k_legendre against the FP32 pipe: the FP32 operations of the work it
+        # does (legendre_ops) against 128 FP32 lanes per SM at the maximum SM
+        # clock sampled during the main timed region
         if leg[0]:
-            ops = 41.0 * npairs * (nalm - (2 * lmax + 1))
+            ops = legendre_ops(w.nside, lmax)
             nsm = torch.cuda.get_device_properties(dev).multi_processor_count
             mhz = float(clk.get("sm_max_mhz") or 2070.0) if isinstance(clk, dict) else 2070.0
             peak_alu = nsm * 128 * mhz * 1e6
