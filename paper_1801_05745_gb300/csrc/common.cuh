@@ -90,11 +90,13 @@ struct BinCounters {
   unsigned long long q2;        // entries in queue 2
   unsigned long long dense;     // keys written by the compaction stage
   unsigned long long ntiles;    // tiles of the second scatter pass
-  unsigned long long range;     // adjoint inputs outside the fixed-point range
   unsigned long long ovf;       // images marked for the exact pass (queue 1 was full)
-  // bounded device waits that ran out: last, so that a binning call's reset
-  // (everything before it) keeps it until ufc_synchronize reports it
+  // bounded device waits that ran out: behind what a binning call's reset
+  // clears, so that it is kept until ufc_synchronize reports it
   unsigned long long timeouts;
+  // adjoint inputs outside the fixed-point range, cleared by the adjoint's own
+  // reduction: outside the reset too, which may run on another stream meanwhile
+  unsigned long long range;
 };
 
 // ---- index checks of checked builds ----------------------------------------

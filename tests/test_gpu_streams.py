@@ -236,3 +236,28 @@ def test_batched_call_overlaps_with_binning_and_kappa(orc):
     for a, b in got:
         for u, v in zip(a, b):
             assert torch.equal(u, v)
+
+
+def test_adjoint_range_report_beside_binning(orc):
+    """A cotangent outside the adjoint's fixed-point range is reported while binning
+    calls, which clear their counters, run on another stream."""
+    api, ctx = api_ctx()
+    nside, S = 64, 3
+    chi, xs, boxes, _, _ = _batch(api, orc, 1, 2_000, 16, 6)
+    counts = torch.ones((S, 12 * nside * nside), dtype=torch.int32, device="cuda")
+    counts[1, ::3] = 2
+    g = torch.zeros(12 * nside * nside, dtype=torch.float32, device="cuda")
+    g[7] = 3.0e4
+    A, dA, dC = np.linspace(0.01, 0.02, S), np.zeros((5, S)), np.zeros(5)
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    torch.cuda.synchronize()
+    for _ in range(20):
+        with torch.cuda.stream(streams[0]):
+            for _ in range(30):
+                ctx.bin(xs[0], boxes[0], chi, 16)
+        with torch.cuda.stream(streams[1]):
+            with pytest.raises(api.UfcError, match="fixed-point range"):
+                ctx.kappa_backward(counts, A, 0.04, dA, dC, 1.0, 0.0, g)
+    torch.cuda.synchronize()
+    g[7] = 1.0
+    ctx.kappa_backward(counts, A, 0.04, dA, dC, 1.0, 0.0, g)       # and it was cleared
