@@ -28,6 +28,13 @@
  *  - Every call returns UFC_OK or an error status; ufc_last_error() then
  *    holds a one-line message.  Invalid arguments never reach the GPU.
  *  - A context is not thread-safe: use one per host thread.
+ *  - Calls of one context share its workspace within four groups: binning and
+ *    keys; kappa maps, moments, PDFs and adjoints; harmonic transforms; and
+ *    ufc_batched_stats (which with UFC_BATCH_LAUNCHES, large maps or periodic
+ *    images uses the first two groups' as well).  Calls of one group have to be
+ *    ordered on the device when they are enqueued on different streams.  Calls
+ *    of different groups may overlap, and ufc_kappa_stats_noalloc (but for other
+ *    calls of itself), ufc_stats_vector and ufc_welford_* with any call.
  */
 #ifndef UFALCON_H
 #define UFALCON_H
@@ -105,8 +112,8 @@ ufc_status ufc_destroy(ufc_ctx *ctx);
 /* Sets the CUDA stream (a cudaStream_t, NULL = legacy default stream). */
 ufc_status ufc_set_stream(ufc_ctx *ctx, void *stream);
 /* Waits for all work enqueued by this context; reports device-side errors:
- * UFC_ERR_TIMEOUT when a bounded wait of the fast binning stage (on its
- * particle copies) ran out since the last report, in which case that
+ * UFC_ERR_TIMEOUT when a bounded wait of the binning's scatter passes (on
+ * their tiles' copies) ran out since the last report, in which case that
  * binning call's counts are incomplete; else UFC_ERR_INTERNAL when an index
  * test failed since the last report (checked builds, and
  * ufc_check_selftest).  The context stays usable. */
@@ -353,7 +360,7 @@ ufc_status ufc_kappa_stats_noalloc(ufc_ctx *ctx, const int32_t *counts_dev,
  * once more per further byte).  dA [5][nshell], dC [5] come from
  * ufc_kappa_coeffs (or ufc_delta_coeffs).  grad_theta [5] (host) receives
  * dL/dtheta; G [nshell] and H (host) may be NULL.  The per-shell sums are
- * exact 128-bit fixed-point sums of the map quantised to 44 bits relative to
+ * exact 128-bit fixed-point sums of the map quantised to 43 bits relative to
  * its maximum (|kappa_p| and |g_p| below 2^14, else UFC_ERR_UNSUPPORTED).
  * Synchronises. */
 ufc_status ufc_kappa_backward(ufc_ctx *ctx, const int32_t *counts_dev,

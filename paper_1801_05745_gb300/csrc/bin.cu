@@ -430,7 +430,7 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
 
 // Self-test of the bounded wait: an mbarrier that expects one arrival which
 // never comes; the wait gives up after `limit` polls and reports it like the
-// fast stage does (the kernel then returns normally).
+// scatter passes do (the kernel then returns normally).
 __global__ void k_wait_selftest(long long limit, unsigned long long* timeouts) {
   __shared__ __align__(8) uint64_t bar;
   if (threadIdx.x != 0) return;
@@ -475,7 +475,7 @@ __device__ __noinline__ int32_t key_exact_slow(const ShellTable& st, int32_t lo,
 // ufc_bin_host).
 //
 // Bound by instruction issue: about 6.3 warp instructions per particle in a box half of whose
-// particles are keyed, three quarters of the issue slots (ALU pipe 58%, FMA 28%, DRAM 25%).
+// particles are keyed, 82% of the issue slots (ALU pipe 56%, FMA 28%, DRAM 29%).
 // Two boxes of 512^3 particles at Nside 512 take 1.55 ms; 1.61 when the block shared bulk
 // copies of 3840 particles behind mbarriers (ring bookkeeping per chunk), 1.80 with circular
 // lists, range tests on the shell after the table and the periodic path's image loop as well.

@@ -19,10 +19,10 @@
 // bytes each in shared memory.
 //
 // What bounds them: the FP32 pipe and the shared-memory latency of 2 blocks of
-// 16 warps per SM.  The 4095 rings of Nside 1024 take 0.57 ms forward (3.93 ms
+// 16 warps per SM.  The 4095 rings of Nside 1024 take 0.49 ms forward (3.93 ms
 // with direct length-i sums and full-length complex FFTs of the belt's real
-// rings), the 2047 of Nside 512 0.38 ms back (0.50 ms; its column-wise reads of
-// G, 16 bytes per row, are what is left there).
+// rings) and 0.59 back at lmax 3071, the 2047 of Nside 512 0.135 ms back at lmax
+// 1535 (its column-wise reads of G, 16 bytes per row, are what is left there).
 #include <algorithm>
 #include <cmath>
 
@@ -320,7 +320,7 @@ constexpr int kPartUsed = 3 * 256 + 128;
 // as many threads as a short ring leaves free, each adding its own in increasing
 // m, and the parts added in order.  (One thread per H_k left the rings next to the
 // poles, 3 to 9 sums of hundreds of dependent loads, as the tail of the kernel: 350
-// us at Nside 512, lmax 1535, now 134.)
+// us at Nside 512, lmax 1535, now 135.)
 __global__ void __launch_bounds__(kRingThreads, 2)
 k_ring_synth(const float4* __restrict__ G, const float4* __restrict__ T, int32_t N,
              int32_t lmax, int32_t nrings, int cap, const int* __restrict__ bad,

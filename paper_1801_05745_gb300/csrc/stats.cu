@@ -392,10 +392,12 @@ k_kappa_finish(const double* __restrict__ part, float ch, float cl, int npix,
 // pixels per thread, a few blocks per SM so that one block's arithmetic overlaps
 // another's loads.
 //
-// Bound by the latency that is left: 60 shells at Nside 1024 take 750 us for 3.0 GB
-// read once (4.0 TB/s, 60% of the copy rate; 53% issue, FMA pipe 49%), with waits
-// for loads and the barriers around phase 2; 140 shells at Nside 512 554 us (3.2
-// TB/s).  Two reads with 64-bit integer multiply-adds took 1080 and 1370 us.  A
+// Bound by the latency that is left: 60 shells at Nside 1024 take 730 us for 3.0 GB
+// read once (4.1 TB/s, 61% of the copy rate; 55% issue, DRAM 50%), with waits for
+// loads and the barriers around phase 2; 140 shells at Nside 512 501 us (3.5 TB/s).
+// Two reads with 64-bit integer multiply-adds took 1050 and 1330 us.  Counts of 256
+// and more cost a tile a second read and product: 919 us for the counts of 2 x 1024^3
+// binned particles (1050 in the two reads), 988 where every tile has them (1005).  A
 // batch of 8 shells in flight while 8 are added (80 registers, three blocks per
 // SM) against none: 930; 4 shells: 765; two blocks with 16: 830.  256-pixel tiles for
 // every shell count: 780.  Phase 2's pixels split over idle warps: 875 (its sums take
@@ -410,9 +412,10 @@ k_kappa_finish(const double* __restrict__ part, float ch, float cl, int npix,
 // Quantisation: each quantity as two integers (quant2: 43 bits relative to the
 // scale) with a power-of-two scale from the block's running maximum over the
 // tiles it has seen; when a tile raises a maximum, the sums so far are first
-// flushed at the old scale into the block's 128-bit fixed-point rows, which
-// take every flush at its own scale exactly.  Every pixel is therefore
-// quantised at least as finely as a single scale from the global maxima would.
+// flushed at the old scale into the block's 128-bit fixed-point rows, each flush
+// exactly or, where the map is so small that the rows end before its digits,
+// rounded once to nearest.  Every pixel is therefore quantised at least as finely
+// as a single scale from the global maxima would.
 //
 // Phase 2: the per-shell sums sum_p q_p n_bp are a matrix product, shells x
 // pixels times pixels x quantities, on the tensor cores: the integers as signed
@@ -970,7 +973,7 @@ __device__ __forceinline__ void moments_block(const float* __restrict__ kappa, i
   // Over the lanes in double-float, over the halves and warps in FP64 by the lanes of
   // one warp, in fixed orders.  (FP64 kept its pipe 79% busy in a batch of small maps when
   // it added the lanes, 74% when every warp converted its sums: 150 maps of Nside 64 took
-  // 174 us, then 119, now 70.)
+  // 174 us, then 119, now 68.)
   const int w = threadIdx.x >> 5, ln = threadIdx.x & 31;
   float4* part = reinterpret_cast<float4*>(red);       // [3][kMT / 32]
   dfx q[3] = {a2, a3, a4};
@@ -1035,7 +1038,8 @@ __device__ __forceinline__ void moments_final_block(const double* ksum_part, int
 // bounds the pass is the latency of a pixel's chain (load, shared-memory histogram, double-float
 // sums): with 2 blocks per SM and one pixel at a time it took 200 us for the
 // 12.6 M pixels of Nside 1024, with four scalar loads in flight 59, with four
-// pixels per load and the next load in flight 51 (6 blocks per SM 53, 8 55).
+// pixels per load and the next load in flight 51 (6 blocks per SM 53, 8 55), 55 with the
+// sums renormalised every four additions.
 static int moments_grid(int num_sms, int npix) {
   return std::min(4 * num_sms, (npix + 4 * kMT - 1) / (4 * kMT));
 }

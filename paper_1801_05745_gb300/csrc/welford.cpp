@@ -1,6 +1,7 @@
 // Welford update and Chan merge of covariance states on host memory (Eq. 10,
 // the realisation-sharded path): the same formulas, in the same order, as
-// k_welford_update and k_welford_merge of the device library.
+// k_welford_update and k_welford_merge of the device library (which forms
+// delta (1 / n) where this divides).
 #include <cmath>
 #include <cstdint>
 #include <vector>
