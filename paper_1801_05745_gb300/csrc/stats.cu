@@ -1200,9 +1200,10 @@ k_welford_mean(const double* __restrict__ v, int nvec, int d, double* __restrict
 }
 
 // One vector into a state of up to kWfOne components (a map at a time) by one
-// cluster in one launch: the operations of the two kernels above.  A second launch
-// costs such a caller more than the arithmetic on 8 SMs: bin, kappa, vector and
-// update of a map of Nside 64 took 128 us before, 132 with two launches.
+// cluster in one launch: the operations of the two kernels above.  Such a caller is
+// bound by the host, and a second launch costs it more than the arithmetic on 8 SMs:
+// bin, kappa, vector and update of a map of Nside 64 take 104 us with one launch,
+// 110 with two (medians of 12 processes each).
 constexpr int kWfOne = 256, kWfOneThreads = 512;
 __global__ void __cluster_dims__(kWfCluster, 1, 1) __launch_bounds__(kWfOneThreads)
 k_welford_one(const double* __restrict__ v, int d, double* __restrict__ st) {
